@@ -244,7 +244,7 @@ int bvf_run_acoustic(bvf_ctx *ctx, int n_steps, const bvf_capture *cap, void *st
  * owns an x-y tile 32 voxels wide and stress_rows (stress kernel) or
  * velocity_rows (velocity kernel) rows high, 4, 8 or 16, and marches kchunk
  * z-planes.  0 selects the default: 8 rows for the stress and 16 for the
- * velocity kernel, and a z-chunk that fills the GPU about six times.  Heights
+ * velocity kernel, and z-chunks chosen per kernel from the grid's size.  Heights
  * other than 8 apply to contexts with two SLS mechanisms (n_sls = 2, the
  * method's); other contexts use 8.  bvf_set_tile keeps the choice for later
  * bvf_run_acoustic calls; bvf_get_tile reports the heights and the stress

@@ -38,6 +38,7 @@
 // nx % 16 != 0) and L <= 2.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <type_traits>
 
@@ -188,14 +189,6 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const bool live = i < nx && j < ny;              // nx is even: i + 1 < nx as well
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
-    if (tid == 0) {
-        tma::mbar_init(&bars[0], 1);
-        tma::mbar_init(&bars[1], 1);
-        tma::mbar_init_fence();
-        *s_abort = -1;
-    }
-    __syncthreads();
-
     // ring slots: A holds plane pl in slot (pl-k0)%2, B in (pl-k0+2)%6,
     // C in (pl-k0+1)%6, the index in (pl-k0)%3
     constexpr unsigned A_BYTES = Lay::SA * Lay::ES, B_BYTES = Lay::SB * Lay::ES;
@@ -218,14 +211,26 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
         tma::load3d(smb + Lay::off_i + slot * IT_SLOT, &tm.idx, x0, y0, pl, bar);
     };
 
+    // the index does not change during a run, so its copies go out before the
+    // wait for the previous kernel of the stream
     if (tid == 0) {
+        tma::mbar_init(&bars[0], 1);
+        tma::mbar_init(&bars[1], 1);
+        tma::mbar_init_fence();
+        *s_abort = -1;
         if (REUSE) tma::fence_async_smem();
         tma::mbar_expect_tx(&bars[0], A_BYTES + 4 * B_BYTES + 4 * C_BYTES + 2 * IT);
+        ldI(k0, 0, &bars[0]);
+        ldI(k0 + 1, 1, &bars[0]);
+    }
+    if (!REUSE) {
+        tma::pdl_wait();
+        tma::pdl_launch_next();
+    }
+    if (tid == 0) {
         ldA(k0, 0, &bars[0]);
         for (int d = 0; d < 4; ++d) ldB(k0 - 2 + d, d, &bars[0]);
         for (int d = 0; d < 4; ++d) ldC(k0 - 1 + d, d, &bars[0]);
-        ldI(k0, 0, &bars[0]);
-        ldI(k0 + 1, 1, &bars[0]);
     }
 
     const st::Dx ix = st::make_dx(p.inv_dx);
@@ -464,7 +469,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
 {
     using Lay = StressLayout<L, T, TH>;
     using Bx = Box<T, TH>;
-    constexpr int IT = Idx<TH>::BYTES, IT_SLOT = Idx<TH>::SLOT, NT = TX * TH;
+    constexpr int IT = Idx<TH>::BYTES, IT_SLOT = Idx<TH>::SLOT;
     constexpr int VW = Bx::BW, VT = Bx::VT;
     const T *smt = reinterpret_cast<const T *>(smb);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smb + Lay::off_bar);
@@ -477,31 +482,44 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const bool live = i < nx && j < ny;
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
-    for (int m = tid; m < p.n_mat; m += NT) s_lut[m] = st::make_stress_coef(p.lut[m], p.Lf);
+    constexpr unsigned VT_BYTES = VT * Lay::ES;
+    auto oV = [&](int pl) { return Lay::off_v + ((pl - k0 + 2) % Lay::RV) * 3 * (int)VT_BYTES; };
+    auto oI = [&](int pl) { return Lay::off_i + ((pl - k0) % Lay::RI) * IT_SLOT; };   // bytes
+    // test hook: plane kk's copies are armed but not issued
+    auto held = [&](int kk) { return p.hold == 2 && kk == p.hold_plane + 2; };
+    // what plane kk adds to the rings: velocities of kk + 2, the index of kk + 1
+    auto issue = [&](int kk, uint64_t *bar) {
+        tma::mbar_expect_tx(bar, 3 * VT_BYTES + IT);
+        if (held(kk)) return;
+        for (int a = 0; a < 3; ++a)
+            tma::load3d(smb + oV(kk + 2) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, kk + 2, bar);
+        tma::load3d(smb + oI(kk + 1), &tm.idx, x0, y0, kk + 1, bar);
+    };
+    // the material table and the index do not change during a run, so their
+    // copies go out before the wait for the previous kernel of the stream
+    const unsigned lut_bytes = (unsigned)p.n_mat * (unsigned)sizeof(st::StressCoef);
     if (tid == 0) {
         for (int b = 0; b < 3; ++b) tma::mbar_init(&bars[b], 1);
         tma::mbar_init_fence();
         *s_abort = -1;
-    }
-    __syncthreads();
-
-    constexpr unsigned VT_BYTES = VT * Lay::ES;
-    auto oV = [&](int pl) { return Lay::off_v + ((pl - k0 + 2) % Lay::RV) * 3 * (int)VT_BYTES; };
-    auto oI = [&](int pl) { return Lay::off_i + ((pl - k0) % Lay::RI) * IT_SLOT; };   // bytes
-    auto issue = [&](int kk, uint64_t *bar, bool first) {
-        const unsigned nv = first ? 5 : 1;
-        tma::mbar_expect_tx(bar, nv * 3 * VT_BYTES + (first ? 2 : 1) * IT);
-        if (p.hold == 2 && kk == p.hold_plane + 2) return;    // test hook: armed, none issued
-        for (int pl = first ? kk - 2 : kk + 2; pl <= kk + 2; ++pl)
-            for (int a = 0; a < 3; ++a)
-                tma::load3d(smb + oV(pl) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, pl, bar);
-        for (int pl = first ? kk : kk + 1; pl <= kk + 1; ++pl)
-            tma::load3d(smb + oI(pl), &tm.idx, x0, y0, pl, bar);
-    };
-    if (tid == 0) {
         if (REUSE) tma::fence_async_smem();
-        issue(k0, &bars[0], true);
-        if (k0 + 1 < k1) issue(k0 + 1, &bars[1], false);
+        tma::mbar_expect_tx(&bars[0], 15 * VT_BYTES + 2 * IT + lut_bytes);
+        if (!held(k0)) {
+            tma::load_bulk(s_lut, p.slut, lut_bytes, &bars[0]);
+            tma::load3d(smb + oI(k0), &tm.idx, x0, y0, k0, &bars[0]);
+            tma::load3d(smb + oI(k0 + 1), &tm.idx, x0, y0, k0 + 1, &bars[0]);
+        }
+    }
+    if (!REUSE) {
+        tma::pdl_wait();
+        tma::pdl_launch_next();
+    }
+    if (tid == 0) {
+        for (int pl = k0 - 2; pl <= k0 + 2 && !held(k0); ++pl)
+            for (int a = 0; a < 3; ++a)
+                tma::load3d(smb + oV(pl) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, pl,
+                            &bars[0]);
+        if (k0 + 1 < k1) issue(k0 + 1, &bars[1]);
     }
 
     const st::Dx ix = st::make_dx(p.inv_dx);
@@ -575,7 +593,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
         if (*s_abort >= 0) break;        // a wait of the previous plane ran out
         if (tid == 0 && k + 2 < k1) {
             tma::fence_async_smem();
-            issue(k + 2, &bars[(it + 2) % 3], false);
+            issue(k + 2, &bars[(it + 2) % 3]);
         }
         if (PREFETCH) prefetch_plane(k + 1);
         const int q = k * (nx * ny) + j * nx + i;
@@ -794,7 +812,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
     using T = __half;
     using Lay = StressLayout<L, T, TH>;
     using Bx = Box<T, TH>;
-    constexpr int IT = Idx<TH>::BYTES, IT_SLOT = Idx<TH>::SLOT, NT = PX * TH;
+    constexpr int IT = Idx<TH>::BYTES, IT_SLOT = Idx<TH>::SLOT;
     constexpr int VW = Bx::BW, VT = Bx::VT;
     const T *smt = reinterpret_cast<const T *>(smb);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smb + Lay::off_bar);
@@ -807,31 +825,44 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const bool live = i < nx && j < ny;                // nx is even: i + 1 < nx as well
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
-    for (int m = tid; m < p.n_mat; m += NT) s_lut[m] = st::make_stress_coef(p.lut[m], p.Lf);
+    constexpr unsigned VT_BYTES = VT * Lay::ES;
+    auto oV = [&](int pl) { return Lay::off_v + ((pl - k0 + 2) % Lay::RV) * 3 * (int)VT_BYTES; };
+    auto oI = [&](int pl) { return Lay::off_i + ((pl - k0) % Lay::RI) * IT_SLOT; };   // bytes
+    // test hook: plane kk's copies are armed but not issued
+    auto held = [&](int kk) { return p.hold == 2 && kk == p.hold_plane + 2; };
+    // what plane kk adds to the rings: velocities of kk + 2, the index of kk + 1
+    auto issue = [&](int kk, uint64_t *bar) {
+        tma::mbar_expect_tx(bar, 3 * VT_BYTES + IT);
+        if (held(kk)) return;
+        for (int a = 0; a < 3; ++a)
+            tma::load3d(smb + oV(kk + 2) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, kk + 2, bar);
+        tma::load3d(smb + oI(kk + 1), &tm.idx, x0, y0, kk + 1, bar);
+    };
+    // the material table and the index do not change during a run, so their
+    // copies go out before the wait for the previous kernel of the stream
+    const unsigned lut_bytes = (unsigned)p.n_mat * (unsigned)sizeof(st::StressCoef);
     if (tid == 0) {
         for (int b = 0; b < 3; ++b) tma::mbar_init(&bars[b], 1);
         tma::mbar_init_fence();
         *s_abort = -1;
-    }
-    __syncthreads();
-
-    constexpr unsigned VT_BYTES = VT * Lay::ES;
-    auto oV = [&](int pl) { return Lay::off_v + ((pl - k0 + 2) % Lay::RV) * 3 * (int)VT_BYTES; };
-    auto oI = [&](int pl) { return Lay::off_i + ((pl - k0) % Lay::RI) * IT_SLOT; };   // bytes
-    auto issue = [&](int kk, uint64_t *bar, bool first) {
-        const unsigned nv = first ? 5 : 1;
-        tma::mbar_expect_tx(bar, nv * 3 * VT_BYTES + (first ? 2 : 1) * IT);
-        if (p.hold == 2 && kk == p.hold_plane + 2) return;    // test hook: armed, none issued
-        for (int pl = first ? kk - 2 : kk + 2; pl <= kk + 2; ++pl)
-            for (int a = 0; a < 3; ++a)
-                tma::load3d(smb + oV(pl) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, pl, bar);
-        for (int pl = first ? kk : kk + 1; pl <= kk + 1; ++pl)
-            tma::load3d(smb + oI(pl), &tm.idx, x0, y0, pl, bar);
-    };
-    if (tid == 0) {
         if (REUSE) tma::fence_async_smem();
-        issue(k0, &bars[0], true);
-        if (k0 + 1 < k1) issue(k0 + 1, &bars[1], false);
+        tma::mbar_expect_tx(&bars[0], 15 * VT_BYTES + 2 * IT + lut_bytes);
+        if (!held(k0)) {
+            tma::load_bulk(s_lut, p.slut, lut_bytes, &bars[0]);
+            tma::load3d(smb + oI(k0), &tm.idx, x0, y0, k0, &bars[0]);
+            tma::load3d(smb + oI(k0 + 1), &tm.idx, x0, y0, k0 + 1, &bars[0]);
+        }
+    }
+    if (!REUSE) {
+        tma::pdl_wait();
+        tma::pdl_launch_next();
+    }
+    if (tid == 0) {
+        for (int pl = k0 - 2; pl <= k0 + 2 && !held(k0); ++pl)
+            for (int a = 0; a < 3; ++a)
+                tma::load3d(smb + oV(pl) + a * VT_BYTES, &tm.v[a], x0 - Bx::XO, y0 - 2, pl,
+                            &bars[0]);
+        if (k0 + 1 < k1) issue(k0 + 1, &bars[1]);
     }
 
     const st::Dx ix = st::make_dx(p.inv_dx);
@@ -865,7 +896,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
         if (*s_abort >= 0) break;        // a wait of the previous plane ran out
         if (tid == 0 && k + 2 < k1) {
             tma::fence_async_smem();
-            issue(k + 2, &bars[(it + 2) % 3], false);
+            issue(k + 2, &bars[(it + 2) % 3]);
         }
         const int q = k * (nx * ny) + j * nx + i;
         // the pair's streams, packed, in flight while the ring wait and the
@@ -1266,23 +1297,30 @@ static cudaError_t raise_smem_once(K kernel, size_t bytes, std::atomic<int> &don
     return e;
 }
 
-static int chunk_of(const AcParams &p, int th)
+// z-planes per block of a launch: the context's choice, else the rule's (with
+// the test hook armed at least 8, so that the plane it names has look-ahead
+// copies).  Beside other domains' kernels the SMs are full whatever one launch
+// does, and long chunks cost the least in all: 16 domains of 96 to 200 cells
+// in one graph take 101.2 ms with the batch rule's 8 to 10 planes, 104.5 with
+// the chunks that are the fastest for a domain alone.
+static int chunk_or(const AcParams &p, int th, int rule)
 {
-    return p.kchunk > 0 ? p.kchunk : default_kchunk_tma(p.nx, p.ny, p.nz, th);
+    if (p.kchunk > 0) return p.kchunk;
+    if (p.crowd) return default_kchunk_tma(p.nx, p.ny, p.nz, th);
+    return p.hold ? std::min(p.nz, std::max(8, rule)) : rule;
 }
 
 template <typename T, int TH>
 static cudaError_t launch_velocity_tma_t(const AcParams &p, const VelocityTmaMaps &tm,
                                          cudaStream_t s)
 {
-    const int kc = chunk_of(p, TH);
+    const int kc = chunk_or(p, TH, velocity_kchunk(p.nx, p.ny, p.nz, TH));
     const size_t sm = VelLayout<T, TH>::bytes(p.n_mat);
     static std::atomic<int> done{0};
     cudaError_t e = raise_smem_once(k_velocity_tma<T, TH>,
                                     VelLayout<T, TH>::bytes(BVF_MAX_MATERIALS), done);
     if (e != cudaSuccess) return e;
-    k_velocity_tma<T, TH><<<grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s>>>(p, kc, tm);
-    return cudaGetLastError();
+    return launch_pdl(k_velocity_tma<T, TH>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p, kc, tm);
 }
 
 // tile heights other than TY are built for L = 2 (the method's two
@@ -1307,7 +1345,7 @@ cudaError_t launch_velocity_tma(const AcParams &p, const VelocityTmaMaps &tm, cu
 template <int L, typename T, int TH>
 static cudaError_t launch_stress_tma_t(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s)
 {
-    const int kc = chunk_of(p, TH);
+    const int kc = chunk_or(p, TH, stress_kchunk(p.nx, p.ny, p.nz, TH, p.h16));
     const size_t sm = StressLayout<L, T, TH>::bytes(p.n_mat);
     static std::atomic<int> done{0};
     if constexpr (std::is_same<T, __half>::value && L > 0) {
@@ -1316,15 +1354,16 @@ static cudaError_t launch_stress_tma_t(const AcParams &p, const StressTmaMaps &t
         cudaError_t e = raise_smem_once(k_stress_tma_h2<L, MB, TH>,
                                         StressLayout<L, T, TH>::bytes(BVF_MAX_MATERIALS), done);
         if (e != cudaSuccess) return e;
-        k_stress_tma_h2<L, MB, TH><<<grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s>>>(p, kc, tm);
+        return launch_pdl(k_stress_tma_h2<L, MB, TH>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p,
+                          kc, tm);
     } else {
         constexpr int MB = 4 * TY / TH;
         cudaError_t e = raise_smem_once(k_stress_tma<L, MB, T, TH>,
                                         StressLayout<L, T, TH>::bytes(BVF_MAX_MATERIALS), done);
         if (e != cudaSuccess) return e;
-        k_stress_tma<L, MB, T, TH><<<grid_tma<TH>(p, kc), dim3(TX, TH, 1), sm, s>>>(p, kc, tm);
+        return launch_pdl(k_stress_tma<L, MB, T, TH>, grid_tma<TH>(p, kc), dim3(TX, TH, 1), sm, s, p,
+                          kc, tm);
     }
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -1408,19 +1447,50 @@ cudaError_t launch_batch_step(const BatchParams &bp, int L, int h16, int n_mat_m
     }
 }
 
-// z-chunk length of the TMA kernels: about six waves of four resident blocks
-// per SM on 152 SMs (13 planes on the 240 x 240 x 200 grid; 8 to 16 measure
-// within 3 % of each other there, 25 is 13 % slower).
+static long long xy_tiles(int nx, int ny, int th)
+{
+    return (long long)((nx + TX - 1) / TX) * ((ny + th - 1) / th);
+}
+// planes per block that give at least `blocks` blocks, at least `least`
+static int planes_for(long long tiles, int nz, long long blocks, int least)
+{
+    const long long chunks = std::max(1LL, (blocks + tiles - 1) / tiles);
+    return std::min(nz, std::max(least, (int)((nz + chunks - 1) / chunks)));
+}
+
+// z-chunk length in batched sweeps (persistent kernels, and graphs or streams
+// of several domains): about six waves of four
+// resident blocks per SM on 152 SMs, at least 8 planes an item (an item
+// restarts its rings).
 int default_kchunk_tma(int nx, int ny, int nz, int tile_y)
 {
-    const int th = tile_y > 0 ? tile_y : TY;
-    const long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + th - 1) / th);
-    const long long target = 152LL * 4 * 6;
-    long long chunks = (target + tiles - 1) / tiles;
-    if (chunks < 1) chunks = 1;
-    int kc = (int)((nz + chunks - 1) / chunks);
-    if (kc < 8) kc = 8;
-    return kc > nz ? nz : kc;
+    return planes_for(xy_tiles(nx, ny, tile_y > 0 ? tile_y : TY), nz, 152LL * 4 * 6, 8);
+}
+
+// z-chunk length of the velocity kernel: about six waves, at least 2 planes.
+// A plane costs a block about 2 us of latency whatever the grid, so few long
+// chunks leave the SMs waiting on a serial chain: 64^3 with 8 planes 18.3 us,
+// with 2 planes 10.3 us; 96^3 21.1 and 16.4 us.  One plane a block re-reads
+// five planes of halo for it: 11.9 us at 64^3.
+int velocity_kchunk(int nx, int ny, int nz, int th)
+{
+    return planes_for(xy_tiles(nx, ny, th), nz, 152LL * 4 * 6, 2);
+}
+
+// z-chunk length of the stress kernel.  FP32 storage: about six waves, 2 to 6
+// planes (64^3: 8 planes 28.8 us, 2 planes 18.4; 240 x 240 x 200: 13 planes
+// 330.7 us, 6 planes 322.7; 360 x 360 x 300: 43 planes 1087 us, 6 planes 1047:
+// the z-neighbours of short chunks are still in L2).  FP16 storage, paired
+// tile: about ten waves of it, 2 to 5 planes (160^3: 8 planes 104 us, 3 planes
+// 96; 240 x 240 x 200: 13 planes 273.6 us, 5 planes 263.5).  Where chunks of 2
+// do not fill the GPU twice, the second wave is mostly empty, and single
+// planes spread it better (64 x 64 x 96 FP32: 28.0 us a step with 2, 26.2
+// with 1; FP16 at 64^3 20.1 and 18.4).
+int stress_kchunk(int nx, int ny, int nz, int th, int h16)
+{
+    const long long tiles = xy_tiles(nx, ny, th), wave = 152LL * 4 * TY / th;
+    if (tiles * ((nz + 1) / 2) < 2 * wave) return 1;
+    return std::min(planes_for(tiles, nz, wave * (h16 ? 10 : 6), 2), h16 ? 5 : 6);
 }
 
 }  // namespace bvf

@@ -55,6 +55,7 @@ struct bvf_ctx {
     int dft_count = 0;
     uint8_t *index = nullptr;
     MatCoef *lut = nullptr;
+    void *slut = nullptr;             // st::StressCoef per material (made from lut)
     float *buoy = nullptr;            // material-pair buoyancy table
     float2 *pml = nullptr;
     float2 *src = nullptr;
@@ -82,6 +83,7 @@ struct bvf_ctx {
     long long steps = 0, launches = 0, thermal_steps = 0;
     double courant = 0.0;
     int kchunk = 0;                   // z-planes per block (0 = default)
+    bool crowd = false;               // enqueued beside other domains (batch calls)
     bvf_tile tile{0, 0, 0};           // tile of the TMA kernels (bvf_set_tile; 0 = default)
     bool tma = false;                 // velocity kernel fed by TMA
     bool tma_stress = false;          // stress kernel fed by TMA
@@ -410,6 +412,7 @@ AcParams make_params(bvf_ctx *c)
     }
     p.idx = c->index;
     p.lut = c->lut;
+    p.slut = c->slut;
     p.buoy = c->buoy;
     p.vx = field_ptr(c, BVF_FIELD_VX);
     p.vy = field_ptr(c, BVF_FIELD_VY);
@@ -437,6 +440,7 @@ AcParams make_params(bvf_ctx *c)
     const bvf_tile t = effective_tile(c);
     p.tile_y = t.stress_rows;
     p.tile_yv = t.velocity_rows;
+    p.crowd = c->crowd;
     p.wait_limit = tma::kWaitLimit;
     p.hold = 0;
     p.hold_plane = -1;
@@ -578,7 +582,7 @@ const char *bvf_last_error(const bvf_ctx *ctx)
 void bvf_destroy(bvf_ctx *c)
 {
     if (!c) return;
-    void *bufs[] = {c->fields, c->psi, c->peak, c->dftC, c->dftS, c->index, c->lut, c->buoy,
+    void *bufs[] = {c->fields, c->psi, c->peak, c->dftC, c->dftS, c->index, c->lut, c->slut, c->buoy,
                     c->pml, c->src, c->flag, c->scratch_u, c->T2, c->Q, c->cemf, c->tlut,
                     c->kface, c->index_p, c->h_index_d, c->h_peak_d, c->h_T_d, c->h_Tmax_d,
                     c->h_amp_d, c->h_cem_d};
@@ -650,6 +654,7 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     if ((e = cudaMalloc(&c->peak, c->N * sizeof(float))) != cudaSuccess ||
         (e = cudaMalloc(&c->index, c->N)) != cudaSuccess ||
         (e = cudaMalloc(&c->lut, BVF_MAX_MATERIALS * sizeof(MatCoef))) != cudaSuccess ||
+        (e = cudaMalloc(&c->slut, BVF_MAX_MATERIALS * 32)) != cudaSuccess ||
         (e = cudaMalloc(&c->buoy, (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float))) !=
             cudaSuccess ||
         (e = cudaMalloc(&c->pml, 6 * (size_t)c->nmax * sizeof(float2))) != cudaSuccess ||
@@ -760,8 +765,9 @@ int bvf_set_materials(bvf_ctx *c, const uint8_t *d_index, const bvf_material *h_
        "copy buoyancy");
     CK(cudaMemcpy(c->pml, pml.data(), pml.size() * sizeof(float2), cudaMemcpyHostToDevice), "copy pml");
     CK(cudaMemset(c->scratch_u, 0, sizeof(unsigned)), "memset");
+    CK(launch_stress_table(c->lut, n_mat, (float)c->L, c->slut, 0), "stress table");
     CK(launch_index_max(c->index, c->N, c->scratch_u, 0), "index scan");
-    c->launches++;
+    c->launches += 2;
     unsigned mx = 0;
     CK(cudaMemcpy(&mx, c->scratch_u, sizeof(unsigned), cudaMemcpyDeviceToHost), "index scan");
     if ((int)mx >= n_mat) {
@@ -1367,8 +1373,18 @@ int bvf_plan(bvf_ctx *skull, bvf_ctx *water, const uint8_t *d_index, const bvf_m
         if ((rc = bvf_reset(c, cs)) != BVF_OK) return done(rc);
         if ((rc = bvf_set_source(c, k_src, src, bowl->c0, BVF_ENV_RAMP_CW, 0, cs)) != BVF_OK)
             return done(rc);
-        if ((rc = bvf_run_acoustic(c, pp->n_steps, &cap, cs)) != BVF_OK) return done(rc);
     }
+    // Side by side, the two runs are enqueued in turns of a few steps: a run's
+    // launches would otherwise fill the launch queue and hold the other run
+    // back until most of the first had finished.  With a time budget each run
+    // is one call, as the budget counts from its start.
+    const bool turns = !pp->serial && !(skull->budget_s > 0.0) && !(water->budget_s > 0.0);
+    const int turn = turns ? 8 : pp->n_steps;
+    for (int n = 0; n < pp->n_steps; n += turn)
+        for (bvf_ctx *c : runs)
+            if ((rc = bvf_run_acoustic(c, std::min(turn, pp->n_steps - n), &cap,
+                                       c == water ? ws : stream)) != BVF_OK)
+                return done(rc);
     if ((rc = bvf_get_amp_phase(skull, d_amp, nullptr, stream)) != BVF_OK) return done(rc);
     if ((rc = bvf_get_amp_phase(water, amp_w, nullptr, ws)) != BVF_OK) return done(rc);
     if (forked) {
@@ -1564,6 +1580,16 @@ int bvf_batch_run(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int
     return BVF_OK;
 }
 
+// one domain's steps on `s`, beside the other domains' (crowd: see chunk_or)
+static int run_beside(bvf_batch *b, int d, int n_steps, const bvf_capture *caps, cudaStream_t s)
+{
+    bvf_ctx *c = b->ctx[d];
+    c->crowd = b->ctx.size() > 1;
+    const int rc = bvf_run_acoustic(c, n_steps, caps ? &caps[d] : nullptr, s);
+    c->crowd = false;
+    return rc;
+}
+
 int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *caps,
                           int n_streams, void *stream)
 {
@@ -1588,8 +1614,7 @@ int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *c
         CK_FREE(cudaStreamWaitEvent(b->side[k], b->fork, 0), "bvf_batch_run_streams");
     // domains dealt round-robin; each side stream runs its domains one after another
     for (int d = 0; d < n; ++d) {
-        const int rc = bvf_run_acoustic(b->ctx[d], n_steps[d], caps ? &caps[d] : nullptr,
-                                        b->side[d % n_streams]);
+        const int rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_streams]);
         if (rc != BVF_OK) return rc;
         b->launches += 2LL * n_steps[d];
     }
@@ -1661,8 +1686,7 @@ int bvf_batch_run_graph(bvf_batch *b, const int *n_steps, const bvf_capture *cap
         for (int k = 0; k < n_branches && e == cudaSuccess; ++k)
             e = cudaStreamWaitEvent(b->side[k], b->fork, 0);
         for (int d = 0; d < n && e == cudaSuccess && rc == BVF_OK; ++d)
-            rc = bvf_run_acoustic(b->ctx[d], n_steps[d], caps ? &caps[d] : nullptr,
-                                  b->side[d % n_branches]);
+            rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_branches]);
         for (int k = 0; k < n_branches && e == cudaSuccess; ++k) {
             e = cudaEventRecord(b->side_ev[k], b->side[k]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->side_ev[k], 0);
@@ -1822,8 +1846,8 @@ int bvf_get_tile(const bvf_ctx *c, bvf_tile *out)
     if (!c || !out) return fail(nullptr, BVF_E_ARG, "bvf_get_tile: NULL argument");
     *out = effective_tile(c);
     out->kchunk = c->kchunk > 0 ? std::min(c->kchunk, c->g.nz)
-                                : (c->tma ? default_kchunk_tma(c->g.nx, c->g.ny, c->g.nz,
-                                                               out->stress_rows)
+                                : (c->tma ? stress_kchunk(c->g.nx, c->g.ny, c->g.nz,
+                                                          out->stress_rows, c->h16)
                                           : default_kchunk(c->g.nx, c->g.ny, c->g.nz));
     return BVF_OK;
 }

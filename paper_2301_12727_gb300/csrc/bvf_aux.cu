@@ -28,6 +28,14 @@ __global__ void k_index_max(const uint8_t *__restrict__ idx, size_t n, unsigned 
     if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
+static_assert(sizeof(st::StressCoef) == 32, "bvf_ctx::slut holds 32 bytes per material");
+__global__ void k_stress_table(const MatCoef *__restrict__ lut, int n, float Lf,
+                               st::StressCoef *__restrict__ out)
+{
+    const int m = threadIdx.x;
+    if (m < n) out[m] = st::make_stress_coef(lut[m], Lf);
+}
+
 template <typename T>
 __global__ void k_pressure(const T *__restrict__ a, const T *__restrict__ b,
                            const T *__restrict__ c, float scale, float *__restrict__ out, size_t n)
@@ -532,6 +540,12 @@ cudaError_t launch_conj_plane(const double *C, const double *S, size_t n,
     if (e != cudaSuccess) return e;
     k_plane_absmax<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, d_max);
     k_conj_normalise<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, d_max, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stress_table(const MatCoef *lut, int n, float Lf, void *slut, cudaStream_t s)
+{
+    k_stress_table<<<1, BVF_MAX_MATERIALS, 0, s>>>(lut, n, Lf, static_cast<st::StressCoef *>(slut));
     return cudaGetLastError();
 }
 

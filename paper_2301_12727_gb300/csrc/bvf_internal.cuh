@@ -78,6 +78,7 @@ struct AcParams {
     float ca[BVF_MAX_SLS], ncb[BVF_MAX_SLS];
     const uint8_t *idx;
     const MatCoef *lut;
+    const void *slut;    // st::StressCoef per material, made from lut when the table is set
     const float *buoy;   // 2 / (rho_a + rho_b) of every material pair, [a * n_mat + b]
     void *vx, *vy, *vz, *sxx, *syy, *szz, *sxy, *sxz, *syz;   // float or __half
     void *mem;           // memory variables, element mem_index(l, c, q)
@@ -94,7 +95,7 @@ struct AcParams {
     double *dftC, *dftS;
     StepParam st;        // this step's source and capture parameters
     int *flag;
-    int kchunk;          // z-planes per block (0 = default_kchunk)
+    int kchunk;          // z-planes per block (0 = the kernel's own rule)
     // bounded TMA waits: polls per mbarrier wait before a block gives up
     // (sets bit 2 of *flag, issues no further copies, drains the copies it
     // has issued, and stops).  hold = 1 (velocity) or 2 (stress) makes that
@@ -106,6 +107,7 @@ struct AcParams {
     // rows of an x-y tile of the TMA-fed stress and velocity kernels: 4, 8 or
     // 16 (heights other than 8 with L = 2 only)
     int tile_y, tile_yv;
+    int crowd;           // other domains' kernels run beside this one (batched sweeps)
 };
 
 // Tensor maps of the TMA-fed acoustic kernels (x-y boxes of one z-plane).
@@ -173,12 +175,35 @@ struct ThParams {
     int hold_plane;
 };
 
+// Launch with programmatic stream serialization: the kernel may start while
+// the previous kernel of its stream drains, so the start-up of a block
+// (barriers, tensor maps, tables) overlaps the tail before it.  The kernel
+// must call tma::pdl_wait() before it touches anything another kernel writes.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                       const A &...args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // message returned by bvf_last_error(NULL) for a failed context-free call
 void set_context_free_error(const char *msg);
 
 // z-planes per block of the z-marching acoustic kernels for a grid
 int default_kchunk(int nx, int ny, int nz);
-int default_kchunk_tma(int nx, int ny, int nz, int tile_y = 8);
+int default_kchunk_tma(int nx, int ny, int nz, int tile_y = 8);   // batched sweeps
+int velocity_kchunk(int nx, int ny, int nz, int th);
+int stress_kchunk(int nx, int ny, int nz, int th, int h16);
 
 // Persistent batch kernels: one velocity and one stress launch advance every
 // domain of `dom` by one step (the step number is read from *d_step, which a
@@ -193,6 +218,8 @@ cudaError_t launch_velocity(const AcParams &p, cudaStream_t s);
 cudaError_t launch_stress(const AcParams &p, cudaStream_t s);
 cudaError_t launch_velocity_tma(const AcParams &p, const VelocityTmaMaps &tm, cudaStream_t s);
 cudaError_t launch_stress_tma(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s);
+// st::StressCoef of each of n materials (slut: n * 32 bytes, 16-byte aligned)
+cudaError_t launch_stress_table(const MatCoef *lut, int n, float Lf, void *slut, cudaStream_t s);
 cudaError_t launch_index_max(const uint8_t *idx, size_t n, unsigned *d_out, cudaStream_t s);
 cudaError_t launch_pressure(const void *sxx, const void *syy, const void *szz, int h16,
                             float scale, float *out, size_t n, cudaStream_t s);

@@ -94,6 +94,26 @@ __device__ __forceinline__ void load3d(void *dst, const CUtensorMap *map, int x,
         : "memory");
 }
 
+// global -> shared copy of `bytes` consecutive bytes (both addresses and the
+// size multiples of 16), counted on `bar`
+__device__ __forceinline__ void load_bulk(void *dst, const void *src, unsigned bytes, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            saddr(dst)),
+        "l"(src), "r"(bytes), "r"(saddr(bar))
+        : "memory");
+}
+
+// Programmatic dependent launch (see launch_pdl): wait until the kernels this
+// one depends on have finished and their writes are visible / let the next
+// kernel of the stream start its prologue.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // shared -> global tile store; out-of-range elements are not written
 __device__ __forceinline__ void store3d(const CUtensorMap *map, int x, int y, int z, const void *src)
 {
