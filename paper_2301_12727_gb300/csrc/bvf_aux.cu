@@ -84,81 +84,65 @@ __global__ void k_amp_phase(const double *__restrict__ C, const double *__restri
     }
 }
 
-// One thread per plane point, elements staged through shared memory.
 // p = pref * sum_e dA_e (sin(k r) + i cos(k r)) / r   with pref = k p0 / (2 pi):
 // the i k p0 / (2 pi) prefactor times exp(-i k r) = cos kr - i sin kr.
-// Elements with complex weights w_e (phased arrays): the element's term is
+// Elements with complex weights w_e (phased arrays, WT): the element's term is
 // multiplied by w_e = wr + i wi.
-__global__ void __launch_bounds__(kThreads) k_rs_weighted(const float4 *__restrict__ el,
-                                                          const float2 *__restrict__ wt, int ne,
-                                                          int nx, int ny, float dx, float zp,
-                                                          float k_over_pi, double pref,
-                                                          float2 *__restrict__ out)
-{
-    __shared__ float4 s_el[kThreads];
-    __shared__ float2 s_w[kThreads];
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = q < nx * ny;
-    const float x = live ? (q % nx) * dx : 0.0f;
-    const float y = live ? (q / nx) * dx : 0.0f;
-    double re = 0.0, im = 0.0;
-    for (int base = 0; base < ne; base += kThreads) {
-        if (base + threadIdx.x < ne) {
-            s_el[threadIdx.x] = el[base + threadIdx.x];
-            s_w[threadIdx.x] = wt[base + threadIdx.x];
-        }
-        __syncthreads();
-        const int cnt = min(kThreads, ne - base);
-        float pre = 0.0f, pim = 0.0f;
-        for (int e = 0; e < cnt; ++e) {
-            const float4 E = s_el[e];
-            const float2 W = s_w[e];
-            const float ddx = x - E.x, ddy = y - E.y, ddz = zp - E.z;
-            const float r = sqrtf(fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz)));
-            float sn, cs;
-            sincospif(k_over_pi * r, &sn, &cs);
-            const float w = E.w / r;
-            // (wr + i wi)(sin kr + i cos kr)
-            pre = fmaf(w, fmaf(W.x, sn, -W.y * cs), pre);
-            pim = fmaf(w, fmaf(W.x, cs, W.y * sn), pim);
-        }
-        re += pre;
-        im += pim;
-        __syncthreads();
-    }
-    if (live) out[q] = make_float2((float)(pref * re), (float)(pref * im));
-}
+//
+// The sum runs in tiles of 256 elements, FP32 within a tile and FP64 over the
+// tiles in their order.  A block of 32 points x 8 threads takes 8 tiles at a
+// time, one per thread of a point, and the first thread of the point adds the
+// 8 partial sums in order, so the result does not depend on the split.  The
+// sum is bound by its instructions (square root, sincospi and division of
+// every pair): one thread per point gave 225 blocks on 152 SMs at 240 x 240
+// points, half the SMs with one block of 8 warps, and 976 us; this takes
+// 650 us.  The elements (98 KB there) come from the L1, the same address for a
+// point's whole warp.
+constexpr int kRsTile = 256;             // elements per FP32 partial sum
+constexpr int kRsPts = 32, kRsGroups = 8;
 
-__global__ void __launch_bounds__(kThreads) k_rs(const float4 *__restrict__ el, int ne, int nx,
-                                                 int ny, float dx, float zp, float k_over_pi,
-                                                 double pref, float2 *__restrict__ out)
+template <bool WT>
+__global__ void __launch_bounds__(kRsPts *kRsGroups)
+    k_rs(const float4 *__restrict__ el, const float2 *__restrict__ wt, int ne, int nx, int ny,
+         float dx, float zp, float k_over_pi, double pref, float2 *__restrict__ out)
 {
-    __shared__ float4 s_el[kThreads];
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ float2 s_part[kRsGroups][kRsPts];
+    const int pt = threadIdx.x, g = threadIdx.y;
+    const int q = blockIdx.x * kRsPts + pt;
     const bool live = q < nx * ny;
     const float x = live ? (q % nx) * dx : 0.0f;
     const float y = live ? (q / nx) * dx : 0.0f;
     double re = 0.0, im = 0.0;
-    for (int base = 0; base < ne; base += kThreads) {
-        if (base + threadIdx.x < ne) s_el[threadIdx.x] = el[base + threadIdx.x];
-        __syncthreads();
-        const int cnt = min(kThreads, ne - base);
-        float pre = 0.0f, pim = 0.0f;   // partial sums of one tile in FP32
-        for (int e = 0; e < cnt; ++e) {
-            const float4 E = s_el[e];
+    for (int base = 0; base < ne; base += kRsTile * kRsGroups) {
+        const int e0 = base + g * kRsTile, e1 = min(ne, e0 + kRsTile);
+        float pre = 0.0f, pim = 0.0f;
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) {
+            const float4 E = __ldg(el + e);
             const float ddx = x - E.x, ddy = y - E.y, ddz = zp - E.z;
             const float r = sqrtf(fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz)));
             float sn, cs;
             sincospif(k_over_pi * r, &sn, &cs);
             const float w = E.w / r;
-            pre = fmaf(w, sn, pre);
-            pim = fmaf(w, cs, pim);
+            if (WT) {                    // (wr + i wi)(sin kr + i cos kr)
+                const float2 W = __ldg(wt + e);
+                pre = fmaf(w, fmaf(W.x, sn, -W.y * cs), pre);
+                pim = fmaf(w, fmaf(W.x, cs, W.y * sn), pim);
+            } else {
+                pre = fmaf(w, sn, pre);
+                pim = fmaf(w, cs, pim);
+            }
         }
-        re += pre;
-        im += pim;
+        s_part[g][pt] = make_float2(pre, pim);
+        __syncthreads();
+        if (g == 0)
+            for (int t = 0; t < kRsGroups && base + t * kRsTile < ne; ++t) {
+                re += s_part[t][pt].x;
+                im += s_part[t][pt].y;
+            }
         __syncthreads();
     }
-    if (live) out[q] = make_float2((float)(pref * re), (float)(pref * im));
+    if (g == 0 && live) out[q] = make_float2((float)(pref * re), (float)(pref * im));
 }
 
 __global__ void k_heat_source(const uint8_t *__restrict__ idx, const ThermCoef *__restrict__ lut,
@@ -628,9 +612,8 @@ cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, int cou
 cudaError_t launch_rs(const float4 *el, int ne, int nx, int ny, float dx, float zp, float k_over_pi,
                       double pref, float2 *out, cudaStream_t s)
 {
-    const int n = nx * ny;
-    k_rs<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(el, ne, nx, ny, dx, zp, k_over_pi,
-                                                           pref, out);
+    k_rs<false><<<(nx * ny + kRsPts - 1) / kRsPts, dim3(kRsPts, kRsGroups), 0, s>>>(
+        el, nullptr, ne, nx, ny, dx, zp, k_over_pi, pref, out);
     return cudaGetLastError();
 }
 
@@ -638,9 +621,8 @@ cudaError_t launch_rs_weighted(const float4 *el, const float2 *wt, int ne, int n
                                float dx, float zp, float k_over_pi, double pref, float2 *out,
                                cudaStream_t s)
 {
-    const int n = nx * ny;
-    k_rs_weighted<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(el, wt, ne, nx, ny, dx, zp,
-                                                                    k_over_pi, pref, out);
+    k_rs<true><<<(nx * ny + kRsPts - 1) / kRsPts, dim3(kRsPts, kRsGroups), 0, s>>>(
+        el, wt, ne, nx, ny, dx, zp, k_over_pi, pref, out);
     return cudaGetLastError();
 }
 
