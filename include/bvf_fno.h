@@ -146,9 +146,9 @@ int bvf_gemm_bf16(const bvf_gemm *g, int *d_flag, void *stream);
  * The same network with every contraction on the BF16 tensor-core product
  * (bvf_gemm_bf16): the lift, W v + b and the projection as channel products;
  * each Fourier layer's truncated transform as three products (x: real ->
- * kept modes, y and z: complex, as real 2 x 2 blocks) with axis permutes in
- * between, the inverse likewise with the real-inverse weights c(kx)/N (c = 1
- * for kx = 0, 2 otherwise); the mode mix in FP32 (no counterpart in the
+ * kept modes, y and z: complex, as real 2 x 2 blocks), the inverse likewise
+ * with the real-inverse weights c(kx)/N (c = 1 for kx = 0, 2 otherwise), its x
+ * stage in one pass with the layer's channel product; the mode mix in FP32 (no counterpart in the
  * paper: planning-time inference and training of the surrogate).  A context
  * is sized for one grid and up to max_batch samples and keeps FP32 master
  * weights, their gradient, Adam moments and every activation the backward pass

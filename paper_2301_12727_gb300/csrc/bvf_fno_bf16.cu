@@ -12,9 +12,10 @@
 //   y: rows (b, c, z, kx) x [part][y]  ->  [part][ky]   (e^{-i theta} as a
 //      real 2 x 2 block)
 //   z: rows (b, c, ky, kx) x [part][z]  ->  [part][kz]
-// with axis permutes in between; the inverse (irfftn of the kept half
-// spectrum) is the same chain backwards with e^{+i theta} and, on x, the
-// weights c(kx)/N (c = 1 for kx = 0, 2 otherwise).  The mode mix (per mode a
+// each reading and writing its neighbours' axis order; the inverse (irfftn of
+// the kept half spectrum) is the same chain backwards with e^{+i theta} and,
+// on x, the weights c(kx)/N (c = 1 for kx = 0, 2 otherwise); its x stage runs
+// in one pass with the layer's channel mix (bvf_row_bf16.cu).  The mode mix (per mode a
 // W x W complex matrix) is a small SIMT kernel.
 //
 // Backward (gradients of the loss below): the adjoint of the inverse is the
@@ -37,14 +38,11 @@
 #include <string>
 #include <vector>
 
-#include "../../include/bvf_fno.h"
-#include "bvf_internal.cuh"
+#include "bvf_fno_bf16.cuh"
 
-namespace bvf {
-cudaError_t launch_gemm_bf16(const bvf_gemm &g, int *flag, cudaStream_t s);
-}
-
+using bvf::GemmX;
 using bvf::launch_gemm_bf16;
+using bvf::RowBf16;
 
 namespace {
 
@@ -65,24 +63,6 @@ int b16_fail(int code, const std::string &msg)
     } while (0)
 
 __host__ __device__ __forceinline__ int slot_freq(int j, int m) { return j < m ? j : j - 2 * m; }
-
-// out[p][c][q][a] = in[p][a][q][c]
-__global__ void k_permute(const float *__restrict__ in, float *__restrict__ out, long long P, int A,
-                          int Q, int C)
-{
-    const long long n = P * A * Q * C;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        // t indexes the output [p][c][q][a]
-        const int a = (int)(t % A);
-        long long r = t / A;
-        const int q = (int)(r % Q);
-        r /= Q;
-        const int c = (int)(r % C);
-        const long long p = r / C;
-        out[t] = in[((p * A + a) * Q + q) * C + c];
-    }
-}
 
 // spectrum position of mode (kz, ky, kx), part, in a channel's 8 m^3 floats
 __device__ __forceinline__ int spec_pos(int kz, int ky, int kx, int part, int m)
@@ -293,6 +273,7 @@ struct bvf_fno_bf16 {
     double *sums = nullptr;
     int *flag = nullptr;
     std::vector<void *> all;
+    int n_sm = 152;
     int ksplit = 1;                     // K split of the voxel-sum products
 };
 
@@ -398,18 +379,23 @@ bvf_gemm rowmajor(const float *A, const float *B, float *C, long long rows, int 
     return g;
 }
 
+int gemm(bvf_fno_bf16 *t, const GemmX &x, cudaStream_t s, const char *what)
+{
+    BCK(launch_gemm_bf16(x, t->flag, s), what);
+    return BVF_OK;
+}
 int gemm(bvf_fno_bf16 *t, const bvf_gemm &g, cudaStream_t s, const char *what)
 {
-    BCK(launch_gemm_bf16(g, t->flag, s), what);
-    return BVF_OK;
+    GemmX x;
+    x.g = g;
+    return gemm(t, x, s, what);
 }
 
-int permute(const float *in, float *out, long long P, int A, int Q, int C, cudaStream_t s)
-{
-    k_permute<<<grid_for(P * A * Q * C), 256, 0, s>>>(in, out, P, A, Q, C);
-    BCK(cudaGetLastError(), "permute");
-    return BVF_OK;
-}
+// Between the stages of a transform the axes change places.  Each product
+// reads and writes its neighbours' order directly (GemmX): with separate
+// permutes every stage's output was read and written once more, 1.56 of 28.2
+// ms of a forward at 240 x 240 x 200 and 2.05 of 17.3 ms of a gradient at
+// 64 x 64 x 96, batch 4.
 
 // forward transform of BC real volumes -> BC spectra (weighted: the x stage
 // carries c(kx)/N, the adjoint of the inverse)
@@ -417,38 +403,66 @@ int spec_fwd(bvf_fno_bf16 *t, const float *in, long long BC, bool weighted, floa
 {
     const int nx = t->nx, ny = t->ny, nz = t->nz, m = t->d.modes;
     int rc;
-    if ((rc = gemm(t, rowmajor(in, weighted ? t->Fxw : t->Fx, t->w1, BC * nz * ny, nx, 2 * m), s,
-                   "spectral x")) != BVF_OK)
-        return rc;
-    if ((rc = permute(t->w1, t->w2, BC * nz, ny, 2, m, s)) != BVF_OK) return rc;
-    if ((rc = gemm(t, rowmajor(t->w2, t->Fy, t->w1, BC * nz * m, 2 * ny, 4 * m), s, "spectral y")) !=
-        BVF_OK)
-        return rc;
-    if ((rc = permute(t->w1, t->w2, BC, nz, 2 * m, 2 * m, s)) != BVF_OK) return rc;
-    return gemm(t, rowmajor(t->w2, t->Fz, S, BC * 2 * m * m, 2 * nz, 4 * m), s, "spectral z");
+    // x: rows (bc, z, y) -> w1 [bc][z][part][kx][y]
+    GemmX x;
+    x.g = rowmajor(in, weighted ? t->Fxw : t->Fx, t->w1, BC * nz * ny, nx, 2 * m);
+    x.rc = ny;
+    x.scm1 = 2LL * m * ny;
+    x.g.scm = 1;
+    x.g.scn = ny;
+    if ((rc = gemm(t, x, s, "spectral x")) != BVF_OK) return rc;
+    // y: rows (bc, kx, z), K (part, y) -> w2 [bc][part][ky][kx][z]
+    x = GemmX();
+    x.g = rowmajor(t->w1, t->Fy, t->w2, BC * nz * m, 2 * ny, 4 * m);
+    x.ra = nz;
+    x.ra2 = m;
+    x.g.sam = 2LL * m * ny;
+    x.sam1 = ny;
+    x.sam2 = 2LL * m * ny * nz;
+    x.ka = ny;
+    x.sak1 = (long long)m * ny;
+    x.rc = m * nz;
+    x.scm1 = 4LL * m * m * nz;
+    x.g.scm = 1;
+    x.g.scn = (long long)m * nz;
+    if ((rc = gemm(t, x, s, "spectral y")) != BVF_OK) return rc;
+    // z: rows (bc, ky, kx), K (part, z) -> S [bc][ky][kx][part][kz]
+    x = GemmX();
+    x.g = rowmajor(t->w2, t->Fz, S, BC * 2 * m * m, 2 * nz, 4 * m);
+    x.ra = 2 * m * m;
+    x.g.sam = nz;
+    x.sam2 = 4LL * m * m * nz;
+    x.ka = nz;
+    x.sak1 = 2LL * m * m * nz;
+    return gemm(t, x, s, "spectral z");
 }
 
-// inverse transform of BC spectra into BC real volumes: out = beta out +
-// Inv(S) (weighted: c(kx)/N, the real inverse of the kept half spectrum;
-// plain: the adjoint of the forward transform), then act (2: times GELU'(pre))
-int spec_inv(bvf_fno_bf16 *t, const float *S, long long BC, bool weighted, float *out, float beta,
-             int act, const float *pre, cudaStream_t s)
+// the z and y stages of the inverse transform of BC spectra: what its x stage
+// reads, w2 [bc][z][y][part][kx]
+int spec_inv_zy(bvf_fno_bf16 *t, const float *S, long long BC, cudaStream_t s)
 {
-    const int nx = t->nx, ny = t->ny, nz = t->nz, m = t->d.modes;
-    int rc;
-    if ((rc = gemm(t, rowmajor(S, t->Gz, t->w1, BC * 2 * m * m, 4 * m, 2 * nz), s, "inverse z")) !=
-        BVF_OK)
-        return rc;
-    if ((rc = permute(t->w1, t->w2, BC, 2 * m, 2 * m, nz, s)) != BVF_OK) return rc;
-    if ((rc = gemm(t, rowmajor(t->w2, t->Gy, t->w1, BC * nz * m, 4 * m, 2 * ny), s, "inverse y")) !=
-        BVF_OK)
-        return rc;
-    if ((rc = permute(t->w1, t->w2, BC * nz, m, 2, ny, s)) != BVF_OK) return rc;
-    bvf_gemm g = rowmajor(t->w2, weighted ? t->Gxw : t->Gx, out, BC * nz * ny, 2 * m, nx);
-    g.beta = beta;
-    g.act = act;
-    g.C_pre = const_cast<float *>(pre);
-    return gemm(t, g, s, "inverse x");
+    const int ny = t->ny, nz = t->nz, m = t->d.modes;
+    // z: rows (bc, ky, kx) -> w1 [bc][ky][kx][part][z]
+    const int rc = gemm(t, rowmajor(S, t->Gz, t->w1, BC * 2 * m * m, 4 * m, 2 * nz), s, "inverse z");
+    if (rc != BVF_OK) return rc;
+    // y: rows (bc, z, kx), K (part, ky)
+    GemmX x;
+    x.g = rowmajor(t->w1, t->Gy, t->w2, BC * nz * m, 4 * m, 2 * ny);
+    x.ra = m;
+    x.ra2 = nz;
+    x.g.sam = 2LL * nz;
+    x.sam1 = 1;
+    x.sam2 = 4LL * m * m * nz;
+    x.ka = 2 * m;
+    x.g.sak = 2LL * m * nz;
+    x.sak1 = nz;
+    x.rc = m;
+    x.scm1 = 2LL * m * ny;
+    x.g.scm = 1;
+    x.nc = ny;
+    x.g.scn = 2 * m;
+    x.scn1 = m;
+    return gemm(t, x, s, "inverse y");
 }
 
 // channel mix out[b][o][p] (+)= sum_c Wt[o][c] in[b][c][p] (Wt row-major [O][C])
@@ -518,6 +532,37 @@ int chan_sum(const float *x, int B, int C, int N, float *out, cudaStream_t s)
     return BVF_OK;
 }
 
+// One row pass over `batch` samples: out = act(Inv_x(w2) + mix of v + bias)
+// with the channel weights Wm(o, c) at o wso + c wsc (v has cin channels); G
+// the x stage's matrix, NULL for no spectral term.  act as in bvf_gemm.  Rows
+// too long for shared memory take the two products, with the sum through
+// `out`.
+int row_pass(bvf_fno_bf16 *t, int batch, const float *v, int cin, const float *Wm, int wso, int wsc,
+             const float *bias, const float *G, int act, float *pre, float *out, cudaStream_t s)
+{
+    const int W = t->d.width, m = t->d.modes, N = t->N;
+    if (bvf::row_bf16_fits(W, m, t->nx)) {
+        RowBf16 q{v, (long long)cin * N, cin, Wm, wso, wsc, bias, G ? t->w2 : nullptr, G, pre, act,
+                  out, batch, t->nx, t->ny * t->nz, m, N, t->n_sm, t->flag};
+        BCK(bvf::launch_row_bf16(q, W, s), "row pass");
+        return BVF_OK;
+    }
+    if (G) {
+        const int rc = gemm(t, rowmajor(t->w2, G, out, (long long)batch * W * t->nz * t->ny, 2 * m,
+                                        t->nx), s, "inverse x");
+        if (rc != BVF_OK) return rc;
+    }
+    bvf_gemm g = chan(v, cin, Wm, out, W, N, batch);
+    g.sbk = wsc;
+    g.sbn = wso;
+    g.beta = G ? 1.0f : 0.0f;
+    g.bias = bias;
+    g.bias_mode = bias ? 1 : 0;
+    g.act = act;
+    g.C_pre = pre;
+    return gemm(t, g, s, "pointwise");
+}
+
 // forward pass of `batch` samples into `out` ([batch][c_out][N]); with `keep`
 // every activation the backward pass needs is kept, without it (inference)
 // the pre-activations are not written
@@ -528,10 +573,9 @@ int forward(bvf_fno_bf16 *t, int batch, const float *in, float *out, bool keep, 
     const Off o = offsets(d);
     const float *w = t->w;
     int rc;
-    bvf_gemm g = chan(in, d.c_in, w + o.Wp, t->v[0], W, N, batch);
-    g.bias = w + o.bp;
-    g.bias_mode = 1;
-    if ((rc = gemm(t, g, s, "lift")) != BVF_OK) return rc;
+    if ((rc = row_pass(t, batch, in, d.c_in, w + o.Wp, d.c_in, 1, w + o.bp, nullptr, 0, nullptr,
+                       t->v[0], s)) != BVF_OK)
+        return rc;
     for (int l = 0; l < L; ++l) {
         const float *lw = w + o.lay0 + l * o.lf;
         const float *R = lw, *Wl = lw + (size_t)4 * m * m * m * W * W * 2, *bl = Wl + (size_t)W * W;
@@ -539,24 +583,23 @@ int forward(bvf_fno_bf16 *t, int batch, const float *in, float *out, bool keep, 
         k_mix_fwd<<<grid_for((long long)batch * 4 * m * m * m * W), 256, 0, s>>>(t->X[l], R, batch, W,
                                                                                    m, t->S1);
         BCK(cudaGetLastError(), "mix");
-        if ((rc = spec_inv(t, t->S1, (long long)batch * W, true, t->v[l + 1], 0.0f, 0, nullptr, s)) !=
-            BVF_OK)
+        if ((rc = spec_inv_zy(t, t->S1, (long long)batch * W, s)) != BVF_OK) return rc;
+        const int act = l < L - 1;
+        if ((rc = row_pass(t, batch, t->v[l], W, Wl, W, 1, bl, t->Gxw, act,
+                           act && keep ? t->s[l] : nullptr, t->v[l + 1], s)) != BVF_OK)
             return rc;
-        bvf_gemm p = chan(t->v[l], W, Wl, t->v[l + 1], W, N, batch);
-        p.beta = 1.0f;
-        p.bias = bl;
-        p.bias_mode = 1;
-        if (l < L - 1) {
-            p.act = 1;
-            p.C_pre = keep ? t->s[l] : nullptr;
-        }
-        if ((rc = gemm(t, p, s, "pointwise")) != BVF_OK) return rc;
     }
-    g = chan(t->v[L], W, w + o.Q1, t->h, d.hidden, N, batch);
+    if (!keep) {
+        BCK(bvf::launch_project_bf16(t->v[L], w + o.Q1, w + o.q1, w + o.Q2, w + o.q2, W, d.hidden,
+                                     d.c_out, out, N, batch, t->n_sm, t->flag, s),
+            "projection");
+        return BVF_OK;
+    }
+    bvf_gemm g = chan(t->v[L], W, w + o.Q1, t->h, d.hidden, N, batch);
     g.bias = w + o.q1;
     g.bias_mode = 1;
     g.act = 1;
-    g.C_pre = keep ? t->pre1 : nullptr;
+    g.C_pre = t->pre1;
     if ((rc = gemm(t, g, s, "projection 1")) != BVF_OK) return rc;
     g = chan(t->h, d.hidden, w + o.Q2, out, d.c_out, N, batch);
     g.bias = w + o.q2;
@@ -606,7 +649,6 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
         float *gR = gl, *gW = gl + (size_t)4 * m * m * m * W * W * 2, *gb = gW + (size_t)W * W;
         if ((rc = chan_sum(ds, batch, W, N, gb, s)) != BVF_OK) return rc;
         if ((rc = gemm(t, wgrad(ds, W, t->v[l], W, gW, N, batch, ks), s, "dW")) != BVF_OK) return rc;
-        if ((rc = gemm(t, chanT(ds, W, Wl, dn, W, N, batch), s, "d pointwise")) != BVF_OK) return rc;
         if ((rc = spec_fwd(t, ds, (long long)batch * W, true, t->S1, s)) != BVF_OK) return rc;
         k_mix_dR<<<grid_for((long long)4 * m * m * m * W * W), 256, 0, s>>>(t->S1, t->X[l], batch, W,
                                                                             m, gR);
@@ -614,8 +656,9 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
                                                                                  m, t->S2);
         BCK(cudaGetLastError(), "d mix");
         // dn = d v_l; for l > 0 it becomes d s_{l-1} = d v_l GELU'(s_{l-1})
-        if ((rc = spec_inv(t, t->S2, (long long)batch * W, false, dn, 1.0f, l > 0 ? 2 : 0,
-                           l > 0 ? t->s[l - 1] : nullptr, s)) != BVF_OK)
+        if ((rc = spec_inv_zy(t, t->S2, (long long)batch * W, s)) != BVF_OK) return rc;
+        if ((rc = row_pass(t, batch, ds, W, Wl, 1, W, nullptr, t->Gx, l > 0 ? 2 : 0,
+                           l > 0 ? t->s[l - 1] : nullptr, dn, s)) != BVF_OK)
             return rc;
         std::swap(ds, dn);
     }
@@ -674,6 +717,10 @@ int bvf_fno_bf16_create(bvf_fno_bf16 **out, const bvf_fno_dims *d, const float *
     };
     const size_t N = t->N, B = max_batch, W = d->width, H = d->hidden, S = 8 * (size_t)m * m * m;
     int rc = BVF_OK;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&t->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fail(b16_fail(BVF_E_CUDA, "bvf_fno_bf16_create: device"));
     for (float **p : {&t->w, &t->g, &t->m1, &t->m2})
         if ((rc = dalloc(t, p, n, "weights")) != BVF_OK) return fail(rc);
     std::vector<std::vector<float>> mats;

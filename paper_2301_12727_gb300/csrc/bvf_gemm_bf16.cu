@@ -19,15 +19,13 @@
 // Waits are bounded: a block whose wait runs out stops issuing products,
 // waits (bounded) for those in flight, frees its tensor memory, sets bit 2 of
 // the flag and ends.
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
-#include <atomic>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
-#include "../../include/bvf_fno.h"
-#include "bvf_internal.cuh"
+#include "bvf_fno_bf16.cuh"
 #include "bvf_tc.cuh"
 #include "bvf_tma.cuh"
 
@@ -48,30 +46,58 @@ struct GemmLayout {
     static constexpr int STAGE = A_BYTES + B_BYTES;
     static constexpr int off_bar = NS * STAGE;
     static constexpr int off_tmem = off_bar + 16;
-    static constexpr int bytes = off_tmem + 16;
+    static constexpr int off_rows = off_tmem + 16;     // [128] row starts of A, then of C
+    static constexpr int bytes = off_rows + 2 * 128 * 8;
     static_assert(NS * STAGE >= 4 * 32 * 33 * 4, "the epilogue's transpose buffers fit the stages");
     static constexpr uint32_t SBO = GSEG * 128;      // byte step between 8-row groups
 };
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
-{
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
+using tc::pack_bf16;
 
-// Rows [0, rows) x K-chunk [k0, k0 + GK) of a strided FP32 operand (element
-// (r, k) at src[r * srow + k * sk]; zero for r >= valid or k >= K) written as
-// BF16 in K-major core matrices.  With sk == 1 consecutive threads take
-// consecutive 8-element pieces of one row, otherwise consecutive rows, so the
-// global reads are coalesced in both layouts.
+// Rows [0, rows) x K-chunk [k0, k0 + GK) of an FP32 operand (element (r, k) at
+// src[start(r) + kof(k)]; zero for r >= valid or k >= K) written as BF16 in
+// K-major core matrices.  Where k is contiguous (kc), consecutive threads
+// take consecutive 8-element pieces of one row, otherwise consecutive rows,
+// so the global reads are coalesced in both layouts.  vec: the pieces load
+// as two float4 (aligned rows, four-element groups never straddle K or a part
+// of it); four pieces are in flight per thread, against eight floats of one:
+// the staging is bound by the latency of its loads.
+template <class Start, class Kof>
 __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__restrict__ src,
-                                           long long srow, long long sk, int rows, int valid,
-                                           int k0, int K, int tid)
+                                           Start start, Kof kof, bool kc, bool vec, int rows,
+                                           int valid, int k0, int K, int tid)
 {
     const int segs = rows * GSEG;
+    if (vec) {
+        constexpr int U = 4;
+        for (int s0 = tid; s0 < segs; s0 += 128 * U) {
+            float4 v[U][2];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int s = s0 + 128 * u, r = s / GSEG, k = k0 + (s % GSEG) * 8;
+                const bool on = s < segs && r < valid;
+                const float *row = src + (on ? start(r) : 0);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    v[u][h] = (on && k + 4 * h < K)
+                                  ? __ldg(reinterpret_cast<const float4 *>(row + kof(k + 4 * h)))
+                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int s = s0 + 128 * u;
+                if (s < segs)
+                    *reinterpret_cast<uint4 *>(dst + tc::kmaj_off16(s / GSEG, (s % GSEG) * 8, GK)) =
+                        make_uint4(pack_bf16(v[u][0].x, v[u][0].y), pack_bf16(v[u][0].z, v[u][0].w),
+                                   pack_bf16(v[u][1].x, v[u][1].y), pack_bf16(v[u][1].z, v[u][1].w));
+            }
+        }
+        return;
+    }
+#pragma unroll 2
     for (int s = tid; s < segs; s += 128) {
         int r, k8;
-        if (sk == 1) {
+        if (kc) {
             r = s / GSEG;
             k8 = (s % GSEG) * 8;
         } else {
@@ -79,11 +105,12 @@ __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__re
             k8 = (s / rows) * 8;
         }
         float v[8];
-        const float *row = src + (long long)r * srow;
+        const bool on = r < valid;
+        const float *row = src + (on ? start(r) : 0);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int k = k0 + k8 + j;
-            v[j] = (r < valid && k < K) ? __ldg(row + (long long)k * sk) : 0.0f;
+            v[j] = (on && k < K) ? __ldg(row + kof(k)) : 0.0f;
         }
         *reinterpret_cast<uint4 *>(dst + tc::kmaj_off16(r, k8, GK)) =
             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
@@ -91,20 +118,10 @@ __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__re
     }
 }
 
-__device__ __forceinline__ float gelu_exact(float s)
-{
-    return 0.5f * s * (1.0f + erff(s * 0.70710678118654752f));
-}
-// d GELU / ds = Phi(s) + s phi(s)
-__device__ __forceinline__ float gelu_grad(float s)
-{
-    return 0.5f * (1.0f + erff(s * 0.70710678118654752f)) +
-           s * 0.39894228040143268f * expf(-0.5f * s * s);
-}
-
 template <int BN, int NS>
-__global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ bvf_gemm g, int *flag)
+__global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX gx, int *flag)
 {
+    const bvf_gemm &g = gx.g;
     extern __shared__ __align__(128) unsigned char sm[];
     using Lay = GemmLayout<BN, NS>;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + Lay::off_bar);
@@ -115,9 +132,24 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ bvf_g
     const int n_chunks = (g.K + GK - 1) / GK;
     const int per = (n_chunks + g.ksplit - 1) / g.ksplit;
     const int c_begin = split * per, c_end = min(n_chunks, c_begin + per);
-    const float *A = g.A + (long long)b * g.sab + (long long)m0 * g.sam;
+    const float *A = g.A + (long long)b * g.sab;
     const float *B = g.B + (long long)b * g.sbb + (long long)n0 * g.sbn;
     const int va = min(128, g.M - m0), vb = min(BN, g.N - n0);
+    // where the tile's rows start in A and C
+    long long *s_ar = reinterpret_cast<long long *>(sm + Lay::off_rows), *s_cr = s_ar + 128;
+    {
+        const int r = m0 + tid;
+        s_ar[tid] = gx.ra ? (r / (gx.ra * gx.ra2)) * gx.sam2 + (r / gx.ra % gx.ra2) * gx.sam1 +
+                                (r % gx.ra) * g.sam
+                          : (long long)r * g.sam;
+        s_cr[tid] = gx.rc ? (r / gx.rc) * gx.scm1 + (r % gx.rc) * g.scm : (long long)r * g.scm;
+    }
+    auto a_row = [&](int r) { return s_ar[r]; };
+    auto a_col = [&](int k) -> long long {
+        return gx.ka ? (k < gx.ka ? k * g.sak : gx.sak1 + (k - gx.ka) * g.sak) : k * g.sak;
+    };
+    auto b_row = [&](int r) { return (long long)r * g.sbn; };
+    auto b_col = [&](int k) { return (long long)k * g.sbk; };
     if (tid == 0) {
         tma::mbar_init(&bar[0], 1);
         tma::mbar_init(&bar[1], 1);
@@ -145,8 +177,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ bvf_g
                 break;
             }
         }
-        stage_tile(sa, A, g.sam, g.sak, 128, va, c * GK, g.K, tid);
-        stage_tile(sb, B, g.sbn, g.sbk, BN, vb, c * GK, g.K, tid);
+        stage_tile(sa, A, a_row, a_col, g.sak == 1, gx.vec & 1, 128, va, c * GK, g.K, tid);
+        stage_tile(sb, B, b_row, b_col, g.sbk == 1, gx.vec & 2, BN, vb, c * GK, g.K, tid);
         tma::fence_async_smem();
         tc::fence_before();
         __syncthreads();
@@ -176,10 +208,10 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ bvf_g
         tc::fence_after();
         // element (mm, n) of the tile: alpha, beta C, bias, activation, store
         auto finish = [&](int mm, int n, float acc) {
-            float *cp = g.C + (long long)b * g.scb + (long long)mm * g.scm + (long long)n * g.scn;
-            float *pp = g.C_pre ? g.C_pre + (long long)b * g.scb + (long long)mm * g.scm +
-                                      (long long)n * g.scn
-                                : nullptr;
+            const long long nn = gx.nc && n >= gx.nc ? gx.scn1 + (n - gx.nc) * g.scn : n * g.scn;
+            const long long at = (long long)b * g.scb + s_cr[mm - m0] + nn;
+            float *cp = g.C + at;
+            float *pp = g.C_pre ? g.C_pre + at : nullptr;
             float v = g.alpha * acc;
             if (g.ksplit > 1) {
                 if (nc > 0) atomicAdd(cp, v);
@@ -242,8 +274,9 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ bvf_g
 }
 
 template <int BN, int NS>
-cudaError_t launch_gemm_ns(const bvf_gemm &g, int *flag, cudaStream_t s)
+cudaError_t launch_gemm_ns(const GemmX &x, int *flag, cudaStream_t s)
 {
+    const bvf_gemm &g = x.g;
     const dim3 grid((g.M + 127) / 128, (g.N + BN - 1) / BN, g.batch * g.ksplit);
     // the shared-memory limit is raised once per process, so that later
     // launches make no other runtime call (a forward can be recorded in a graph)
@@ -255,31 +288,40 @@ cudaError_t launch_gemm_ns(const bvf_gemm &g, int *flag, cudaStream_t s)
         if (e != cudaSuccess) return e;
         raised.store(1, std::memory_order_release);
     }
-    k_gemm_bf16<BN, NS><<<grid, 128, GemmLayout<BN, NS>::bytes, s>>>(g, flag);
+    k_gemm_bf16<BN, NS><<<grid, 128, GemmLayout<BN, NS>::bytes, s>>>(x, flag);
     return cudaGetLastError();
 }
 
 // one stage when the product is a single K chunk
 template <int BN>
-cudaError_t launch_gemm_t(const bvf_gemm &g, int *flag, cudaStream_t s)
+cudaError_t launch_gemm_t(const GemmX &x, int *flag, cudaStream_t s)
 {
-    const int per_split = ((g.K + GK - 1) / GK + g.ksplit - 1) / g.ksplit;
-    return per_split <= 1 ? launch_gemm_ns<BN, 1>(g, flag, s) : launch_gemm_ns<BN, 2>(g, flag, s);
+    const int per_split = ((x.g.K + GK - 1) / GK + x.g.ksplit - 1) / x.g.ksplit;
+    return per_split <= 1 ? launch_gemm_ns<BN, 1>(x, flag, s) : launch_gemm_ns<BN, 2>(x, flag, s);
 }
 
 }  // namespace
 
 // BN: the smallest tile width of 32, 64, 128, 256 that holds N (256 beyond),
 // at most 64 for a single-chunk product
-cudaError_t launch_gemm_bf16(const bvf_gemm &g, int *flag, cudaStream_t s)
+cudaError_t launch_gemm_bf16(const GemmX &gx, int *flag, cudaStream_t s)
 {
-    if (g.N <= 32) return launch_gemm_t<32>(g, flag, s);
+    GemmX x = gx;
+    const bvf_gemm &g = x.g;
+    auto al4 = [](long long v) { return v % 4 == 0; };
+    auto al16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    x.vec = (g.sak == 1 && g.K % 4 == 0 && al16(g.A) && al4(g.sam) && al4(g.sab) && al4(x.sam1) &&
+             al4(x.sam2) && al4(x.ka) && al4(x.sak1))
+                ? 1
+                : 0;
+    if (g.sbk == 1 && g.K % 4 == 0 && al16(g.B) && al4(g.sbn) && al4(g.sbb)) x.vec |= 2;
+    if (g.N <= 32) return launch_gemm_t<32>(x, flag, s);
     // a single-chunk product restages its small A tile per N tile but keeps
     // 64 TMEM columns per block, so up to 8 blocks share an SM's 512
     const int per_split = ((g.K + GK - 1) / GK + g.ksplit - 1) / g.ksplit;
-    if (g.N <= 64 || per_split <= 1) return launch_gemm_t<64>(g, flag, s);
-    if (g.N <= 128) return launch_gemm_t<128>(g, flag, s);
-    return launch_gemm_t<256>(g, flag, s);
+    if (g.N <= 64 || per_split <= 1) return launch_gemm_t<64>(x, flag, s);
+    if (g.N <= 128) return launch_gemm_t<128>(x, flag, s);
+    return launch_gemm_t<256>(x, flag, s);
 }
 
 }  // namespace bvf
@@ -294,7 +336,9 @@ extern "C" int bvf_gemm_bf16(const bvf_gemm *g, int *d_flag, void *stream)
         bvf::set_context_free_error("bvf_gemm_bf16: bad argument");
         return BVF_E_ARG;
     }
-    const cudaError_t e = bvf::launch_gemm_bf16(*g, d_flag, static_cast<cudaStream_t>(stream));
+    bvf::GemmX x;
+    x.g = *g;
+    const cudaError_t e = bvf::launch_gemm_bf16(x, d_flag, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
         bvf::set_context_free_error(cudaGetErrorString(e));
         return BVF_E_CUDA;

@@ -10,6 +10,7 @@
 // back to registers.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 #include "bvf_tma.cuh"
@@ -111,6 +112,13 @@ __device__ __forceinline__ void ld8(uint32_t taddr, float (&r)[8])
                  : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < 8; ++i) r[i] = __uint_as_float(u[i]);
+}
+
+// two values rounded to BF16 (to nearest), the first in the low half
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
 }
 
 // byte offset of element (row, k) in a K-major TF32 operand with K columns
