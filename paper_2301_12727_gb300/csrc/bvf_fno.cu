@@ -192,76 +192,139 @@ __global__ void k_dftx(const float *__restrict__ v, int rows, int nx, int m,
     }
 }
 
-// complex a * e^{s i theta} with the table entry t = (cos, sin) and s = +-1
-__device__ __forceinline__ float2 cmul_tw(float2 a, float2 t, float s)
+// --------------------------------------------- transforms along y and z
+// Only 2m of the n frequencies of an axis survive, in classes f = 0 .. m of
+// slots: f = 0 and f = m (slot m, frequency -m) alone, 0 < f < m with -f (slot
+// 2m - f).  A direct sum over the kept frequencies shares its products twice:
+// +f and -f need the same four sums (a cos, b cos, a sin, b sin), and the
+// samples j and n - j have the same cosine and opposite sines, so they are
+// folded to a(j) + a(n - j) and a(j) - a(n - j) first (forward) or leave as a
+// pair (inverse): a quarter of the multiplications of a sum per slot.  MC: an
+// upper bound of the classes, m + 1 <= MC (9, 13 or 17).
+// At 240 x 240 x 200 (width 32, m 12) a sum per slot took 249 (y), 83 (z), 62
+// (inverse z) and 196 us (inverse y), now 131, 28, 40 and 102; at 64 x 64 x 96
+// the four took 150 of 296 us a layer, now 74.
+
+// half-range of an axis: j = 0 .. n/2, with n - j as the partner of j where
+// they differ
+__device__ __forceinline__ int half_len(int n) { return n / 2 + 1; }
+__device__ __forceinline__ bool has_partner(int j, int n) { return j > 0 && 2 * j != n; }
+
+// four sums of a class -> the spectra at +f (e^{-i theta}) and -f
+__device__ __forceinline__ float2 spec_plus(float4 s) { return make_float2(s.x + s.w, s.y - s.z); }
+__device__ __forceinline__ float2 spec_minus(float4 s) { return make_float2(s.x - s.w, s.y + s.z); }
+// s += (a+ cos, b+ cos, a- sin, b- sin), p = (a+, b+, a-, b-), t = (cos, sin)
+__device__ __forceinline__ void class_add(float4 &s, float4 p, float2 t)
 {
-    return make_float2(a.x * t.x - s * a.y * t.y, a.y * t.x + s * a.x * t.y);
+    s.x = fmaf(p.x, t.x, s.x);
+    s.y = fmaf(p.y, t.x, s.y);
+    s.z = fmaf(p.z, t.y, s.z);
+    s.w = fmaf(p.w, t.y, s.w);
+}
+__device__ __forceinline__ float4 fold(float2 a, float2 b, bool both)
+{
+    return both ? make_float4(a.x + b.x, a.y + b.y, a.x - b.x, a.y - b.y)
+                : make_float4(a.x, a.y, a.x, a.y);
+}
+// the pair of spectral values of a class, as P = G+ + G- and D = G+ - G-
+// (a class of one slot: P = D = G): the sample at j is
+// (P.x c - D.y s, P.y c + D.x s), at n - j with the sign of s turned
+__device__ __forceinline__ float4 unfold(float2 gp, float2 gm, bool both)
+{
+    return both ? make_float4(gp.x + gm.x, gp.y + gm.y, gp.x - gm.x, gp.y - gm.y)
+                : make_float4(gp.x, gp.y, gp.x, gp.y);
 }
 
-// ------------------------------------------------------ forward DFT along y
-// B[c][z][jy][kx] = sum_y A[c][z][y][kx] e^{-2 pi i f(jy) y / ny}; one block
-// per (c, z) slab; each thread takes the mode slots jy and jy + m of one kx
-// (the same A column against two twiddle rows).
-__global__ void k_dfty(const float2 *__restrict__ A, int ny, int m,
+// B[slab][jy][kx] = sum_y A[slab][y][kx] e^{-2 pi i f(jy) y / ny} for the slabs
+// (c, z).  Blocks walk over slabs: fold the slab's rows into shared memory,
+// then thread (class, kx) sums the half-range; the class twiddles stay in
+// shared memory.  Bound by its reads of A and the fold's shared-memory traffic.
+__global__ void k_dfty(const float2 *__restrict__ A, int slabs, int ny, int m,
                        const float2 *__restrict__ ty, float2 *__restrict__ B)
 {
-    extern __shared__ float2 s_y[];
-    float2 *s_a = s_y;                  // [ny][m]
-    const long slab = blockIdx.x;
-    const float2 *a = A + slab * ny * m;
-    for (int e = threadIdx.x; e < ny * m; e += blockDim.x) s_a[e] = a[e];
-    __syncthreads();
-    const int t = threadIdx.x;
-    if (t >= m * m) return;
-    const int jy = t / m, kx = t - jy * m;           // jy in [0, m); the pair is jy + m
-    const float2 *tw0 = ty + (long)jy * ny, *tw1 = ty + (long)(jy + m) * ny;
-    float2 a0[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}}, a1[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
-    int y = 0;
-    for (; y + 2 <= ny; y += 2) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const float2 v = s_a[(y + q) * m + kx];
-            const float2 p0 = cmul_tw(v, __ldg(tw0 + y + q), -1.0f);
-            const float2 p1 = cmul_tw(v, __ldg(tw1 + y + q), -1.0f);
-            a0[q].x += p0.x;
-            a0[q].y += p0.y;
-            a1[q].x += p1.x;
-            a1[q].y += p1.y;
+    extern __shared__ __align__(16) float4 s_y4[];
+    const int nh = half_len(ny), nc = m + 1;
+    float4 *s_a = s_y4;                                        // [nh][m]
+    float2 *s_t = reinterpret_cast<float2 *>(s_y4 + nh * m);   // [nc][nh]
+    for (int e = threadIdx.x; e < nc * nh; e += blockDim.x) {
+        const int f = e / nh, y = e - f * nh;
+        s_t[e] = ty[(long)f * ny + y];
+    }
+    const int t = threadIdx.x, f = t / m, kx = t - f * m;
+    for (int slab = blockIdx.x; slab < slabs; slab += gridDim.x) {
+        const float2 *a = A + (long)slab * ny * m;
+        __syncthreads();
+        for (int e = threadIdx.x; e < nh * m; e += blockDim.x) {
+            const int y = e / m, k = e - y * m;
+            const bool both = has_partner(y, ny);
+            s_a[e] = fold(a[e], both ? a[(ny - y) * m + k] : make_float2(0.0f, 0.0f), both);
+        }
+        __syncthreads();
+        if (t < nc * m) {
+            float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const float4 *p = s_a + kx;
+            const float2 *tw = s_t + f * nh;
+#pragma unroll 4
+            for (int y = 0; y < nh; ++y) class_add(s, p[y * m], tw[y]);
+            float2 *out = B + (long)slab * 2 * m * m + kx;
+            out[f * m] = spec_plus(s);
+            if (f > 0 && f < m) out[(2 * m - f) * m] = spec_minus(s);
         }
     }
-    for (; y < ny; ++y) {
-        const float2 v = s_a[y * m + kx];
-        const float2 p0 = cmul_tw(v, __ldg(tw0 + y), -1.0f);
-        const float2 p1 = cmul_tw(v, __ldg(tw1 + y), -1.0f);
-        a0[0].x += p0.x;
-        a0[0].y += p0.y;
-        a1[0].x += p1.x;
-        a1[0].y += p1.y;
-    }
-    B[(slab * 2 * m + jy) * m + kx] = make_float2(a0[0].x + a0[1].x, a0[0].y + a0[1].y);
-    B[(slab * 2 * m + jy + m) * m + kx] = make_float2(a1[0].x + a1[1].x, a1[0].y + a1[1].y);
 }
 
-// ------------------------------------------------------ forward DFT along z
-// H[c][jz][q] = sum_z B[c][z][q] e^{-2 pi i f(jz) z / nz}, q = (jy, kx).
-__global__ void k_dftz(const float2 *__restrict__ B, int nz, int m, int width,
-                       const float2 *__restrict__ tz, float2 *__restrict__ H)
+// H[c][jz][q] = sum_z B[c][z][q] e^{-2 pi i f(jz) z / nz}, q = (jy, kx).  Thread
+// (q, g) sums every class over the half-range planes z = g, g + 8, ...; the
+// eight partial sums of a q meet in shared memory.
+constexpr int kZg = 8;
+template <int MC>
+__global__ void __launch_bounds__(32 * kZg)
+    k_dftz(const float2 *__restrict__ B, int nz, int m, const float2 *__restrict__ tz,
+           float2 *__restrict__ H)
 {
-    const int M2 = 2 * m * m;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)width * 2 * m * M2) return;
-    const int q = (int)(t % M2);
-    const long rest = t / M2;
-    const int jz = (int)(rest % (2 * m)), c = (int)(rest / (2 * m));
-    const float2 *b = B + (long)c * nz * M2 + q;
-    const float2 *tw = tz + (long)jz * nz;
-    float2 acc = make_float2(0.0f, 0.0f);
-    for (int z = 0; z < nz; ++z) {
-        const float2 p = cmul_tw(b[(long)z * M2], __ldg(tw + z), -1.0f);
-        acc.x += p.x;
-        acc.y += p.y;
+    __shared__ float4 s_p[kZg / 2][MC][32];
+    const int M2 = 2 * m * m, nh = half_len(nz);
+    const int lane = threadIdx.x, g = threadIdx.y, q = blockIdx.x * 32 + lane, c = blockIdx.y;
+    float4 s[MC];
+#pragma unroll
+    for (int f = 0; f < MC; ++f) s[f] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (q < M2) {
+        const float2 *b = B + (long)c * nz * M2 + q;
+#pragma unroll 2
+        for (int z = g; z < nh; z += kZg) {
+            const bool both = has_partner(z, nz);
+            const float4 p = fold(b[(long)z * M2],
+                                  both ? b[(long)(nz - z) * M2] : make_float2(0.0f, 0.0f), both);
+#pragma unroll
+            for (int f = 0; f < MC; ++f)
+                if (f <= m) class_add(s[f], p, __ldg(tz + (long)f * nz + z));
+        }
     }
-    H[t] = acc;     // t = (c * 2m + jz) * M2 + q
+#pragma unroll
+    for (int h = kZg / 2; h > 0; h >>= 1) {
+        __syncthreads();
+        if (g >= h && g < 2 * h) {
+#pragma unroll
+            for (int f = 0; f < MC; ++f) s_p[g - h][f][lane] = s[f];
+        }
+        __syncthreads();
+        if (g < h) {
+#pragma unroll
+            for (int f = 0; f < MC; ++f) {
+                const float4 p = s_p[g][f][lane];
+                s[f] = make_float4(s[f].x + p.x, s[f].y + p.y, s[f].z + p.z, s[f].w + p.w);
+            }
+        }
+    }
+    if (g == 0 && q < M2) {
+        float2 *h = H + (long)c * 2 * m * M2 + q;
+#pragma unroll
+        for (int f = 0; f < MC; ++f)
+            if (f <= m) {
+                h[(long)f * M2] = spec_plus(s[f]);
+                if (f > 0 && f < m) h[(long)(2 * m - f) * M2] = spec_minus(s[f]);
+            }
+    }
 }
 
 // ------------------------------------------------------------ mode mixing
@@ -278,6 +341,7 @@ __global__ void k_mix(const float2 *__restrict__ H, const float2 *__restrict__ R
     if (mode >= n_modes) return;
     const float2 *r = R + (long)mode * width * width + o;
     float2 acc = make_float2(0.0f, 0.0f);
+#pragma unroll 8
     for (int c = 0; c < width; ++c) {
         const float2 w = r[(long)c * width], h = s_h[ty * width + c];
         acc.x = fmaf(w.x, h.x, fmaf(-w.y, h.y, acc.x));
@@ -286,58 +350,70 @@ __global__ void k_mix(const float2 *__restrict__ H, const float2 *__restrict__ R
     G[(long)o * n_modes + mode] = acc;
 }
 
-// ------------------------------------------------------ inverse along z
-// B'[o][z][q] = sum_jz G[o][jz][q] e^{+2 pi i f(jz) z / nz}
-__global__ void k_idftz(const float2 *__restrict__ G, int nz, int m, int width,
-                        const float2 *__restrict__ tz, float2 *__restrict__ Bp)
+// ------------------------------------------------- inverse along z and y
+// B'[o][z][q] = sum_jz G[o][jz][q] e^{+2 pi i f(jz) z / nz}: thread (q, g) holds
+// the classes of its q and writes the planes z and nz - z for z = g, g + 8, ...
+template <int MC>
+__global__ void __launch_bounds__(32 * kZg)
+    k_idftz(const float2 *__restrict__ G, int nz, int m, const float2 *__restrict__ tz,
+            float2 *__restrict__ Bp)
 {
-    const int M2 = 2 * m * m;
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (long)width * nz * M2) return;
-    const int q = (int)(t % M2);
-    const long rest = t / M2;
-    const int z = (int)(rest % nz), o = (int)(rest / nz);
-    const float2 *g = G + (long)o * 2 * m * M2 + q;
-    float2 acc = make_float2(0.0f, 0.0f);
-    for (int jz = 0; jz < 2 * m; ++jz) {
-        const float2 p = cmul_tw(g[(long)jz * M2], __ldg(tz + (long)jz * nz + z), 1.0f);
-        acc.x += p.x;
-        acc.y += p.y;
+    const int M2 = 2 * m * m, nh = half_len(nz);
+    const int q = blockIdx.x * 32 + threadIdx.x, o = blockIdx.y;
+    if (q >= M2) return;
+    const float2 *gq = G + (long)o * 2 * m * M2 + q;
+    float4 p[MC];
+#pragma unroll
+    for (int f = 0; f < MC; ++f) {
+        const bool both = f > 0 && f < m;
+        p[f] = f <= m ? unfold(gq[(long)f * M2],
+                               both ? gq[(long)(2 * m - f) * M2] : make_float2(0.0f, 0.0f), both)
+                      : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
-    Bp[t] = acc;    // t = (o * nz + z) * M2 + q
+    float2 *out = Bp + (long)o * nz * M2 + q;
+    for (int z = threadIdx.y; z < nh; z += kZg) {
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // P.x c, P.y c, D.x s, D.y s
+#pragma unroll
+        for (int f = 0; f < MC; ++f)
+            if (f <= m) class_add(s, p[f], __ldg(tz + (long)f * nz + z));
+        out[(long)z * M2] = make_float2(s.x - s.w, s.y + s.z);
+        if (has_partner(z, nz)) out[(long)(nz - z) * M2] = make_float2(s.x + s.w, s.y - s.z);
+    }
 }
 
-// ------------------------------------------------------ inverse along y
-// A'[o][z][y][kx] = sum_jy B'[o][z][jy][kx] e^{+2 pi i f(jy) y / ny}; one block
-// per (o, z) slab.
-__global__ void k_idfty(const float2 *__restrict__ Bp, int ny, int m,
+// A'[slab][y][kx] = sum_jy B'[slab][jy][kx] e^{+2 pi i f(jy) y / ny}.  Blocks
+// walk over the slabs (o, z); a thread writes y and ny - y of one kx, the
+// slab's classes and the twiddles come from shared memory.
+__global__ void k_idfty(const float2 *__restrict__ Bp, int slabs, int ny, int m,
                         const float2 *__restrict__ ty, float2 *__restrict__ Ap)
 {
-    extern __shared__ float2 s_y[];
-    const int M2 = 2 * m * m;
-    float2 *s_b = s_y;               // [2m][m]
-    const long slab = blockIdx.x;
-    for (int e = threadIdx.x; e < M2; e += blockDim.x) s_b[e] = Bp[slab * M2 + e];
-    __syncthreads();
-    float2 *out = Ap + slab * ny * m;
-    // two y per thread (y0, y0 + 1) share each spectral value
-    const int npairs = (ny + 1) / 2;
-    for (int e = threadIdx.x; e < npairs * m; e += blockDim.x) {
-        const int yp = e / m, kx = e - yp * m;
-        const int y0 = 2 * yp, y1 = y0 + 1 < ny ? y0 + 1 : y0;
-        float2 acc0 = make_float2(0.0f, 0.0f), acc1 = make_float2(0.0f, 0.0f);
-        for (int jy = 0; jy < 2 * m; ++jy) {
-            const float2 b = s_b[jy * m + kx];
-            const float2 *tw = ty + (long)jy * ny;
-            const float2 p0 = cmul_tw(b, __ldg(tw + y0), 1.0f);
-            const float2 p1 = cmul_tw(b, __ldg(tw + y1), 1.0f);
-            acc0.x += p0.x;
-            acc0.y += p0.y;
-            acc1.x += p1.x;
-            acc1.y += p1.y;
+    extern __shared__ __align__(16) float4 s_y4[];
+    const int nh = half_len(ny), nc = m + 1, M2 = 2 * m * m;
+    float4 *s_b = s_y4;                                         // [nc][m]
+    float2 *s_t = reinterpret_cast<float2 *>(s_y4 + nc * m);    // [nh][nc]
+    for (int e = threadIdx.x; e < nc * nh; e += blockDim.x) {
+        const int f = e / nh, y = e - f * nh;
+        s_t[y * nc + f] = ty[(long)f * ny + y];
+    }
+    for (int slab = blockIdx.x; slab < slabs; slab += gridDim.x) {
+        const float2 *b = Bp + (long)slab * M2;
+        __syncthreads();
+        for (int e = threadIdx.x; e < nc * m; e += blockDim.x) {
+            const int f = e / m, kx = e - f * m;
+            const bool both = f > 0 && f < m;
+            s_b[e] = unfold(b[e], both ? b[(2 * m - f) * m + kx] : make_float2(0.0f, 0.0f), both);
         }
-        out[y0 * m + kx] = acc0;
-        if (y0 + 1 < ny) out[(y0 + 1) * m + kx] = acc1;
+        __syncthreads();
+        float2 *out = Ap + (long)slab * ny * m;
+        for (int e = threadIdx.x; e < nh * m; e += blockDim.x) {
+            const int y = e / m, kx = e - y * m;
+            float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const float2 *tw = s_t + y * nc;
+#pragma unroll 4
+            for (int f = 0; f < nc; ++f) class_add(s, s_b[f * m + kx], tw[f]);
+            out[e] = make_float2(s.x - s.w, s.y + s.z);
+            if (has_partner(y, ny)) out[(ny - y) * m + kx] = make_float2(s.x + s.w, s.y - s.z);
+        }
     }
 }
 
@@ -876,7 +952,7 @@ struct ProjTcLayout {
     }
 };
 
-template <int W, int COUT>     // COUT: output count rounded up to 1 or 8
+template <int W, int COUT>     // COUT: output count rounded up to 1, 2, 4 or 8
 __global__ void __launch_bounds__(256, 2)
 k_project_tc(const float *__restrict__ v, const float *__restrict__ Q1, const float *__restrict__ q1,
              const float *__restrict__ Q2, const float *__restrict__ q2, int hidden, int c_out,
@@ -1423,9 +1499,18 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     }
     FCK(mark(0), "event");
 
-    const size_t sy = (size_t)ny * m * sizeof(float2);
-    FCK(smem_at_least<k_dfty>(sy),
-        "bvf_fno_forward: dfty smem");
+    // y transforms: shared memory of a block, and blocks that fill the GPU
+    const size_t nhy = ny / 2 + 1, tw_y = (size_t)(m + 1) * nhy * sizeof(float2);
+    const size_t sy = nhy * m * sizeof(float4) + tw_y;
+    const size_t siy = (size_t)(m + 1) * m * sizeof(float4) + tw_y;
+    FCK(smem_at_least<k_dfty>(sy), "bvf_fno_forward: dfty smem");
+    FCK(smem_at_least<k_idfty>(siy), "bvf_fno_forward: idfty smem");
+    const int slabs = W * nz, ty_threads = ((m + 1) * m + 31) / 32 * 32;
+    auto y_grid = [&](size_t smem, int threads) {
+        const int fit = (int)std::min<size_t>(2048 / threads, (size_t)227 * 1024 / (smem + 1024));
+        return std::min(slabs, n_sm * std::max(1, fit));
+    };
+    const dim3 zg((2 * m * m + 31) / 32, W), zb(32, kZg);
     const size_t s_out = ((size_t)W * W + W + 1) * sizeof(float) + (size_t)W * m * sizeof(float2);
     const int rows_x = W * nz * ny;
     const int bo = std::min(256, ((nx + 31) / 32) * 32);
@@ -1441,11 +1526,15 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
             FCK(cudaGetLastError(), "bvf_fno_forward: dftx");
         }
         FCK(mark(1), "event");
-        k_dfty<<<W * nz, std::max(32, ((m * m + 31) / 32) * 32), sy, s>>>(f->A, ny, m, ty, f->B);
+        k_dfty<<<y_grid(sy, ty_threads), ty_threads, sy, s>>>(f->A, slabs, ny, m, ty, f->B);
         FCK(cudaGetLastError(), "bvf_fno_forward: dfty");
         FCK(mark(2), "event");
-        const long nh = (long)W * 2 * m * M2;
-        k_dftz<<<(unsigned)((nh + TB - 1) / TB), TB, 0, s>>>(f->B, nz, m, W, tz, f->H);
+        if (m < 9)
+            k_dftz<9><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
+        else if (m < 13)
+            k_dftz<13><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
+        else
+            k_dftz<17><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
         FCK(cudaGetLastError(), "bvf_fno_forward: dftz");
         FCK(mark(3), "event");
         const dim3 mb(W, 256 / W);
@@ -1453,11 +1542,15 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
                                                                                  n_modes, f->G);
         FCK(cudaGetLastError(), "bvf_fno_forward: mix");
         FCK(mark(4), "event");
-        const long nb = (long)W * nz * M2;
-        k_idftz<<<(unsigned)((nb + TB - 1) / TB), TB, 0, s>>>(f->G, nz, m, W, tz, f->B);
+        if (m < 9)
+            k_idftz<9><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
+        else if (m < 13)
+            k_idftz<13><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
+        else
+            k_idftz<17><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
         FCK(cudaGetLastError(), "bvf_fno_forward: idftz");
         FCK(mark(5), "event");
-        k_idfty<<<W * nz, TB, (size_t)M2 * sizeof(float2), s>>>(f->B, ny, m, ty, f->A);
+        k_idfty<<<y_grid(siy, TB), TB, siy, s>>>(f->B, slabs, ny, m, ty, f->A);
         FCK(cudaGetLastError(), "bvf_fno_forward: idfty");
         FCK(mark(6), "event");
         const int act = l < d.n_layers - 1;
@@ -1480,7 +1573,7 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
         std::swap(vc, vn);
     }
     {
-        const int cp = d.c_out == 1 ? 1 : 8;
+        const int cp = d.c_out <= 2 ? d.c_out : (d.c_out <= 4 ? 4 : 8);
         const ProjTcLayout pl(W, d.hidden, cp);
         const long tiles = (N64 + 127) / 128;
         const int per_sm = std::max(1, std::min(2, 512 / pl.ncols));
@@ -1491,21 +1584,20 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     if (e == cudaSuccess)                                                                      \
         k_project_tc<WW, CP><<<grid, 256, pl.bytes, s>>>(vc, Q1, q1, Q2, q2, d.hidden, d.c_out, \
                                                         d_out, N, f->flag);
-        if (cp == 1) {
-            switch (W) {
-            case 16: BVF_PRJ(16, 1) break;
-            case 32: BVF_PRJ(32, 1) break;
-            case 48: BVF_PRJ(48, 1) break;
-            default: BVF_PRJ(64, 1) break;
-            }
-        } else {
-            switch (W) {
-            case 16: BVF_PRJ(16, 8) break;
-            case 32: BVF_PRJ(32, 8) break;
-            case 48: BVF_PRJ(48, 8) break;
-            default: BVF_PRJ(64, 8) break;
-            }
+#define BVF_PRJ_W(CP)                     \
+    switch (W) {                          \
+    case 16: BVF_PRJ(16, CP) break;       \
+    case 32: BVF_PRJ(32, CP) break;       \
+    case 48: BVF_PRJ(48, CP) break;       \
+    default: BVF_PRJ(64, CP) break;       \
+    }
+        switch (cp) {
+        case 1: BVF_PRJ_W(1) break;
+        case 2: BVF_PRJ_W(2) break;
+        case 4: BVF_PRJ_W(4) break;
+        default: BVF_PRJ_W(8) break;
         }
+#undef BVF_PRJ_W
 #undef BVF_PRJ
         FCK(e, "bvf_fno_forward: project smem");
     }
