@@ -202,12 +202,12 @@ __global__ void k_dftx(const float *__restrict__ v, int rows, int nx, int m,
 // pair (inverse): a quarter of the multiplications of a sum per slot.  MC: an
 // upper bound of the classes, m + 1 <= MC (9, 13 or 17).
 // At 240 x 240 x 200 (width 32, m 12) a sum per slot took 249 (y), 83 (z), 62
-// (inverse z) and 196 us (inverse y), now 131, 28, 40 and 102; at 64 x 64 x 96
-// the four took 150 of 296 us a layer, now 74.
+// (inverse z) and 196 us (inverse y), now 87, 14, 16 and 78; at 64 x 64 x 96
+// the four took 150 of 296 us a layer, now 57.
 
 // half-range of an axis: j = 0 .. n/2, with n - j as the partner of j where
 // they differ
-__device__ __forceinline__ int half_len(int n) { return n / 2 + 1; }
+__host__ __device__ __forceinline__ int half_len(int n) { return n / 2 + 1; }
 __device__ __forceinline__ bool has_partner(int j, int n) { return j > 0 && 2 * j != n; }
 
 // four sums of a class -> the spectra at +f (e^{-i theta}) and -f
@@ -235,186 +235,303 @@ __device__ __forceinline__ float4 unfold(float2 gp, float2 gm, bool both)
                 : make_float4(gp.x, gp.y, gp.x, gp.y);
 }
 
-// B[slab][jy][kx] = sum_y A[slab][y][kx] e^{-2 pi i f(jy) y / ny} for the slabs
-// (c, z).  Blocks walk over slabs: fold the slab's rows into shared memory,
-// then thread (class, kx) sums the half-range; the class twiddles stay in
-// shared memory.  Bound by its reads of A and the fold's shared-memory traffic.
-__global__ void k_dfty(const float2 *__restrict__ A, int slabs, int ny, int m,
-                       const float2 *__restrict__ ty, float2 *__restrict__ B)
+// Both axes are columns of one shape: in[outer][j < n][inner], the sum over j
+// for every (outer, inner) column; y: outer (c, z), inner kx; z: outer c, inner
+// (jy, kx).  A thread holds every class of its column (4 (m + 1) sums) and
+// reads its samples once, neighbouring threads neighbouring columns; up to 8
+// threads share a column, sample pairs j = g, g + G, ..., where there are too
+// few columns to fill the GPU.  tab[j][f]: the class twiddles of sample j, read
+// two classes at a time at an address the whole warp shares.  (One block per
+// slab with the folded rows in shared memory, one thread per class and kx,
+// took 131 us for y at 240 x 240 x 200: bound by its shared-memory reads, one
+// 16-byte pair for every four products.)
+// A thread takes NC = 2 neighbouring columns where inner is even (16-byte
+// accesses, and each twiddle read serves eight products): with one column the
+// kernels waited on their loads (21 % and 26 % of issue slots used, 148 and
+// 113 us for y at 240 x 240 x 200).
+constexpr int kColGroups = 8;
+__host__ __device__ __forceinline__ int class_pitch(int m) { return (m + 2) / 2 * 2; }
+
+constexpr int kColDepth = 5;      // sample pairs in flight per thread
+template <int BYTES>              // 8 or 16, both addresses aligned to it
+__device__ __forceinline__ void cp_async(void *dst, const void *src)
 {
-    extern __shared__ __align__(16) float4 s_y4[];
-    const int nh = half_len(ny), nc = m + 1;
-    float4 *s_a = s_y4;                                        // [nh][m]
-    float2 *s_t = reinterpret_cast<float2 *>(s_y4 + nh * m);   // [nc][nh]
-    for (int e = threadIdx.x; e < nc * nh; e += blockDim.x) {
-        const int f = e / nh, y = e - f * nh;
-        s_t[e] = ty[(long)f * ny + y];
-    }
-    const int t = threadIdx.x, f = t / m, kx = t - f * m;
-    for (int slab = blockIdx.x; slab < slabs; slab += gridDim.x) {
-        const float2 *a = A + (long)slab * ny * m;
-        __syncthreads();
-        for (int e = threadIdx.x; e < nh * m; e += blockDim.x) {
-            const int y = e / m, k = e - y * m;
-            const bool both = has_partner(y, ny);
-            s_a[e] = fold(a[e], both ? a[(ny - y) * m + k] : make_float2(0.0f, 0.0f), both);
-        }
-        __syncthreads();
-        if (t < nc * m) {
-            float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            const float4 *p = s_a + kx;
-            const float2 *tw = s_t + f * nh;
-#pragma unroll 4
-            for (int y = 0; y < nh; ++y) class_add(s, p[y * m], tw[y]);
-            float2 *out = B + (long)slab * 2 * m * m + kx;
-            out[f * m] = spec_plus(s);
-            if (f > 0 && f < m) out[(2 * m - f) * m] = spec_minus(s);
-        }
-    }
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(bvf::tma::saddr(dst)), "l"(src),
+                 "n"(BYTES)
+                 : "memory");
 }
 
-// H[c][jz][q] = sum_z B[c][z][q] e^{-2 pi i f(jz) z / nz}, q = (jy, kx).  Thread
-// (q, g) sums every class over the half-range planes z = g, g + 8, ...; the
-// eight partial sums of a q meet in shared memory.
-constexpr int kZg = 8;
-template <int MC>
-__global__ void __launch_bounds__(32 * kZg)
-    k_dftz(const float2 *__restrict__ B, int nz, int m, const float2 *__restrict__ tz,
-           float2 *__restrict__ H)
+template <int NC>
+struct Cols {
+    float2 v[NC];
+};
+template <int NC>
+__device__ __forceinline__ Cols<NC> ld_cols(const float2 *p)
 {
-    __shared__ float4 s_p[kZg / 2][MC][32];
-    const int M2 = 2 * m * m, nh = half_len(nz);
-    const int lane = threadIdx.x, g = threadIdx.y, q = blockIdx.x * 32 + lane, c = blockIdx.y;
-    float4 s[MC];
+    Cols<NC> c;
+    if constexpr (NC == 2) {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        c.v[0] = make_float2(q.x, q.y);
+        c.v[1] = make_float2(q.z, q.w);
+    } else {
+        c.v[0] = *p;
+    }
+    return c;
+}
+template <int NC>
+__device__ __forceinline__ void st_cols(float2 *p, const Cols<NC> &c)
+{
+    if constexpr (NC == 2)
+        *reinterpret_cast<float4 *>(p) = make_float4(c.v[0].x, c.v[0].y, c.v[1].x, c.v[1].y);
+    else
+        *p = c.v[0];
+}
+
+// cols counts groups of NC columns; inner is in columns
+template <int MC, int NC>
+__global__ void __launch_bounds__(32 * kColGroups)
+    k_dft_axis(const float2 *in, int cols, int inner, int n, int m,
+               const float2 *__restrict__ tab, float2 *out)
+{
+    extern __shared__ float4 s_p[];      // the copy ring; then [G / 2][MC][32] partial sums
+    const int lane = threadIdx.x, g = threadIdx.y, G = blockDim.y, nh = half_len(n);
+    const int col = blockIdx.x * 32 + lane;
+    const bool live = col < cols;
+    // idle threads shadow the last column; they store nothing
+    const long cc = (long)(live ? col : cols - 1) * NC, o = cc / inner, i = cc - o * inner;
+    const float4 *t4 = reinterpret_cast<const float4 *>(tab);
+    const int tp = class_pitch(m) / 2;
+    float4 s[NC][MC + 1];
 #pragma unroll
-    for (int f = 0; f < MC; ++f) s[f] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (q < M2) {
-        const float2 *b = B + (long)c * nz * M2 + q;
-#pragma unroll 2
-        for (int z = g; z < nh; z += kZg) {
-            const bool both = has_partner(z, nz);
-            const float4 p = fold(b[(long)z * M2],
-                                  both ? b[(long)(nz - z) * M2] : make_float2(0.0f, 0.0f), both);
+    for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int f = 0; f < MC; ++f)
-                if (f <= m) class_add(s[f], p, __ldg(tz + (long)f * nz + z));
+        for (int f = 0; f <= MC; ++f) s[c][f] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float2 *a = in + o * n * inner + i;
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
+    // The samples of a pair travel through a ring of kColDepth slots of this
+    // thread's own in shared memory (asynchronous copies, read back by the
+    // thread that issued them): a pair ahead in registers kept 12 KB per SM in
+    // flight and waited on every load.  A sample without a partner is copied
+    // twice.
+    constexpr int CB = NC * (int)sizeof(float2);
+    const int nth = 32 * G, me = g * 32 + lane;
+    char *ring = reinterpret_cast<char *>(s_p);
+    auto slot = [&](int d, int w) { return ring + ((d * 2 + w) * nth + me) * CB; };
+    auto copy = [&](int j, int d) {
+        if (j < nh) {
+            cp_async<CB>(slot(d, 0), a + (long)j * inner);
+            cp_async<CB>(slot(d, 1), a + (long)(has_partner(j, n) ? n - j : j) * inner);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int d = 0; d < kColDepth - 1; ++d) copy(g + d * G, d);
+    int d = 0;
+    for (int j = g; j < nh; j += G) {
+        float4 tw[(MC + 1) / 2];                 // all in flight before the sums
+#pragma unroll
+        for (int f = 0; f < MC; f += 2)
+            if (f <= m) tw[f / 2] = __ldg(t4 + j * tp + f / 2);
+        copy(j + (kColDepth - 1) * G, d == 0 ? kColDepth - 1 : d - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kColDepth - 1) : "memory");
+        const Cols<NC> u = ld_cols<NC>(reinterpret_cast<const float2 *>(slot(d, 0)));
+        const Cols<NC> v = ld_cols<NC>(reinterpret_cast<const float2 *>(slot(d, 1)));
+        d = d + 1 == kColDepth ? 0 : d + 1;
+        const bool both = has_partner(j, n);
+        float4 p[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) p[c] = fold(u.v[c], v.v[c], both);
+#pragma unroll
+        for (int f = 0; f < MC; f += 2)
+            if (f <= m) {
+                const float4 t = tw[f / 2];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    class_add(s[c][f], p[c], make_float2(t.x, t.y));
+                    class_add(s[c][f + 1], p[c], make_float2(t.z, t.w));
+                }
+            }
     }
 #pragma unroll
-    for (int h = kZg / 2; h > 0; h >>= 1) {
-        __syncthreads();
-        if (g >= h && g < 2 * h) {
+    for (int c = 0; c < NC; ++c)
+        for (int h = G / 2; h > 0; h >>= 1) {
+            __syncthreads();
+            if (g >= h && g < 2 * h) {
 #pragma unroll
-            for (int f = 0; f < MC; ++f) s_p[g - h][f][lane] = s[f];
-        }
-        __syncthreads();
-        if (g < h) {
+                for (int f = 0; f < MC; ++f) s_p[((g - h) * MC + f) * 32 + lane] = s[c][f];
+            }
+            __syncthreads();
+            if (g < h) {
 #pragma unroll
-            for (int f = 0; f < MC; ++f) {
-                const float4 p = s_p[g][f][lane];
-                s[f] = make_float4(s[f].x + p.x, s[f].y + p.y, s[f].z + p.z, s[f].w + p.w);
+                for (int f = 0; f < MC; ++f) {
+                    const float4 p = s_p[(g * MC + f) * 32 + lane];
+                    s[c][f] = make_float4(s[c][f].x + p.x, s[c][f].y + p.y, s[c][f].z + p.z,
+                                          s[c][f].w + p.w);
+                }
             }
         }
-    }
-    if (g == 0 && q < M2) {
-        float2 *h = H + (long)c * 2 * m * M2 + q;
+    if (g == 0 && live) {
+        float2 *h = out + o * 2 * m * inner + i;
 #pragma unroll
         for (int f = 0; f < MC; ++f)
             if (f <= m) {
-                h[(long)f * M2] = spec_plus(s[f]);
-                if (f > 0 && f < m) h[(long)(2 * m - f) * M2] = spec_minus(s[f]);
+                Cols<NC> x, y;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    x.v[c] = spec_plus(s[c][f]);
+                    y.v[c] = spec_minus(s[c][f]);
+                }
+                st_cols<NC>(h + (long)f * inner, x);
+                if (f > 0 && f < m) st_cols<NC>(h + (long)(2 * m - f) * inner, y);
             }
     }
 }
 
+// The inverse: out[outer][j][inner] = sum_slot in[outer][slot][inner]
+// e^{+2 pi i f j / n}.  A thread holds its columns' classes and writes the
+// samples j and n - j for j = g, g + G, ...
+template <int MC, int NC>
+__global__ void __launch_bounds__(32 * kColGroups)
+    k_idft_axis(const float2 *in, int cols, int inner, int n, int m,
+                const float2 *__restrict__ tab, float2 *out)
+{
+    const int col = blockIdx.x * 32 + threadIdx.x, nh = half_len(n);
+    if (col >= cols) return;
+    const long cc = (long)col * NC, o = cc / inner, i = cc - o * inner;
+    const float4 *t4 = reinterpret_cast<const float4 *>(tab);
+    const int tp = class_pitch(m) / 2;
+    const float2 *g = in + o * 2 * m * inner + i;
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
+    float4 p[NC][MC + 1];
+#pragma unroll
+    for (int f = 0; f <= MC; ++f) {
+        const bool on = f <= m && f < MC, both = f > 0 && f < m;
+        Cols<NC> x, y;
+        if (on) {
+            x = ld_cols<NC>(g + (long)f * inner);
+            y = ld_cols<NC>(g + (long)(both ? 2 * m - f : f) * inner);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            p[c][f] = on ? unfold(x.v[c], y.v[c], both) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    float2 *a = out + o * n * inner + i;
+    // this sample's twiddles and, with registers to spare (one column), the
+    // next one's (z at 64 x 64 x 96: 14.1 -> 12.3 us; with two columns they
+    // push the block from 128 to 190 registers, 18.1 -> 26.0 us for y)
+    constexpr bool AHEAD = NC == 1;
+    float4 tw[(MC + 1) / 2], nw[(MC + 1) / 2];
+    auto twiddles = [&](int j, float4 (&t)[(MC + 1) / 2]) {
+#pragma unroll
+        for (int f = 0; f < MC; f += 2)
+            if (f <= m) t[f / 2] = __ldg(t4 + j * tp + f / 2);
+    };
+    if (AHEAD && (int)threadIdx.y < nh) twiddles(threadIdx.y, tw);
+    for (int j = threadIdx.y; j < nh; j += blockDim.y) {
+        if (AHEAD && j + (int)blockDim.y < nh) twiddles(j + blockDim.y, nw);
+        float4 s[NC];                              // P.x c, P.y c, D.x s, D.y s
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int f = 0; f < MC; f += 2)
+            if (f <= m) {
+                const float4 t = AHEAD ? tw[f / 2] : __ldg(t4 + j * tp + f / 2);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    class_add(s[c], p[c][f], make_float2(t.x, t.y));
+                    class_add(s[c], p[c][f + 1], make_float2(t.z, t.w));
+                }
+            }
+        Cols<NC> x, y;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            x.v[c] = make_float2(s[c].x - s[c].w, s[c].y + s[c].z);
+            y.v[c] = make_float2(s[c].x + s[c].w, s[c].y - s[c].z);
+        }
+        st_cols<NC>(a + (long)j * inner, x);
+        if (has_partner(j, n)) st_cols<NC>(a + (long)(n - j) * inner, y);
+        if (AHEAD) {
+#pragma unroll
+            for (int f = 0; f < (MC + 1) / 2; ++f) tw[f] = nw[f];
+        }
+    }
+}
+
+// threads sharing a column: the fewest of 1, 2, 4, 8 that give 14 warps per SM
+inline int col_groups(long cols, int n_sm)
+{
+    int g = 1;
+    while (g < kColGroups && cols * g < 32L * 14 * n_sm) g *= 2;
+    return g;
+}
+
+template <bool INV, int NC>
+cudaError_t launch_axis_nc(const float2 *in, long outer, int inner, int n, int m, const float2 *tab,
+                           float2 *out, int n_sm, cudaStream_t s)
+{
+    const int cols = (int)(outer * inner / NC);
+    const int G = col_groups(cols, n_sm);
+    const dim3 grid((cols + 31) / 32), block(32, G);
+    auto go = [&](auto kernel, int mc) {
+        const size_t smem = INV ? 0
+                                : std::max((size_t)(G / 2) * mc * 32 * sizeof(float4),
+                                           (size_t)kColDepth * 2 * 32 * G * NC * sizeof(float2));
+        return bvf::launch_pdl(kernel, grid, block, smem, s, in, cols, inner, n, m, tab, out);
+    };
+    if (m < 9) return go(INV ? k_idft_axis<9, NC> : k_dft_axis<9, NC>, 9);
+    if (m < 13) return go(INV ? k_idft_axis<13, NC> : k_dft_axis<13, NC>, 13);
+    return go(INV ? k_idft_axis<17, NC> : k_dft_axis<17, NC>, 17);
+}
+
+template <bool INV>
+cudaError_t launch_axis(const float2 *in, long outer, int inner, int n, int m, const float2 *tab,
+                        float2 *out, int n_sm, cudaStream_t s)
+{
+    // the inverse holds its columns' classes and has nothing to wait for but
+    // their first load: with few columns it takes single ones (z at 64 x 64 x
+    // 96: 14.0 us, 16.3 with pairs; the forward 12.7 and 9.9)
+    const bool few = outer * inner / 2 * kColGroups < 32L * 14 * n_sm;
+    return inner % 2 == 0 && !(INV && few)
+               ? launch_axis_nc<INV, 2>(in, outer, inner, n, m, tab, out, n_sm, s)
+               : launch_axis_nc<INV, 1>(in, outer, inner, n, m, tab, out, n_sm, s);
+}
+
 // ------------------------------------------------------------ mode mixing
-// G[o][mode] = sum_c R[mode][c][o] H[c][mode]; block (width, 256/width modes).
-__global__ void k_mix(const float2 *__restrict__ H, const float2 *__restrict__ R, int width,
-                      int n_modes, float2 *__restrict__ G)
+// G[o][mode] = sum_c R[mode][c][o] H[c][mode]; block (width / 2, modes): a
+// thread takes two outputs, so the weights, which bound the kernel (56 MB a
+// layer at width 32, m 12), stream in as 16-byte loads, eight in flight.
+__global__ void k_mix(const float2 *H, const float2 *__restrict__ R, int width, int n_modes,
+                      float2 *G)
 {
     extern __shared__ float2 s_h[];              // [blockDim.y][width]
-    const int o = threadIdx.x, ty = threadIdx.y;
+    const int t = threadIdx.x, ty = threadIdx.y;
     const int mode = blockIdx.x * blockDim.y + ty;
-    for (int c = o; c < width; c += blockDim.x)
+    if (mode < n_modes) {
+        // a mode's weights are width * width * 8 bytes: its threads bring the
+        // lines into L2 while the transform before still runs
+        const char *w = reinterpret_cast<const char *>(R + (long)mode * width * width);
+        for (int l = t; l < width * width / 16; l += blockDim.x) bvf::tma::prefetch_l2(w + 128 * l);
+    }
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
+    for (int c = t; c < width; c += blockDim.x)
         s_h[ty * width + c] = mode < n_modes ? H[(long)c * n_modes + mode] : make_float2(0.f, 0.f);
     __syncthreads();
     if (mode >= n_modes) return;
-    const float2 *r = R + (long)mode * width * width + o;
-    float2 acc = make_float2(0.0f, 0.0f);
+    const float4 *r = reinterpret_cast<const float4 *>(R + (long)mode * width * width) + t;
+    float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
 #pragma unroll 8
     for (int c = 0; c < width; ++c) {
-        const float2 w = r[(long)c * width], h = s_h[ty * width + c];
-        acc.x = fmaf(w.x, h.x, fmaf(-w.y, h.y, acc.x));
-        acc.y = fmaf(w.x, h.y, fmaf(w.y, h.x, acc.y));
+        const float4 w = __ldg(r + c * (width / 2));
+        const float2 h = s_h[ty * width + c];
+        a0.x = fmaf(w.x, h.x, fmaf(-w.y, h.y, a0.x));
+        a0.y = fmaf(w.x, h.y, fmaf(w.y, h.x, a0.y));
+        a1.x = fmaf(w.z, h.x, fmaf(-w.w, h.y, a1.x));
+        a1.y = fmaf(w.z, h.y, fmaf(w.w, h.x, a1.y));
     }
-    G[(long)o * n_modes + mode] = acc;
-}
-
-// ------------------------------------------------- inverse along z and y
-// B'[o][z][q] = sum_jz G[o][jz][q] e^{+2 pi i f(jz) z / nz}: thread (q, g) holds
-// the classes of its q and writes the planes z and nz - z for z = g, g + 8, ...
-template <int MC>
-__global__ void __launch_bounds__(32 * kZg)
-    k_idftz(const float2 *__restrict__ G, int nz, int m, const float2 *__restrict__ tz,
-            float2 *__restrict__ Bp)
-{
-    const int M2 = 2 * m * m, nh = half_len(nz);
-    const int q = blockIdx.x * 32 + threadIdx.x, o = blockIdx.y;
-    if (q >= M2) return;
-    const float2 *gq = G + (long)o * 2 * m * M2 + q;
-    float4 p[MC];
-#pragma unroll
-    for (int f = 0; f < MC; ++f) {
-        const bool both = f > 0 && f < m;
-        p[f] = f <= m ? unfold(gq[(long)f * M2],
-                               both ? gq[(long)(2 * m - f) * M2] : make_float2(0.0f, 0.0f), both)
-                      : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-    float2 *out = Bp + (long)o * nz * M2 + q;
-    for (int z = threadIdx.y; z < nh; z += kZg) {
-        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // P.x c, P.y c, D.x s, D.y s
-#pragma unroll
-        for (int f = 0; f < MC; ++f)
-            if (f <= m) class_add(s, p[f], __ldg(tz + (long)f * nz + z));
-        out[(long)z * M2] = make_float2(s.x - s.w, s.y + s.z);
-        if (has_partner(z, nz)) out[(long)(nz - z) * M2] = make_float2(s.x + s.w, s.y - s.z);
-    }
-}
-
-// A'[slab][y][kx] = sum_jy B'[slab][jy][kx] e^{+2 pi i f(jy) y / ny}.  Blocks
-// walk over the slabs (o, z); a thread writes y and ny - y of one kx, the
-// slab's classes and the twiddles come from shared memory.
-__global__ void k_idfty(const float2 *__restrict__ Bp, int slabs, int ny, int m,
-                        const float2 *__restrict__ ty, float2 *__restrict__ Ap)
-{
-    extern __shared__ __align__(16) float4 s_y4[];
-    const int nh = half_len(ny), nc = m + 1, M2 = 2 * m * m;
-    float4 *s_b = s_y4;                                         // [nc][m]
-    float2 *s_t = reinterpret_cast<float2 *>(s_y4 + nc * m);    // [nh][nc]
-    for (int e = threadIdx.x; e < nc * nh; e += blockDim.x) {
-        const int f = e / nh, y = e - f * nh;
-        s_t[y * nc + f] = ty[(long)f * ny + y];
-    }
-    for (int slab = blockIdx.x; slab < slabs; slab += gridDim.x) {
-        const float2 *b = Bp + (long)slab * M2;
-        __syncthreads();
-        for (int e = threadIdx.x; e < nc * m; e += blockDim.x) {
-            const int f = e / m, kx = e - f * m;
-            const bool both = f > 0 && f < m;
-            s_b[e] = unfold(b[e], both ? b[(2 * m - f) * m + kx] : make_float2(0.0f, 0.0f), both);
-        }
-        __syncthreads();
-        float2 *out = Ap + (long)slab * ny * m;
-        for (int e = threadIdx.x; e < nh * m; e += blockDim.x) {
-            const int y = e / m, kx = e - y * m;
-            float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            const float2 *tw = s_t + y * nc;
-#pragma unroll 4
-            for (int f = 0; f < nc; ++f) class_add(s, s_b[f * m + kx], tw[f]);
-            out[e] = make_float2(s.x - s.w, s.y + s.z);
-            if (has_partner(y, ny)) out[(ny - y) * m + kx] = make_float2(s.x + s.w, s.y - s.z);
-        }
-    }
+    G[(long)(2 * t) * n_modes + mode] = a0;
+    G[(long)(2 * t + 1) * n_modes + mode] = a1;
 }
 
 // ------------------------------- inverse along x + pointwise mix + GELU
@@ -537,11 +654,10 @@ struct RowTcLayout {
 };
 
 template <int W, int KC>     // W output channels; input channels padded to KC (a multiple of 8)
-__global__ void __launch_bounds__(256, 2)
-k_row_tc(const float *__restrict__ vin, int cin, const float2 *__restrict__ Ap,
+__global__ void __launch_bounds__(256, KC < W ? 3 : 2)
+k_row_tc(const float *vin, int cin, const float2 *Ap,
          const float *__restrict__ Wm, const float *__restrict__ b, int nx, int rows, int m,
-         float invN, int act, const float2 *__restrict__ tx, float *__restrict__ vout, int N,
-         int *flag)
+         float invN, int act, const float2 *__restrict__ tx, float *vout, int N, int *flag)
 {
     static_assert(W % 16 == 0 && W <= 64 && KC % 8 == 0, "tile shape");
     extern __shared__ __align__(128) unsigned char s_r[];
@@ -609,29 +725,43 @@ k_row_tc(const float *__restrict__ vin, int cin, const float2 *__restrict__ Ap,
     const uint32_t sbo_t = (uint32_t)(JP / 4) * 128;
     // this thread's channels of its point of a tile, loaded one tile ahead
     float xr[CH];
+    const bool full = cin == KC;
     auto load_v = [&](int row, int t) {
         const int x = 128 * t + pt;
-        const bool ok = x < nx;
-        const long p = (long)row * nx + x;
+        const float *src = vin + (long)half * CH * N + (long)row * nx + x;
+        if (x < nx && full) {
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            const int ch = half * CH + c;
-            xr[c] = (ok && ch < cin) ? vin[(long)ch * N + p] : 0.0f;
+            for (int c = 0; c < CH; ++c, src += N) xr[c] = bvf::tma::ld_stream(src);
+        } else {
+#pragma unroll
+            for (int c = 0; c < CH; ++c, src += N)
+                xr[c] = (x < nx && half * CH + c < cin) ? bvf::tma::ld_stream(src) : 0.0f;
         }
     };
-    // the (o, kx) pairs of A' this thread converts, loaded one row ahead
+    // the (o, kx) pairs of A' this thread converts, loaded one row ahead;
+    // where they lie in A' and in S (-1: none)
     constexpr int PRE = (W * BVF_FNO_MAX_MODES + 255) / 256;
     float2 pre[PRE];
-    auto load_pairs = [&](int row) {
+    long p_src[PRE];
+    int p_dst[PRE];
+    float p_sc[PRE];
 #pragma unroll
-        for (int i = 0; i < PRE; ++i) {
-            const int e = tid + i * 256;
-            if (e < W * m) {
-                const int o = e / m, kx = e - o * m;
-                pre[i] = Ap[((long)o * rows + row) * m + kx];
-            }
-        }
+    for (int i = 0; i < PRE; ++i) {
+        const int e = tid + i * 256, o = e / m, kx = e - o * m;
+        p_src[i] = (long)o * rows * m + kx;
+        p_dst[i] = spec && e < W * m ? (int)tc::kmaj_off(o, 2 * kx, JP) : -1;
+        p_sc[i] = (kx == 0 ? 1.0f : 2.0f) * invN;
+    }
+    auto load_pairs = [&](int row) {
+        const float2 *src = Ap + (long)row * m;
+#pragma unroll
+        for (int i = 0; i < PRE; ++i)
+            if (p_dst[i] >= 0) pre[i] = bvf::tma::ld_stream(src + p_src[i]);
     };
+    // The weights and tables above do not depend on earlier kernels, the rest
+    // does.
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
     int row = blockIdx.x, t = 0, it = 0;
     if (row < rows) {
         load_v(row, 0);
@@ -652,16 +782,12 @@ k_row_tc(const float *__restrict__ vin, int cin, const float2 *__restrict__ Ap,
         if (spec && t == 0) {
 #pragma unroll
             for (int i = 0; i < PRE; ++i) {
-                const int e = tid + i * 256;
-                if (e < W * m) {
-                    const int o = e / m, kx = e - o * m;
-                    const float sc = (kx == 0 ? 1.0f : 2.0f) * invN;
+                if (p_dst[i] >= 0) {
                     uint32_t h0, l0, h1, l1;
-                    tf32_split(pre[i].x * sc, h0, l0);
-                    tf32_split(-pre[i].y * sc, h1, l1);
-                    const uint32_t off = tc::kmaj_off(o, 2 * kx, JP);
-                    *reinterpret_cast<uint2 *>(sSh + off) = make_uint2(h0, h1);
-                    *reinterpret_cast<uint2 *>(sSl + off) = make_uint2(l0, l1);
+                    tf32_split(pre[i].x * p_sc[i], h0, l0);
+                    tf32_split(-pre[i].y * p_sc[i], h1, l1);
+                    *reinterpret_cast<uint2 *>(sSh + p_dst[i]) = make_uint2(h0, h1);
+                    *reinterpret_cast<uint2 *>(sSl + p_dst[i]) = make_uint2(l0, l1);
                 }
             }
         }
@@ -704,7 +830,7 @@ k_row_tc(const float *__restrict__ vin, int cin, const float2 *__restrict__ Ap,
         tc::fence_after();
         if (ready) {
             const int x = 128 * t + pt;
-            const long p = (long)row * nx + x;
+            float *dst = vout + (long)half * (W / 2) * N + (long)row * nx + x;
 #pragma unroll
             for (int c0 = 0; c0 < W / 2; c0 += 8) {
                 float r[8];
@@ -715,10 +841,12 @@ k_row_tc(const float *__restrict__ vin, int cin, const float2 *__restrict__ Ap,
 #pragma unroll
                     for (int i = 0; i < 8; i += 2) {
                         const int o = half * (W / 2) + c0 + i;
-                        float2 val = make_float2(r[i] + sb[o], r[i + 1] + sb[o + 1]);
+                        const float2 bo = *reinterpret_cast<const float2 *>(sb + o);
+                        float2 val = make_float2(r[i] + bo.x, r[i + 1] + bo.y);
                         if (act) val = gelu2(val);
-                        vout[(long)o * N + p] = val.x;
-                        vout[(long)(o + 1) * N + p] = val.y;
+                        dst[0] = val.x;
+                        dst[N] = val.y;
+                        dst += 2L * N;
                     }
                 }
             }
@@ -770,10 +898,10 @@ struct DftxTcLayout {
 
 template <int NB, bool VEC>     // NB: T rows (16 or 32); VEC: rows start on 16 bytes (nx % 4 == 0)
 __global__ void __launch_bounds__(256, 2)
-k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__restrict__ tx,
-          float2 *__restrict__ A, int *flag)
+k_dftx_tc(const float *v, long R, int nx, int m, const float2 *__restrict__ tx, float2 *A,
+          int *flag)
 {
-    extern __shared__ __align__(128) unsigned char s_d[];
+    extern __shared__ __align__(1024) unsigned char s_d[];
     const DftxTcLayout L(NB, nx);
     const int nxp = L.nxp, nch = nxp / kDxC;
     unsigned char *sA = s_d + L.sA, *sBh = s_d + L.sB, *sBl = sBh + NB * nxp * 4;
@@ -809,11 +937,14 @@ k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__re
     tc::fence_after();
     const uint32_t tbase = *tslot;
     const uint32_t idesc = tc::idesc_tf32(128, NB);
-    constexpr uint32_t SBO_A = (kDxC / 4) * 128;
     const uint32_t sbo_b = (uint32_t)(nxp / 4) * 128;
-    // warp w stages rows 16 w .. 16 w + 15 of a chunk: 8 rows by 4 groups of
-    // 4 x per access (512 contiguous bytes in shared memory)
-    const int r_lo = 16 * warp + (lane & 7), kg = lane >> 3;
+    // warp w stages rows 16 w .. 16 w + 15 of a chunk, 8 rows by 4 groups of 4 x
+    // per access.  Four neighbouring lanes read one row's 64 bytes, so a
+    // quarter warp touches two lines (eight when it took eight rows: the
+    // accesses' wavefronts then filled 85 % of the L1 pipe and bound the
+    // kernel); in the 64-byte swizzle the quarter's two rows by four groups
+    // land in distinct banks.
+    const int r_lo = 16 * warp + (lane >> 2), kg = lane & 3;
     const long tiles = (R + 127) / 128;
     auto load = [&](long tile, int ch, float4 (&dst)[2]) {
         const int x = ch * kDxC + 4 * kg;
@@ -822,7 +953,7 @@ k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__re
             const long i = tile * 128 + r_lo + 8 * q;
             const float *src = v + i * nx + x;
             if (VEC) {
-                dst[q] = (i < R && x < nx) ? *reinterpret_cast<const float4 *>(src)
+                dst[q] = (i < R && x < nx) ? bvf::tma::ld_stream(reinterpret_cast<const float4 *>(src))
                                            : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             } else {
                 const bool ok = i < R;
@@ -832,6 +963,8 @@ k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__re
             }
         }
     };
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
     float4 cur[2], nxt[2];
     long tile = blockIdx.x;
     if (tile < tiles) load(tile, 0, cur);
@@ -861,7 +994,7 @@ k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__re
                 tf32_split(cur[q].y, h[1], l[1]);
                 tf32_split(cur[q].z, h[2], l[2]);
                 tf32_split(cur[q].w, h[3], l[3]);
-                const uint32_t off = tc::kmaj_off(r_lo + 8 * q, 4 * kg, kDxC);
+                const uint32_t off = tc::sw64_off(r_lo + 8 * q, kg);
                 *reinterpret_cast<uint4 *>(ah + off) = make_uint4(h[0], h[1], h[2], h[3]);
                 *reinterpret_cast<uint4 *>(al + off) = make_uint4(l[0], l[1], l[2], l[3]);
             }
@@ -875,10 +1008,11 @@ k_dftx_tc(const float *__restrict__ v, long R, int nx, int m, const float2 *__re
                 tc::fence_after();
 #pragma unroll
                 for (int ks = 0; ks < kDxC / 8; ++ks) {
-                    const uint32_t ko = ks * 2 * 128, kb = (ch * (kDxC / 8) + ks) * 2 * 128;
-                    mma3_tc(tbase, tc::smem_desc(ah + ko, 128, SBO_A),
-                            tc::smem_desc(al + ko, 128, SBO_A), tc::smem_desc(sBh + kb, 128, sbo_b),
-                            tc::smem_desc(sBl + kb, 128, sbo_b), idesc, ch > 0 || ks > 0);
+                    const uint32_t ko = ks * 32, kb = (ch * (kDxC / 8) + ks) * 2 * 128;
+                    mma3_tc(tbase, tc::smem_desc_sw(ah + ko, 512, tc::kSwizzle64),
+                            tc::smem_desc_sw(al + ko, 512, tc::kSwizzle64),
+                            tc::smem_desc(sBh + kb, 128, sbo_b), tc::smem_desc(sBl + kb, 128, sbo_b),
+                            idesc, ch > 0 || ks > 0);
                 }
                 tc::commit(&bar[st]);
             }
@@ -953,8 +1087,8 @@ struct ProjTcLayout {
 };
 
 template <int W, int COUT>     // COUT: output count rounded up to 1, 2, 4 or 8
-__global__ void __launch_bounds__(256, 2)
-k_project_tc(const float *__restrict__ v, const float *__restrict__ Q1, const float *__restrict__ q1,
+__global__ void __launch_bounds__(256, 3)
+k_project_tc(const float *v, const float *__restrict__ Q1, const float *__restrict__ q1,
              const float *__restrict__ Q2, const float *__restrict__ q2, int hidden, int c_out,
              float *__restrict__ out, int N, int *flag)
 {
@@ -1006,8 +1140,10 @@ k_project_tc(const float *__restrict__ v, const float *__restrict__ Q1, const fl
         const long p = tile * 128 + pt;
         const bool ok = p < N;
 #pragma unroll
-        for (int c = 0; c < CH; ++c) xr[c] = ok ? v[(long)(half * CH + c) * N + p] : 0.0f;
+        for (int c = 0; c < CH; ++c) xr[c] = ok ? bvf::tma::ld_stream(v + (long)(half * CH + c) * N + p) : 0.0f;
     };
+    bvf::tma::pdl_wait();
+    bvf::tma::pdl_launch_next();
     if ((long)blockIdx.x < tiles) load(blockIdx.x);
     int it = 0;
     bool gave_up = false;
@@ -1050,22 +1186,20 @@ k_project_tc(const float *__restrict__ v, const float *__restrict__ Q1, const fl
 #pragma unroll
         for (int k = 0; k < COUT; ++k) o[k] = 0.0f;
         if (ready) {
-            // 32-column chunks alternate between the two warp halves
-            for (int c0 = 32 * half; c0 < HP; c0 += 64) {
-                float r[32];
-                tc::ld32(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, r);
+            // 16-column chunks alternate between the two warp halves
+            for (int c0 = 16 * half; c0 < HP; c0 += 32) {
+                float r[16];
+                tc::ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, r);
                 tc::wait_ld();
-                const int nv = min(32, HP - c0);
 #pragma unroll
-                for (int i = 0; i < 32; i += 2) {      // nv is a multiple of 16
-                    if (i < nv) {
-                        const float2 h =
-                            gelu2(make_float2(r[i] + sq1[c0 + i], r[i + 1] + sq1[c0 + i + 1]));
+                for (int i = 0; i < 16; i += 2) {
+                    const float2 b = *reinterpret_cast<const float2 *>(sq1 + c0 + i);
+                    const float2 h = gelu2(make_float2(r[i] + b.x, r[i + 1] + b.y));
 #pragma unroll
-                        for (int k = 0; k < COUT; ++k) {
-                            o[k] = fmaf(sq2[k * HP + c0 + i], h.x, o[k]);
-                            o[k] = fmaf(sq2[k * HP + c0 + i + 1], h.y, o[k]);
-                        }
+                    for (int k = 0; k < COUT; ++k) {
+                        const float2 w = *reinterpret_cast<const float2 *>(sq2 + k * HP + c0 + i);
+                        o[k] = fmaf(w.x, h.x, o[k]);
+                        o[k] = fmaf(w.y, h.y, o[k]);
                     }
                 }
             }
@@ -1139,7 +1273,7 @@ struct bvf_fno {
     int *flag = nullptr;                     // device: bit 1 = a bounded wait ran out
     // grid-dependent state
     int nx = 0, ny = 0, nz = 0;
-    float2 *tw = nullptr;                    // twiddle tables [m][nx], [2m][ny], [2m][nz]
+    float2 *tw = nullptr;                    // twiddle tables: classes of y, of z, [m][nx]
     size_t tw_cap = 0;
     float *v0 = nullptr, *v1 = nullptr;
     size_t v_cap = 0;
@@ -1181,6 +1315,19 @@ int grow(T **p, size_t *cap, size_t n, const char *what)
     FCK(cudaMalloc(p, n * sizeof(T)), what);
     *cap = n;
     return BVF_OK;
+}
+
+// the same twiddles by class, [j <= n/2][class f] (class m: frequency -m; the
+// pitch's pad is zero): the layout of k_dft_axis
+void class_table(std::vector<float2> &t, int m, int n)
+{
+    for (int j = 0; j < half_len(n); ++j)
+        for (int f = 0; f < class_pitch(m); ++f) {
+            const long r = (((long)slot_freq(f, m) * j) % n + n) % n;
+            const double a = kTwoPi * (double)r / (double)n;
+            t.push_back(f <= m ? make_float2((float)std::cos(a), (float)std::sin(a))
+                               : make_float2(0.0f, 0.0f));
+        }
 }
 
 // e^{+2 pi i f j / n} for j < n and each signed frequency f of `freqs`
@@ -1225,16 +1372,13 @@ int prepare_grid(bvf_fno *f, int nx, int ny, int nz)
         FCK(cudaMalloc(&f->G, hn * sizeof(float2)), "workspace G");
         f->h_cap = hn;
     }
-    // twiddle tables: [m][nx] for kx = 0 .. m-1, [2m][ny] and [2m][nz] for the
-    // signed slots of y and z
-    std::vector<int> fx(m), fs(2 * m);
+    // twiddle tables: by class for y and z, then [m][nx] for kx = 0 .. m-1
+    std::vector<int> fx(m);
     for (int k = 0; k < m; ++k) fx[k] = k;
-    for (int j = 0; j < 2 * m; ++j) fs[j] = slot_freq(j, m);
     std::vector<float2> t;
-    t.reserve((size_t)m * nx + (size_t)2 * m * (ny + nz));
+    class_table(t, m, ny);
+    class_table(t, m, nz);
     mode_table(t, fx, nx);
-    mode_table(t, fs, ny);
-    mode_table(t, fs, nz);
     if ((rc = grow(&f->tw, &f->tw_cap, t.size(), "twiddle table")) != BVF_OK) return rc;
     FCK(cudaMemcpy(f->tw, t.data(), t.size() * sizeof(float2), cudaMemcpyHostToDevice),
         "twiddle upload");
@@ -1275,9 +1419,8 @@ cudaError_t launch_row_tc_k(int grid, int bytes, cudaStream_t s, const float *vi
 {
     cudaError_t e = smem_at_least<k_row_tc<W, KC>>((size_t)bytes);
     if (e != cudaSuccess) return e;
-    k_row_tc<W, KC><<<grid, 256, bytes, s>>>(vin, cin, Ap, Wm, bm, nx, rows, m, invN, act, tx,
-                                             vout, N, flag);
-    return cudaGetLastError();
+    return bvf::launch_pdl(k_row_tc<W, KC>, grid, 256, bytes, s, vin, cin, Ap, Wm, bm, nx, rows, m,
+                           invN, act, tx, vout, N, flag);
 }
 
 // input channels padded to 8 or 16 (the lift) or to W (a Fourier layer)
@@ -1303,6 +1446,9 @@ cudaError_t launch_dftx_tc(int grid, int bytes, cudaStream_t s, const float *v, 
 {
     cudaError_t e = smem_at_least<k_dftx_tc<NB, VEC>>((size_t)bytes);
     if (e != cudaSuccess) return e;
+    // not started early: its two blocks per SM then land unevenly behind a
+    // lift that was started early itself (8.64 ms an inference at 240 x 240 x
+    // 200 against 7.62)
     k_dftx_tc<NB, VEC><<<grid, 256, bytes, s>>>(v, R, nx, m, tx, A, flag);
     return cudaGetLastError();
 }
@@ -1413,7 +1559,8 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     f->last_stream = s;
     const int N = (int)N64;
     const int M2 = 2 * m * m, n_modes = 2 * m * M2;
-    const float2 *tx = f->tw, *ty = tx + (size_t)m * nx, *tz = ty + (size_t)2 * m * ny;
+    const float2 *ty = f->tw, *tz = ty + (size_t)half_len(ny) * class_pitch(m),
+                 *tx = tz + (size_t)half_len(nz) * class_pitch(m);
 
     // stage events
     const int n_ev_need = 2 + 7 * d.n_layers + 1;
@@ -1460,14 +1607,14 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     FCK(cudaGetDevice(&dev), "bvf_fno_forward: device");
     FCK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev), "sm count");
     // resident blocks per SM: two where shared memory allows (launch bounds)
-    auto blocks_per_sm = [](int bytes) {
-        return std::max(1, std::min(2, (227 * 1024) / (bytes + 1024)));
+    auto blocks_per_sm = [](int bytes, int most = 2) {
+        return std::max(1, std::min(most, (227 * 1024) / (bytes + 1024)));
     };
     auto row_pass = [&](const float *vin, int cin, const float2 *Ap, const float *Wm,
                         const float *bm, int act, float *vout, float2 *An) -> cudaError_t {
         const int kc = Ap ? W : kc_lift;
         const RowTcLayout rl(W, kc, m, nx, Ap != nullptr);
-        const int grid = std::min(rows_p, n_sm * blocks_per_sm(rl.bytes));
+        const int grid = std::min(rows_p, n_sm * blocks_per_sm(rl.bytes, kc < W ? 3 : 2));
         cudaError_t e;
 #define BVF_ROW(WW)                                                                            \
     e = launch_row_tc<WW>(kc, grid, rl.bytes, s, vin, cin, Ap, Wm, bm, nx, rows_p, m, invN, act, \
@@ -1499,18 +1646,6 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     }
     FCK(mark(0), "event");
 
-    // y transforms: shared memory of a block, and blocks that fill the GPU
-    const size_t nhy = ny / 2 + 1, tw_y = (size_t)(m + 1) * nhy * sizeof(float2);
-    const size_t sy = nhy * m * sizeof(float4) + tw_y;
-    const size_t siy = (size_t)(m + 1) * m * sizeof(float4) + tw_y;
-    FCK(smem_at_least<k_dfty>(sy), "bvf_fno_forward: dfty smem");
-    FCK(smem_at_least<k_idfty>(siy), "bvf_fno_forward: idfty smem");
-    const int slabs = W * nz, ty_threads = ((m + 1) * m + 31) / 32 * 32;
-    auto y_grid = [&](size_t smem, int threads) {
-        const int fit = (int)std::min<size_t>(2048 / threads, (size_t)227 * 1024 / (smem + 1024));
-        return std::min(slabs, n_sm * std::max(1, fit));
-    };
-    const dim3 zg((2 * m * m + 31) / 32, W), zb(32, kZg);
     const size_t s_out = ((size_t)W * W + W + 1) * sizeof(float) + (size_t)W * m * sizeof(float2);
     const int rows_x = W * nz * ny;
     const int bo = std::min(256, ((nx + 31) / 32) * 32);
@@ -1526,32 +1661,20 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
             FCK(cudaGetLastError(), "bvf_fno_forward: dftx");
         }
         FCK(mark(1), "event");
-        k_dfty<<<y_grid(sy, ty_threads), ty_threads, sy, s>>>(f->A, slabs, ny, m, ty, f->B);
-        FCK(cudaGetLastError(), "bvf_fno_forward: dfty");
+        FCK(launch_axis<false>(f->A, (long)W * nz, m, ny, m, ty, f->B, n_sm, s),
+            "bvf_fno_forward: dft y");
         FCK(mark(2), "event");
-        if (m < 9)
-            k_dftz<9><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
-        else if (m < 13)
-            k_dftz<13><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
-        else
-            k_dftz<17><<<zg, zb, 0, s>>>(f->B, nz, m, tz, f->H);
-        FCK(cudaGetLastError(), "bvf_fno_forward: dftz");
+        FCK(launch_axis<false>(f->B, W, M2, nz, m, tz, f->H, n_sm, s), "bvf_fno_forward: dft z");
         FCK(mark(3), "event");
-        const dim3 mb(W, 256 / W);
-        k_mix<<<(n_modes + mb.y - 1) / mb.y, mb, mb.y * W * sizeof(float2), s>>>(f->H, R, W,
-                                                                                 n_modes, f->G);
-        FCK(cudaGetLastError(), "bvf_fno_forward: mix");
+        const dim3 mb(W / 2, 256 / (W / 2));
+        FCK(bvf::launch_pdl(k_mix, (n_modes + mb.y - 1) / mb.y, mb, mb.y * W * sizeof(float2), s, f->H,
+                            R, W, n_modes, f->G),
+            "bvf_fno_forward: mix");
         FCK(mark(4), "event");
-        if (m < 9)
-            k_idftz<9><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
-        else if (m < 13)
-            k_idftz<13><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
-        else
-            k_idftz<17><<<zg, zb, 0, s>>>(f->G, nz, m, tz, f->B);
-        FCK(cudaGetLastError(), "bvf_fno_forward: idftz");
+        FCK(launch_axis<true>(f->G, W, M2, nz, m, tz, f->B, n_sm, s), "bvf_fno_forward: idft z");
         FCK(mark(5), "event");
-        k_idfty<<<y_grid(siy, TB), TB, siy, s>>>(f->B, slabs, ny, m, ty, f->A);
-        FCK(cudaGetLastError(), "bvf_fno_forward: idfty");
+        FCK(launch_axis<true>(f->B, (long)W * nz, m, ny, m, ty, f->A, n_sm, s),
+            "bvf_fno_forward: idft y");
         FCK(mark(6), "event");
         const int act = l < d.n_layers - 1;
         if (fused) {
@@ -1576,14 +1699,15 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
         const int cp = d.c_out <= 2 ? d.c_out : (d.c_out <= 4 ? 4 : 8);
         const ProjTcLayout pl(W, d.hidden, cp);
         const long tiles = (N64 + 127) / 128;
-        const int per_sm = std::max(1, std::min(2, 512 / pl.ncols));
+        const int per_sm =
+            std::max(1, std::min({3, 512 / pl.ncols, (227 * 1024) / (pl.bytes + 1024)}));
         const int grid = (int)std::min<long>(tiles, (long)n_sm * per_sm);
         cudaError_t e = cudaSuccess;
 #define BVF_PRJ(WW, CP)                                                                      \
     e = smem_at_least<k_project_tc<WW, CP>>((size_t)pl.bytes);                                 \
     if (e == cudaSuccess)                                                                      \
-        k_project_tc<WW, CP><<<grid, 256, pl.bytes, s>>>(vc, Q1, q1, Q2, q2, d.hidden, d.c_out, \
-                                                        d_out, N, f->flag);
+        e = bvf::launch_pdl(k_project_tc<WW, CP>, grid, 256, pl.bytes, s, vc, Q1, q1, Q2, q2,    \
+                            d.hidden, d.c_out, d_out, N, f->flag);
 #define BVF_PRJ_W(CP)                     \
     switch (W) {                          \
     case 16: BVF_PRJ(16, CP) break;       \

@@ -7,8 +7,8 @@
 // A block of 128 threads computes a 128 x BN tile of C:
 //   * K runs in chunks of 64; the chunk's A (128 x 64) and B (BN x 64) tiles
 //     are read from their strided FP32 arrays, rounded to BF16 and written to
-//     shared memory in the canonical K-major layout (8 rows x 16 bytes per
-//     core matrix), two stages deep, so the threads stage chunk c+1 while the
+//     shared memory K-major with a 128-byte swizzle (without one the eight
+//     pieces of a row share their banks), two stages deep, so the threads stage chunk c+1 while the
 //     tensor cores multiply chunk c;
 //   * thread 0 issues four tcgen05.mma.kind::f16 (K = 16 each) per chunk into
 //     the TMEM accumulator and commits them to the stage's mbarrier;
@@ -35,7 +35,6 @@ namespace {
 
 constexpr int GK = 64;                 // K chunk (BF16 elements): 128 bytes per row
 constexpr int GSEG = GK / 8;           // 16-byte core-matrix rows per tile row and chunk
-
 // NS shared-memory stages of GK-wide K chunks: two overlap the staging of a
 // chunk with the products of the previous one; products of a single chunk
 // (K <= GK) take one, so twice as many blocks fit per SM.
@@ -49,21 +48,20 @@ struct GemmLayout {
     static constexpr int off_rows = off_tmem + 16;     // [128] row starts of A, then of C
     static constexpr int bytes = off_rows + 2 * 128 * 8;
     static_assert(NS * STAGE >= 4 * 32 * 33 * 4, "the epilogue's transpose buffers fit the stages");
-    static constexpr uint32_t SBO = GSEG * 128;      // byte step between 8-row groups
 };
 
 using tc::pack_bf16;
 
 // Rows [0, rows) x K-chunk [k0, k0 + GK) of an FP32 operand (element (r, k) at
-// src[start(r) + kof(k)]; zero for r >= valid or k >= K) written as BF16 in
-// K-major core matrices.  Where k is contiguous (kc), consecutive threads
+// src[start(r) + kof(k)]; zero for r >= valid or k >= K) written as BF16,
+// K-major, swizzled.  Where k is contiguous (kc), consecutive threads
 // take consecutive 8-element pieces of one row, otherwise consecutive rows,
 // so the global reads are coalesced in both layouts.  vec: the pieces load
 // as two float4 (aligned rows, four-element groups never straddle K or a part
 // of it); four pieces are in flight per thread, against eight floats of one:
 // the staging is bound by the latency of its loads.
 template <class Start, class Kof>
-__device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__restrict__ src,
+__device__ __forceinline__ void stage_tile(unsigned char *dst, const float *src,
                                            Start start, Kof kof, bool kc, bool vec, int rows,
                                            int valid, int k0, int K, int tid)
 {
@@ -80,14 +78,14 @@ __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__re
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
                     v[u][h] = (on && k + 4 * h < K)
-                                  ? __ldg(reinterpret_cast<const float4 *>(row + kof(k + 4 * h)))
+                                  ? *reinterpret_cast<const float4 *>(row + kof(k + 4 * h))
                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int s = s0 + 128 * u;
                 if (s < segs)
-                    *reinterpret_cast<uint4 *>(dst + tc::kmaj_off16(s / GSEG, (s % GSEG) * 8, GK)) =
+                    *reinterpret_cast<uint4 *>(dst + tc::sw128_off(s / GSEG, s % GSEG)) =
                         make_uint4(pack_bf16(v[u][0].x, v[u][0].y), pack_bf16(v[u][0].z, v[u][0].w),
                                    pack_bf16(v[u][1].x, v[u][1].y), pack_bf16(v[u][1].z, v[u][1].w));
             }
@@ -110,9 +108,9 @@ __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *__re
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int k = k0 + k8 + j;
-            v[j] = (on && k < K) ? __ldg(row + kof(k)) : 0.0f;
+            v[j] = (on && k < K) ? row[kof(k)] : 0.0f;
         }
-        *reinterpret_cast<uint4 *>(dst + tc::kmaj_off16(r, k8, GK)) =
+        *reinterpret_cast<uint4 *>(dst + tc::sw128_off(r, k8 >> 3)) =
             make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
                        pack_bf16(v[6], v[7]));
     }
@@ -122,7 +120,7 @@ template <int BN, int NS>
 __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX gx, int *flag)
 {
     const bvf_gemm &g = gx.g;
-    extern __shared__ __align__(128) unsigned char sm[];
+    extern __shared__ __align__(1024) unsigned char sm[];
     using Lay = GemmLayout<BN, NS>;
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + Lay::off_bar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + Lay::off_tmem);
@@ -162,6 +160,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    tma::pdl_wait();
+    tma::pdl_launch_next();
     const uint32_t tbase = *tslot;
     const uint32_t idesc = tc::idesc_bf16(128, BN);
 
@@ -186,9 +186,9 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
             tc::fence_after();
 #pragma unroll
             for (int ks = 0; ks < GK / 16; ++ks) {
-                const uint32_t ko = ks * 2 * 128;        // two core matrices per K step of 16
-                tc::mma_f16(tbase, tc::smem_desc(sa + ko, 128, Lay::SBO),
-                            tc::smem_desc(sb + ko, 128, Lay::SBO), idesc, (nc > 0 || ks > 0) ? 1 : 0);
+                // 32 bytes of each row per K step of 16
+                tc::mma_f16(tbase, tc::smem_desc_sw(sa + 32 * ks, 1024, tc::kSwizzle128),
+                            tc::smem_desc_sw(sb + 32 * ks, 1024, tc::kSwizzle128), idesc, (nc > 0 || ks > 0) ? 1 : 0);
             }
             tc::commit(&bar[st]);
         }
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
                 return;
             }
             if (g.beta != 0.0f) v = fmaf(g.beta, *cp, v);
-            if (g.bias_mode == 1) v += __ldg(g.bias + n);
-            else if (g.bias_mode == 2) v += __ldg(g.bias + mm);
+            if (g.bias_mode == 1) v += g.bias[n];
+            else if (g.bias_mode == 2) v += g.bias[mm];
             if (g.act == 1) {
                 if (pp) *pp = v;
                 v = gelu_exact(v);
@@ -288,8 +288,7 @@ cudaError_t launch_gemm_ns(const GemmX &x, int *flag, cudaStream_t s)
         if (e != cudaSuccess) return e;
         raised.store(1, std::memory_order_release);
     }
-    k_gemm_bf16<BN, NS><<<grid, 128, GemmLayout<BN, NS>::bytes, s>>>(x, flag);
-    return cudaGetLastError();
+    return launch_pdl(k_gemm_bf16<BN, NS>, grid, 128, GemmLayout<BN, NS>::bytes, s, x, flag);
 }
 
 // one stage when the product is a single K chunk

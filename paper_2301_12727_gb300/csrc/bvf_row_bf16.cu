@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
             const int ch = half * CH + c;
-            xv[c] = (ok && ch < q.cin) ? __ldg(src + (long long)ch * N) : 0.0f;
+            xv[c] = (ok && ch < q.cin) ? tma::ld_stream(src + (long long)ch * N) : 0.0f;
         }
     };
     constexpr int PRE = (W * RP * 16 + 255) / 256;   // pairs per thread at m = 16
@@ -153,10 +153,14 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
             if (e < W * RP * m) {
                 const int o = e / (RP * m), r = e - o * RP * m;   // r: pair of the o's RP rows
                 if (row0 + r / m < rows)
-                    pre[i] = __ldg(reinterpret_cast<const float2 *>(src + (long long)o * rows * (2 * m)) + r);
+                    pre[i] = tma::ld_stream(
+                        reinterpret_cast<const float2 *>(src + (long long)o * rows * (2 * m)) + r);
             }
         }
     };
+    // weights and tables are in place: the rest depends on earlier kernels
+    tma::pdl_wait();
+    tma::pdl_launch_next();
     int item = blockIdx.x, t = 0, phase = 0;
     if (item < items) {
         load_v(item, 0);
@@ -225,7 +229,7 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
                 if (spec) tc::ld8(ta, s);
                 if (ok && q.act == 2) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) pv[i] = __ldg(q.pre + at + (long long)(o0 + i) * N);
+                    for (int i = 0; i < 8; ++i) pv[i] = tma::ld_stream(q.pre + at + (long long)(o0 + i) * N);
                 }
                 tc::wait_ld();
                 if (ok) {
@@ -287,7 +291,7 @@ struct ProjBLayout {
 
 template <int W>
 __global__ void __launch_bounds__(256, 3)
-    k_project_bf16(const float *__restrict__ v, const float *__restrict__ Q1,
+    k_project_bf16(const float *v, const float *__restrict__ Q1,
                    const float *__restrict__ q1, const float *__restrict__ Q2,
                    const float *__restrict__ q2, int hidden, int c_out, float *__restrict__ out,
                    int N, int B, int *flag)
@@ -339,8 +343,10 @@ __global__ void __launch_bounds__(256, 3)
         const float *src = v + (long long)b * W * N + p;
 #pragma unroll
         for (int c = 0; c < CH; ++c)
-            xv[c] = p < N ? __ldg(src + (long long)(half * CH + c) * N) : 0.0f;
+            xv[c] = p < N ? tma::ld_stream(src + (long long)(half * CH + c) * N) : 0.0f;
     };
+    tma::pdl_wait();
+    tma::pdl_launch_next();
     if ((int)blockIdx.x < tiles) load(blockIdx.x);
     int phase = 0;
     bool gave_up = false;
@@ -450,8 +456,7 @@ cudaError_t launch_row_k(const RowBf16 &q, const RowBLayout &L, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const int items = q.B * ((q.rows + RP - 1) / RP);
     const int grid = std::min(items, q.n_sm * blocks_per_sm(L.bytes, 2 * W <= 64 ? 64 : 128));
-    k_row_bf16<W, KC, RP><<<grid, 256, L.bytes, s>>>(q);
-    return cudaGetLastError();
+    return launch_pdl(k_row_bf16<W, KC, RP>, grid, 256, L.bytes, s, q);
 }
 
 template <int W, int KC>
@@ -500,8 +505,8 @@ cudaError_t launch_project_bf16(const float *v, const float *Q1, const float *q1
 #define BVF_PROJ(WW)                                                                             \
     e = raise_smem<k_project_bf16<WW>>();                                                          \
     if (e == cudaSuccess)                                                                          \
-        k_project_bf16<WW><<<grid, 256, L.bytes, s>>>(v, Q1, q1, Q2, q2, hidden, c_out, out, N, B, \
-                                                     flag);
+        e = launch_pdl(k_project_bf16<WW>, grid, 256, L.bytes, s, v, Q1, q1, Q2, q2, hidden, c_out, \
+                       out, N, B, flag);
     switch (width) {
     case 16: BVF_PROJ(16) break;
     case 32: BVF_PROJ(32) break;
@@ -509,7 +514,7 @@ cudaError_t launch_project_bf16(const float *v, const float *Q1, const float *q1
     default: BVF_PROJ(64) break;
     }
 #undef BVF_PROJ
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return e;
 }
 
 }  // namespace bvf

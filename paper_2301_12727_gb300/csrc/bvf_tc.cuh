@@ -26,6 +26,29 @@ __device__ __forceinline__ uint64_t smem_desc(const void *p, uint32_t lbo, uint3
     return d;
 }
 
+// Swizzled K-major operands: 8-row groups of 64- or 128-byte rows, sbo bytes
+// apart, each group aligned to its 512 or 1024 bytes; 16-byte piece c of row r
+// sits at piece c ^ ((r / 2) % 4) (64 bytes) or c ^ (r % 8) (128 bytes).  Both
+// eight rows of one piece and the pieces of one row fall into different
+// banks.  A K step moves the address by its bytes within the row.
+constexpr uint64_t kSwizzle128 = 2, kSwizzle64 = 4;
+__device__ __forceinline__ uint64_t smem_desc_sw(const void *p, uint32_t sbo, uint64_t mode)
+{
+    uint64_t d = (uint64_t)((bvf::tma::saddr(p) >> 4) & 0x3FFFu);
+    d |= (uint64_t)1 << 16;                      // LBO: unused with a swizzle
+    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)1 << 46;
+    return d | mode << 61;
+}
+__host__ __device__ __forceinline__ uint32_t sw64_off(int row, int piece)
+{
+    return (uint32_t)((row >> 3) * 512 + (row & 7) * 64 + ((piece ^ ((row >> 1) & 3)) << 4));
+}
+__host__ __device__ __forceinline__ uint32_t sw128_off(int row, int piece)
+{
+    return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((piece ^ (row & 7)) << 4));
+}
+
 // kind::tf32 instruction descriptor: D FP32, A and B TF32, both K-major
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 {
@@ -100,6 +123,20 @@ __device__ __forceinline__ void ld32(uint32_t taddr, float (&r)[32])
                  : "r"(taddr));
 #pragma unroll
     for (int i = 0; i < 32; ++i) r[i] = __uint_as_float(u[i]);
+}
+
+// 16 consecutive columns of this warp's 32 lanes
+__device__ __forceinline__ void ld16(uint32_t taddr, float (&r)[16])
+{
+    uint32_t u[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]),
+                   "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]),
+                   "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+                 : "r"(taddr));
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = __uint_as_float(u[i]);
 }
 
 // 8 consecutive columns of this warp's 32 lanes (the narrow form of ld32)
