@@ -32,10 +32,12 @@
 // The state is stored as T = float or __half (scaled FP16 storage; the
 // arithmetic is FP32 either way).  A TMA box must start on a 16-byte boundary
 // in x, so the x-halo is XO = 16 / sizeof(T) columns: 4 floats or 8 halves.
-// Used when nx % 8 == 0 (state rows are whole multiples of 16 bytes in both
-// storages, every pair lies inside the grid and every paired access is
-// aligned; the index is mapped from a copy with rows padded to 16 bytes when
-// nx % 16 != 0) and L <= 2.
+// Used with L <= 2.  The rows of the context's arrays lie p.pitch elements
+// apart, a multiple of 8: rows are whole multiples of 16 bytes in both
+// storages and every paired access is aligned; where nx itself is not a
+// multiple of 8 the row's pad is never read by another voxel (the tensor maps
+// end at nx and fill zeros).  The index is mapped from a copy with rows padded
+// to 16 bytes when nx % 16 != 0.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -164,12 +166,14 @@ struct VelLayout {
                   "TMA destinations must stay 128-byte aligned");
 };
 
-// One tile (bx, by) of the grid over z-chunk bz.  REUSE: the block runs
+// One tile (bx, by) of the grid over z-chunk bz.  PAD: rows are padded (pitch >
+// nx, nx may be odd); compiled apart because the checks cost 1 % of a step at
+// 240 x 240 x 200.  REUSE: the block runs
 // further tiles afterwards (persistent batch kernel), so its mbarriers are
 // invalidated at the end and the first copies are fenced against the
 // previous tile's reads of the same shared memory.  Returns true (in every
 // thread) when a ring wait ran out; the tile's results are then incomplete.
-template <typename T, bool REUSE, int TH = TY>
+template <typename T, bool REUSE, int TH = TY, bool PAD = false>
 __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityTmaMaps &tm,
                                               int kchunk, int bx, int by, int bz,
                                               unsigned char *smb)
@@ -186,8 +190,8 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * PX + tx;
     const int x0 = bx * TX, y0 = by * TH;
     const int i = x0 + 2 * tx, j = y0 + ty;         // the pair (i, i+1) of row j
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const bool live = i < nx && j < ny;              // nx is even: i + 1 < nx as well
+    const int nx = p.nx, ny = p.ny, nz = p.nz, pitch = PAD ? p.pitch : nx;
+    const bool live = i < nx && j < ny;
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
     // ring slots: A holds plane pl in slot (pl-k0)%2, B in (pl-k0+2)%6,
     // C in (pl-k0+1)%6, the index in (pl-k0)%3
@@ -242,16 +246,17 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
     const int cxy = (ty + 2) * VW + 2 * tx + Bx::XO;
     const int cz = ty * TX + 2 * tx;
     const int cI = ty * IW + 2 * tx;
-    const int xs[2] = {slab_pos(i, nx, p.P), slab_pos(i + 1, nx, p.P)};
+    // (the second voxel of an odd row's last pair lies in the row's pad)
+    const int xs[2] = {slab_pos(i, nx, p.P), !PAD || i + 1 < nx ? slab_pos(i + 1, nx, p.P) : -1};
     const int ys = slab_pos(j, ny, p.P);
-    const int Sxs = nz * ny * p.W, Sys = nz * p.W * nx, Szs = p.W * ny * nx;
+    const int Sxs = nz * ny * p.W, Sys = nz * p.W * pitch, Szs = p.W * ny * pitch;
     const float2 *pmlx = p.pml, *pmly = p.pml + 2 * p.nmax, *pmlz = p.pml + 4 * p.nmax;
     T *__restrict__ vxg = static_cast<T *>(p.vx);
     T *__restrict__ vyg = static_cast<T *>(p.vy);
     T *__restrict__ vzg = static_cast<T *>(p.vz);
-    // the pair's second voxel is not the last point in x (the first never is)
-    const bool ix1 = i + 1 < nx - 1, jy1 = j < ny - 1;
-    const int plane = nx * ny, col = j * nx + i;
+    // the pair's voxels are not the last point in x (the first is in odd rows only)
+    const bool ix0 = !PAD || i < nx - 1, ix1 = i + 1 < nx - 1, jy1 = j < ny - 1;
+    const int plane = pitch * ny, col = j * pitch + i;
     // velocities of the plane being computed, loaded one plane ahead
     float2 ux = pair(0.0f, 0.0f), uy = ux, uz = ux;
     if (live) {
@@ -262,8 +267,8 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
     int q = k0 * plane + col;                       // this pair in plane k
     int ox[2] = {(k0 * ny + j) * p.W + xs[0],       // in the x-slab (xs >= 0)
                  (k0 * ny + j) * p.W + xs[1]};
-    int oy = (k0 * p.W + ys) * nx + i;              // in the y-slab (ys >= 0)
-    const int dox = ny * p.W, doy = p.W * nx;
+    int oy = (k0 * p.W + ys) * pitch + i;              // in the y-slab (ys >= 0)
+    const int dox = ny * p.W, doy = p.W * pitch;
 
     unsigned mpar = 0;                              // parity of (k - k0) / R
     bool stop = false;
@@ -360,7 +365,7 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
                     const float2 h = __ldg(&pmlx[p.nmax + i + l]), w = __ldg(&pmlx[i + l]);
                     float t, d;
                     d = st::cpml_v(qx[l][0], h.x, h.y, lane(ax1, l), t);
-                    if (l == 0 || ix1) p.psx[ox[l]] = t;
+                    if (l == 0 ? ix0 : ix1) p.psx[ox[l]] = t;
                     set_lane(ax1, l, d);
                     d = st::cpml_v(qx[l][1], w.x, w.y, lane(ay1, l), t);
                     if (jy1) p.psx[Sxs + ox[l]] = t;
@@ -373,7 +378,7 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
                     const float2 h = __ldg(&pmly[p.nmax + j]), w = __ldg(&pmly[j]);
                     float2 t;
                     ax2 = st::cpml_v(qy[0], splat<float2>(w.x), splat<float2>(w.y), ax2, t);
-                    st::st2_or_1(p.psy + oy, t, ix1);
+                    if (ix0) st::st2_or_1(p.psy + oy, t, ix1);
                     ay2 = st::cpml_v(qy[1], splat<float2>(h.x), splat<float2>(h.y), ay2, t);
                     if (jy1) st::st2(p.psy + Sys + oy, t);
                     az2 = st::cpml_v(qy[2], splat<float2>(w.x), splat<float2>(w.y), az2, t);
@@ -383,7 +388,7 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
                     const float2 h = __ldg(&pmlz[p.nmax + k]), w = __ldg(&pmlz[k]);
                     float2 t;
                     ax3 = st::cpml_v(qz[0], splat<float2>(w.x), splat<float2>(w.y), ax3, t);
-                    st::st2_or_1(p.psz + oz, t, ix1);
+                    if (ix0) st::st2_or_1(p.psz + oz, t, ix1);
                     ay3 = st::cpml_v(qz[1], splat<float2>(w.x), splat<float2>(w.y), ay3, t);
                     if (jy1) st::st2(p.psz + Szs + oz, t);
                     az3 = st::cpml_v(qz[2], splat<float2>(h.x), splat<float2>(h.y), az3, t);
@@ -399,7 +404,7 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
                                         st::buoyancy(p.buoy, nm, mb, I0[IW + 1]));
                 const float2 bzv = pair(st::buoyancy(p.buoy, nm, ma, I1[0]),
                                         st::buoyancy(p.buoy, nm, mb, I1[1]));
-                st::st2_or_1(vxg + q, st::vel_step(dt, bxv, ux, ax1, ax2, ax3), ix1);
+                if (ix0) st::st2_or_1(vxg + q, st::vel_step(dt, bxv, ux, ax1, ax2, ax3), ix1);
                 if (jy1) st::st2(vyg + q, st::vel_step(dt, byv, uy, ay1, ay2, ay3));
                 if (kz1) st::st2(vzg + q, st::vel_step(dt, bzv, uz, az1, az2, az3));
             }
@@ -427,13 +432,13 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
 
 // six resident blocks of 128 threads per SM at the default height (80
 // registers); the thread count times blocks per SM is kept for other heights
-template <typename T, int TH>
+template <typename T, int TH, bool PAD>
 __global__ void __launch_bounds__(PX * TH, 6 * TY / TH)
     k_velocity_tma(const __grid_constant__ AcParams p, int kchunk,
                    const __grid_constant__ VelocityTmaMaps tm)
 {
     extern __shared__ __align__(1024) unsigned char smb[];
-    velocity_tile<T, false, TH>(p, tm, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
+    velocity_tile<T, false, TH, PAD>(p, tm, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
 }
 
 // ------------------------------------------------------------------ stress
@@ -462,7 +467,7 @@ struct StressLayout {
 constexpr int SNTH = TX * TY;
 
 // One tile (bx, by) over z-chunk bz; REUSE and the result as for velocity_tile.
-template <int L, typename T, bool REUSE, int TH = TY>
+template <int L, typename T, bool REUSE, int TH = TY, bool PAD = false>
 __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMaps &tm,
                                             const StepParam &st, int kchunk, int bx, int by,
                                             int bz, unsigned char *smb)
@@ -479,7 +484,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const int x0 = bx * TX, y0 = by * TH;
     const int i = x0 + tx, j = y0 + ty;
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
+    const int nx = p.nx, ny = p.ny, nz = p.nz, pitch = PAD ? p.pitch : nx;
     const bool live = i < nx && j < ny;
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
     constexpr unsigned VT_BYTES = VT * Lay::ES;
@@ -526,7 +531,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
     const int cv = (ty + 2) * VW + tx + Bx::XO;
     const int ci = ty * IW + tx;
     const int xs = slab_pos(i, nx, p.P), ys = slab_pos(j, ny, p.P);
-    const int Sxs = nz * ny * p.W, Sys = nz * p.W * nx, Szs = p.W * ny * nx;
+    const int Sxs = nz * ny * p.W, Sys = nz * p.W * pitch, Szs = p.W * ny * pitch;
     const float2 *pmlx = p.pml, *pmly = p.pml + 2 * p.nmax, *pmlz = p.pml + 4 * p.nmax;
     T *const gs[6] = {static_cast<T *>(p.sxx), static_cast<T *>(p.syy), static_cast<T *>(p.szz),
                       static_cast<T *>(p.sxy), static_cast<T *>(p.sxz), static_cast<T *>(p.syz)};
@@ -558,12 +563,13 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
     const T *st0 = static_cast<const T *>(p.sxx);     // stresses: consecutive arrays, fstride apart
     auto prefetch_plane = [&](int kp) {
         if (kp >= k1 || y0 + pf_r >= ny || pf_a >= n_lines) return;
-        const size_t e = (size_t)kp * nx * ny + (size_t)(y0 + pf_r) * nx + x0;
+        const size_t e = ((size_t)kp * ny + (size_t)(y0 + pf_r)) * pitch + x0;
         int a = pf_a;
         const char *ln;
         if (a < 6 * LS) {
             ln = reinterpret_cast<const char *>(st0 + (size_t)(a / LS) * p.fstride + e) + (a % LS) * 128;
         } else if ((a -= 6 * LS) < (L > 0 ? 6 * LM : 0)) {
+            if (a % LM && x0 + (a % LM) * (32 / LM) >= nx) return;
             ln = reinterpret_cast<const char *>(mem + mem_index(0, a / LM, e, p.fstride, L)) +
                  (a % LM) * 128;
         } else {
@@ -596,7 +602,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
             issue(k + 2, &bars[(it + 2) % 3]);
         }
         if (PREFETCH) prefetch_plane(k + 1);
-        const int q = k * (nx * ny) + j * nx + i;
+        const int q = k * (pitch * ny) + j * pitch + i;
         // per-voxel loads first, in flight while the ring wait and the
         // derivatives proceed
         float sv[6], rv[L > 0 ? L : 1][6];
@@ -605,8 +611,8 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
         // CPML memories of this voxel: components 3-5 of each slab it lies in,
         // i.e. [normal, then the two shear derivatives along that axis]
         const int zs = slab_pos(k, nz, p.P);
-        const int ox = (k * ny + j) * p.W + xs, oy = (k * p.W + ys) * nx + i,
-                  oz = (zs * ny + j) * nx + i;
+        const int ox = (k * ny + j) * p.W + xs, oy = (k * p.W + ys) * pitch + i,
+                  oz = (zs * ny + j) * pitch + i;
         float qx[3] = {0.0f, 0.0f, 0.0f}, qy[3] = {0.0f, 0.0f, 0.0f}, qz[3] = {0.0f, 0.0f, 0.0f};
         if (lv) {
             if (EDGE && xs >= 0) {
@@ -663,7 +669,7 @@ __device__ __forceinline__ bool stress_tile(const AcParams &p, const StressTmaMa
             if (zs >= 0) ezz = st::cpml_pre(p.psz + 3 * Szs + oz, qz[0], __ldg(&pmlz[k]), ezz);
             float srcv = 0.0f;
             if ((st.flags & kStepSource) && k == p.k_src) {
-                const float2 a = p.src[j * nx + i];
+                const float2 a = p.src[j * pitch + i];
                 srcv = st::source_value<float>(p.src_scale, a.x, a.y, st.src_ws, st.src_wc);
             }
             st::normal_update<L>(p, c0, exx, eyy, ezz, srcv, sv, rv);
@@ -804,7 +810,7 @@ __device__ __forceinline__ uint2 pack_mem2(float2 r0, float2 r1)
     return w;
 }
 
-template <int L, bool REUSE, int TH = TY>
+template <int L, bool REUSE, int TH = TY, bool PAD = false>
 __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTmaMaps &tm,
                                                const StepParam &st, int kchunk, int bx, int by,
                                                int bz, unsigned char *smb)
@@ -822,8 +828,8 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * PX + tx;
     const int x0 = bx * TX, y0 = by * TH;
     const int i = x0 + 2 * tx, j = y0 + ty;           // the pair (i, i+1) of row j
-    const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const bool live = i < nx && j < ny;                // nx is even: i + 1 < nx as well
+    const int nx = p.nx, ny = p.ny, nz = p.nz, pitch = PAD ? p.pitch : nx;
+    const bool live = i < nx && j < ny;
     const int k0 = bz * kchunk, k1 = min(nz, k0 + kchunk);
     constexpr unsigned VT_BYTES = VT * Lay::ES;
     auto oV = [&](int pl) { return Lay::off_v + ((pl - k0 + 2) % Lay::RV) * 3 * (int)VT_BYTES; };
@@ -868,15 +874,17 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
     const st::Dx ix = st::make_dx(p.inv_dx);
     const int cv = (ty + 2) * VW + 2 * tx + Bx::XO;    // even: every pair read is aligned
     const int ci = ty * IW + 2 * tx;
-    const int xs[2] = {slab_pos(i, nx, p.P), slab_pos(i + 1, nx, p.P)};
+    // (the second voxel of an odd row's last pair lies in the row's pad)
+    const bool two = !PAD || i + 1 < nx;
+    const int xs[2] = {slab_pos(i, nx, p.P), two ? slab_pos(i + 1, nx, p.P) : -1};
     const int ys = slab_pos(j, ny, p.P);
-    const int Sxs = nz * ny * p.W, Sys = nz * p.W * nx, Szs = p.W * ny * nx;
+    const int Sxs = nz * ny * p.W, Sys = nz * p.W * pitch, Szs = p.W * ny * pitch;
     const float2 *pmlx = p.pml, *pmly = p.pml + 2 * p.nmax, *pmlz = p.pml + 4 * p.nmax;
     T *const gs[6] = {static_cast<T *>(p.sxx), static_cast<T *>(p.syy), static_cast<T *>(p.szz),
                       static_cast<T *>(p.sxy), static_cast<T *>(p.sxz), static_cast<T *>(p.syz)};
     T *__restrict__ mem = static_cast<T *>(p.mem);
-    // the pair's second voxel is not the last point in x (the first never is)
-    const bool ix1 = i + 1 < nx - 1;
+    // the pair's voxels are not the last point in x (the first is in odd rows only)
+    const bool ix0 = !PAD || i < nx - 1, ix1 = i + 1 < nx - 1;
 
     const int vbase = Lay::off_v / Lay::ES, vend = vbase + Lay::RV * 3 * VT;
     const int ibase = Lay::off_i, iend = ibase + Lay::RI * IT_SLOT;
@@ -898,7 +906,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
             tma::fence_async_smem();
             issue(k + 2, &bars[(it + 2) % 3]);
         }
-        const int q = k * (nx * ny) + j * nx + i;
+        const int q = k * (pitch * ny) + j * pitch + i;
         // the pair's streams, packed, in flight while the ring wait and the
         // derivatives proceed
         __half2 sp[6];
@@ -908,7 +916,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
         double2 dC = make_double2(0.0, 0.0), dS = dC;
         const int zs = slab_pos(k, nz, p.P);
         const int ox[2] = {(k * ny + j) * p.W + xs[0], (k * ny + j) * p.W + xs[1]};
-        const int oy = (k * p.W + ys) * nx + i, oz = (zs * ny + j) * nx + i;
+        const int oy = (k * p.W + ys) * pitch + i, oz = (zs * ny + j) * pitch + i;
         float qx[2][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
         float2 qy[3] = {pair(0.0f, 0.0f), pair(0.0f, 0.0f), pair(0.0f, 0.0f)};
         float2 qz[3] = {qy[0], qy[0], qy[0]};
@@ -1014,7 +1022,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
             }
             float2 srcv = pair(0.0f, 0.0f);
             if ((st.flags & kStepSource) && k == p.k_src) {
-                const float4 a = *reinterpret_cast<const float4 *>(p.src + j * nx + i);
+                const float4 a = *reinterpret_cast<const float4 *>(p.src + j * pitch + i);
                 srcv = st::source_value<float2>(p.src_scale, pair(a.x, a.z), pair(a.y, a.w),
                                                 st.src_ws, st.src_wc);
             }
@@ -1025,7 +1033,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
                                          pair(ca.nmu2U, cb.nmu2U), pair(ca.nmu2T, cb.nmu2T), exx,
                                          eyy, ezz, srcv, sv, rv);
             const float2 pr = st::pressure(sv);
-            if (!isfinite(pr.x) || !isfinite(pr.y)) atomicOr(p.flag, 1);
+            if (!isfinite(pr.x) || (two && !isfinite(pr.y))) atomicOr(p.flag, 1);
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) {
                 put_s(cc, true);
@@ -1046,7 +1054,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
                     const float2 h = __ldg(&pmly[p.nmax + j]);
                     float2 t;
                     a = st::cpml_v(qy[1], splat<float2>(h.x), splat<float2>(h.y), a, t);
-                    if (jy1) st::st2_or_1(p.psy + 4 * Sys + oy, t, ix1);
+                    if (jy1 && ix0) st::st2_or_1(p.psy + 4 * Sys + oy, t, ix1);
                 }
                 if (EDGE) {
 #pragma unroll
@@ -1055,14 +1063,14 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
                         const float2 h = __ldg(&pmlx[p.nmax + i + l]);
                         float t;
                         set_lane(b, l, st::cpml_v(qx[l][1], h.x, h.y, lane(b, l), t));
-                        if (jy1 && (l == 0 || ix1)) p.psx[4 * Sxs + ox[l]] = t;
+                        if (jy1 && (l == 0 ? ix0 : ix1)) p.psx[4 * Sxs + ox[l]] = t;
                     }
                 }
                 float2 psic, thec;
                 coef(mb, I0[IW], I0[IW + 1], I0[2], I0[IW + 1], I0[IW + 2], psic, thec);
                 unpack(3);
                 st::shear_update<L, float2>(p, psic, thec, st::vadd(a, b), 3, sv, rv);
-                if (jy1) {
+                if (jy1 && ix0) {
                     put_s(3, ix1);
                     put_r(3, ix1);
                 }
@@ -1075,7 +1083,7 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
                     const float2 h = __ldg(&pmlz[p.nmax + k]);
                     float2 t;
                     a = st::cpml_v(qz[1], splat<float2>(h.x), splat<float2>(h.y), a, t);
-                    if (kz1) st::st2_or_1(p.psz + 4 * Szs + oz, t, ix1);
+                    if (kz1 && ix0) st::st2_or_1(p.psz + 4 * Szs + oz, t, ix1);
                 }
                 if (EDGE) {
 #pragma unroll
@@ -1084,14 +1092,14 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
                         const float2 h = __ldg(&pmlx[p.nmax + i + l]);
                         float t;
                         set_lane(b, l, st::cpml_v(qx[l][2], h.x, h.y, lane(b, l), t));
-                        if (kz1 && (l == 0 || ix1)) p.psx[5 * Sxs + ox[l]] = t;
+                        if (kz1 && (l == 0 ? ix0 : ix1)) p.psx[5 * Sxs + ox[l]] = t;
                     }
                 }
                 float2 psic, thec;
                 coef(mb, I1[0], I1[1], I0[2], I1[1], I1[2], psic, thec);
                 unpack(4);
                 st::shear_update<L, float2>(p, psic, thec, st::vadd(a, b), 4, sv, rv);
-                if (kz1) {
+                if (kz1 && ix0) {
                     put_s(4, ix1);
                     put_r(4, ix1);
                 }
@@ -1155,22 +1163,22 @@ __device__ __forceinline__ bool stress_tile_h2(const AcParams &p, const StressTm
     return ab >= 0;
 }
 
-template <int L, int MINB, int TH>
+template <int L, int MINB, int TH, bool PAD>
 __global__ void __launch_bounds__(PX * TH, MINB)
     k_stress_tma_h2(const __grid_constant__ AcParams p, int kchunk,
                     const __grid_constant__ StressTmaMaps tm)
 {
     extern __shared__ __align__(1024) unsigned char smb[];
-    stress_tile_h2<L, false, TH>(p, tm, p.st, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
+    stress_tile_h2<L, false, TH, PAD>(p, tm, p.st, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
 }
 
-template <int L, int MINB, typename T, int TH>
+template <int L, int MINB, typename T, int TH, bool PAD>
 __global__ void __launch_bounds__(TX * TH, MINB)
     k_stress_tma(const __grid_constant__ AcParams p, int kchunk,
                  const __grid_constant__ StressTmaMaps tm)
 {
     extern __shared__ __align__(1024) unsigned char smb[];
-    stress_tile<L, T, false, TH>(p, tm, p.st, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
+    stress_tile<L, T, false, TH, PAD>(p, tm, p.st, kchunk, blockIdx.x, blockIdx.y, blockIdx.z, smb);
 }
 
 // ------------------------------------------------------------------ batch
@@ -1310,39 +1318,43 @@ static int chunk_or(const AcParams &p, int th, int rule)
     return p.hold ? std::min(p.nz, std::max(8, rule)) : rule;
 }
 
-template <typename T, int TH>
+template <typename T, int TH, bool PAD>
 static cudaError_t launch_velocity_tma_t(const AcParams &p, const VelocityTmaMaps &tm,
                                          cudaStream_t s)
 {
     const int kc = chunk_or(p, TH, velocity_kchunk(p.nx, p.ny, p.nz, TH));
     const size_t sm = VelLayout<T, TH>::bytes(p.n_mat);
     static std::atomic<int> done{0};
-    cudaError_t e = raise_smem_once(k_velocity_tma<T, TH>,
+    cudaError_t e = raise_smem_once(k_velocity_tma<T, TH, PAD>,
                                     VelLayout<T, TH>::bytes(BVF_MAX_MATERIALS), done);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_velocity_tma<T, TH>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p, kc, tm);
+    return launch_pdl(k_velocity_tma<T, TH, PAD>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p, kc, tm);
 }
 
 // tile heights other than TY are built for L = 2 (the method's two
 // mechanisms); other L take TY
-template <typename T>
+template <typename T, bool PAD>
 static cudaError_t launch_velocity_tma_h(const AcParams &p, const VelocityTmaMaps &tm,
                                          cudaStream_t s)
 {
-    if (p.L == 2 && p.tile_yv == 4) return launch_velocity_tma_t<T, 4>(p, tm, s);
-    if (p.L == 2 && p.tile_yv == 16) return launch_velocity_tma_t<T, 16>(p, tm, s);
-    return launch_velocity_tma_t<T, TY>(p, tm, s);
+    if (p.L == 2 && p.tile_yv == 4) return launch_velocity_tma_t<T, 4, PAD>(p, tm, s);
+    if (p.L == 2 && p.tile_yv == 16) return launch_velocity_tma_t<T, 16, PAD>(p, tm, s);
+    return launch_velocity_tma_t<T, TY, PAD>(p, tm, s);
 }
 
 cudaError_t launch_velocity_tma(const AcParams &p, const VelocityTmaMaps &tm, cudaStream_t s)
 {
-    return p.h16 ? launch_velocity_tma_h<__half>(p, tm, s) : launch_velocity_tma_h<float>(p, tm, s);
+    if (p.pitch != p.nx)
+        return p.h16 ? launch_velocity_tma_h<__half, true>(p, tm, s)
+                     : launch_velocity_tma_h<float, true>(p, tm, s);
+    return p.h16 ? launch_velocity_tma_h<__half, false>(p, tm, s)
+                 : launch_velocity_tma_h<float, false>(p, tm, s);
 }
 
 // Resident blocks per SM at height TH: the thread count times blocks per SM
 // of the default height (four blocks of 256 threads for the scalar tile, five
 // of 128 for the paired FP16 tile) is kept, so are the registers per thread.
-template <int L, typename T, int TH>
+template <int L, typename T, int TH, bool PAD>
 static cudaError_t launch_stress_tma_t(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s)
 {
     const int kc = chunk_or(p, TH, stress_kchunk(p.nx, p.ny, p.nz, TH, p.h16));
@@ -1351,31 +1363,31 @@ static cudaError_t launch_stress_tma_t(const AcParams &p, const StressTmaMaps &t
     if constexpr (std::is_same<T, __half>::value && L > 0) {
         // FP16 storage: the paired tile (see stress_tile_h2)
         constexpr int MB = kStressH2Blocks * TY / TH > 0 ? kStressH2Blocks * TY / TH : 1;
-        cudaError_t e = raise_smem_once(k_stress_tma_h2<L, MB, TH>,
+        cudaError_t e = raise_smem_once(k_stress_tma_h2<L, MB, TH, PAD>,
                                         StressLayout<L, T, TH>::bytes(BVF_MAX_MATERIALS), done);
         if (e != cudaSuccess) return e;
-        return launch_pdl(k_stress_tma_h2<L, MB, TH>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p,
+        return launch_pdl(k_stress_tma_h2<L, MB, TH, PAD>, grid_tma<TH>(p, kc), dim3(PX, TH, 1), sm, s, p,
                           kc, tm);
     } else {
         constexpr int MB = 4 * TY / TH;
-        cudaError_t e = raise_smem_once(k_stress_tma<L, MB, T, TH>,
+        cudaError_t e = raise_smem_once(k_stress_tma<L, MB, T, TH, PAD>,
                                         StressLayout<L, T, TH>::bytes(BVF_MAX_MATERIALS), done);
         if (e != cudaSuccess) return e;
-        return launch_pdl(k_stress_tma<L, MB, T, TH>, grid_tma<TH>(p, kc), dim3(TX, TH, 1), sm, s, p,
+        return launch_pdl(k_stress_tma<L, MB, T, TH, PAD>, grid_tma<TH>(p, kc), dim3(TX, TH, 1), sm, s, p,
                           kc, tm);
     }
 }
 
-template <typename T>
+template <typename T, bool PAD>
 static cudaError_t launch_stress_tma_l(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s)
 {
     switch (p.L) {
-    case 0: return launch_stress_tma_t<0, T, TY>(p, tm, s);
-    case 1: return launch_stress_tma_t<1, T, TY>(p, tm, s);
+    case 0: return launch_stress_tma_t<0, T, TY, PAD>(p, tm, s);
+    case 1: return launch_stress_tma_t<1, T, TY, PAD>(p, tm, s);
     case 2:
-        if (p.tile_y == 4) return launch_stress_tma_t<2, T, 4>(p, tm, s);
-        if (p.tile_y == 16) return launch_stress_tma_t<2, T, 16>(p, tm, s);
-        return launch_stress_tma_t<2, T, TY>(p, tm, s);
+        if (p.tile_y == 4) return launch_stress_tma_t<2, T, 4, PAD>(p, tm, s);
+        if (p.tile_y == 16) return launch_stress_tma_t<2, T, 16, PAD>(p, tm, s);
+        return launch_stress_tma_t<2, T, TY, PAD>(p, tm, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1384,7 +1396,11 @@ static cudaError_t launch_stress_tma_l(const AcParams &p, const StressTmaMaps &t
 // shared memory each in FP32 storage).
 cudaError_t launch_stress_tma(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s)
 {
-    return p.h16 ? launch_stress_tma_l<__half>(p, tm, s) : launch_stress_tma_l<float>(p, tm, s);
+    if (p.pitch != p.nx)
+        return p.h16 ? launch_stress_tma_l<__half, true>(p, tm, s)
+                     : launch_stress_tma_l<float, true>(p, tm, s);
+    return p.h16 ? launch_stress_tma_l<__half, false>(p, tm, s)
+                 : launch_stress_tma_l<float, false>(p, tm, s);
 }
 
 template <int L, typename T>

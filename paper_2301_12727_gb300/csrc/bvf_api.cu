@@ -41,7 +41,9 @@ struct bvf_ctx {
     bvf_grid g{};
     bvf_physics ph{};
     int L = 0;
-    size_t N = 0, fstride = 0;
+    size_t N = 0, fstride = 0;        // voxels; elements of one state array
+    int pitch = 0;                    // row length of the context's arrays (nx, or nx rounded up to 8)
+    size_t NP = 0;                    // elements of pitch * ny * nz
     int h16 = 0;                      // state stored as scaled FP16
     size_t es = 4;                    // bytes per state element
     double s_sig = 1.0, s_v = 1.0, s_r = 1.0;   // storage scales of sigma, v, r
@@ -307,14 +309,15 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
     return fn;
 }
 
-// 3-D map of an nx*ny*nz array (x fastest) with a bx x by x 1 box; points
+// 3-D map of an nx*ny*nz array (x fastest, rows pitch elements apart, 0: nx)
+// with a bx x by x 1 box; points
 // outside the array read as zero.
 bool encode_map(CUtensorMap *m, void *base, int nx, int ny, int nz, CUtensorMapDataType type,
-                size_t es, unsigned bx, unsigned by)
+                size_t es, unsigned bx, unsigned by, int pitch = 0)
 {
     auto enc = tensor_map_encoder();
     if (!enc) return false;
-    const size_t row = (size_t)nx * es;
+    const size_t row = (size_t)(pitch ? pitch : nx) * es;
     const cuuint64_t dims[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nz};
     const cuuint64_t strides[2] = {(cuuint64_t)row, (cuuint64_t)row * ny};
     const cuuint32_t box[3] = {bx, by, 1};
@@ -325,15 +328,15 @@ bool encode_map(CUtensorMap *m, void *base, int nx, int ny, int nz, CUtensorMapD
 }
 
 // Tensor maps of the TMA-fed kernels.  They need state rows that are whole
-// multiples of 16 bytes in both storages and an even nx for the voxel pairs
-// (nx % 8 == 0; the index is read from its padded copy when nx % 16 != 0) and
-// at most 2 SLS mechanisms; other grids use the direct kernels.
+// multiples of 16 bytes in both storages and aligned voxel pairs (a pitch that
+// is a multiple of 8; the index is read from its padded copy when nx % 16 !=
+// 0) and at most 2 SLS mechanisms; other grids use the direct kernels.
 void setup_maps(bvf_ctx *c)
 {
     c->tma = false;
     c->tma_stress = false;
     const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
-    if (nx % 8 != 0 || c->L > 2 || std::getenv("BVF_NO_TMA")) return;
+    if (c->pitch % 8 != 0 || c->L > 2 || std::getenv("BVF_NO_TMA")) return;
     const auto ST = c->h16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const auto U8 = CU_TENSOR_MAP_DATA_TYPE_UINT8;
     const size_t es = c->es;
@@ -348,12 +351,13 @@ void setup_maps(bvf_ctx *c)
     auto encode_for = [&](unsigned th, StressTmaMaps &sm, VelocityTmaMaps &vm) {
         bool ok = true;
         for (int v = 0; v < 3; ++v)
-            ok = ok && encode_map(&sm.v[v], fld(BVF_FIELD_VX + v), nx, ny, nz, ST, es, bw, th + 4);
+            ok = ok && encode_map(&sm.v[v], fld(BVF_FIELD_VX + v), nx, ny, nz, ST, es, bw, th + 4,
+                                  c->pitch);
         const unsigned w6[6] = {bw, 32, 32, bw, bw, 32},
                        h6[6] = {th, th + 4, th, th + 4, th, th + 4};
         for (int g6 = 0; g6 < 6; ++g6)
             ok = ok && encode_map(&vm.sg[g6], fld(BVF_FIELD_SXX + g6), nx, ny, nz, ST, es, w6[g6],
-                                  h6[g6]);
+                                  h6[g6], c->pitch);
         ok = ok && encode_map(&sm.idx, c->index_p ? c->index_p : c->index, idx_nx, ny, nz, U8, 1,
                               48, th + 1);
         vm.idx = sm.idx;
@@ -393,6 +397,7 @@ AcParams make_params(bvf_ctx *c)
     p.nx = c->g.nx;
     p.ny = c->g.ny;
     p.nz = c->g.nz;
+    p.pitch = c->pitch;
     p.P = c->P;
     p.W = c->W;
     p.L = c->L;
@@ -472,10 +477,10 @@ StepParam step_param(const bvf_ctx *c, const bvf_capture &cp, long long n)
 int ensure_dft(bvf_ctx *c, cudaStream_t s)
 {
     if (c->dftC) return BVF_OK;
-    CK(cudaMalloc(&c->dftC, c->N * sizeof(double)), "dft buffers");
-    CK(cudaMalloc(&c->dftS, c->N * sizeof(double)), "dft buffers");
-    CK(cudaMemsetAsync(c->dftC, 0, c->N * sizeof(double), s), "dft buffers");
-    CK(cudaMemsetAsync(c->dftS, 0, c->N * sizeof(double), s), "dft buffers");
+    CK(cudaMalloc(&c->dftC, c->NP * sizeof(double)), "dft buffers");
+    CK(cudaMalloc(&c->dftS, c->NP * sizeof(double)), "dft buffers");
+    CK(cudaMemsetAsync(c->dftC, 0, c->NP * sizeof(double), s), "dft buffers");
+    CK(cudaMemsetAsync(c->dftS, 0, c->NP * sizeof(double), s), "dft buffers");
     return BVF_OK;
 }
 
@@ -536,8 +541,10 @@ StateSections state_sections(const bvf_ctx *c)
 {
     auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };
     StateSections t{};
-    t.fields = (9 + 6 * (size_t)c->L) * c->fstride * c->es;
-    t.psi = kNumCpmlSlots * (c->slab_x + c->slab_y + c->slab_z) * sizeof(float);
+    // dense rows whatever the context's pitch
+    t.fields = (9 + 6 * (size_t)c->L) * ((c->N + 63) & ~(size_t)63) * c->es;
+    const size_t rows_yz = (size_t)c->W * (c->g.nz + c->g.ny);
+    t.psi = kNumCpmlSlots * (c->slab_x + rows_yz * c->g.nx) * sizeof(float);
     t.peak = c->N * sizeof(float);
     t.dft = c->N * sizeof(double);
     t.flag = sizeof(int);
@@ -549,6 +556,119 @@ StateSections state_sections(const bvf_ctx *c)
     t.off_flag = t.off_S + up(t.dft);
     t.total = t.off_flag + 256;
     return t;
+}
+
+// rows of nx elements of `es` bytes between an array of the context (rows
+// pitch apart) and a dense one
+cudaError_t copy_rows(const bvf_ctx *c, void *dense, void *own, size_t rows, size_t es, bool out,
+                      cudaStream_t s)
+{
+    const size_t w = (size_t)c->g.nx * es, p = (size_t)c->pitch * es;
+    if (w == p)
+        return cudaMemcpyAsync(out ? dense : own, out ? own : dense, rows * w,
+                               cudaMemcpyDeviceToDevice, s);
+    return out ? cudaMemcpy2DAsync(dense, w, own, p, w, rows, cudaMemcpyDeviceToDevice, s)
+               : cudaMemcpy2DAsync(own, p, dense, w, w, rows, cudaMemcpyDeviceToDevice, s);
+}
+
+// the snapshot's arrays between the context and the buffer at b
+cudaError_t copy_sections(const bvf_ctx *c, const StateSections &t, char *b, bool out,
+                          cudaStream_t s)
+{
+    const size_t rows = (size_t)c->g.ny * c->g.nz, lf = (c->N + 63) & ~(size_t)63;
+    char *f = static_cast<char *>(c->fields);
+    cudaError_t e = cudaSuccess;
+    if (c->pitch == c->g.nx) {
+        e = cudaMemcpyAsync(out ? b + t.off_fields : f, out ? f : b + t.off_fields, t.fields,
+                            cudaMemcpyDeviceToDevice, s);
+        if (e == cudaSuccess && t.psi)
+            e = cudaMemcpyAsync(out ? b + t.off_psi : (char *)c->psi,
+                                out ? (char *)c->psi : b + t.off_psi, t.psi,
+                                cudaMemcpyDeviceToDevice, s);
+    } else {
+        if (out) e = cudaMemsetAsync(b + t.off_fields, 0, t.fields, s);
+        // 9 arrays of rows of nx elements, then 6 of rows of nx L (the
+        // mechanisms of a voxel are adjacent)
+        for (int a = 0; a < 15 && e == cudaSuccess; ++a) {
+            const size_t L = c->L, n = a < 9 ? (size_t)a : 9 + (size_t)(a - 9) * L;
+            const size_t es = c->es * (a < 9 ? 1 : L);
+            if (es)
+                e = copy_rows(c, b + t.off_fields + n * lf * c->es, f + n * c->fstride * c->es, rows,
+                              es, out, s);
+        }
+        if (e == cudaSuccess && t.psi) {
+            char *d = b + t.off_psi, *own = reinterpret_cast<char *>(c->psi);
+            const size_t bx = kNumCpmlSlots * c->slab_x * sizeof(float);
+            e = cudaMemcpyAsync(out ? d : own, out ? own : d, bx, cudaMemcpyDeviceToDevice, s);
+            if (e == cudaSuccess)
+                e = copy_rows(c, d + bx, own + bx, (size_t)kNumCpmlSlots * c->W * (c->g.nz + c->g.ny),
+                              sizeof(float), out, s);
+        }
+    }
+    if (e == cudaSuccess) e = copy_rows(c, b + t.off_peak, c->peak, rows, sizeof(float), out, s);
+    if (c->dftC) {
+        if (e == cudaSuccess) e = copy_rows(c, b + t.off_C, c->dftC, rows, sizeof(double), out, s);
+        if (e == cudaSuccess) e = copy_rows(c, b + t.off_S, c->dftS, rows, sizeof(double), out, s);
+    }
+    return e;
+}
+
+Rows rows_of(const bvf_ctx *c) { return Rows{(unsigned)c->g.nx, (unsigned)c->pitch}; }
+
+void free_state(bvf_ctx *c)
+{
+    void **bufs[] = {&c->fields, (void **)&c->psi, (void **)&c->peak, (void **)&c->index,
+                     (void **)&c->lut, &c->slut, (void **)&c->buoy, (void **)&c->pml,
+                     (void **)&c->src, (void **)&c->flag, (void **)&c->scratch_u,
+                     (void **)&c->index_p};
+    for (void **b : bufs) {
+        if (*b) cudaFree(*b);
+        *b = nullptr;
+    }
+}
+
+// Device state of a context with rows of `pitch` elements, zeroed, and the
+// tensor maps over it.  On failure some buffers may be left (free_state).
+cudaError_t alloc_state(bvf_ctx *c, int pitch)
+{
+    const bvf_grid &g = c->g;
+    c->pitch = pitch;
+    c->NP = (size_t)pitch * g.ny * g.nz;
+    c->fstride = (c->NP + 63) & ~(size_t)63;
+    c->slab_x = (size_t)g.nz * g.ny * c->W;
+    c->slab_y = (size_t)g.nz * c->W * pitch;
+    c->slab_z = (size_t)c->W * g.ny * pitch;
+    c->index_pitch = (size_t)(g.nx + 15) / 16 * 16;
+    const size_t nf = 9 + 6 * (size_t)c->L;
+    const size_t npsi = kNumCpmlSlots * (c->slab_x + c->slab_y + c->slab_z);
+    const size_t idx_p = pitch % 8 == 0 && g.nx % 16 != 0 ? c->index_pitch * g.ny * g.nz : 0;
+    struct {
+        void **p;
+        size_t bytes;
+        bool zero;
+    } bufs[] = {
+        {&c->fields, nf * c->fstride * c->es, true},
+        {(void **)&c->psi, npsi * sizeof(float), true},
+        {(void **)&c->peak, c->NP * sizeof(float), true},
+        {(void **)&c->index, c->N, true},
+        {(void **)&c->lut, BVF_MAX_MATERIALS * sizeof(MatCoef), false},
+        {&c->slut, BVF_MAX_MATERIALS * 32, false},
+        {(void **)&c->buoy, (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float), false},
+        {(void **)&c->pml, 6 * (size_t)c->nmax * sizeof(float2), true},
+        {(void **)&c->src, (size_t)pitch * g.ny * sizeof(float2), false},
+        {(void **)&c->flag, sizeof(int), true},
+        {(void **)&c->scratch_u, sizeof(unsigned), false},
+        {(void **)&c->index_p, idx_p, true},
+    };
+    cudaError_t e = cudaSuccess;
+    for (auto &b : bufs) {
+        if (!b.bytes) continue;
+        if ((e = cudaMalloc(b.p, b.bytes)) != cudaSuccess) return e;
+        if (b.zero && (e = cudaMemset(*b.p, 0, b.bytes)) != cudaSuccess) return e;
+    }
+    if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+    setup_maps(c);
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -623,7 +743,6 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     c->ph = *phys;
     c->L = phys->n_sls;
     c->N = (size_t)g.nx * g.ny * g.nz;
-    c->fstride = (c->N + 63) & ~(size_t)63;
     c->h16 = phys->storage == BVF_STORAGE_F16;
     c->es = c->h16 ? 2 : 4;
     if (c->h16) {
@@ -637,48 +756,29 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     c->P = g.n_pml;
     c->W = g.n_pml > 0 ? 2 * g.n_pml + 1 : 0;
     c->nmax = std::max(g.nx, std::max(g.ny, g.nz));
-    c->slab_x = (size_t)g.nz * g.ny * c->W;
-    c->slab_y = (size_t)g.nz * c->W * g.nx;
-    c->slab_z = (size_t)c->W * g.ny * g.nx;
     c->tau_sigma = relaxation_times(phys->f0, c->L);
     if (const char *kc = std::getenv("BVF_KCHUNK")) c->kchunk = std::max(0, std::atoi(kc));
-
-    auto cleanup = [&](int code) { bvf_destroy(c); return code; };
-    cudaError_t e;
-    const size_t nf = 9 + 6 * (size_t)c->L;
-    if ((e = cudaMalloc(&c->fields, nf * c->fstride * c->es)) != cudaSuccess)
-        return cleanup(cuda_fail(nullptr, e, "bvf_create: fields"));
-    const size_t npsi = kNumCpmlSlots * (c->slab_x + c->slab_y + c->slab_z);
-    if (npsi && (e = cudaMalloc(&c->psi, npsi * sizeof(float))) != cudaSuccess)
-        return cleanup(cuda_fail(nullptr, e, "bvf_create: cpml"));
-    if ((e = cudaMalloc(&c->peak, c->N * sizeof(float))) != cudaSuccess ||
-        (e = cudaMalloc(&c->index, c->N)) != cudaSuccess ||
-        (e = cudaMalloc(&c->lut, BVF_MAX_MATERIALS * sizeof(MatCoef))) != cudaSuccess ||
-        (e = cudaMalloc(&c->slut, BVF_MAX_MATERIALS * 32)) != cudaSuccess ||
-        (e = cudaMalloc(&c->buoy, (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float))) !=
-            cudaSuccess ||
-        (e = cudaMalloc(&c->pml, 6 * (size_t)c->nmax * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMalloc(&c->src, (size_t)g.nx * g.ny * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMalloc(&c->flag, sizeof(int))) != cudaSuccess ||
-        (e = cudaMalloc(&c->scratch_u, sizeof(unsigned))) != cudaSuccess)
-        return cleanup(cuda_fail(nullptr, e, "bvf_create: buffers"));
-    if ((e = cudaMemset(c->fields, 0, nf * c->fstride * c->es)) != cudaSuccess ||
-        (npsi && (e = cudaMemset(c->psi, 0, npsi * sizeof(float))) != cudaSuccess) ||
-        (e = cudaMemset(c->peak, 0, c->N * sizeof(float))) != cudaSuccess ||
-        (e = cudaMemset(c->index, 0, c->N)) != cudaSuccess ||
-        (e = cudaMemset(c->pml, 0, 6 * (size_t)c->nmax * sizeof(float2))) != cudaSuccess ||
-        (e = cudaMemset(c->flag, 0, sizeof(int))) != cudaSuccess ||
-        (e = cudaDeviceSynchronize()) != cudaSuccess)
-        return cleanup(cuda_fail(nullptr, e, "bvf_create: zero fill"));
-    if (g.nx % 8 == 0 && g.nx % 16 != 0) {
-        c->index_pitch = (size_t)(g.nx + 15) / 16 * 16;
-        const size_t bytes = c->index_pitch * g.ny * g.nz;
-        if ((e = cudaMalloc(&c->index_p, bytes)) != cudaSuccess ||
-            (e = cudaMemset(c->index_p, 0, bytes)) != cudaSuccess ||
-            (e = cudaDeviceSynchronize()) != cudaSuccess)
-            return cleanup(cuda_fail(nullptr, e, "bvf_create: padded index"));
+    // Rows padded to a multiple of 8 let the TMA-fed kernels take any nx: the
+    // direct kernels, which load every halo by hand, need 653 us a step at 197
+    // x 211 x 163 against 320.  Up to a quarter more memory (nx of about 29
+    // and up); without it (or where a switch keeps a kernel direct) rows stay
+    // dense.
+    const int padded = (g.nx + 7) / 8 * 8;
+    const char *st_env = std::getenv("BVF_STRESS_TMA");
+    const bool pad = padded != g.nx && 4LL * padded <= 5LL * g.nx && c->L <= 2 &&
+                     (double)padded * g.ny * g.nz < 2147483648.0 && tensor_map_encoder() &&
+                     !std::getenv("BVF_NO_TMA") && !(st_env && st_env[0] == '0');
+    cudaError_t e = pad ? alloc_state(c, padded) : cudaErrorMemoryAllocation;
+    if (e != cudaSuccess || !c->tma) {
+        free_state(c);
+        (void)cudaGetLastError();
+        e = alloc_state(c, g.nx);
     }
-    setup_maps(c);
+    if (e != cudaSuccess) {
+        const int rc = cuda_fail(nullptr, e, "bvf_create: buffers");
+        bvf_destroy(c);
+        return rc;
+    }
     *out = c;
     return BVF_OK;
 }
@@ -796,8 +896,8 @@ int bvf_set_source(bvf_ctx *c, int k_plane, const float *d_plane, double c0, int
         (env != BVF_ENV_BURST && env != BVF_ENV_RAMP_CW) || (env == BVF_ENV_BURST && n_cycles < 1))
         return fail(c, BVF_E_ARG, "bvf_set_source: bad plane, speed, envelope or cycle count");
     cudaStream_t s = (cudaStream_t)stream;
-    CK(cudaMemcpyAsync(c->src, d_plane, (size_t)c->g.nx * c->g.ny * sizeof(float2),
-                       cudaMemcpyDeviceToDevice, s), "copy source plane");
+    CK(copy_rows(c, const_cast<float *>(d_plane), c->src, c->g.ny, sizeof(float2), false, s),
+       "copy source plane");
     c->k_src = k_plane;
     c->c0 = c0;
     c->envelope = env;
@@ -814,10 +914,10 @@ int bvf_reset(bvf_ctx *c, void *stream)
     CK(cudaMemsetAsync(c->fields, 0, nf * c->fstride * c->es, s), "reset");
     const size_t npsi = kNumCpmlSlots * (c->slab_x + c->slab_y + c->slab_z);
     if (npsi) CK(cudaMemsetAsync(c->psi, 0, npsi * sizeof(float), s), "reset");
-    CK(cudaMemsetAsync(c->peak, 0, c->N * sizeof(float), s), "reset");
+    CK(cudaMemsetAsync(c->peak, 0, c->NP * sizeof(float), s), "reset");
     if (c->dftC) {
-        CK(cudaMemsetAsync(c->dftC, 0, c->N * sizeof(double), s), "reset");
-        CK(cudaMemsetAsync(c->dftS, 0, c->N * sizeof(double), s), "reset");
+        CK(cudaMemsetAsync(c->dftC, 0, c->NP * sizeof(double), s), "reset");
+        CK(cudaMemsetAsync(c->dftS, 0, c->NP * sizeof(double), s), "reset");
     }
     CK(cudaMemsetAsync(c->flag, 0, sizeof(int), s), "reset");
     c->dft_count = 0;
@@ -902,11 +1002,12 @@ int bvf_get_field(bvf_ctx *c, int which, float *d_out, void *stream)
     if (!c || !d_out || which < 0 || which >= 9 + 6 * c->L)
         return fail(c, BVF_E_ARG, "bvf_get_field: bad context, pointer or field id");
     if (!c->h16 && field_stride(c, which) == 1)
-        CK(cudaMemcpyAsync(d_out, field_ptr(c, which), c->N * sizeof(float),
-                           cudaMemcpyDeviceToDevice, (cudaStream_t)stream), "get field");
+        CK(copy_rows(c, d_out, field_ptr(c, which), (size_t)c->g.ny * c->g.nz, sizeof(float), true,
+                     (cudaStream_t)stream), "get field");
     else {
         CK(launch_field_out(field_ptr(c, which), c->h16, field_stride(c, which),
-                            (float)field_scale(c, which), d_out, c->N, (cudaStream_t)stream),
+                            (float)field_scale(c, which), d_out, c->N, rows_of(c),
+                            (cudaStream_t)stream),
            "get field");
         c->launches++;
     }
@@ -918,12 +1019,12 @@ int bvf_set_field(bvf_ctx *c, int which, const float *d_in, void *stream)
     if (!c || !d_in || which < 0 || which >= 9 + 6 * c->L)
         return fail(c, BVF_E_ARG, "bvf_set_field: bad context, pointer or field id");
     if (!c->h16 && field_stride(c, which) == 1)
-        CK(cudaMemcpyAsync(field_ptr(c, which), d_in, c->N * sizeof(float),
-                           cudaMemcpyDeviceToDevice, (cudaStream_t)stream), "set field");
+        CK(copy_rows(c, const_cast<float *>(d_in), field_ptr(c, which), (size_t)c->g.ny * c->g.nz,
+                     sizeof(float), false, (cudaStream_t)stream), "set field");
     else {
         CK(launch_field_in(d_in, c->h16, field_stride(c, which),
                            (float)(1.0 / field_scale(c, which)), field_ptr(c, which), c->N,
-                           (cudaStream_t)stream), "set field");
+                           rows_of(c), (cudaStream_t)stream), "set field");
         c->launches++;
     }
     return BVF_OK;
@@ -934,7 +1035,7 @@ int bvf_get_pressure(bvf_ctx *c, float *d_out, void *stream)
     if (!c || !d_out) return fail(c, BVF_E_ARG, "bvf_get_pressure: NULL argument");
     CK(launch_pressure(field_ptr(c, BVF_FIELD_SXX), field_ptr(c, BVF_FIELD_SYY),
                        field_ptr(c, BVF_FIELD_SZZ), c->h16, (float)c->s_sig, d_out, c->N,
-                       (cudaStream_t)stream),
+                       rows_of(c), (cudaStream_t)stream),
        "pressure kernel");
     c->launches++;
     return BVF_OK;
@@ -944,10 +1045,11 @@ int bvf_get_peak(bvf_ctx *c, float *d_out, void *stream)
 {
     if (!c || !d_out) return fail(c, BVF_E_ARG, "bvf_get_peak: NULL argument");
     if (!c->h16)
-        CK(cudaMemcpyAsync(d_out, c->peak, c->N * sizeof(float), cudaMemcpyDeviceToDevice,
-                           (cudaStream_t)stream), "get peak");
+        CK(copy_rows(c, d_out, c->peak, (size_t)c->g.ny * c->g.nz, sizeof(float), true,
+                     (cudaStream_t)stream), "get peak");
     else {
-        CK(launch_scale_copy(c->peak, (float)c->s_sig, d_out, c->N, (cudaStream_t)stream),
+        CK(launch_scale_copy(c->peak, (float)c->s_sig, d_out, c->N, rows_of(c),
+                             (cudaStream_t)stream),
            "get peak");
         c->launches++;
     }
@@ -959,7 +1061,7 @@ int bvf_get_amp_phase(bvf_ctx *c, double *d_amp, double *d_phase, void *stream)
     if (!c) return fail(nullptr, BVF_E_ARG, "bvf_get_amp_phase: NULL context");
     if (!c->dftC || c->dft_count <= 0)
         return fail(c, BVF_E_ARG, "bvf_get_amp_phase: no step was captured");
-    CK(launch_amp_phase(c->dftC, c->dftS, c->N, c->dft_count, c->s_sig, d_amp, d_phase,
+    CK(launch_amp_phase(c->dftC, c->dftS, c->N, rows_of(c), c->dft_count, c->s_sig, d_amp, d_phase,
                         (cudaStream_t)stream), "amp/phase kernel");
     c->launches++;
     return BVF_OK;
@@ -1429,7 +1531,7 @@ int bvf_batch_create(bvf_ctx *const *ctxs, int n, bvf_batch **out)
         const bvf_ctx *c = ctxs[d];
         if (!c || !c->have_materials)
             return fail(nullptr, BVF_E_ARG, "bvf_batch_create: NULL context or materials not set");
-        if (!c->tma || !c->tma_stress)
+        if (!c->tma || !c->tma_stress || c->g.nx % 8 != 0)
             return fail(nullptr, BVF_E_ARG,
                         "bvf_batch_create: every grid needs nx % 8 == 0 and at most 2 SLS");
         if (c->L != ctxs[0]->L || c->h16 != ctxs[0]->h16)
@@ -1940,8 +2042,8 @@ int bvf_test_withhold_copy(bvf_ctx *c, int kernel, int plane, unsigned wait_limi
     if ((kernel < 1 || kernel > 3) || plane < 0 || plane >= c->g.nz)
         return fail(c, BVF_E_ARG,
                     "bvf_test_withhold_copy: kernel must be 1, 2 or 3, plane inside the grid");
-    if (kernel < 3 ? !(kernel == 1 ? c->tma : c->tma_stress)
-                   : (c->g.nx % 8 != 0 || std::getenv("BVF_NO_TMA") != nullptr))
+    if (c->g.nx % 8 != 0 || (kernel < 3 ? !(kernel == 1 ? c->tma : c->tma_stress)
+                                        : std::getenv("BVF_NO_TMA") != nullptr))
         return fail(c, BVF_E_ARG, "bvf_test_withhold_copy: this context does not use the TMA-fed kernel");
     c->hold = kernel;
     c->hold_plane = plane;
@@ -1980,15 +2082,9 @@ int bvf_state_save(bvf_ctx *c, void *d_buf, size_t bytes, void *stream)
     h.bytes = t.total;
     // pageable source: the copy is staged before the call returns
     CK(cudaMemcpyAsync(b, &h, sizeof h, cudaMemcpyHostToDevice, s), "bvf_state_save");
-    CK(cudaMemcpyAsync(b + t.off_fields, c->fields, t.fields, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
-    if (t.psi) CK(cudaMemcpyAsync(b + t.off_psi, c->psi, t.psi, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
-    CK(cudaMemcpyAsync(b + t.off_peak, c->peak, t.peak, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
-    if (c->dftC) {
-        CK(cudaMemcpyAsync(b + t.off_C, c->dftC, t.dft, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
-        CK(cudaMemcpyAsync(b + t.off_S, c->dftS, t.dft, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
-    } else {
+    CK(copy_sections(c, t, b, true, s), "bvf_state_save");
+    if (!c->dftC)
         CK(cudaMemsetAsync(b + t.off_C, 0, 2 * (t.off_S - t.off_C), s), "bvf_state_save");
-    }
     CK(cudaMemcpyAsync(b + t.off_flag, c->flag, t.flag, cudaMemcpyDeviceToDevice, s), "bvf_state_save");
     return BVF_OK;
 }
@@ -2013,13 +2109,7 @@ int bvf_state_load(bvf_ctx *c, const void *d_buf, size_t bytes, void *stream)
         const int rc = ensure_dft(c, s);
         if (rc != BVF_OK) return rc;
     }
-    CK(cudaMemcpyAsync(c->fields, b + t.off_fields, t.fields, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
-    if (t.psi) CK(cudaMemcpyAsync(c->psi, b + t.off_psi, t.psi, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
-    CK(cudaMemcpyAsync(c->peak, b + t.off_peak, t.peak, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
-    if (c->dftC) {
-        CK(cudaMemcpyAsync(c->dftC, b + t.off_C, t.dft, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
-        CK(cudaMemcpyAsync(c->dftS, b + t.off_S, t.dft, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
-    }
+    CK(copy_sections(c, t, const_cast<char *>(b), false, s), "bvf_state_load");
     CK(cudaMemcpyAsync(c->flag, b + t.off_flag, t.flag, cudaMemcpyDeviceToDevice, s), "bvf_state_load");
     c->steps = h.steps;
     c->dft_count = (int)h.dft_count;
@@ -2116,8 +2206,8 @@ int bvf_time_reversal_plane(bvf_ctx *c, int ti, int tj, int tk, int k_src, int n
     const bvf_capture cap{-1, n_steps - 2 * M + 1, 2 * M};
     if (rc == BVF_OK) rc = bvf_run_acoustic(c, n_steps, &cap, stream);
     if (rc != BVF_OK) return done(rc);
-    e = launch_conj_plane(c->dftC + (size_t)k_src * plane, c->dftS + (size_t)k_src * plane, plane,
-                          d_max, reinterpret_cast<float2 *>(d_plane), s);
+    const size_t at = (size_t)k_src * c->pitch * ny;
+    e = launch_conj_plane(c->dftC + at, c->dftS + at, plane, rows_of(c), d_max, reinterpret_cast<float2 *>(d_plane), s);
     if (e != cudaSuccess) return done(cuda_fail(c, e, "bvf_time_reversal_plane: conjugate plane"));
     c->launches += 2;
     rc = bvf_synchronize(c, stream);

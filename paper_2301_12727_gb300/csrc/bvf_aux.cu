@@ -18,6 +18,14 @@ inline unsigned blocks_for(size_t n, int per_block = kThreads, unsigned cap = 15
     return (unsigned)(b < cap ? (b ? b : 1) : cap);
 }
 
+// element q of a dense array in one with row pitch r.pitch
+__device__ __forceinline__ size_t in_rows(size_t q, Rows r)
+{
+    if (r.pitch == r.nx) return q;
+    const unsigned row = (unsigned)q / r.nx;
+    return (size_t)row * r.pitch + ((unsigned)q - row * r.nx);
+}
+
 __global__ void k_index_max(const uint8_t *__restrict__ idx, size_t n, unsigned *out)
 {
     unsigned m = 0;
@@ -38,47 +46,51 @@ __global__ void k_stress_table(const MatCoef *__restrict__ lut, int n, float Lf,
 
 template <typename T>
 __global__ void k_pressure(const T *__restrict__ a, const T *__restrict__ b,
-                           const T *__restrict__ c, float scale, float *__restrict__ out, size_t n)
+                           const T *__restrict__ c, float scale, float *__restrict__ out, size_t n,
+                           Rows r)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-         q += (size_t)gridDim.x * blockDim.x)
-        out[q] = -(st::tof(a[q]) + st::tof(b[q]) + st::tof(c[q])) / 3.0f * scale;
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = in_rows(q, r);
+        out[q] = -(st::tof(a[i]) + st::tof(b[i]) + st::tof(c[i])) / 3.0f * scale;
+    }
 }
 
 // state array (element q at f[q * stride]) <-> FP32 values in physical units
 // (scale = the storage scale)
 template <typename T>
 __global__ void k_field_out(const T *__restrict__ f, size_t stride, float scale,
-                            float *__restrict__ out, size_t n)
+                            float *__restrict__ out, size_t n, Rows r)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x)
-        out[q] = st::tof(f[q * stride]) * scale;
+        out[q] = st::tof(f[in_rows(q, r) * stride]) * scale;
 }
 template <typename T>
 __global__ void k_field_in(const float *__restrict__ in, size_t stride, float inv_scale,
-                           T *__restrict__ f, size_t n)
+                           T *__restrict__ f, size_t n, Rows r)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x)
-        st::stv(f + q * stride, in[q] * inv_scale);
+        st::stv(f + in_rows(q, r) * stride, in[q] * inv_scale);
 }
 // out = in * scale, or out = scale where in is NULL (fill)
 __global__ void k_scale_copy(const float *__restrict__ in, float scale, float *__restrict__ out,
-                             size_t n)
+                             size_t n, Rows r)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x)
-        out[q] = in ? in[q] * scale : scale;
+        out[q] = in ? in[in_rows(q, r)] * scale : scale;
 }
 
 // p(t) = A cos(w t + phi): C = A N/2 cos phi, S = -A N/2 sin phi
 __global__ void k_amp_phase(const double *__restrict__ C, const double *__restrict__ S, size_t n,
-                            double inv_half_n, double scale, double *amp, double *ph)
+                            Rows r, double inv_half_n, double scale, double *amp, double *ph)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x) {
-        const double c = C[q], s = S[q];
+        const size_t i = in_rows(q, r);
+        const double c = C[i], s = S[i];
         if (amp) amp[q] = sqrt(c * c + s * s) * inv_half_n * scale;
         if (ph) ph[q] = atan2(-s, c);
     }
@@ -495,35 +507,40 @@ __global__ void __launch_bounds__(1024) k_plane_sums(
 // (non-negative doubles order like their bit patterns, so one 64-bit
 // atomicMax keeps it); second pass: the normalised conjugate.
 __global__ void k_plane_absmax(const double *__restrict__ C, const double *__restrict__ S,
-                               size_t n, unsigned long long *out)
+                               size_t n, Rows r, unsigned long long *out)
 {
     double m = 0.0;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-         q += (size_t)gridDim.x * blockDim.x)
-        m = fmax(m, C[q] * C[q] + S[q] * S[q]);
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = in_rows(q, r);
+        m = fmax(m, C[i] * C[i] + S[i] * S[i]);
+    }
     for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
 __global__ void k_conj_normalise(const double *__restrict__ C, const double *__restrict__ S,
-                                 size_t n, const unsigned long long *mx, float2 *__restrict__ out)
+                                 size_t n, Rows r, const unsigned long long *mx,
+                                 float2 *__restrict__ out)
 {
     const double m2 = __longlong_as_double((long long)*mx);
     const double inv = m2 > 0.0 ? 1.0 / sqrt(m2) : 0.0;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
-         q += (size_t)gridDim.x * blockDim.x)
-        out[q] = make_float2((float)(C[q] * inv), (float)(S[q] * inv));
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = in_rows(q, r);
+        out[q] = make_float2((float)(C[i] * inv), (float)(S[i] * inv));
+    }
 }
 
 }  // namespace
 
-cudaError_t launch_conj_plane(const double *C, const double *S, size_t n,
+cudaError_t launch_conj_plane(const double *C, const double *S, size_t n, Rows r,
                               unsigned long long *d_max, float2 *out, cudaStream_t s)
 {
     cudaError_t e = cudaMemsetAsync(d_max, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    k_plane_absmax<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, d_max);
-    k_conj_normalise<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, d_max, out);
+    k_plane_absmax<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, r, d_max);
+    k_conj_normalise<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, r, d_max, out);
     return cudaGetLastError();
 }
 
@@ -540,40 +557,40 @@ cudaError_t launch_index_max(const uint8_t *idx, size_t n, unsigned *d_out, cuda
 }
 
 cudaError_t launch_pressure(const void *sxx, const void *syy, const void *szz, int h16,
-                            float scale, float *out, size_t n, cudaStream_t s)
+                            float scale, float *out, size_t n, Rows r, cudaStream_t s)
 {
     if (h16)
         k_pressure<__half><<<blocks_for(n), kThreads, 0, s>>>(
             static_cast<const __half *>(sxx), static_cast<const __half *>(syy),
-            static_cast<const __half *>(szz), scale, out, n);
+            static_cast<const __half *>(szz), scale, out, n, r);
     else
         k_pressure<float><<<blocks_for(n), kThreads, 0, s>>>(
             static_cast<const float *>(sxx), static_cast<const float *>(syy),
-            static_cast<const float *>(szz), scale, out, n);
+            static_cast<const float *>(szz), scale, out, n, r);
     return cudaGetLastError();
 }
 
 cudaError_t launch_field_out(const void *f, int h16, size_t stride, float scale, float *out,
-                             size_t n, cudaStream_t s)
+                             size_t n, Rows r, cudaStream_t s)
 {
     if (h16)
         k_field_out<__half><<<blocks_for(n), kThreads, 0, s>>>(static_cast<const __half *>(f),
-                                                              stride, scale, out, n);
+                                                              stride, scale, out, n, r);
     else
         k_field_out<float><<<blocks_for(n), kThreads, 0, s>>>(static_cast<const float *>(f),
-                                                             stride, scale, out, n);
+                                                             stride, scale, out, n, r);
     return cudaGetLastError();
 }
 
 cudaError_t launch_field_in(const float *in, int h16, size_t stride, float inv_scale, void *f,
-                            size_t n, cudaStream_t s)
+                            size_t n, Rows r, cudaStream_t s)
 {
     if (h16)
         k_field_in<__half><<<blocks_for(n), kThreads, 0, s>>>(in, stride, inv_scale,
-                                                             static_cast<__half *>(f), n);
+                                                             static_cast<__half *>(f), n, r);
     else
         k_field_in<float><<<blocks_for(n), kThreads, 0, s>>>(in, stride, inv_scale,
-                                                            static_cast<float *>(f), n);
+                                                            static_cast<float *>(f), n, r);
     return cudaGetLastError();
 }
 
@@ -592,20 +609,21 @@ cudaError_t launch_add_const(float *x, float c, size_t n, cudaStream_t s)
 
 cudaError_t launch_fill(float *out, float value, size_t n, cudaStream_t s)
 {
-    k_scale_copy<<<blocks_for(n), kThreads, 0, s>>>(nullptr, value, out, n);
+    k_scale_copy<<<blocks_for(n), kThreads, 0, s>>>(nullptr, value, out, n, Rows{1, 1});
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_copy(const float *in, float scale, float *out, size_t n, cudaStream_t s)
+cudaError_t launch_scale_copy(const float *in, float scale, float *out, size_t n, Rows r,
+                              cudaStream_t s)
 {
-    k_scale_copy<<<blocks_for(n), kThreads, 0, s>>>(in, scale, out, n);
+    k_scale_copy<<<blocks_for(n), kThreads, 0, s>>>(in, scale, out, n, r);
     return cudaGetLastError();
 }
 
-cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, int count, double scale,
-                             double *amp, double *ph, cudaStream_t s)
+cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, Rows r, int count,
+                             double scale, double *amp, double *ph, cudaStream_t s)
 {
-    k_amp_phase<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, 2.0 / count, scale, amp, ph);
+    k_amp_phase<<<blocks_for(n), kThreads, 0, s>>>(C, S, n, r, 2.0 / count, scale, amp, ph);
     return cudaGetLastError();
 }
 

@@ -70,6 +70,7 @@ enum { kStepSource = 1, kStepPeak = 2, kStepDft = 4 };
 // Captured p (peak map, DFT sums) is in units of S_sigma.
 struct AcParams {
     int nx, ny, nz;
+    int pitch;           // row length of the state, peak, DFT, source and CPML arrays (>= nx)
     int P, W;            // CPML cells per face; slab width 2P+1 (0 if no CPML)
     int L;               // SLS mechanisms
     int n_mat;
@@ -83,7 +84,7 @@ struct AcParams {
     void *vx, *vy, *vz, *sxx, *syy, *szz, *sxy, *sxz, *syz;   // float or __half
     void *mem;           // memory variables, element mem_index(l, c, q)
     size_t fstride;
-    float *psx, *psy, *psz;   // CPML slabs: x [6][nz][ny][W], y [6][nz][W][nx], z [6][W][ny][nx]
+    float *psx, *psy, *psz;   // CPML slabs: x [6][nz][ny][W], y [6][nz][W][pitch], z [6][W][ny][pitch]
     const float2 *pml;   // (a, b) at [axis][h][s], h = 0 integer / 1 half point
     int nmax;
     // source plane
@@ -221,24 +222,30 @@ cudaError_t launch_stress_tma(const AcParams &p, const StressTmaMaps &tm, cudaSt
 // st::StressCoef of each of n materials (slut: n * 32 bytes, 16-byte aligned)
 cudaError_t launch_stress_table(const MatCoef *lut, int n, float Lf, void *slut, cudaStream_t s);
 cudaError_t launch_index_max(const uint8_t *idx, size_t n, unsigned *d_out, cudaStream_t s);
+// Read-outs of the context's arrays, whose rows of nx elements lie pitch apart,
+// into the caller's dense ones (launch_field_in: the other way).
+struct Rows {
+    unsigned nx, pitch;
+};
 cudaError_t launch_pressure(const void *sxx, const void *syy, const void *szz, int h16,
-                            float scale, float *out, size_t n, cudaStream_t s);
+                            float scale, float *out, size_t n, Rows r, cudaStream_t s);
 cudaError_t launch_field_out(const void *f, int h16, size_t stride, float scale, float *out,
-                             size_t n, cudaStream_t s);
+                             size_t n, Rows r, cudaStream_t s);
 cudaError_t launch_field_in(const float *in, int h16, size_t stride, float inv_scale, void *f,
-                            size_t n, cudaStream_t s);
-cudaError_t launch_scale_copy(const float *in, float scale, float *out, size_t n, cudaStream_t s);
+                            size_t n, Rows r, cudaStream_t s);
+cudaError_t launch_scale_copy(const float *in, float scale, float *out, size_t n, Rows r,
+                              cudaStream_t s);
 cudaError_t launch_fill(float *out, float value, size_t n, cudaStream_t s);
 // x[i] += c (round to nearest)
 cudaError_t launch_add_const(float *x, float c, size_t n, cudaStream_t s);
-cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, int count, double scale,
-                             double *amp, double *ph, cudaStream_t s);
+cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, Rows r, int count,
+                             double scale, double *amp, double *ph, cudaStream_t s);
 cudaError_t launch_rs(const float4 *el, int ne, int nx, int ny, float dx, float zp, float k_over_pi,
                       double pref, float2 *out, cudaStream_t s);
 cudaError_t launch_rs_weighted(const float4 *el, const float2 *wt, int ne, int nx, int ny,
                                float dx, float zp, float k_over_pi, double pref, float2 *out,
                                cudaStream_t s);
-cudaError_t launch_conj_plane(const double *C, const double *S, size_t n,
+cudaError_t launch_conj_plane(const double *C, const double *S, size_t n, Rows r,
                               unsigned long long *d_max, float2 *out, cudaStream_t s);
 cudaError_t launch_heat_source(const uint8_t *idx, const ThermCoef *lut, int n_mat,
                                const double *amp, double p_scale, float *Q, size_t n,
