@@ -64,6 +64,8 @@ struct bvf_ctx {
     int *flag = nullptr;
     unsigned *scratch_u = nullptr;
     float *T2 = nullptr, *Q = nullptr, *cemf = nullptr;
+    int *q_bad = nullptr;             // the heat source holds a non-finite value
+    uint8_t *cls = nullptr, *cls_of = nullptr;   // conduction class per voxel (rows of index_pitch), per material
     ThermCoef *tlut = nullptr;
     float *kface = nullptr;      // [n_mat][n_mat] face conductivities of the BHTE
     // the material index with rows padded to a multiple of 16 bytes, read by
@@ -703,7 +705,7 @@ void bvf_destroy(bvf_ctx *c)
 {
     if (!c) return;
     void *bufs[] = {c->fields, c->psi, c->peak, c->dftC, c->dftS, c->index, c->lut, c->slut, c->buoy,
-                    c->pml, c->src, c->flag, c->scratch_u, c->T2, c->Q, c->cemf, c->tlut,
+                    c->pml, c->src, c->flag, c->scratch_u, c->T2, c->Q, c->cemf, c->q_bad, c->cls, c->cls_of, c->tlut,
                     c->kface, c->index_p, c->h_index_d, c->h_peak_d, c->h_T_d, c->h_Tmax_d,
                     c->h_amp_d, c->h_cem_d};
     for (void *b : bufs)
@@ -1093,27 +1095,81 @@ int bvf_run_thermal(bvf_ctx *c, const bvf_thermal *th, const double *d_amp, floa
         CK(cudaMalloc(&c->T2, c->N * sizeof(float)), "thermal buffers");
         CK(cudaMalloc(&c->Q, c->N * sizeof(float)), "thermal buffers");
         CK(cudaMalloc(&c->cemf, c->N * sizeof(float)), "thermal buffers");
+        CK(cudaMalloc(&c->q_bad, sizeof(int)), "thermal buffers");
         CK(cudaMalloc(&c->tlut, BVF_MAX_MATERIALS * sizeof(ThermCoef)), "thermal buffers");
         CK(cudaMalloc(&c->kface, (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float)),
            "thermal buffers");
     }
-    // harmonic-mean face conductivity of every material pair (Sec. 2.4 FTCS
-    // stencil), in FP64 then rounded once
-    std::vector<float> kf((size_t)n_mat * n_mat);
-    for (int a = 0; a < n_mat; ++a)
-        for (int b = 0; b < n_mat; ++b) {
-            const double ka = c->table[a].k_th, kb = c->table[b].k_th;
-            kf[(size_t)a * n_mat + b] = (ka + kb > 0.0) ? (float)(2.0 * ka * kb / (ka + kb)) : 0.0f;
-        }
+    // TMA-fed steps where the rows are whole multiples of 16 bytes and both
+    // temperature buffers can be mapped (BVF_NO_TMA forces the direct kernel)
+    const bool want_tma = c->g.nx % 8 == 0 && !std::getenv("BVF_NO_TMA");
+    if (want_tma && !c->cls) {
+        const size_t bytes = c->index_pitch * c->g.ny * c->g.nz;
+        CK(cudaMalloc(&c->cls_of, BVF_MAX_MATERIALS), "thermal buffers");
+        CK(cudaMalloc(&c->cls, bytes), "thermal buffers");
+        CK(cudaMemsetAsync(c->cls, 0, bytes, s), "thermal buffers");
+    }
+    ThermTmaMaps tmaps[2];
+    bool th_tma = false;
+    if (want_tma) {
+        const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
+        const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+        const auto U8 = CU_TENSOR_MAP_DATA_TYPE_UINT8;
+        // one map per temperature buffer, chosen per step
+        th_tma = encode_map(&tmaps[0].T, d_T, nx, ny, nz, F32, 4, 40, 18) &&
+                 encode_map(&tmaps[1].T, c->T2, nx, ny, nz, F32, 4, 40, 18) &&
+                 encode_map(&tmaps[0].cls, c->cls, (int)c->index_pitch, ny, nz, U8, 1, 64, 18) &&
+                 encode_map(&tmaps[0].idx, c->index_p ? c->index_p : c->index,
+                            c->index_p ? (int)c->index_pitch : nx, ny, nz, U8, 1, 32, 16) &&
+                 encode_map(&tmaps[0].Q, c->Q, nx, ny, nz, F32, 4, 32, 16) &&
+                 encode_map(&tmaps[0].Tmax, d_Tmax, nx, ny, nz, F32, 4, 32, 16) &&
+                 encode_map(&tmaps[0].cemf, c->cemf, nx, ny, nz, F32, 4, 32, 16);
+        tmaps[1].cls = tmaps[0].cls;
+        tmaps[1].idx = tmaps[0].idx;
+        tmaps[1].Q = tmaps[0].Q;
+        tmaps[1].Tmax = tmaps[0].Tmax;
+        tmaps[1].cemf = tmaps[0].cemf;
+    }
+    // conduction classes: the materials of one conductivity (skull bins, for
+    // one, share theirs), so that faces inside a tissue need no pair look-up
+    std::vector<double> ks;
+    std::vector<uint8_t> cls_of(BVF_MAX_MATERIALS, 0);
+    for (int m = 0; m < n_mat; ++m) {
+        const size_t at = std::find(ks.begin(), ks.end(), c->table[m].k_th) - ks.begin();
+        if (at == ks.size()) ks.push_back(c->table[m].k_th);
+        cls_of[m] = (uint8_t)at;
+    }
+    const int n_cls = (int)ks.size();
+    // harmonic-mean face conductivity of every pair (Sec. 2.4 FTCS stencil), in
+    // FP64 then rounded once: of materials for the direct kernel, of classes
+    // for the TMA-fed one
+    auto face = [](double ka, double kb) {
+        return (ka + kb > 0.0) ? (float)(2.0 * ka * kb / (ka + kb)) : 0.0f;
+    };
+    const int nk = th_tma ? n_cls : n_mat;
+    std::vector<float> kf((size_t)nk * nk);
+    for (int a = 0; a < nk; ++a)
+        for (int b = 0; b < nk; ++b)
+            kf[(size_t)a * nk + b] =
+                th_tma ? face(ks[a], ks[b]) : face(c->table[a].k_th, c->table[b].k_th);
     // the diagonal rides with each material's coefficients: the kernels take
-    // it for a voxel whose six neighbours share its material
-    for (int m = 0; m < n_mat; ++m) tl[m].k = kf[(size_t)m * n_mat + m];
+    // it for a voxel whose six neighbours share its material (or class)
+    for (int m = 0; m < n_mat; ++m) tl[m].k = face(c->table[m].k_th, c->table[m].k_th);
+    if (th_tma) {
+        CK(cudaMemcpyAsync(c->cls_of, cls_of.data(), cls_of.size(), cudaMemcpyHostToDevice, s),
+           "thermal classes");
+        CK(launch_classes(c->index, c->cls_of, c->cls, c->N,
+                          Rows{(unsigned)c->g.nx, (unsigned)c->index_pitch}, s), "thermal classes");
+        c->launches++;
+    }
     CK(cudaMemsetAsync(c->cemf, 0, c->N * sizeof(float), s), "thermal buffers");
     CK(cudaMemcpyAsync(c->tlut, tl.data(), n_mat * sizeof(ThermCoef), cudaMemcpyHostToDevice, s),
        "thermal lut");
     CK(cudaMemcpyAsync(c->kface, kf.data(), kf.size() * sizeof(float), cudaMemcpyHostToDevice, s),
        "thermal face table");
-    CK(launch_heat_source(c->index, c->tlut, n_mat, d_amp, th->p_scale, c->Q, c->N, s), "heat source");
+    CK(cudaMemsetAsync(c->q_bad, 0, sizeof(int), s), "thermal buffers");
+    CK(launch_heat_source(c->index, c->tlut, n_mat, d_amp, th->p_scale, c->Q, c->N, c->q_bad, s),
+       "heat source");
     c->launches++;
     ThParams p{};
     p.nx = c->g.nx;
@@ -1127,33 +1183,14 @@ int bvf_run_thermal(bvf_ctx *c, const bvf_thermal *th, const double *d_amp, floa
     p.lut = c->tlut;
     p.kface = c->kface;
     p.n_mat = n_mat;
+    p.n_cls = n_cls;
     p.Q = c->Q;
+    p.q_bad = c->q_bad;
     p.Tmax = d_Tmax;
     p.cemf = c->cemf;
     p.cem = d_cem43;
     const int total = th->n_on + th->n_off;
     float *a = d_T, *b = c->T2;
-    // TMA-fed steps where the index rows are whole multiples of 16 bytes and
-    // both temperature buffers can be mapped (BVF_NO_TMA forces the direct
-    // kernel); one map per temperature buffer, chosen per step
-    ThermTmaMaps tmaps[2];
-    bool th_tma = false;
-    if (c->g.nx % 8 == 0 && !std::getenv("BVF_NO_TMA")) {
-        const int nx = c->g.nx, ny = c->g.ny, nz = c->g.nz;
-        const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-        th_tma = encode_map(&tmaps[0].T, d_T, nx, ny, nz, F32, 4, 40, 18) &&
-                 encode_map(&tmaps[1].T, c->T2, nx, ny, nz, F32, 4, 40, 18) &&
-                 encode_map(&tmaps[0].idx, c->index_p ? c->index_p : c->index,
-                            c->index_p ? (int)c->index_pitch : nx, ny, nz,
-                            CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, 64, 18) &&
-                 encode_map(&tmaps[0].Q, c->Q, nx, ny, nz, F32, 4, 32, 16) &&
-                 encode_map(&tmaps[0].Tmax, d_Tmax, nx, ny, nz, F32, 4, 32, 16) &&
-                 encode_map(&tmaps[0].cemf, c->cemf, nx, ny, nz, F32, 4, 32, 16);
-        tmaps[1].idx = tmaps[0].idx;
-        tmaps[1].Q = tmaps[0].Q;
-        tmaps[1].Tmax = tmaps[0].Tmax;
-        tmaps[1].cemf = tmaps[0].cemf;
-    }
     p.kz = thermal_kchunk(c->g.nx, c->g.ny, c->g.nz, th_tma, n_mat);
     // the kernels advance the rise T - T_a (see ThParams); T and T_max are
     // converted in the caller's buffers on entry and back on every exit

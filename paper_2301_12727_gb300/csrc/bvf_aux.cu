@@ -3,6 +3,8 @@
 // and the E_L reductions (Sec. 2.4, Eq. 2).
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "bvf_stencil.cuh"
 #include "bvf_tma.cuh"
 
@@ -159,13 +161,26 @@ __global__ void __launch_bounds__(kRsPts *kRsGroups)
 
 __global__ void k_heat_source(const uint8_t *__restrict__ idx, const ThermCoef *__restrict__ lut,
                               const double *__restrict__ amp, double p_scale,
-                              float *__restrict__ Q, size_t n)
+                              float *__restrict__ Q, size_t n, int *q_bad)
 {
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
          q += (size_t)gridDim.x * blockDim.x) {
         const float A = amp ? (float)(p_scale * amp[q]) : 0.0f;
-        Q[q] = lut[idx[q]].qfac * A * A;
+        const float h = lut[idx[q]].qfac * A * A;
+        Q[q] = h;
+        if (!isfinite(h)) *q_bad = 1;
     }
+}
+
+__global__ void k_classes(const uint8_t *__restrict__ idx, const uint8_t *__restrict__ cls,
+                          uint8_t *__restrict__ out, size_t n, Rows r)
+{
+    __shared__ uint8_t s_c[BVF_MAX_MATERIALS];
+    for (int m = threadIdx.x; m < BVF_MAX_MATERIALS; m += blockDim.x) s_c[m] = cls[m];
+    __syncthreads();
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n;
+         q += (size_t)gridDim.x * blockDim.x)
+        out[in_rows(q, r)] = s_c[idx[q]];
 }
 
 // Pennes forward-Euler step on the rise; border voxels held at T_a (rise 0);
@@ -289,45 +304,93 @@ __global__ void __launch_bounds__(256) k_thermal(ThParams p)
     }
 }
 
-// TMA-fed step (grids with nx % 8 == 0).  A block of 32 x 8 threads owns a
-// 32 x 16 x-y tile (thread (tx, ty) the voxels of rows ty and ty + 8) and
+// The same step for two x-neighbours, arithmetic on pairs (bit for bit two
+// calls of thermal_update): face conductivities k[] in the order x-, x+, y-,
+// y+, z-, z+, nperf = -perfw and inv_rhoc of the two centres.
+__device__ __forceinline__ float2 thermal_update2(const ThParams &p, const float2 (&k)[6],
+                                                  float2 nperfw, float2 inv_rhoc, float2 Tc,
+                                                  float2 Tw, float2 Te, float2 Ts, float2 Tq,
+                                                  float2 Tm, float2 Tp, float2 Q)
+{
+    using st::splat;
+    float2 lap = st::vmul(k[0], st::vsub(Tw, Tc));
+    lap = st::vfma(k[1], st::vsub(Te, Tc), lap);
+    lap = st::vfma(k[2], st::vsub(Ts, Tc), lap);
+    lap = st::vfma(k[3], st::vsub(Tq, Tc), lap);
+    lap = st::vfma(k[4], st::vsub(Tm, Tc), lap);
+    lap = st::vfma(k[5], st::vsub(Tp, Tc), lap);
+    const float2 nperf = st::vmul(nperfw, Tc);
+    const float2 rhs =
+        st::vfma(splat<float2>(p.dc), Q, st::vfma(lap, splat<float2>(p.inv_dx2), nperf));
+    return st::vfma(st::vmul(splat<float2>(p.dt), rhs), inv_rhoc, Tc);
+}
+
+// thermal_outputs for the pair at q, q + 1 (q even)
+__device__ __forceinline__ void thermal_outputs2(const ThParams &p, size_t q, float2 Tn, float2 Tmax,
+                                                 float2 cemf)
+{
+    st::st2(p.Tmax + q, make_float2(fmaxf(Tmax.x, Tn.x), fmaxf(Tmax.y, Tn.y)));
+    const float2 l2r = make_float2((Tn.x >= p.rise43) ? -1.0f : -2.0f,
+                                   (Tn.y >= p.rise43) ? -1.0f : -2.0f);
+    const float2 x = st::vmul(l2r, st::vsub(st::splat<float2>(p.rise43), Tn));
+    const float2 part =
+        st::vfma(st::splat<float2>(p.dt60), make_float2(exp2f(x.x), exp2f(x.y)), cemf);
+    if (p.flush) {
+        p.cem[q] += (double)part.x;
+        p.cem[q + 1] += (double)part.y;
+        st::st2(p.cemf + q, make_float2(0.0f, 0.0f));
+    } else {
+        st::st2(p.cemf + q, part);
+    }
+}
+
+// TMA-fed step (grids with nx % 8 == 0).  A block of 16 x 16 threads owns a
+// 32 x 16 x-y tile (thread (tx, ty) the pair x0 + 2 tx, + 1 of row y0 + ty) and
 // walks a z-chunk.  Every input of a plane arrives through the tensor-memory
-// accelerator in a four-plane shared-memory ring: T and the material index
-// as halo'd boxes (T: x0-4 .. x0+35, index: x0-16 .. x0+47, both
-// y0-1 .. y0+16; a TMA box starts on a 16-byte boundary, out-of-range
-// elements read as zero and only feed border voxels, which are held at T_a),
-// Q, T_max and the dose partial as 32 x 16 boxes.  Plane k reads planes k-1,
-// k, k+1 of the ring while plane k+2 is in flight, so the kernel's loads run
-// two planes ahead of its arithmetic; results are stored directly.  One
-// thread issues the copies; waits are bounded as in the acoustic kernels (a
-// time-out sets bit 2 of the flag after the block's armed copies have
-// landed).
-constexpr int kThRing = 4;                                             // planes k-1 .. k+2
+// accelerator in shared-memory rings: T and the conduction class as halo'd
+// boxes (T: x0-4 .. x0+35, class: x0-16 .. x0+47, both y0-1 .. y0+16; a TMA
+// box starts on a 16-byte boundary, out-of-range elements read as zero and
+// only feed border voxels, which are held at T_a), the material, Q (while the
+// source is on), T_max and the dose partial as 32 x 16 boxes.  Plane k reads
+// planes k-1, k, k+1 while k+2 and k+3 are in flight; results are stored
+// directly.  One thread issues the copies; waits are bounded as in the
+// acoustic kernels (a time-out sets bit 2 of the flag after the block's armed
+// copies have landed).
+//
+// At 240 x 240 x 200 the copies and stores alone take 60 us of a step (four
+// planes of ring, one of them in flight: 62), a voxel a time with a pair
+// look-up for every bone voxel took 84.9 in all.  Pairs (8-byte shared-memory
+// and global accesses, the class as 16-bit words, one comparison of all
+// twelve, packed arithmetic) and classes instead of materials (the 125 bone
+// bins of the skull share one conductivity) bring it to 74.4, 67.3 in one
+// tissue.
+constexpr int kThRing = 5, kThVRing = 4;     // T and index planes k-1 .. k+3; streams k .. k+3
 constexpr int kThTileY = 16;
 constexpr int kThTW = 40, kThTH = kThTileY + 2, kThTBytes = kThTW * kThTH * 4;   // 2880 B
 constexpr int kThTSlot = 2944;                                         // 23 x 128 B
 constexpr int kThIW = 64, kThIBytes = kThIW * kThTH;                   // 1152 B
 constexpr int kThVBytes = 32 * kThTileY * 4;                           // Q, T_max, partial: 2048 B
-constexpr int kThSlot = kThTSlot + kThIBytes + 3 * kThVBytes;          // one plane: 10240 B
-constexpr int kThOffBar = kThRing * kThSlot;
+constexpr int kThSlot = kThTSlot + kThIBytes, kThVSlot = 3 * kThVBytes + 512;
+constexpr int kThMBytes = 32 * kThTileY;                               // own materials: 512 B
+constexpr int kThOffV = kThRing * kThSlot;
+constexpr int kThOffBar = kThOffV + kThVRing * kThVSlot;
 constexpr int kThOffAbort = kThOffBar + 8 * kThRing;
 constexpr int kThOffLut = (kThOffAbort + (int)sizeof(int) + 15) / 16 * 16;
-constexpr unsigned kThPlaneBytes = kThTBytes + kThIBytes + 3 * kThVBytes;
 static_assert(kThTSlot % 128 == 0 && kThTSlot >= kThTBytes && kThIBytes % 128 == 0 &&
                   kThVBytes % 128 == 0 && kThSlot % 128 == 0 && kThOffLut % 16 == 0,
               "ring slots 128-byte aligned, coefficients 16");
 
-__global__ void __launch_bounds__(256, 5)
+__global__ void __launch_bounds__(256, 4)
     k_thermal_tma(ThParams p, const __grid_constant__ ThermTmaMaps tm, int *flag)
 {
     extern __shared__ __align__(128) unsigned char smb[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smb + kThOffBar);
     volatile int *s_abort = reinterpret_cast<volatile int *>(smb + kThOffAbort);
     ThermCoef *s_th = reinterpret_cast<ThermCoef *>(smb + kThOffLut);
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 16 + tx;
     for (int m = tid; m < p.n_mat; m += 256) s_th[m] = p.lut[m];
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * kThTileY, i = x0 + tx;
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * kThTileY, i = x0 + 2 * tx, j = y0 + ty;
     const int k0 = blockIdx.z * p.kz, k1 = min(nz, k0 + p.kz);
     if (tid == 0) {
         for (int b = 0; b < kThRing; ++b) tma::mbar_init(&bars[b], 1);
@@ -335,25 +398,33 @@ __global__ void __launch_bounds__(256, 5)
         *s_abort = -1;
     }
     __syncthreads();
-    // plane pl of the chunk's window k0-1 .. k1 sits in slot (pl - k0 + 1) % 4,
-    // the (pl - k0 + 1) / 4-th phase of that slot's barrier; a slot holds T,
-    // the index, Q, T_max and the partial of its plane, in that order
-    auto slot = [&](int pl) { return (pl - k0 + 1) & (kThRing - 1); };
-    auto parity = [&](int pl) { return (unsigned)((pl - k0 + 1) >> 2) & 1u; };
+    // the coefficients are in place; the rest is the step before's
+    tma::pdl_wait();
+    tma::pdl_launch_next();
+    // T and the index of plane pl of the chunk's window k0-1 .. k1 sit in slot
+    // (pl - k0 + 1) % 5 of their ring, the (pl - k0 + 1) / 5-th phase of that
+    // slot's barrier; Q, T_max and the partial of an own plane in slot
+    // (pl - k0) % 4 of theirs, on the same barrier
+    auto slot = [&](int pl) { return (pl - k0 + 1) % kThRing; };
+    auto parity = [&](int pl) { return (unsigned)((pl - k0 + 1) / kThRing) & 1u; };
+    const bool heat = p.dc != 0.0f || *p.q_bad != 0;
     auto issue = [&](int pl) {
         uint64_t *bar = &bars[slot(pl)];
         unsigned char *d = smb + slot(pl) * kThSlot;
         // the per-voxel streams only for the chunk's own planes; its two
         // neighbour planes supply T and the index
         const bool own = pl >= k0 && pl < k1;
-        tma::mbar_expect_tx(bar, own ? kThPlaneBytes : (unsigned)(kThTBytes + kThIBytes));
+        tma::mbar_expect_tx(bar, (unsigned)(kThTBytes + kThIBytes) +
+                                     (own ? (heat ? 3u : 2u) * kThVBytes + kThMBytes : 0u));
         if (p.hold_plane >= 0 && pl == p.hold_plane) return;   // test hook: armed, none issued
         tma::load3d(d, &tm.T, x0 - 4, y0 - 1, pl, bar);
-        tma::load3d(d + kThTSlot, &tm.idx, x0 - 16, y0 - 1, pl, bar);
+        tma::load3d(d + kThTSlot, &tm.cls, x0 - 16, y0 - 1, pl, bar);
         if (own) {
-            tma::load3d(d + kThTSlot + kThIBytes, &tm.Q, x0, y0, pl, bar);
-            tma::load3d(d + kThTSlot + kThIBytes + kThVBytes, &tm.Tmax, x0, y0, pl, bar);
-            tma::load3d(d + kThTSlot + kThIBytes + 2 * kThVBytes, &tm.cemf, x0, y0, pl, bar);
+            unsigned char *e = smb + kThOffV + (pl - k0) % kThVRing * kThVSlot;
+            if (heat) tma::load3d(e, &tm.Q, x0, y0, pl, bar);
+            tma::load3d(e + kThVBytes, &tm.Tmax, x0, y0, pl, bar);
+            tma::load3d(e + 2 * kThVBytes, &tm.cemf, x0, y0, pl, bar);
+            tma::load3d(e + 3 * kThVBytes, &tm.idx, x0, y0, pl, bar);
         }
     };
     auto wait = [&](int pl) { return tma::mbar_wait(&bars[slot(pl)], parity(pl), p.wait_limit); };
@@ -362,65 +433,91 @@ __global__ void __launch_bounds__(256, 5)
         for (int pl = k0 - 1; pl <= first_last; ++pl) issue(pl);
     int issued = first_last;
 
-    // the thread's two voxels: rows j = y0 + ty + 8 h, h = 0, 1
-    bool live[2], border[2];
-    int ct[2], ci[2], cv[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int j = y0 + ty + 8 * h;
-        live[h] = i < nx && j < ny;
-        border[h] = i == 0 || j == 0 || i == nx - 1 || j == ny - 1;
-        ct[h] = (ty + 8 * h + 1) * kThTW + tx + 4;
-        ci[h] = (ty + 8 * h + 1) * kThIW + tx + 16;
-        cv[h] = (ty + 8 * h) * 32 + tx;
-    }
+    // nx is even: a pair lies inside the grid or outside
+    const bool live = i < nx && j < ny, xb0 = i == 0, xb1 = i + 1 == nx - 1;
+    const bool yb = j == 0 || j == ny - 1;
+    const int c = (ty + 1) * kThTW + 2 * tx + 4, d = (ty + 1) * kThIW + 2 * tx + 16;
+    const int cv = ty * 32 + 2 * tx;
     const size_t SZ = (size_t)nx * ny;
-    size_t q0 = (size_t)k0 * SZ + (size_t)(y0 + ty) * nx + i;     // row ty of plane k
-    const size_t q8 = (size_t)8 * nx;                                // row ty + 8
-    for (int k = k0; k < k1; ++k, q0 += SZ) {
+    size_t q = (size_t)k0 * SZ + (size_t)j * nx + i;
+    // the pair of plane k: S, Sm, Sp the ring slots of planes k, k-1, k+1, V0
+    // the streams of plane k
+    auto pair_step = [&](const unsigned char *S, const unsigned char *Sm, const unsigned char *Sp,
+                         const float *V0, bool border) {
+        const float *T0 = reinterpret_cast<const float *>(S);
+        const unsigned char *I0 = S + kThTSlot;
+        const float2 Q = heat ? st::ld2(V0 + cv) : make_float2(0.0f, 0.0f), Tmax = st::ld2(V0 + cv + kThVBytes / 4),
+                     cemf = st::ld2(V0 + cv + kThVBytes / 2);
+        float2 Tn = make_float2(0.0f, 0.0f);
+        if (!border) {
+            auto w16 = [](const unsigned char *p16) {
+                return (unsigned)*reinterpret_cast<const unsigned short *>(p16);
+            };
+            const float2 Tc = st::ld2(T0 + c), Tl = st::ld2(T0 + c - 2), Tr = st::ld2(T0 + c + 2);
+            const float2 Ts = st::ld2(T0 + c - kThTW), Tq = st::ld2(T0 + c + kThTW);
+            const float2 Tm = st::ld2(reinterpret_cast<const float *>(Sm) + c);
+            const float2 Tp = st::ld2(reinterpret_cast<const float *>(Sp) + c);
+            const float2 Tw = make_float2(Tl.y, Tc.x), Te = make_float2(Tc.y, Tr.x);
+            const unsigned m2 = w16(I0 + d), ml = w16(I0 + d - 2) >> 8, mr = w16(I0 + d + 2) & 255u;
+            const unsigned ms = w16(I0 + d - kThIW), mq = w16(I0 + d + kThIW);
+            const unsigned mm = w16(Sm + kThTSlot + d), mp = w16(Sp + kThTSlot + d);
+            // m..: conduction classes; own materials for the other coefficients
+            const unsigned ca = m2 & 255u, cb = m2 >> 8, one = ca * 0x0101u;
+            const unsigned own =
+                w16(reinterpret_cast<const unsigned char *>(V0 + 3 * (kThVBytes / 4)) + cv);
+            const ThermCoef a = s_th[own & 255u], b = s_th[own >> 8];
+            float2 k[6];
+            if (((m2 ^ one) | (ms ^ one) | (mq ^ one) | (mm ^ one) | (mp ^ one) | (ml ^ ca) |
+                 (mr ^ ca)) == 0u) {
+#pragma unroll
+                for (int f = 0; f < 6; ++f) k[f] = st::splat<float2>(a.k);
+            } else {
+                const float *ka = p.kface + ca * p.n_cls, *kb = p.kface + cb * p.n_cls;
+                k[0] = make_float2(__ldg(ka + ml), __ldg(kb + ca));
+                k[1] = make_float2(__ldg(ka + cb), __ldg(kb + mr));
+                k[2] = make_float2(__ldg(ka + (ms & 255u)), __ldg(kb + (ms >> 8)));
+                k[3] = make_float2(__ldg(ka + (mq & 255u)), __ldg(kb + (mq >> 8)));
+                k[4] = make_float2(__ldg(ka + (mm & 255u)), __ldg(kb + (mm >> 8)));
+                k[5] = make_float2(__ldg(ka + (mp & 255u)), __ldg(kb + (mp >> 8)));
+            }
+            const float2 nperfw = make_float2(-a.perfw, -b.perfw),
+                         irc = make_float2(a.inv_rhoc, b.inv_rhoc);
+            Tn = thermal_update2(p, k, nperfw, irc, Tc, Tw, Te, Ts, Tq, Tm, Tp, Q);
+            if (xb0) Tn.x = 0.0f;
+            if (xb1) Tn.y = 0.0f;
+        }
+        st::st2(p.Tn + q, Tn);
+        thermal_outputs2(p, q, Tn, Tmax, cemf);
+    };
+    // slots of planes k-1, k, k+1 and of plane k's streams, rotated per plane;
+    // parity of plane k+1's barrier
+    int sm1 = 0, sc = 1, sp1 = 2, sv = 0;
+    unsigned ph = 0;
+    for (int k = k0; k < k1; ++k, q += SZ) {
         __syncthreads();
-        if (*s_abort >= 0) break;                 // a wait of the previous plane ran out
-        if (k + 2 <= k1 && k + 2 > issued) {      // into the slot plane k-2 has freed
+        if (*s_abort >= 0) break;             // a wait of the previous plane ran out
+        if (k + 3 <= k1 && k + 3 > issued) {  // into the slots planes k-2 and k-1 have freed
             if (tid == 0) {
                 tma::fence_async_smem();
-                issue(k + 2);
+                issue(k + 3);
             }
-            issued = k + 2;
+            issued = k + 3;
         }
         bool ready = true;
         if (k == k0) ready = wait(k0 - 1) && wait(k0);
-        ready = ready && wait(k + 1);
-        if (!ready) *s_abort = k;
-        if (!ready) continue;                     // leaves at the next barrier
-        const unsigned char *S0 = smb + slot(k) * kThSlot;
-        const unsigned char *Sz0 = smb + slot(k - 1) * kThSlot;
-        const unsigned char *Sz1 = smb + slot(k + 1) * kThSlot;
-        const float *T0 = reinterpret_cast<const float *>(S0);
-        const float *Tz0 = reinterpret_cast<const float *>(Sz0);
-        const float *Tz1 = reinterpret_cast<const float *>(Sz1);
-        const unsigned char *I0 = S0 + kThTSlot, *Iz0 = Sz0 + kThTSlot, *Iz1 = Sz1 + kThTSlot;
-        const float *V0 = reinterpret_cast<const float *>(S0 + kThTSlot + kThIBytes);
-        const bool zb = k == 0 || k == nz - 1;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (!live[h]) continue;
-            const float Q = V0[cv[h]], Tmax = V0[cv[h] + kThVBytes / 4],
-                        cemf = V0[cv[h] + kThVBytes / 2];
-            float Tn;
-            if (border[h] || zb) {
-                Tn = 0.0f;
-            } else {
-                const int c = ct[h], d = ci[h];
-                const int mc = I0[d];
-                Tn = thermal_update(p, s_th[mc], mc, p.kface + mc * p.n_mat, T0[c], T0[c - 1],
-                                    I0[d - 1], T0[c + 1], I0[d + 1], T0[c - kThTW], I0[d - kThIW],
-                                    T0[c + kThTW], I0[d + kThIW], Tz0[c], Iz0[d], Tz1[c], Iz1[d],
-                                    Q);
-            }
-            const size_t q = q0 + h * q8;
-            p.Tn[q] = Tn;
-            thermal_outputs(p, q, Tn, Tmax, cemf);
+        ready = ready && tma::mbar_wait(&bars[sp1], ph, p.wait_limit);
+        if (!ready) *s_abort = k;             // leaves at the next barrier
+        if (ready && live)
+            pair_step(smb + sc * kThSlot, smb + sm1 * kThSlot, smb + sp1 * kThSlot,
+                      reinterpret_cast<const float *>(smb + kThOffV + sv * kThVSlot),
+                      yb || k == 0 || k == nz - 1);
+        sm1 = sc;
+        sc = sp1;
+        if (++sp1 == kThRing) {
+            sp1 = 0;
+            ph ^= 1u;
         }
+        sv = sv + 1 == kThVRing ? 0 : sv + 1;
     }
     __syncthreads();
     const int ab = *s_abort;
@@ -644,25 +741,39 @@ cudaError_t launch_rs_weighted(const float4 *el, const float2 *wt, int ne, int n
     return cudaGetLastError();
 }
 
+cudaError_t launch_classes(const uint8_t *idx, const uint8_t *cls, uint8_t *out, size_t n, Rows r,
+                           cudaStream_t s)
+{
+    k_classes<<<blocks_for(n), kThreads, 0, s>>>(idx, cls, out, n, r);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_heat_source(const uint8_t *idx, const ThermCoef *lut, int n_mat,
                                const double *amp, double p_scale, float *Q, size_t n,
-                               cudaStream_t s)
+                               int *q_bad, cudaStream_t s)
 {
     (void)n_mat;
-    k_heat_source<<<blocks_for(n), kThreads, 0, s>>>(idx, lut, amp, p_scale, Q, n);
+    k_heat_source<<<blocks_for(n), kThreads, 0, s>>>(idx, lut, amp, p_scale, Q, n, q_bad);
     return cudaGetLastError();
+}
+
+static cudaError_t raise_thermal_smem()
+{
+    return cudaFuncSetAttribute(k_thermal_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kThOffLut + BVF_MAX_MATERIALS * (int)sizeof(ThermCoef));
 }
 
 // The z-chunk of a BHTE launch: blocks of a chunk run in waves of
 // (resident blocks per SM) x (SMs); a block's time is about its planes plus
 // two (the z-neighbour planes and the pipeline fill), so the chunk length kz
-// in 4 .. 32 that minimises waves(kz) x (kz + 2) is taken.
+// in 1 .. 32 that minimises waves(kz) x (kz + 2) is taken.
 int thermal_kchunk(int nx, int ny, int nz, bool tma, int n_mat)
 {
     int dev = 0, n_sm = 152, per_sm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = tma ? kThOffLut + n_mat * sizeof(ThermCoef) : n_mat * sizeof(ThermCoef);
+    if (tma) raise_thermal_smem();
     const cudaError_t e =
         tma ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_thermal_tma, 256, smem)
             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_thermal, 256, smem);
@@ -672,7 +783,7 @@ int thermal_kchunk(int nx, int ny, int nz, bool tma, int n_mat)
     const long long slots = (long long)per_sm * n_sm;
     int best = 16;
     long long best_cost = -1;
-    for (int kz = 4; kz <= 32; ++kz) {
+    for (int kz = 1; kz <= 32; ++kz) {
         const long long blocks = tiles * ((nz + kz - 1) / kz);
         const long long cost = ((blocks + slots - 1) / slots) * (kz + 2);
         if (best_cost < 0 || cost < best_cost) {
@@ -689,8 +800,16 @@ cudaError_t launch_thermal_step(const ThParams &p, const ThermTmaMaps *tm, int *
     dim3 blk(32, 8, 1);
     dim3 grd((p.nx + 31) / 32, (p.ny + 7) / 8, (p.nz + p.kz - 1) / p.kz);
     if (tm) {
+        // the shared-memory limit is raised once per process (graph capture)
+        static std::atomic<int> raised{0};
+        if (!raised.load(std::memory_order_acquire)) {
+            const cudaError_t e = raise_thermal_smem();
+            if (e != cudaSuccess) return e;
+            raised.store(1, std::memory_order_release);
+        }
         grd.y = (p.ny + kThTileY - 1) / kThTileY;
-        k_thermal_tma<<<grd, blk, kThOffLut + p.n_mat * sizeof(ThermCoef), s>>>(p, *tm, flag);
+        return launch_pdl(k_thermal_tma, grd, dim3(16, 16, 1),
+                          kThOffLut + p.n_mat * sizeof(ThermCoef), s, p, *tm, flag);
     } else {
         k_thermal<<<grd, blk, p.n_mat * sizeof(ThermCoef), s>>>(p);
     }

@@ -158,8 +158,11 @@ struct ThParams {
     float rise43;            // 43 C - T_a: the CEM43 threshold as a rise
     const uint8_t *idx;
     const ThermCoef *lut;
-    const float *kface;      // [n_mat][n_mat] harmonic-mean face conductivity (FP64-derived)
-    int n_mat;
+    // harmonic-mean face conductivity (FP64-derived): of every material pair
+    // (direct kernel), or of every pair of conduction classes (TMA-fed kernel;
+    // a class is the materials of one k_th)
+    const float *kface;
+    int n_mat, n_cls;
     const float *T;
     float *Tn;
     const float *Q;
@@ -167,6 +170,7 @@ struct ThParams {
     float *cemf;
     double *cem;
     int flush;
+    const int *q_bad;        // set where the heat source holds a value that is not finite
     int kz;                  // z-planes per block (thermal_kchunk)
     // bounded waits of the TMA-fed step: polls per wait; hold_plane >= 0 makes
     // the kernel arm that plane's barrier but issue none of its copies (the
@@ -249,13 +253,17 @@ cudaError_t launch_conj_plane(const double *C, const double *S, size_t n, Rows r
                               unsigned long long *d_max, float2 *out, cudaStream_t s);
 cudaError_t launch_heat_source(const uint8_t *idx, const ThermCoef *lut, int n_mat,
                                const double *amp, double p_scale, float *Q, size_t n,
-                               cudaStream_t s);
+                               int *q_bad, cudaStream_t s);
 // Tensor maps of the TMA-fed BHTE step: the input temperature (40 x 18 x 1
-// float box), the material index (64 x 18 x 1 byte box), and the heat
-// source, T_max and the FP32 dose partial (32 x 16 x 1 float boxes).
+// float box), the conduction class (64 x 18 x 1 byte box), the material index
+// (32 x 16 x 1 byte box), and the heat source, T_max and the FP32 dose partial
+// (32 x 16 x 1 float boxes).
 struct ThermTmaMaps {
-    CUtensorMap T, idx, Q, Tmax, cemf;
+    CUtensorMap T, cls, idx, Q, Tmax, cemf;
 };
+// out[row * pitch + x] = cls[idx[row * nx + x]] (cls: 256 bytes on the device)
+cudaError_t launch_classes(const uint8_t *idx, const uint8_t *cls, uint8_t *out, size_t n, Rows r,
+                           cudaStream_t s);
 // z-planes per block of the BHTE kernels for a grid (tma: the TMA-fed kernel)
 int thermal_kchunk(int nx, int ny, int nz, bool tma, int n_mat);
 // one BHTE step; tm == NULL takes the direct kernel
