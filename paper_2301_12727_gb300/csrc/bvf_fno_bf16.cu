@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -152,6 +153,177 @@ __global__ void k_mix_dR(const float *__restrict__ dY, const float *__restrict__
     }
 }
 
+// ------------------------------------------------------- tiled mode mix
+// The mix and its adjoints move a layer's spectral weights (W x W complex per
+// mode, 56.6 MB at width 32, m 12) and do little else.  A block takes KZ modes
+// of one (ky, kx), which lie together in the spectra: their spectra of all
+// samples and channels sit in shared memory, the weights of a mode stream
+// through once for the whole batch, and results leave as they came in.  One
+// thread per output that fetched every operand itself took 65 us (mix), 215
+// (adjoint) and 235 (weight gradient) a layer at batch 4; now 49, and 98 for
+// both adjoints.  Sums run in the same order as there.
+//
+// spectra tile: [b * W + c][part][KZ], channel rows padded by one float
+struct MixTile {
+    int B, W, m, KZ, pitch;
+    __host__ __device__ MixTile(int B_, int W_, int m_, int kz) : B(B_), W(W_), m(m_), KZ(kz)
+    {
+        pitch = 2 * kz + 1;
+    }
+    __host__ __device__ size_t bytes() const { return (size_t)B * W * pitch * sizeof(float); }
+};
+// copy the tile of modes kz0 .. kz0 + n - 1 at (ky, kx) = yx between a spectrum
+// array and shared memory
+__device__ __forceinline__ void tile_io(float *tile, const MixTile &t, float *X, int yx, int kz0,
+                                        int n, bool store)
+{
+    const int S2 = 2 * t.m;
+    const size_t S = (size_t)8 * t.m * t.m * t.m;
+    for (int e = threadIdx.x; e < t.B * t.W * 2 * t.KZ; e += blockDim.x) {
+        const int z = e % t.KZ, part = e / t.KZ % 2, bc = e / (2 * t.KZ);
+        if (z >= n) continue;
+        float *x = X + bc * S + ((size_t)yx * 2 + part) * S2 + kz0 + z;
+        float *p = tile + bc * t.pitch + part * t.KZ + z;
+        if (store)
+            *x = *p;
+        else
+            *p = *x;
+    }
+}
+
+// Y[b][o][mode] = sum_c R[mode][c][o] X[b][c][mode]: 16 lanes take two outputs
+// each (W / 2 in passes), for BT samples at a time
+template <int BT>
+__global__ void __launch_bounds__(256) k_mix_fwd_tile(float *X, const float *R, MixTile t, float *Y)
+{
+    extern __shared__ float s_mix[];
+    float *sx = s_mix, *sy = s_mix + t.bytes() / sizeof(float);
+    const int yx = blockIdx.x, kz0 = blockIdx.y * t.KZ, n = min(t.KZ, 2 * t.m - kz0);
+    tile_io(sx, t, X, yx, kz0, n, false);
+    __syncthreads();
+    const int W = t.W, lane = threadIdx.x & 15, groups = blockDim.x >> 4;
+    for (int w = threadIdx.x >> 4; w < n * (W / 32 + (W % 32 != 0)); w += groups) {
+        const int z = w % n, o2 = w / n * 16 + lane;          // output pair
+        if (2 * o2 >= W) continue;
+        const size_t mode = (size_t)(kz0 + z) * 2 * t.m * t.m + yx;
+        const float4 *r = reinterpret_cast<const float4 *>(R + mode * W * W * 2) + o2;
+        for (int b0 = 0; b0 < t.B; b0 += BT) {
+            float2 y0[BT], y1[BT];
+#pragma unroll
+            for (int b = 0; b < BT; ++b) y0[b] = y1[b] = make_float2(0.0f, 0.0f);
+#pragma unroll 8
+            for (int c = 0; c < W; ++c) {
+                const float4 q = r[c * (W / 2)];
+#pragma unroll
+                for (int b = 0; b < BT; ++b) {
+                    if (b0 + b >= t.B) break;
+                    const float *x = sx + ((b0 + b) * W + c) * t.pitch + z;
+                    const float xr = x[0], xi = x[t.KZ];
+                    y0[b].x = fmaf(q.x, xr, fmaf(-q.y, xi, y0[b].x));
+                    y0[b].y = fmaf(q.x, xi, fmaf(q.y, xr, y0[b].y));
+                    y1[b].x = fmaf(q.z, xr, fmaf(-q.w, xi, y1[b].x));
+                    y1[b].y = fmaf(q.z, xi, fmaf(q.w, xr, y1[b].y));
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                if (b0 + b >= t.B) break;
+                float *y = sy + ((b0 + b) * W + 2 * o2) * t.pitch + z;
+                y[0] = y0[b].x;
+                y[t.KZ] = y0[b].y;
+                y[t.pitch] = y1[b].x;
+                y[t.pitch + t.KZ] = y1[b].y;
+            }
+        }
+    }
+    __syncthreads();
+    tile_io(sy, t, Y, yx, kz0, n, true);
+}
+
+// dX[b][c][mode] = sum_o conj(R[mode][c][o]) dY[b][o][mode] and
+// dR[mode][c][o] = sum_b dY[b][o][mode] conj(X[b][c][mode]): a warp brings one
+// mode's weights into shared memory (rows padded), sums its lanes' channels
+// over the outputs, and writes the mode's weight gradient.  dX replaces X in
+// its tile.
+__global__ void __launch_bounds__(256) k_mix_bwd_tile(float *dY, float *X, const float *R, MixTile t,
+                                                      float *dR, float *dX)
+{
+    extern __shared__ float s_mix[];
+    const int W = t.W, tile = (int)(t.bytes() / sizeof(float));
+    float *sy = s_mix, *sx = sy + tile, *sd = sx + tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int rp = W + 1;
+    float2 *sr = reinterpret_cast<float2 *>(s_mix + (3 * tile + 1) / 2 * 2) + warp * W * rp;
+    const int yx = blockIdx.x, kz0 = blockIdx.y * t.KZ, n = min(t.KZ, 2 * t.m - kz0);
+    tile_io(sy, t, dY, yx, kz0, n, false);
+    tile_io(sx, t, X, yx, kz0, n, false);
+    __syncthreads();
+    for (int z = warp; z < n; z += warps) {
+        const size_t mode = (size_t)(kz0 + z) * 2 * t.m * t.m + yx;
+        const float4 *r = reinterpret_cast<const float4 *>(R + mode * W * W * 2);
+        float4 *g = reinterpret_cast<float4 *>(dR + mode * W * W * 2);
+        __syncwarp();
+#pragma unroll 4
+        for (int e = lane; e < W * W / 2; e += 32) {
+            const float4 q = r[e];
+            const int c = e / (W / 2), o = 2 * (e - c * (W / 2));
+            sr[c * rp + o] = make_float2(q.x, q.y);
+            sr[c * rp + o + 1] = make_float2(q.z, q.w);
+            float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int b = 0; b < t.B; ++b) {
+                const float *x = sx + (b * W + c) * t.pitch + z, *y = sy + (b * W + o) * t.pitch + z;
+                const float xr = x[0], xi = x[t.KZ];
+                const float yr = y[0], yi = y[t.KZ], zr = y[t.pitch], zi = y[t.pitch + t.KZ];
+                a.x = fmaf(yr, xr, fmaf(yi, xi, a.x));
+                a.y = fmaf(yi, xr, fmaf(-yr, xi, a.y));
+                a.z = fmaf(zr, xr, fmaf(zi, xi, a.z));
+                a.w = fmaf(zi, xr, fmaf(-zr, xi, a.w));
+            }
+            g[e] = a;
+        }
+        __syncwarp();
+        for (int c = lane; c < W; c += 32)
+            for (int b = 0; b < t.B; ++b) {
+                float xr = 0.0f, xi = 0.0f;
+#pragma unroll 8
+                for (int o = 0; o < W; ++o) {
+                    const float *y = sy + (b * W + o) * t.pitch + z;
+                    const float yr = y[0], yi = y[t.KZ];
+                    const float2 w = sr[c * rp + o];
+                    xr = fmaf(w.x, yr, fmaf(w.y, yi, xr));
+                    xi = fmaf(w.x, yi, fmaf(-w.y, yr, xi));
+                }
+                float *d = sd + (b * W + c) * t.pitch + z;
+                d[0] = xr;
+                d[t.KZ] = xi;
+            }
+    }
+    __syncthreads();
+    tile_io(sd, t, dX, yx, kz0, n, true);
+}
+
+// modes of a tile: as many of the 2m as leave room for two blocks per SM (`per`
+// tiles and `extra` bytes a block), 0 if not even one fits
+constexpr size_t kMixSmem = 110 * 1024;
+inline int mix_modes(int B, int W, int m, int per, size_t extra)
+{
+    for (int kz = 2 * m; kz >= 1; kz = kz > 8 ? (kz + 1) / 2 : kz - 1)
+        if (per * MixTile(B, W, m, kz).bytes() + extra <= kMixSmem) return kz;
+    return 0;
+}
+
+// a kernel's shared-memory limit, raised once per process
+template <auto Kernel>
+cudaError_t mix_smem()
+{
+    static std::atomic<int> done{0};
+    if (done.load(std::memory_order_acquire)) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem);
+    if (e == cudaSuccess) done.store(1, std::memory_order_release);
+    return e;
+}
+
 // out[c] += sum over samples and voxels of x[b][c][p]
 __global__ void k_chan_sum(const float *__restrict__ x, int B, int C, int N, float *__restrict__ out)
 {
@@ -159,8 +331,23 @@ __global__ void k_chan_sum(const float *__restrict__ x, int B, int C, int N, flo
     float acc = 0.0f;
     for (int b = 0; b < B; ++b) {
         const float *xc = x + ((size_t)b * C + c) * N;
-        for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x)
-            acc += xc[p];
+        const int step = gridDim.x * blockDim.x, t = blockIdx.x * blockDim.x + threadIdx.x;
+        if (N % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+            // four 16-byte loads in flight
+            const float4 *x4 = reinterpret_cast<const float4 *>(xc);
+            const int n4 = N / 4;
+            for (int p = t; p < n4; p += 4 * step) {
+                float4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    v[u] = p + u * step < n4 ? __ldg(x4 + p + u * step)
+                                             : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc += (v[u].x + v[u].y) + (v[u].z + v[u].w);
+            }
+        } else {
+            for (int p = t; p < N; p += step) acc += xc[p];
+        }
     }
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     __shared__ float sh[32];
@@ -532,6 +719,50 @@ int chan_sum(const float *x, int B, int C, int N, float *out, cudaStream_t s)
     return BVF_OK;
 }
 
+// Y = R X per mode
+int mix_forward(bvf_fno_bf16 *t, int batch, float *X, const float *Rw, float *Y, cudaStream_t s)
+{
+    const int W = t->d.width, m = t->d.modes, kz = mix_modes(batch, W, m, 2, 0);
+    if (!kz) {
+        k_mix_fwd<<<grid_for((long long)batch * 4 * m * m * m * W), 256, 0, s>>>(X, Rw, batch, W, m, Y);
+    } else {
+        const MixTile tile(batch, W, m, kz);
+        const dim3 grid(2 * m * m, (2 * m + kz - 1) / kz);
+        const size_t smem = 2 * tile.bytes();
+        if (batch == 1) {
+            BCK(mix_smem<k_mix_fwd_tile<1>>(), "mix");
+            k_mix_fwd_tile<1><<<grid, 256, smem, s>>>(X, Rw, tile, Y);
+        } else {
+            BCK(mix_smem<k_mix_fwd_tile<4>>(), "mix");
+            k_mix_fwd_tile<4><<<grid, 256, smem, s>>>(X, Rw, tile, Y);
+        }
+    }
+    BCK(cudaGetLastError(), "mix");
+    return BVF_OK;
+}
+
+// dR = dY conj(X) summed over the batch, dX = conj(R) dY (gR starts at zero)
+int mix_backward(bvf_fno_bf16 *t, int batch, float *dY, float *X, const float *Rw, float *gR,
+                 float *dX, cudaStream_t s)
+{
+    const int W = t->d.width, m = t->d.modes;
+    const int warps = W <= 32 ? 8 : 2;                    // a warp holds one mode's weights
+    const size_t wb = (size_t)warps * W * (W + 1) * sizeof(float2) + 16;
+    const int kz = mix_modes(batch, W, m, 3, wb);
+    const MixTile tile(batch, W, m, kz ? kz : 1);
+    const size_t smem = 3 * tile.bytes() + wb;
+    if (!kz) {                                            // a batch too large for a tile
+        k_mix_dR<<<grid_for((long long)4 * m * m * m * W * W), 256, 0, s>>>(dY, X, batch, W, m, gR);
+        k_mix_adj<<<grid_for((long long)batch * 4 * m * m * m * W), 256, 0, s>>>(dY, Rw, batch, W, m, dX);
+    } else {
+        BCK(mix_smem<k_mix_bwd_tile>(), "d mix");
+        k_mix_bwd_tile<<<dim3(2 * m * m, (2 * m + kz - 1) / kz), 32 * warps, smem, s>>>(dY, X, Rw, tile,
+                                                                                      gR, dX);
+    }
+    BCK(cudaGetLastError(), "d mix");
+    return BVF_OK;
+}
+
 // One row pass over `batch` samples: out = act(Inv_x(w2) + mix of v + bias)
 // with the channel weights Wm(o, c) at o wso + c wsc (v has cin channels); G
 // the x stage's matrix, NULL for no spectral term.  act as in bvf_gemm.  Rows
@@ -580,9 +811,7 @@ int forward(bvf_fno_bf16 *t, int batch, const float *in, float *out, bool keep, 
         const float *lw = w + o.lay0 + l * o.lf;
         const float *R = lw, *Wl = lw + (size_t)4 * m * m * m * W * W * 2, *bl = Wl + (size_t)W * W;
         if ((rc = spec_fwd(t, t->v[l], (long long)batch * W, false, t->X[l], s)) != BVF_OK) return rc;
-        k_mix_fwd<<<grid_for((long long)batch * 4 * m * m * m * W), 256, 0, s>>>(t->X[l], R, batch, W,
-                                                                                   m, t->S1);
-        BCK(cudaGetLastError(), "mix");
+        if ((rc = mix_forward(t, batch, t->X[l], R, t->S1, s)) != BVF_OK) return rc;
         if ((rc = spec_inv_zy(t, t->S1, (long long)batch * W, s)) != BVF_OK) return rc;
         const int act = l < L - 1;
         if ((rc = row_pass(t, batch, t->v[l], W, Wl, W, 1, bl, t->Gxw, act,
@@ -650,11 +879,7 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
         if ((rc = chan_sum(ds, batch, W, N, gb, s)) != BVF_OK) return rc;
         if ((rc = gemm(t, wgrad(ds, W, t->v[l], W, gW, N, batch, ks), s, "dW")) != BVF_OK) return rc;
         if ((rc = spec_fwd(t, ds, (long long)batch * W, true, t->S1, s)) != BVF_OK) return rc;
-        k_mix_dR<<<grid_for((long long)4 * m * m * m * W * W), 256, 0, s>>>(t->S1, t->X[l], batch, W,
-                                                                            m, gR);
-        k_mix_adj<<<grid_for((long long)batch * 4 * m * m * m * W), 256, 0, s>>>(t->S1, R, batch, W,
-                                                                                 m, t->S2);
-        BCK(cudaGetLastError(), "d mix");
+        if ((rc = mix_backward(t, batch, t->S1, t->X[l], R, gR, t->S2, s)) != BVF_OK) return rc;
         // dn = d v_l; for l > 0 it becomes d s_{l-1} = d v_l GELU'(s_{l-1})
         if ((rc = spec_inv_zy(t, t->S2, (long long)batch * W, s)) != BVF_OK) return rc;
         if ((rc = row_pass(t, batch, ds, W, Wl, 1, W, nullptr, t->Gx, l > 0 ? 2 : 0,
