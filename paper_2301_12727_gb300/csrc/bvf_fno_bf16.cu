@@ -41,6 +41,7 @@
 
 #include "bvf_fno_bf16.cuh"
 
+using bvf::ChanBf16;
 using bvf::GemmX;
 using bvf::launch_gemm_bf16;
 using bvf::RowBf16;
@@ -390,24 +391,22 @@ __global__ void k_loss_grad(const float *__restrict__ out, const float *__restri
                             const float *__restrict__ el, const double *__restrict__ sums, int B,
                             int c_out, int N, float el_weight, float *__restrict__ dout)
 {
-    const long long n = (long long)B * c_out * N;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int p = (int)(t % N);
-        const int k = (int)((t / N) % c_out);
-        const int b = (int)(t / ((long long)c_out * N));
-        const double *s = sums + 3 * b;
-        float g = 0.0f;
-        if (k == 0) {
-            const double rel = sqrt(s[0] / s[1]);
-            g = rel > 0.0 ? (float)(((double)out[t] - y[(size_t)b * N + p]) / (rel * s[1] * B))
-                          : 0.0f;
-        } else if (k == 1 && el) {
-            const double mean = s[2] / N;
-            g = (float)(2.0 * el_weight * (mean - el[b]) / ((double)N * B));
-        }
-        dout[t] = g;
+    // blockIdx.x: sample and channel, whose factor is the same for every voxel
+    const int b = blockIdx.x / c_out, k = blockIdx.x % c_out;
+    const double *s = sums + 3 * b;
+    bool on = false;
+    double f = 0.0;
+    if (k == 0) {
+        const double rel = sqrt(s[0] / s[1]);
+        on = rel > 0.0;
+        if (on) f = 1.0 / (rel * s[1] * B);
+    } else if (k == 1 && el) {
+        f = 2.0 * el_weight * (s[2] / N - el[b]) / ((double)N * B);
     }
+    const float *o = out + (size_t)blockIdx.x * N, *yb = y + (size_t)b * N;
+    float *d = dout + (size_t)blockIdx.x * N;
+    for (int p = blockIdx.y * blockDim.x + threadIdx.x; p < N; p += gridDim.y * blockDim.x)
+        d[p] = k == 0 ? (on ? (float)(((double)o[p] - yb[p]) * f) : 0.0f) : (float)f;
 }
 
 // sum of n floats into *out (FP64)
@@ -677,15 +676,6 @@ bvf_gemm chan(const float *in, int C, const float *Wt, float *out, int O, int N,
     return g;
 }
 
-// transposed channel mix out[b][c][p] = sum_o Wt[o][c] din[b][o][p]
-bvf_gemm chanT(const float *din, int O, const float *Wt, float *out, int C, int N, int B)
-{
-    bvf_gemm g = chan(din, O, Wt, out, C, N, B);
-    g.sbk = C;          // B(k = o, n = c) = Wt[o][c]
-    g.sbn = 1;
-    return g;
-}
-
 // weight gradient G[o][c] += sum_{b,p} d[b][o][p] x[b][c][p]
 bvf_gemm wgrad(const float *d, int O, const float *x, int C, float *G, int N, int B, int ksplit)
 {
@@ -794,6 +784,15 @@ int row_pass(bvf_fno_bf16 *t, int batch, const float *v, int cin, const float *W
     return gemm(t, g, s, "pointwise");
 }
 
+// out = act(Wm v + bias), K input and O output channels (Wm(o, c) at o wso + c wsc)
+int chan_pass(bvf_fno_bf16 *t, int batch, const float *v, int K, const float *Wm, int wso, int wsc,
+              const float *bias, int act, float *pre, float *out, int O, cudaStream_t s)
+{
+    const ChanBf16 q{v, K, O, Wm, wso, wsc, bias, pre, act, out, batch, t->N, t->flag};
+    BCK(bvf::launch_chan_bf16(q, t->n_sm, s), "channel product");
+    return BVF_OK;
+}
+
 // forward pass of `batch` samples into `out` ([batch][c_out][N]); with `keep`
 // every activation the backward pass needs is kept, without it (inference)
 // the pre-activations are not written
@@ -824,16 +823,11 @@ int forward(bvf_fno_bf16 *t, int batch, const float *in, float *out, bool keep, 
             "projection");
         return BVF_OK;
     }
-    bvf_gemm g = chan(t->v[L], W, w + o.Q1, t->h, d.hidden, N, batch);
-    g.bias = w + o.q1;
-    g.bias_mode = 1;
-    g.act = 1;
-    g.C_pre = t->pre1;
-    if ((rc = gemm(t, g, s, "projection 1")) != BVF_OK) return rc;
-    g = chan(t->h, d.hidden, w + o.Q2, out, d.c_out, N, batch);
-    g.bias = w + o.q2;
-    g.bias_mode = 1;
-    return gemm(t, g, s, "projection 2");
+    if ((rc = chan_pass(t, batch, t->v[L], W, w + o.Q1, W, 1, w + o.q1, 1, t->pre1, t->h, d.hidden,
+                        s)) != BVF_OK)
+        return rc;
+    return chan_pass(t, batch, t->h, d.hidden, w + o.Q2, d.hidden, 1, w + o.q2, 0, nullptr, out,
+                     d.c_out, s);
 }
 
 // loss and gradient into t->g (zeroed first); h_loss on the host
@@ -848,7 +842,7 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
     BCK(cudaMemsetAsync(t->sums, 0, 3 * sizeof(double) * batch, s), "loss");
     k_loss_sums<<<dim3(std::min(64, (N + 255) / 256), batch), 256, 0, s>>>(t->out, target, d.c_out,
                                                                           N, t->sums);
-    k_loss_grad<<<grid_for((long long)batch * d.c_out * N), 256, 0, s>>>(
+    k_loss_grad<<<dim3(batch * d.c_out, std::min(256, (N + 255) / 256)), 256, 0, s>>>(
         t->out, target, d.c_out > 1 ? el : nullptr, t->sums, batch, d.c_out, N, (float)el_weight,
         t->dout);
     BCK(cudaGetLastError(), "loss");
@@ -857,17 +851,17 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
     const float *w = t->w;
     const int ks = t->ksplit;
     // projection
-    bvf_gemm g = chanT(t->dout, d.c_out, w + o.Q2, t->dh, H, N, batch);
-    g.act = 2;
-    g.C_pre = t->pre1;                                 // dh -> d pre1
-    if ((rc = gemm(t, g, s, "d projection 2")) != BVF_OK) return rc;
+    if ((rc = chan_pass(t, batch, t->dout, d.c_out, w + o.Q2, 1, H, nullptr, 2, t->pre1, t->dh, H,
+                        s)) != BVF_OK)                 // dh -> d pre1
+        return rc;
     if ((rc = gemm(t, wgrad(t->dout, d.c_out, t->h, H, G + o.Q2, N, batch, ks), s, "dQ2")) != BVF_OK)
         return rc;
     if ((rc = chan_sum(t->dout, batch, d.c_out, N, G + o.q2, s)) != BVF_OK) return rc;
     if ((rc = gemm(t, wgrad(t->dh, H, t->v[L], W, G + o.Q1, N, batch, ks), s, "dQ1")) != BVF_OK)
         return rc;
     if ((rc = chan_sum(t->dh, batch, H, N, G + o.q1, s)) != BVF_OK) return rc;
-    if ((rc = gemm(t, chanT(t->dh, H, w + o.Q1, t->dv, W, N, batch), s, "d projection 1")) != BVF_OK)
+    if ((rc = chan_pass(t, batch, t->dh, H, w + o.Q1, 1, W, nullptr, 0, nullptr, t->dv, W, s)) !=
+        BVF_OK)
         return rc;
     // Fourier layers, top down; ds holds d(pre-activation) of layer l
     float *ds = t->dv, *dn = t->dv2;

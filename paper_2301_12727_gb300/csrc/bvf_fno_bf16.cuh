@@ -52,6 +52,20 @@ struct RowBf16 {
 };
 bool row_bf16_fits(int width, int m, int nx);
 cudaError_t launch_row_bf16(const RowBf16 &q, int width, cudaStream_t s);
+// one channel product (see bvf_row_bf16.cu)
+struct ChanBf16 {
+    const float *v;        // [B][K][N]
+    int K, O;
+    const float *Wm;       // Wm(o, c) at o wso + c wsc
+    int wso, wsc;
+    const float *bias;     // [O] or NULL
+    float *pre;            // act 1: receives the pre-activation (or NULL); act 2: holds it
+    int act;
+    float *out;            // [B][O][N]
+    int B, N;
+    int *flag;
+};
+cudaError_t launch_chan_bf16(const ChanBf16 &q, int n_sm, cudaStream_t s);
 cudaError_t launch_project_bf16(const float *v, const float *Q1, const float *q1, const float *Q2,
                                 const float *q2, int width, int hidden, int c_out, float *out, int N,
                                 int B, int n_sm, int *flag, cudaStream_t s);

@@ -10,6 +10,8 @@
 //     of a stored pre-activation.  Without S it is the lift.
 //   k_project_bf16  both layers of the projection with the hidden
 //     activations in shared memory.
+//   k_chan_bf16     one layer of the projection with its activations kept
+//     (training), and the backward products.
 //
 // What they replace are separate products (bvf_gemm_bf16.cu) with the volume
 // between them in HBM.  At 240 x 240 x 200, width 32, a layer took 904 us for
@@ -431,6 +433,151 @@ __global__ void __launch_bounds__(256, 3)
     if (warp == 0) tc::dealloc(tbase, L.ncols);
 }
 
+// ------------------------------------------------------------ channel product
+// out[o][p] = act( sum_c Wm(o, c) v[c][p] + b[o] ) on 128-point tiles, any K up
+// to 256 input and N up to 256 output channels: the projection's two layers
+// and their backward products when their activations are kept.  All of K is
+// staged at once (16 channels per thread in flight), the weights once per
+// block.  As separate products of one tile a block the four took 1244, 397,
+// 1244 and 397 us at 64 x 64 x 96, batch 4; now 402, 196, 570 (two special
+// functions for each of 50 million values) and 219.
+struct ChanBLayout {
+    int KP, NP, ncols, sA, sB, sb, bar, tmem, bytes;
+    __host__ __device__ ChanBLayout(int K, int N)
+    {
+        KP = (K + 15) & ~15;
+        NP = (N + 15) & ~15;
+        ncols = 32;
+        while (ncols < NP) ncols *= 2;
+        sA = 0;                              // [128][KP]
+        sB = sA + 128 * KP * 2;              // [NP][KP]
+        sb = sB + NP * KP * 2;
+        bar = (sb + NP * 4 + 15) & ~15;
+        tmem = bar + 16;
+        bytes = tmem + 16;
+    }
+};
+
+__global__ void __launch_bounds__(256, 3) k_chan_bf16(const __grid_constant__ ChanBf16 q)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    const ChanBLayout L(q.K, q.O);
+    const int KP = L.KP, NP = L.NP, N = q.N;
+    unsigned char *sA = sm + L.sA, *sB = sm + L.sB;
+    float *sb = reinterpret_cast<float *>(sm + L.sb);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + L.bar);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + L.tmem);
+    const int tid = threadIdx.x, warp = tid >> 5, pt = tid & 127, half = tid >> 7;
+    for (int e = tid; e < NP * (KP / 2); e += 256) {
+        const int o = e / (KP / 2), c = 2 * (e - o * (KP / 2));
+        const float w0 = o < q.O && c < q.K ? q.Wm[o * q.wso + c * q.wsc] : 0.0f;
+        const float w1 = o < q.O && c + 1 < q.K ? q.Wm[o * q.wso + (c + 1) * q.wsc] : 0.0f;
+        *reinterpret_cast<uint32_t *>(sB + tc::kmaj_off16(o, c & ~7, KP) + (c & 7) * 2) =
+            tc::pack_bf16(w0, w1);
+    }
+    for (int o = tid; o < NP; o += 256) sb[o] = q.bias && o < q.O ? q.bias[o] : 0.0f;
+    if (tid == 0) {
+        tma::mbar_init(bar, 1);
+        tma::mbar_init_fence();
+    }
+    if (warp == 0) {
+        tc::alloc(tslot, L.ncols);
+        tc::relinquish();
+    }
+    tma::fence_async_smem();
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tbase = *tslot;
+    const uint32_t idesc = tc::idesc_bf16(128, NP);
+    const uint32_t sbo = (uint32_t)(KP / 8) * 128;
+    const int per = (N + 127) / 128, tiles = per * q.B;
+    tma::pdl_wait();
+    tma::pdl_launch_next();
+    // 16 channels of this thread's point: c0 + 16 half ..
+    float xv[16];
+    auto load = [&](int tile, int c0) {
+        const int b = tile / per, p = (tile - b * per) * 128 + pt, ch = c0 + 16 * half;
+        const float *src = q.v + ((long long)b * q.K + ch) * N + p;
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+            xv[c] = p < N && ch + c < q.K ? tma::ld_stream(src + (long long)c * N) : 0.0f;
+    };
+    if ((int)blockIdx.x < tiles) load(blockIdx.x, 0);
+    int phase = 0;
+    bool gave_up = false;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        for (int c0 = 0; c0 < KP; c0 += 32) {
+            const int ch = c0 + 16 * half;
+            if (ch < KP) {                       // KP is a multiple of 16
+                *reinterpret_cast<uint4 *>(sA + tc::kmaj_off16(pt, ch, KP)) =
+                    make_uint4(tc::pack_bf16(xv[0], xv[1]), tc::pack_bf16(xv[2], xv[3]),
+                               tc::pack_bf16(xv[4], xv[5]), tc::pack_bf16(xv[6], xv[7]));
+                *reinterpret_cast<uint4 *>(sA + tc::kmaj_off16(pt, ch + 8, KP)) =
+                    make_uint4(tc::pack_bf16(xv[8], xv[9]), tc::pack_bf16(xv[10], xv[11]),
+                               tc::pack_bf16(xv[12], xv[13]), tc::pack_bf16(xv[14], xv[15]));
+            }
+            if (c0 + 32 < KP) load(tile, c0 + 32);
+        }
+        tma::fence_async_smem();
+        tc::fence_before();
+        __syncthreads();
+        if (tid == 0) {
+            tc::fence_after();
+            for (int ks = 0; ks < KP / 16; ++ks)
+                tc::mma_f16(tbase, tc::smem_desc(sA + ks * 256, 128, sbo),
+                            tc::smem_desc(sB + ks * 256, 128, sbo), idesc, ks > 0);
+            tc::commit(bar);
+        }
+        if (tile + (int)gridDim.x < tiles) load(tile + gridDim.x, 0);
+        const bool ready = __all_sync(0xffffffffu, tma::mbar_wait(bar, phase & 1, tma::kWaitLimit));
+        tc::fence_after();
+        if (ready) {
+            const int b = tile / per, p = (tile - b * per) * 128 + pt;
+            const long long at = (long long)b * q.O * N + p;
+            for (int c0 = 16 * half; c0 < NP; c0 += 32) {
+                float r[16], pv[16];
+                tc::ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, r);
+                if (p < N && q.act == 2) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        pv[i] = c0 + i < q.O ? tma::ld_stream(q.pre + at + (long long)(c0 + i) * N)
+                                             : 0.0f;
+                }
+                tc::wait_ld();
+                if (p < N) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        if (c0 + i >= q.O) break;
+                        const long long o = at + (long long)(c0 + i) * N;
+                        float v = r[i];
+                        if (q.bias) v = __fadd_rn(v, sb[c0 + i]);
+                        if (q.act == 1) {
+                            if (q.pre) q.pre[o] = v;
+                            v = gelu_exact(v);
+                        } else if (q.act == 2) {
+                            v *= gelu_grad(pv[i]);
+                        }
+                        q.out[o] = v;
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        tc::fence_before();
+        gave_up = __syncthreads_or(!ready) != 0;
+        if (gave_up) break;
+        ++phase;
+    }
+    if (gave_up && tid == 0) {
+        tma::mbar_wait(bar, phase & 1, tma::kWaitLimit);
+        atomicOr(q.flag, 2);
+    }
+    tc::fence_after();
+    __syncthreads();
+    if (warp == 0) tc::dealloc(tbase, L.ncols);
+}
+
 // the shared-memory limit, raised once per process and kernel to the cap, so
 // that later launches make no other runtime call
 template <auto Kernel>
@@ -492,6 +639,15 @@ cudaError_t launch_row_bf16(const RowBf16 &q, int width, cudaStream_t s)
     case 48: return launch_row_w<48, 48>(q, s);
     default: return launch_row_w<64, 64>(q, s);
     }
+}
+
+cudaError_t launch_chan_bf16(const ChanBf16 &q, int n_sm, cudaStream_t s)
+{
+    const ChanBLayout L(q.K, q.O);
+    const cudaError_t e = raise_smem<k_chan_bf16>();
+    if (e != cudaSuccess) return e;
+    const int grid = std::min((q.N + 127) / 128 * q.B, n_sm * blocks_per_sm(L.bytes, L.ncols));
+    return launch_pdl(k_chan_bf16, grid, 256, L.bytes, s, q);
 }
 
 cudaError_t launch_project_bf16(const float *v, const float *Q1, const float *q1, const float *Q2,
