@@ -17,8 +17,8 @@
 // between them in HBM.  At 240 x 240 x 200, width 32, a layer took 904 us for
 // the inverse (1.5 GB written) and 2040 us for the mix (1.5 GB read twice
 // over, 1.5 GB written), the projection 6806 + 2151 us around 5.9 GB of
-// hidden activations; now 1096 us a layer and 1799 us (the whole
-// forward 28.0 -> 10.5 ms).  Every product keeps its
+// hidden activations; now 690 us a layer and 1793 us (the whole
+// forward 28.0 -> 8.5 ms).  Every product keeps its
 // operands' rounding and its order of K steps, and the two sums of a layer
 // meet in FP32 in the epilogue as they did through memory, so the results are
 // the separate products' bit for bit.
@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "bvf_fno_bf16.cuh"
 #include "bvf_tc.cuh"
@@ -65,22 +66,44 @@ struct RowBLayout {
     }
 };
 
-// W output channels; input channels padded to KC (a multiple of 16); RP rows a tile
-template <int W, int KC, int RP>
-__global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ RowBf16 q)
+// e / d by multiplication (d >= 1, e d < 2^30)
+struct SmallDiv {
+    unsigned d, f;
+    __device__ explicit SmallDiv(unsigned d_) : d(d_), f((0x80000000u + d_ - 1) / d_) {}
+    __device__ unsigned quot(unsigned e) const { return __umulhi(2 * e, f); }
+};
+
+// W output channels; input channels padded to KC (a multiple of 16); RP rows a
+// tile; SPEC: with a spectral term (the lift has none).  The products of a
+// tile run under the epilogue of the tile before it: two accumulator sets in
+// tensor memory, one barrier a tile.  With the products waited for in turn,
+// and divisions for the row, branches and 64-bit address products for every
+// output (80 instructions an output, two thirds of the issue slots), a layer
+// took 1179 us at 240 x 240 x 200, width 32, the last one (no GELU) 845 and the
+// lift 787; now 690, 592 and 331.  Bound by issue under a GELU, by its reads
+// and writes (433 us at 6.8 TB/s) without.
+template <int W, int KC, int RP, bool SPEC>
+struct RowBShape {
+    static constexpr int kSet = SPEC ? 2 * W : W;            // columns of a set
+    static constexpr int kCols = 2 * kSet <= 32 ? 32 : (2 * kSet <= 64 ? 64 : (2 * kSet <= 128 ? 128 : 256));
+    static constexpr int kBlocks = SPEC ? (kCols <= 128 ? 3 : 2) : 4;
+};
+
+template <int W, int KC, int RP, bool SPEC>
+__global__ void __launch_bounds__(256, (RowBShape<W, KC, RP, SPEC>::kBlocks))
+    k_row_bf16(const __grid_constant__ RowBf16 q)
 {
     static_assert(W % 16 == 0 && KC % 16 == 0, "tile shape");
+    using Shape = RowBShape<W, KC, RP, SPEC>;
     extern __shared__ __align__(128) unsigned char sm[];
-    const bool spec = q.S != nullptr;
     const int nx = q.nx, m = q.m, rows = q.rows, N = q.N;
-    const RowBLayout L(W, KC, m, nx, spec);
+    const RowBLayout L(W, KC, m, nx, SPEC);
     const int JP = L.JP, KS = L.KS, nxt = L.nxt;
     unsigned char *sA = sm + L.sA, *sT = sm + L.sT, *sW = sm + L.sW, *sS = sm + L.sS;
     float *sb = reinterpret_cast<float *>(sm + L.sb);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + L.bar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + L.tmem);
     const int tid = threadIdx.x, warp = tid >> 5, pt = tid & 127, half = tid >> 7;
-    constexpr int NCOLS = 2 * W <= 32 ? 32 : (2 * W <= 64 ? 64 : 128);
     // this thread's point: row lr of the tile, x (of the first tile)
     const int lr = RP > 1 ? pt / nx : 0, px = pt - lr * nx;
     // block constants: the channel weights, the x table, the zero columns of S
@@ -91,7 +114,7 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
         *reinterpret_cast<uint32_t *>(sW + tc::kmaj_off16(o, c & ~7, KC) + (c & 7) * 2) =
             tc::pack_bf16(w0, w1);
     }
-    if (spec) {
+    if (SPEC) {
         for (int e = tid; e < nxt * 128 * (KS / 2); e += 256) {
             const int t = e / (128 * (KS / 2)), r = e - t * 128 * (KS / 2);
             const int xl = r / (KS / 2), k = 2 * (r - xl * (KS / 2));
@@ -115,7 +138,7 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
         tma::mbar_init_fence();
     }
     if (warp == 0) {
-        tc::alloc(tslot, NCOLS);
+        tc::alloc(tslot, Shape::kCols);
         tc::relinquish();
     }
     tma::fence_async_smem();
@@ -128,48 +151,63 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
     constexpr uint32_t SBO = (KC / 8) * 128;
     const uint32_t sbo_s = (uint32_t)(KS / 8) * 128;
     const int groups = (rows + RP - 1) / RP;         // row groups of a sample
-    const int items = q.B * groups;
 
-    // loaded one tile (channels) or one row group (spectral pairs) ahead
+    struct Pos {
+        int b, g, t;                                 // sample, row group, tile of the row
+    };
+    auto next = [&](Pos p) {
+        if (++p.t == nxt) {
+            p.t = 0;
+            for (p.g += gridDim.x; p.g >= groups; p.g -= groups) ++p.b;
+        }
+        return p;
+    };
+    // this thread's point of a tile: whether there is one, and its index
+    auto point = [&](const Pos &p, long long &at) {
+        const int row = p.g * RP + lr, x = RP > 1 ? px : 128 * p.t + pt;
+        at = (long long)row * nx + x;
+        return RP > 1 ? (lr < RP && row < rows) : x < nx;
+    };
+    // loaded one tile (channels) or one row group (spectral pairs) ahead of staging
     float xv[CH];
-    auto load_v = [&](int it, int t) {
-        const int b = it / groups, row = (it - b * groups) * RP + lr;
-        const int x = RP > 1 ? px : 128 * t + pt;
-        const bool ok = RP > 1 ? (lr < RP && row < rows) : x < nx;
-        const float *src = q.v + (long long)b * q.vb + ((long long)row * nx + x);
+    const bool full = q.cin == KC;
+    auto load_v = [&](const Pos &p) {
+        long long at;
+        const bool ok = point(p, at);
+        const float *src = q.v + p.b * q.vb + (long long)(half * CH) * N + at;
+        if (full) {
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-            const int ch = half * CH + c;
-            xv[c] = (ok && ch < q.cin) ? tma::ld_stream(src + (long long)ch * N) : 0.0f;
+            for (int c = 0; c < CH; ++c) {
+                xv[c] = ok ? tma::ld_stream(src) : 0.0f;
+                src += N;
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                xv[c] = ok && half * CH + c < q.cin ? tma::ld_stream(src) : 0.0f;
+                src += N;
+            }
         }
     };
-    constexpr int PRE = (W * RP * 16 + 255) / 256;   // pairs per thread at m = 16
+    constexpr int PRE = SPEC ? (W * RP * 16 + 255) / 256 : 1;   // pairs per thread at m = 16
     float2 pre[PRE];
-    auto load_s = [&](int it) {
-        const int b = it / groups, row0 = (it - b * groups) * RP;
-        const float *src = q.S + ((long long)b * W * rows + row0) * (2 * m);
+    const SmallDiv by_rm((unsigned)(RP * (SPEC ? m : 1))), by_m((unsigned)(SPEC ? m : 1));
+    auto load_s = [&](const Pos &p) {
+        const int row0 = p.g * RP;
+        const float *src = q.S + ((long long)p.b * W * rows + row0) * (2 * m);
 #pragma unroll
         for (int i = 0; i < PRE; ++i) {
             const int e = tid + i * 256;
             pre[i] = make_float2(0.0f, 0.0f);
             if (e < W * RP * m) {
-                const int o = e / (RP * m), r = e - o * RP * m;   // r: pair of the o's RP rows
-                if (row0 + r / m < rows)
+                const int o = by_rm.quot(e), r = e - o * RP * m;   // r: pair of the o's RP rows
+                if (RP == 1 || row0 + (int)by_m.quot(r) < rows)
                     pre[i] = tma::ld_stream(
                         reinterpret_cast<const float2 *>(src + (long long)o * rows * (2 * m)) + r);
             }
         }
     };
-    // weights and tables are in place: the rest depends on earlier kernels
-    tma::pdl_wait();
-    tma::pdl_launch_next();
-    int item = blockIdx.x, t = 0, phase = 0;
-    if (item < items) {
-        load_v(item, 0);
-        if (spec) load_s(item);
-    }
-    bool gave_up = false;
-    while (item < items) {
+    auto stage = [&](const Pos &p) {
 #pragma unroll
         for (int c8 = 0; c8 < CH / 8; ++c8)
             *reinterpret_cast<uint4 *>(sA + tc::kmaj_off16(pt, half * CH + 8 * c8, KC)) =
@@ -177,12 +215,13 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
                            tc::pack_bf16(xv[8 * c8 + 2], xv[8 * c8 + 3]),
                            tc::pack_bf16(xv[8 * c8 + 4], xv[8 * c8 + 5]),
                            tc::pack_bf16(xv[8 * c8 + 6], xv[8 * c8 + 7]));
-        if (spec && t == 0) {
+        if (SPEC && p.t == 0) {
 #pragma unroll
             for (int i = 0; i < PRE; ++i) {
                 const int e = tid + i * 256;
                 if (e < W * RP * m) {
-                    const int o = e / (RP * m), r = e - o * RP * m, k = (r / m) * JP + 2 * (r % m);
+                    const int o = by_rm.quot(e), r = e - o * RP * m;
+                    const int kr = RP == 1 ? 0 : by_m.quot(r), k = kr * JP + 2 * (r - kr * m);
                     *reinterpret_cast<uint32_t *>(sS + tc::kmaj_off16(o, k & ~7, KS) + (k & 7) * 2) =
                         tc::pack_bf16(pre[i].x, pre[i].y);
                 }
@@ -190,73 +229,110 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
         }
         tma::fence_async_smem();
         tc::fence_before();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after();
-            if (spec)
-                for (int ks = 0; ks < KS / 16; ++ks)
-                    tc::mma_f16(tbase, tc::smem_desc(sT + t * 128 * KS * 2 + ks * 256, 128, sbo_s),
-                                tc::smem_desc(sS + ks * 256, 128, sbo_s), idesc, ks > 0);
+    };
+    // thread 0, after a barrier behind stage(): both sums of a tile into a set
+    auto issue = [&](const Pos &p, int set) {
+        const uint32_t ta = tbase + (uint32_t)(set * Shape::kSet);
+        tc::fence_after();
+        if (SPEC)
+            for (int ks = 0; ks < KS / 16; ++ks)
+                tc::mma_f16(ta, tc::smem_desc(sT + p.t * 128 * KS * 2 + ks * 256, 128, sbo_s),
+                            tc::smem_desc(sS + ks * 256, 128, sbo_s), idesc, ks > 0);
 #pragma unroll
-            for (int ks = 0; ks < KC / 16; ++ks)
-                tc::mma_f16(tbase + W, tc::smem_desc(sA + ks * 256, 128, SBO),
-                            tc::smem_desc(sW + ks * 256, 128, SBO), idesc, ks > 0);
-            tc::commit(bar);
+        for (int ks = 0; ks < KC / 16; ++ks)
+            tc::mma_f16(ta + (SPEC ? W : 0), tc::smem_desc(sA + ks * 256, 128, SBO),
+                        tc::smem_desc(sW + ks * 256, 128, SBO), idesc, ks > 0);
+        tc::commit(bar);
+    };
+    // ACT: 0 none, 1 GELU, 2 times GELU' of the stored value, 3 GELU, value kept
+    auto epilogue = [&](auto act, const Pos &p, int set) {
+        constexpr int ACT = decltype(act)::value;
+        long long at;
+        const bool ok = point(p, at);
+        const int o0 = half * (W / 2);
+        const uint32_t ta = tbase + (uint32_t)(set * Shape::kSet + o0) +
+                            ((uint32_t)(32 * (warp & 3)) << 16);
+        at += ((long long)p.b * W + o0) * N;
+        float *op = q.out + at;
+        float *pp = ACT >= 2 ? q.pre + at : nullptr;
+#pragma unroll 1
+        for (int c0 = 0; c0 < W / 2; c0 += 8) {
+            float d[8], s[8], pv[8];
+            tc::ld8(ta + (SPEC ? W : 0) + c0, d);
+            if (SPEC) tc::ld8(ta + c0, s);
+            if (ACT == 2 && ok) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    pv[i] = tma::ld_stream(pp);
+                    pp += N;
+                }
+            }
+            tc::wait_ld();
+            if (ok) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float v = SPEC ? __fadd_rn(s[i], d[i]) : d[i];
+                    v = __fadd_rn(v, sb[o0 + c0 + i]);
+                    if (ACT == 3) {
+                        *pp = v;
+                        pp += N;
+                    }
+                    if (ACT == 1 || ACT == 3) v = gelu_exact(v);
+                    if (ACT == 2) v *= gelu_grad(pv[i]);
+                    *op = v;
+                    op += N;
+                }
+            }
+            __syncwarp();            // the next tensor-memory load is warp-wide
         }
-        int nitem = item, nt = t + 1;
-        if (nt == nxt) {
-            nt = 0;
-            nitem = item + gridDim.x;
-        }
-        const int b = item / groups, row = (item - b * groups) * RP + lr;
-        const int x = RP > 1 ? px : 128 * t + pt;
-        const bool ok = RP > 1 ? (lr < RP && row < rows) : x < nx;
-        const long long at = (long long)b * W * N + ((long long)row * nx + x);
-        // the next tile's loads and this one's stored pre-activations overlap
-        // the products
-        if (nitem < items) {
-            load_v(nitem, nt);
-            if (spec && nt == 0) load_s(nitem);
-        }
+    };
+    // weights and tables are in place: the rest depends on earlier kernels
+    tma::pdl_wait();
+    tma::pdl_launch_next();
+    Pos cur{0, (int)blockIdx.x, 0};
+    for (; cur.g >= groups; cur.g -= groups) ++cur.b;     // gridDim.x <= B groups
+    load_v(cur);
+    if (SPEC) load_s(cur);
+    stage(cur);
+    __syncthreads();
+    if (tid == 0) issue(cur, 0);
+    Pos nxtp = next(cur);
+    if (nxtp.b < q.B) {
+        load_v(nxtp);
+        if (SPEC && nxtp.t == 0) load_s(nxtp);
+    }
+    int phase = 0;
+    bool gave_up = false;
+    while (cur.b < q.B) {
+        // the products of cur: their operands and the other accumulators are free
         const bool ready =
             __all_sync(0xffffffffu, tma::mbar_wait(bar, phase & 1, tma::kWaitLimit));
         tc::fence_after();
-        if (ready) {
-#pragma unroll 1
-            for (int c0 = 0; c0 < W / 2; c0 += 8) {
-                const int o0 = half * (W / 2) + c0;
-                const uint32_t ta = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)o0;
-                float d[8], s[8], pv[8];
-                tc::ld8(ta + W, d);
-                if (spec) tc::ld8(ta, s);
-                if (ok && q.act == 2) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) pv[i] = tma::ld_stream(q.pre + at + (long long)(o0 + i) * N);
-                }
-                tc::wait_ld();
-                if (ok) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const long long p = at + (long long)(o0 + i) * N;
-                        float v = spec ? __fadd_rn(s[i], d[i]) : d[i];
-                        if (q.bias) v = __fadd_rn(v, sb[o0 + i]);
-                        if (q.act == 1) {
-                            if (q.pre) q.pre[p] = v;
-                            v = gelu_exact(v);
-                        } else if (q.act == 2) {
-                            v *= gelu_grad(pv[i]);
-                        }
-                        q.out[p] = v;
-                    }
-                }
-                __syncwarp();        // the next tensor-memory load is warp-wide
-            }
-        }
-        tc::fence_before();
+        const bool more = nxtp.b < q.B;
+        if (more && ready) stage(nxtp);
         gave_up = __syncthreads_or(!ready) != 0;
         if (gave_up) break;
-        item = nitem;
-        t = nt;
+        Pos after = nxtp;
+        if (more) {
+            if (tid == 0) issue(nxtp, (phase + 1) & 1);
+            after = next(nxtp);
+            if (after.b < q.B) {
+                load_v(after);
+                if (SPEC && after.t == 0) load_s(after);
+            }
+        }
+        const int set = phase & 1;
+        if (!SPEC || q.act == 0)
+            epilogue(std::integral_constant<int, 0>{}, cur, set);
+        else if (q.act == 2)
+            epilogue(std::integral_constant<int, 2>{}, cur, set);
+        else if (q.pre)
+            epilogue(std::integral_constant<int, 3>{}, cur, set);
+        else
+            epilogue(std::integral_constant<int, 1>{}, cur, set);
+        tc::fence_before();
+        cur = nxtp;
+        nxtp = after;
         ++phase;
     }
     if (gave_up && tid == 0) {
@@ -265,7 +341,7 @@ __global__ void __launch_bounds__(256, 3) k_row_bf16(const __grid_constant__ Row
     }
     tc::fence_after();
     __syncthreads();
-    if (warp == 0) tc::dealloc(tbase, NCOLS);
+    if (warp == 0) tc::dealloc(tbase, Shape::kCols);
 }
 
 // ---------------------------------------------------------------- projection
@@ -591,28 +667,33 @@ cudaError_t raise_smem()
     return e;
 }
 
-int blocks_per_sm(int bytes, int ncols)
+int blocks_per_sm(int bytes, int ncols, int most = 3)
 {
-    return std::max(1, std::min({3, (227 * 1024) / (bytes + 1024), 512 / ncols}));
+    return std::max(1, std::min({most, (227 * 1024) / (bytes + 1024), 512 / ncols}));
 }
 
-template <int W, int KC, int RP>
+template <int W, int KC, int RP, bool SPEC>
 cudaError_t launch_row_k(const RowBf16 &q, const RowBLayout &L, cudaStream_t s)
 {
-    const cudaError_t e = raise_smem<k_row_bf16<W, KC, RP>>();
+    using Shape = RowBShape<W, KC, RP, SPEC>;
+    const cudaError_t e = raise_smem<k_row_bf16<W, KC, RP, SPEC>>();
     if (e != cudaSuccess) return e;
     const int items = q.B * ((q.rows + RP - 1) / RP);
-    const int grid = std::min(items, q.n_sm * blocks_per_sm(L.bytes, 2 * W <= 64 ? 64 : 128));
-    return launch_pdl(k_row_bf16<W, KC, RP>, grid, 256, L.bytes, s, q);
+    const int grid = std::min(items, q.n_sm * blocks_per_sm(L.bytes, Shape::kCols, Shape::kBlocks));
+    if (SPEC) return launch_pdl(k_row_bf16<W, KC, RP, SPEC>, grid, 256, L.bytes, s, q);
+    // the lift reads weights that an optimiser step just before it may have
+    // written: an ordinary launch
+    k_row_bf16<W, KC, RP, SPEC><<<grid, 256, L.bytes, s>>>(q);
+    return cudaGetLastError();
 }
 
-template <int W, int KC>
+template <int W, int KC, bool SPEC>
 cudaError_t launch_row_w(const RowBf16 &q, cudaStream_t s)
 {
-    const RowBLayout L(W, KC, q.m, q.nx, q.S != nullptr);
-    if (L.RP == 1) return launch_row_k<W, KC, 1>(q, L, s);
-    if (L.RP == 2) return launch_row_k<W, KC, 2>(q, L, s);
-    return launch_row_k<W, KC, 4>(q, L, s);
+    const RowBLayout L(W, KC, q.m, q.nx, SPEC);
+    if (L.RP == 1) return launch_row_k<W, KC, 1, SPEC>(q, L, s);
+    if (L.RP == 2) return launch_row_k<W, KC, 2, SPEC>(q, L, s);
+    return launch_row_k<W, KC, 4, SPEC>(q, L, s);
 }
 
 }  // namespace
@@ -625,19 +706,19 @@ bool row_bf16_fits(int width, int m, int nx)
 cudaError_t launch_row_bf16(const RowBf16 &q, int width, cudaStream_t s)
 {
     // the lift's 1 .. 16 input channels fill one K step; a layer has W
-    if (!q.S && q.cin <= 16) {
+    if (!q.S) {
         switch (width) {
-        case 16: return launch_row_w<16, 16>(q, s);
-        case 32: return launch_row_w<32, 16>(q, s);
-        case 48: return launch_row_w<48, 16>(q, s);
-        default: return launch_row_w<64, 16>(q, s);
+        case 16: return launch_row_w<16, 16, false>(q, s);
+        case 32: return launch_row_w<32, 16, false>(q, s);
+        case 48: return launch_row_w<48, 16, false>(q, s);
+        default: return launch_row_w<64, 16, false>(q, s);
         }
     }
     switch (width) {
-    case 16: return launch_row_w<16, 16>(q, s);
-    case 32: return launch_row_w<32, 32>(q, s);
-    case 48: return launch_row_w<48, 48>(q, s);
-    default: return launch_row_w<64, 64>(q, s);
+    case 16: return launch_row_w<16, 16, true>(q, s);
+    case 32: return launch_row_w<32, 32, true>(q, s);
+    case 48: return launch_row_w<48, 48, true>(q, s);
+    default: return launch_row_w<64, 64, true>(q, s);
     }
 }
 
