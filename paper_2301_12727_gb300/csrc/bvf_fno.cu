@@ -32,6 +32,7 @@
 #include "bvf_internal.cuh"
 #include "bvf_tc.cuh"
 #include "bvf_tma.cuh"
+#include "bvf_xfwd.cuh"
 
 namespace {
 
@@ -879,7 +880,9 @@ k_row_tc(const float *vin, int cin, const float2 *Ap,
 // with T[j][x] = cos, sin (2 pi kx x / nx) for j = 2 kx, 2 kx + 1 (zero rows
 // up to NB, a multiple of 16).  x runs in chunks of 16 through two staged
 // buffers (A, split, K-major); T is resident, split, for the whole row.  The
-// next chunk's loads are issued before the current chunk is staged.
+// next chunk's loads are issued before the current chunk is staged.  Rows that
+// TMA can fetch take k_xfwd (bvf_xfwd.cu: 298 us against 475 at 240 x 240 x
+// 200, width 32); this kernel takes the others.
 constexpr int kDxC = 16;     // x per chunk
 
 struct DftxTcLayout {
@@ -1628,6 +1631,19 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
 #undef BVF_ROW
         if (e != cudaSuccess || !An) return e;
         const long R = (long)W * rows_p, tiles = (R + 127) / 128;
+        if (bvf::xfwd_fits(true, vout, R, nx, m)) {
+            bvf::XfwdArgs x{};
+            x.v = vout;
+            x.R = R;
+            x.nx = nx;
+            x.m = m;
+            x.tx = tx;
+            x.out = An;
+            x.n_sm = n_sm;
+            x.flag = f->flag;
+            e = bvf::launch_xfwd(true, x, s);
+            if (e != cudaErrorNotSupported) return e;
+        }
         const int g2 = (int)std::min<long>(tiles, (long)n_sm * blocks_per_sm(dl.bytes));
         const bool vec = nx % 4 == 0;
         if (nb == 16)

@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "bvf_fno_bf16.cuh"
+#include "bvf_xfwd.cuh"
 
 using bvf::ChanBf16;
 using bvf::GemmX;
@@ -590,13 +591,29 @@ int spec_fwd(bvf_fno_bf16 *t, const float *in, long long BC, bool weighted, floa
     const int nx = t->nx, ny = t->ny, nz = t->nz, m = t->d.modes;
     int rc;
     // x: rows (bc, z, y) -> w1 [bc][z][part][kx][y]
+    const long long rows = BC * nz * ny;
+    cudaError_t e = cudaErrorNotSupported;
+    if (bvf::xfwd_fits(false, in, rows, nx, m)) {
+        bvf::XfwdArgs q{};
+        q.v = in;
+        q.R = rows;
+        q.nx = nx;
+        q.m = m;
+        q.F = weighted ? t->Fxw : t->Fx;
+        q.outw = t->w1;
+        q.ny = ny;
+        q.n_sm = t->n_sm;
+        q.flag = t->flag;
+        e = bvf::launch_xfwd(false, q, s);
+        if (e != cudaErrorNotSupported) BCK(e, "spectral x");
+    }
     GemmX x;
     x.g = rowmajor(in, weighted ? t->Fxw : t->Fx, t->w1, BC * nz * ny, nx, 2 * m);
     x.rc = ny;
     x.scm1 = 2LL * m * ny;
     x.g.scm = 1;
     x.g.scn = ny;
-    if ((rc = gemm(t, x, s, "spectral x")) != BVF_OK) return rc;
+    if (e == cudaErrorNotSupported && (rc = gemm(t, x, s, "spectral x")) != BVF_OK) return rc;
     // y: rows (bc, kx, z), K (part, y) -> w2 [bc][part][ky][kx][z]
     x = GemmX();
     x.g = rowmajor(t->w1, t->Fy, t->w2, BC * nz * m, 2 * ny, 4 * m);
