@@ -75,40 +75,6 @@ int pick_slots(bool tf, int nb, int nx)
     return 0;
 }
 
-// the two products of a K step with A in tensor memory
-__device__ __forceinline__ void mma_tf32_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, int acc)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
-                 ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc)
-                 : "memory");
-}
-__device__ __forceinline__ void mma_bf16_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, int acc)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-                 ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc)
-                 : "memory");
-}
-// 16 / 8 consecutive columns of this warp's lanes
-__device__ __forceinline__ void st16(uint32_t t, const uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15,%16};" ::"r"(t),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
-__device__ __forceinline__ void st8(uint32_t t, const uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(t),
-                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
-                 "r"(r[7])
-                 : "memory");
-}
-__device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
 __device__ __forceinline__ void load2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
@@ -221,15 +187,15 @@ __global__ void __launch_bounds__(256, 2)
                     h[i] = __float_as_uint(v[i]) & 0xFFFFE000u;
                     l[i] = __float_as_uint(v[i] - __uint_as_float(h[i]));
                 }
-                st16(ta + 16 * half, h);
-                st16(ta + 32 + 16 * half, l);
+                tc::st16(ta + 16 * half, h);
+                tc::st16(ta + 32 + 16 * half, l);
             } else {
                 uint32_t u[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) u[i] = tc::pack_bf16(v[2 * i], v[2 * i + 1]);
-                st8(ta + 8 * half, u);
+                tc::st8(ta + 8 * half, u);
             }
-            wait_st();
+            tc::wait_st();
         }
         tc::fence_before();
         if (__syncthreads_or(!ok)) {
@@ -245,13 +211,13 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
                     for (int ks = 0; ks < kXc / 8; ++ks) {
                         const uint64_t b = tc::smem_desc(sB + (sch * (kXc / 8) + ks) * 256, 128, sbo);
-                        mma_tf32_ta(td, ta + 8 * ks, b, idesc2, sch > 0 || ks > 0);
-                        mma_tf32_ta(td + NB, ta + 32 + 8 * ks, b, idesc, 1);
+                        tc::mma_ta(td, ta + 8 * ks, b, idesc2, sch > 0 || ks > 0);
+                        tc::mma_ta(td + NB, ta + 32 + 8 * ks, b, idesc, 1);
                     }
                 } else {
 #pragma unroll
                     for (int ks = 0; ks < kXc / 16; ++ks)
-                        mma_bf16_ta(td, ta + 8 * ks,
+                        tc::mma_f16_ta(td, ta + 8 * ks,
                                     tc::smem_desc(sB + (sch * (kXc / 16) + ks) * 256, 128, sbo),
                                     idesc, sch > 0 || ks > 0);
                 }
@@ -350,12 +316,6 @@ cudaError_t launch_k(const CUtensorMap &map, const XfwdArgs &q, cudaStream_t s)
     const long long tiles = (q.R + 127) / 128;
     const int per = 2 * (L.bytes + 1024) <= 228 * 1024 ? 2 : 1;
     const int grid = (int)std::min<long long>(tiles, (long long)q.n_sm * per);
-    if (TF) {
-        // not started early, as the kernel it stands in for: behind a lift that
-        // was started early itself its blocks land unevenly
-        k_xfwd<TF, NB><<<grid, 256, L.bytes, s>>>(map, q, slots);
-        return cudaGetLastError();
-    }
     return launch_pdl(k_xfwd<TF, NB>, grid, 256, L.bytes, s, map, q, slots);
 }
 
