@@ -46,6 +46,7 @@ using bvf::ChanBf16;
 using bvf::GemmX;
 using bvf::launch_gemm_bf16;
 using bvf::RowBf16;
+using bvf::WgradBf16;
 
 namespace {
 
@@ -726,6 +727,20 @@ int chan_sum(const float *x, int B, int C, int N, float *out, cudaStream_t s)
     return BVF_OK;
 }
 
+// G += d x^T and g += the sums of d over the batch's points.  Volumes whose
+// rows are no whole 16-byte pieces take a general product and separate sums.
+int weight_grad(bvf_fno_bf16 *t, int batch, const float *dd, int O, const float *x, int C, float *G,
+                float *g, cudaStream_t s)
+{
+    const WgradBf16 q{dd, x, O, C, G, g, batch, t->N, t->flag};
+    if (bvf::wgrad_fits(q)) {
+        BCK(bvf::launch_wgrad_bf16(q, t->n_sm, s), "weight gradient");
+        return BVF_OK;
+    }
+    const int rc = gemm(t, wgrad(dd, O, x, C, G, t->N, batch, t->ksplit), s, "weight gradient");
+    return rc != BVF_OK ? rc : chan_sum(dd, batch, O, t->N, g, s);
+}
+
 // Y = R X per mode
 int mix_forward(bvf_fno_bf16 *t, int batch, float *X, const float *Rw, float *Y, cudaStream_t s)
 {
@@ -866,17 +881,14 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
     BCK(cudaMemsetAsync(t->g, 0, t->n_w * sizeof(float), s), "gradient");
     float *G = t->g;
     const float *w = t->w;
-    const int ks = t->ksplit;
     // projection
     if ((rc = chan_pass(t, batch, t->dout, d.c_out, w + o.Q2, 1, H, nullptr, 2, t->pre1, t->dh, H,
                         s)) != BVF_OK)                 // dh -> d pre1
         return rc;
-    if ((rc = gemm(t, wgrad(t->dout, d.c_out, t->h, H, G + o.Q2, N, batch, ks), s, "dQ2")) != BVF_OK)
+    if ((rc = weight_grad(t, batch, t->dout, d.c_out, t->h, H, G + o.Q2, G + o.q2, s)) != BVF_OK)
         return rc;
-    if ((rc = chan_sum(t->dout, batch, d.c_out, N, G + o.q2, s)) != BVF_OK) return rc;
-    if ((rc = gemm(t, wgrad(t->dh, H, t->v[L], W, G + o.Q1, N, batch, ks), s, "dQ1")) != BVF_OK)
+    if ((rc = weight_grad(t, batch, t->dh, H, t->v[L], W, G + o.Q1, G + o.q1, s)) != BVF_OK)
         return rc;
-    if ((rc = chan_sum(t->dh, batch, H, N, G + o.q1, s)) != BVF_OK) return rc;
     if ((rc = chan_pass(t, batch, t->dh, H, w + o.Q1, 1, W, nullptr, 0, nullptr, t->dv, W, s)) !=
         BVF_OK)
         return rc;
@@ -887,8 +899,7 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
         float *gl = G + o.lay0 + l * o.lf;
         const float *R = lw, *Wl = lw + (size_t)4 * m * m * m * W * W * 2;
         float *gR = gl, *gW = gl + (size_t)4 * m * m * m * W * W * 2, *gb = gW + (size_t)W * W;
-        if ((rc = chan_sum(ds, batch, W, N, gb, s)) != BVF_OK) return rc;
-        if ((rc = gemm(t, wgrad(ds, W, t->v[l], W, gW, N, batch, ks), s, "dW")) != BVF_OK) return rc;
+        if ((rc = weight_grad(t, batch, ds, W, t->v[l], W, gW, gb, s)) != BVF_OK) return rc;
         if ((rc = spec_fwd(t, ds, (long long)batch * W, true, t->S1, s)) != BVF_OK) return rc;
         if ((rc = mix_backward(t, batch, t->S1, t->X[l], R, gR, t->S2, s)) != BVF_OK) return rc;
         // dn = d v_l; for l > 0 it becomes d s_{l-1} = d v_l GELU'(s_{l-1})
@@ -899,9 +910,7 @@ int gradient(bvf_fno_bf16 *t, int batch, const float *in, const float *target, c
         std::swap(ds, dn);
     }
     // lift
-    if ((rc = chan_sum(ds, batch, W, N, G + o.bp, s)) != BVF_OK) return rc;
-    if ((rc = gemm(t, wgrad(ds, W, in, d.c_in, G + o.Wp, N, batch, ks), s, "dWp")) != BVF_OK)
-        return rc;
+    if ((rc = weight_grad(t, batch, ds, W, in, d.c_in, G + o.Wp, G + o.bp, s)) != BVF_OK) return rc;
     if (h_loss) {
         std::vector<double> h(3 * batch);
         BCK(cudaMemcpyAsync(h.data(), t->sums, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s),

@@ -52,6 +52,18 @@ struct RowBf16 {
 };
 bool row_bf16_fits(int width, int m, int nx);
 cudaError_t launch_row_bf16(const RowBf16 &q, int width, cudaStream_t s);
+// weight and bias gradient of a channel mix (see bvf_wgrad_bf16.cu)
+struct WgradBf16 {
+    const float *d;        // [B][O][N]
+    const float *x;        // [B][C][N]
+    int O, C;
+    float *G;              // [O][C], added to
+    float *g;              // [O], added to, or NULL
+    int B, N;
+    int *flag;
+};
+bool wgrad_fits(const WgradBf16 &q);      // rows of whole 16-byte pieces
+cudaError_t launch_wgrad_bf16(const WgradBf16 &q, int n_sm, cudaStream_t s);
 // one channel product (see bvf_row_bf16.cu)
 struct ChanBf16 {
     const float *v;        // [B][K][N]
