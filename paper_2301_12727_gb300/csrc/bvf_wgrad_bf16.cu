@@ -75,17 +75,18 @@ __global__ void __launch_bounds__(256, ITEMS <= 2 ? 4 : 2)
     tc::fence_after();
     const uint32_t tbase = *tslot;
     const uint32_t idesc = tc::idesc_bf16(128, L.CP);
-    // this block's chunks: a run of the batch's, sample by sample
-    const int per = (N + kWgK - 1) / kWgK;
-    const long long all = (long long)per * q.B;
-    const long long begin = all * blockIdx.x / gridDim.x, end = all * (blockIdx.x + 1) / gridDim.x;
-    const int n = (int)(end - begin);
-    int lb = (int)(begin / per), lc = (int)(begin - (long long)lb * per);   // next chunk to load
-    float4 v[ITEMS][2];
+    // this block's chunks: every gridDim.x-th of the batch's, so that the
+    // blocks together read one stretch of each row at a time
+    const int per = (N + kWgK - 1) / kWgK, all = per * q.B;
+    const int n = (int)blockIdx.x < all ? (all - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    int lb = blockIdx.x / per, lc = blockIdx.x - lb * per;                  // next chunk to load
+    constexpr int AHEAD = ITEMS <= 2 ? 2 : 1;
+    float4 v[AHEAD][ITEMS][2];
     float acc[ITEMS];
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) acc[i] = 0.0f;
-    auto load_next = [&]() {
+    auto load_next = [&](float4 (&v)[ITEMS][2]) {
+        if (lb >= q.B) return;
         const float *d = q.d + ((long long)lb * q.O + o0) * N + lc * kWgK;
         const float *x = q.x + (long long)lb * q.C * N + lc * kWgK;
         const int left = N - lc * kWgK;              // a multiple of 4
@@ -99,52 +100,55 @@ __global__ void __launch_bounds__(256, ITEMS <= 2 ? 4 : 2)
                               ? tma::ld_stream(reinterpret_cast<const float4 *>(src + 4 * h))
                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
-        if (++lc == per) {
-            lc = 0;
-            ++lb;
-        }
+        for (lc += gridDim.x; lc >= per; lc -= per) ++lb;
     };
     tma::pdl_wait();
     tma::pdl_launch_next();
-    if (n > 0) load_next();
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u) load_next(v[u]);
     bool gave_up = false;
     int c = 0;
-    for (; c < n; ++c) {
-        const int st = c & 1;
-        unsigned char *sa = sm + st * L.stage, *sb = sa + 128 * 128;
-        // the products that read this stage two chunks ago are done
-        bool ok = true;
-        if (c >= 2)
-            ok = __all_sync(0xffffffffu,
-                            tma::mbar_wait(&bar[st], ((c - 2) >> 1) & 1, tma::kWaitLimit));
-        if (ok) {
+    while (c < n && !gave_up) {
 #pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const int e = tid + 256 * i, r = e >> 3;
-                if (e >= pieces) continue;
-                const float4 a = v[i][0], b = v[i][1];
-                acc[i] += ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
-                unsigned char *dst = r < no ? sa + tc::sw128_off(r, e & 7) : sb + tc::sw128_off(r - no, e & 7);
-                *reinterpret_cast<uint4 *>(dst) =
-                    make_uint4(tc::pack_bf16(a.x, a.y), tc::pack_bf16(a.z, a.w),
-                               tc::pack_bf16(b.x, b.y), tc::pack_bf16(b.z, b.w));
+        for (int u = 0; u < AHEAD; ++u) {
+            if (c >= n) break;
+            const int st = c & 1;
+            unsigned char *sa = sm + st * L.stage, *sb = sa + 128 * 128;
+            // the products that read this stage two chunks ago are done
+            bool ok = true;
+            if (c >= 2)
+                ok = __all_sync(0xffffffffu,
+                                tma::mbar_wait(&bar[st], ((c - 2) >> 1) & 1, tma::kWaitLimit));
+            if (ok) {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    const int e = tid + 256 * i, r = e >> 3;
+                    if (e >= pieces) continue;
+                    const float4 a = v[u][i][0], b = v[u][i][1];
+                    acc[i] += ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
+                    unsigned char *dst = r < no ? sa + tc::sw128_off(r, e & 7) : sb + tc::sw128_off(r - no, e & 7);
+                    *reinterpret_cast<uint4 *>(dst) =
+                        make_uint4(tc::pack_bf16(a.x, a.y), tc::pack_bf16(a.z, a.w),
+                                   tc::pack_bf16(b.x, b.y), tc::pack_bf16(b.z, b.w));
+                }
             }
-        }
-        if (c + 1 < n) load_next();
-        tma::fence_async_smem();
-        tc::fence_before();
-        if (__syncthreads_or(!ok)) {
-            gave_up = true;
-            break;
-        }
-        if (tid == 0) {
-            tc::fence_after();
+            load_next(v[u]);
+            tma::fence_async_smem();
+            tc::fence_before();
+            if (__syncthreads_or(!ok)) {
+                gave_up = true;
+                break;
+            }
+            if (tid == 0) {
+                tc::fence_after();
 #pragma unroll
-            for (int ks = 0; ks < kWgK / 16; ++ks)
-                tc::mma_f16(tbase, tc::smem_desc_sw(sa + 32 * ks, 1024, tc::kSwizzle128),
-                            tc::smem_desc_sw(sb + 32 * ks, 1024, tc::kSwizzle128), idesc,
-                            c > 0 || ks > 0);
-            tc::commit(&bar[st]);
+                for (int ks = 0; ks < kWgK / 16; ++ks)
+                    tc::mma_f16(tbase, tc::smem_desc_sw(sa + 32 * ks, 1024, tc::kSwizzle128),
+                                tc::smem_desc_sw(sb + 32 * ks, 1024, tc::kSwizzle128), idesc,
+                                c > 0 || ks > 0);
+                tc::commit(&bar[st]);
+            }
+            ++c;
         }
     }
     // the last commit covers every earlier product
@@ -158,14 +162,27 @@ __global__ void __launch_bounds__(256, ITEMS <= 2 ? 4 : 2)
         if (tid == 0) atomicOr(q.flag, 2);
     } else if (c > 0) {
         const int o = 32 * (warp & 3) + lane;
+        // four columns an addition where rows of G start on 16 bytes
+        const bool vec = q.C % 4 == 0 && (reinterpret_cast<uintptr_t>(q.G) & 15) == 0;
         for (int k0 = 16 * (warp >> 2); k0 < L.CP; k0 += 32) {
             float r[16];
             tc::ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)k0, r);
             tc::wait_ld();
             if (o < no) {
 #pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    if (k0 + k < q.C) atomicAdd(q.G + (long long)(o0 + o) * q.C + k0 + k, r[k]);
+                for (int k = 0; k < 16; k += 4) {
+                    float *at = q.G + (long long)(o0 + o) * q.C + k0 + k;
+                    if (vec) {
+                        if (k0 + k < q.C)
+                            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at),
+                                         "f"(r[k]), "f"(r[k + 1]), "f"(r[k + 2]), "f"(r[k + 3])
+                                         : "memory");
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            if (k0 + k + h < q.C) atomicAdd(at + h, r[k + h]);
+                    }
+                }
             }
             __syncwarp();
         }
