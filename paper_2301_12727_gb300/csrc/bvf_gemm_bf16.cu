@@ -59,11 +59,12 @@ using tc::pack_bf16;
 // so the global reads are coalesced in both layouts.  vec: the pieces load
 // as two float4 (aligned rows, four-element groups never straddle K or a part
 // of it); four pieces are in flight per thread, against eight floats of one:
-// the staging is bound by the latency of its loads.
+// the staging is bound by the latency of its loads.  own: the row a thread
+// takes of a 128-row tile where k is not contiguous.
 template <class Start, class Kof>
 __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *src,
                                            Start start, Kof kof, bool kc, bool vec, int rows,
-                                           int valid, int k0, int K, int tid)
+                                           int valid, int k0, int K, int tid, int own)
 {
     const int segs = rows * GSEG;
     if (vec) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ void stage_tile(unsigned char *dst, const float *src,
             r = s / GSEG;
             k8 = (s % GSEG) * 8;
         } else {
-            r = s % rows;
+            r = rows == 128 ? own : s % rows;
             k8 = (s / rows) * 8;
         }
         float v[8];
@@ -142,6 +143,17 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
                           : (long long)r * g.sam;
         s_cr[tid] = gx.rc ? (r / gx.rc) * gx.scm1 + (r % gx.rc) * g.scm : (long long)r * g.scm;
     }
+    // Where rows ra apart are neighbours in memory (the inverse y transform: kx
+    // runs fastest through the rows, z through A) the threads take the tile's
+    // rows in A's order, so a warp's loads touch 4 lines instead of 32: at 64 x
+    // 64 x 96, batch 4, that product took 104 us, at 240 x 240 x 200 192 us; with
+    // that and the plain stores below 46 and 114.
+    int own = tid;
+    if (gx.ra > 0 && gx.ra < 128 && gx.sam1 == 1 && g.sam != 1) {
+        const int q = 128 / gx.ra, rem = 128 % gx.ra, big = rem * (q + 1);
+        const int t = tid - big;
+        own = tid < big ? tid / (q + 1) + (tid % (q + 1)) * gx.ra : rem + t / q + (t % q) * gx.ra;
+    }
     auto a_row = [&](int r) { return s_ar[r]; };
     auto a_col = [&](int k) -> long long {
         return gx.ka ? (k < gx.ka ? k * g.sak : gx.sak1 + (k - gx.ka) * g.sak) : k * g.sak;
@@ -177,8 +189,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
                 break;
             }
         }
-        stage_tile(sa, A, a_row, a_col, g.sak == 1, gx.vec & 1, 128, va, c * GK, g.K, tid);
-        stage_tile(sb, B, b_row, b_col, g.sbk == 1, gx.vec & 2, BN, vb, c * GK, g.K, tid);
+        stage_tile(sa, A, a_row, a_col, g.sak == 1, gx.vec & 1, 128, va, c * GK, g.K, tid, own);
+        stage_tile(sb, B, b_row, b_col, g.sbk == 1, gx.vec & 2, BN, vb, c * GK, g.K, tid, tid);
         tma::fence_async_smem();
         tc::fence_before();
         __syncthreads();
@@ -235,10 +247,16 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
         // consecutive columns of one row; otherwise (rows contiguous) it
         // stores straight from the accumulator row.
         const bool by_rows = g.scn == 1 && g.ksplit == 1;
+        // A plain product is stored without the choices of finish(): 32 copies of
+        // those do not fit the instruction cache (4.6 of 12 cycles between a
+        // warp's instructions in the inverse y product were spent on it).
+        const bool plain = g.alpha == 1.0f && g.ksplit == 1 && g.beta == 0.0f && g.bias_mode == 0 &&
+                           g.act == 0;
         float *wbuf = reinterpret_cast<float *>(sm) + warp * (32 * 33);
         const int m = m0 + warp * 32 + lane;
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 32) {
+            __syncwarp();                   // the tensor-memory load is warp-wide
             float r[32];
             if (nc > 0) {
                 tc::ld32(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
@@ -253,10 +271,30 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(const __grid_constant__ GemmX
                 for (int i = 0; i < 32; ++i) wbuf[lane * 33 + i] = r[i];
                 __syncwarp();
                 const int n = n0 + c0 + lane;
+                if (plain) {
+                    float *cp = g.C + (long long)b * g.scb +
+                                (gx.nc && n >= gx.nc ? gx.scn1 + (n - gx.nc) : n);
+                    if (n < g.N)
 #pragma unroll 4
+                        for (int i = 0; i < min(32, g.M - m0 - warp * 32); ++i)
+                            cp[s_cr[warp * 32 + i]] = wbuf[i * 33 + lane];
+                    continue;
+                }
+#pragma unroll 1
                 for (int i = 0; i < 32; ++i) {
                     const int mm = m0 + warp * 32 + i;
                     if (mm < g.M && n < g.N) finish(mm, n, wbuf[i * 33 + lane]);
+                }
+            } else if (plain) {
+                if (m >= g.M) continue;
+                int n = n0 + c0;
+                float *cp = g.C + (long long)b * g.scb + s_cr[m - m0];
+                float *at = cp + (gx.nc && n >= gx.nc ? gx.scn1 + (n - gx.nc) * g.scn : n * g.scn);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    if (n < g.N) *at = r[i];
+                    ++n;
+                    at = gx.nc && n == gx.nc ? cp + gx.scn1 : at + g.scn;
                 }
             } else {
                 if (m >= g.M) continue;

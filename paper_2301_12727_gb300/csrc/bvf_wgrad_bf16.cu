@@ -5,15 +5,17 @@
 //
 // A contraction over millions of points into a few small tiles, so bound by
 // reading d and x once (402 MB, 59 us at 6.8 TB/s, for 32 x 32 channels at 64 x
-// 64 x 96, batch 4).  Blocks take runs of 64-point chunks over the whole batch;
-// a chunk's rows (o of d, then c of x) are loaded a chunk ahead, 32 bytes a
-// thread and row piece, summed for the bias, rounded to BF16 and written to one
-// of two swizzled stages, and only rows that exist are staged: the rows up to
-// the product's 128 stay zero from the start.  The accumulator stays in tensor
+// 64 x 96, batch 4).  Blocks take 64-point chunks of the whole batch in turn, so
+// that together they read one stretch of each row at a time; a chunk's rows (o
+// of d, then c of x) are loaded one or two chunks ahead, 32 bytes a thread and
+// row piece, summed for the bias, rounded to BF16 and written to one of two
+// swizzled stages, and only rows that exist are staged: the rows up to the
+// product's 128 stay zero from the start.  The accumulator stays in tensor
 // memory until the block's last chunk and is then added to G.
 // As general products (one 128-row tile staged per chunk with its zero rows,
 // loads waited for chunk by chunk) and separate sums the layer's pair took 212
-// and 35 us, the hidden layer's 264 and 113; now 155 and 158.
+// and 35 us, the hidden layer's 264 and 113; now 75 and 139 (155 and 158 with a
+// run of chunks per block, one chunk ahead, and G added to value by value).
 //
 // Waits are bounded as in the other tensor-core kernels.
 #include <cuda_bf16.h>

@@ -37,3 +37,20 @@ def test_matches_oracle(nx, ny, nz, m, bf16):
         assert np.linalg.norm(got - ref) <= 3e-2 * np.linalg.norm(ref)
     else:
         assert np.abs(got - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
+def test_long_rows_of_a_wide_layer():
+    """Width 64, 16 modes, rows of 300: the layer output holds one x tile's
+    table and so takes rows that a table for the whole row did not fit."""
+    torch = pytest.importorskip("torch")
+    from oracle import fno as ofno
+    from paper_2301_12727_gb300 import fno, synth
+    dims = dict(c_in=3, width=64, modes=16, n_layers=2, hidden=24, c_out=1)
+    w = synth.fno_weights(dims, 5)
+    a = synth.fno_inputs(3, 300, 32, 33, 6)
+    net = fno.Surrogate(dims, w)
+    got = net(torch.from_numpy(a).cuda()).cpu().numpy()
+    net.synchronize()
+    net.close()
+    ref = ofno.forward(a.astype(np.float64), w.astype(np.float64), **dims)
+    assert np.abs(got - ref).max() <= 2e-5 * np.abs(ref).max()
