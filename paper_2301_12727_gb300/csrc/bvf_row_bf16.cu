@@ -515,8 +515,8 @@ __global__ void __launch_bounds__(256, 3)
 // and their backward products when their activations are kept.  All of K is
 // staged at once (16 channels per thread in flight), the weights once per
 // block.  As separate products of one tile a block the four took 1244, 397,
-// 1244 and 397 us at 64 x 64 x 96, batch 4; now 402, 196, 570 (two special
-// functions for each of 50 million values) and 219.
+// 1244 and 397 us at 64 x 64 x 96, batch 4; now 371, 189, 466 (two special
+// functions for each of 201 million values) and 205.
 struct ChanBLayout {
     int KP, NP, ncols, sA, sB, sb, bar, tmem, bytes;
     __host__ __device__ ChanBLayout(int K, int N)
@@ -579,6 +579,45 @@ __global__ void __launch_bounds__(256, 3) k_chan_bf16(const __grid_constant__ Ch
         for (int c = 0; c < 16; ++c)
             xv[c] = p < N && ch + c < q.K ? tma::ld_stream(src + (long long)c * N) : 0.0f;
     };
+    // ACT: 0 none, 1 GELU (the value kept when asked), 2 times GELU' of the kept one
+    auto epilogue = [&](auto act, int tile) {
+        constexpr int ACT = decltype(act)::value;
+        const int b = tile / per, p = (tile - b * per) * 128 + pt;
+        const bool keep = ACT == 1 && q.pre;
+#pragma unroll 1
+        for (int c0 = 16 * half; c0 < NP; c0 += 32) {
+            const int n = p < N ? min(16, q.O - c0) : 0;
+            const long long at = ((long long)b * q.O + c0) * N + p;
+            float r[16], pv[16];
+            tc::ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, r);
+            if (ACT == 2) {
+                const float *pp = q.pre + at;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    if (i < n) pv[i] = tma::ld_stream(pp);
+                    pp += N;
+                }
+            }
+            tc::wait_ld();
+            float *op = q.out + at, *pp = ACT == 1 ? q.pre + at : nullptr;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                if (i < n) {
+                    float v = q.bias ? __fadd_rn(r[i], sb[c0 + i]) : r[i];
+                    if (ACT == 1) {
+                        if (keep) *pp = v;
+                        v = gelu_exact(v);
+                    } else if (ACT == 2) {
+                        v *= gelu_grad(pv[i]);
+                    }
+                    *op = v;
+                }
+                op += N;
+                if (ACT == 1) pp += N;
+            }
+            __syncwarp();            // the next tensor-memory load is warp-wide
+        }
+    };
     if ((int)blockIdx.x < tiles) load(blockIdx.x, 0);
     int phase = 0;
     bool gave_up = false;
@@ -609,36 +648,12 @@ __global__ void __launch_bounds__(256, 3) k_chan_bf16(const __grid_constant__ Ch
         const bool ready = __all_sync(0xffffffffu, tma::mbar_wait(bar, phase & 1, tma::kWaitLimit));
         tc::fence_after();
         if (ready) {
-            const int b = tile / per, p = (tile - b * per) * 128 + pt;
-            const long long at = (long long)b * q.O * N + p;
-            for (int c0 = 16 * half; c0 < NP; c0 += 32) {
-                float r[16], pv[16];
-                tc::ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, r);
-                if (p < N && q.act == 2) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        pv[i] = c0 + i < q.O ? tma::ld_stream(q.pre + at + (long long)(c0 + i) * N)
-                                             : 0.0f;
-                }
-                tc::wait_ld();
-                if (p < N) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        if (c0 + i >= q.O) break;
-                        const long long o = at + (long long)(c0 + i) * N;
-                        float v = r[i];
-                        if (q.bias) v = __fadd_rn(v, sb[c0 + i]);
-                        if (q.act == 1) {
-                            if (q.pre) q.pre[o] = v;
-                            v = gelu_exact(v);
-                        } else if (q.act == 2) {
-                            v *= gelu_grad(pv[i]);
-                        }
-                        q.out[o] = v;
-                    }
-                }
-                __syncwarp();
-            }
+            if (q.act == 0)
+                epilogue(std::integral_constant<int, 0>{}, tile);
+            else if (q.act == 2)
+                epilogue(std::integral_constant<int, 2>{}, tile);
+            else
+                epilogue(std::integral_constant<int, 1>{}, tile);
         }
         tc::fence_before();
         gave_up = __syncthreads_or(!ready) != 0;
