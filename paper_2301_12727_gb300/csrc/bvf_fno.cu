@@ -12,7 +12,8 @@
 //   - the layer output (inverse x transform, W v + b and GELU) is one
 //     tensor-core product per 128-point tile of a (z, y) row (k_row_tc), and
 //     the next layer's forward x transform is one tall product over all rows
-//     of the new v (k_dftx_tc);
+//     of the new v (k_xfwd of bvf_xfwd.cu, fed by TMA; k_dftx_tc for rows TMA
+//     cannot fetch);
 //   - the lift is the layer output without the spectral term.
 // The projection is a tensor-core product with GELU in its epilogue
 // (k_project_tc).  All three run on the fifth-generation tensor cores

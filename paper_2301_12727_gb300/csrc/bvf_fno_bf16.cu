@@ -1,7 +1,9 @@
 // BF16 path of the surrogate: inference and training of the Fourier neural
 // operator (Li et al., ICLR 2021, Sec. 4; the network of include/bvf_fno.h)
-// with every contraction on the tcgen05 BF16 product of bvf_gemm_bf16.cu
-// (BF16 operands, FP32 accumulation) and FP32 master weights.
+// with every contraction on tcgen05 (BF16 operands, FP32 accumulation; row
+// passes and projection: bvf_row_bf16.cu, forward x transform: bvf_xfwd.cu,
+// weight gradients: bvf_wgrad_bf16.cu, y and z transforms and the general case:
+// bvf_gemm_bf16.cu) and FP32 master weights.
 //
 // Layouts (per sample b, channel c, voxel p = (z ny + y) nx + x):
 //   volumes  [b][c][p];
@@ -21,8 +23,8 @@
 // Backward (gradients of the loss below): the adjoint of the inverse is the
 // forward transform with the weights c(kx)/N, the adjoint of the forward
 // transform is the inverse without them, the mix's adjoints take conj(R);
-// weight gradients are products summed over the batch and the voxels (split
-// K, added atomically), bias gradients channel sums.  GELU's derivative is
+// weight and bias gradients are sums over the batch and the voxels (split,
+// added atomically).  GELU's derivative is
 // applied in the product epilogue from the stored pre-activation.
 //
 // Loss of a batch: the mean over samples of the relative L2 error

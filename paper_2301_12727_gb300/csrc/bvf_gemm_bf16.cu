@@ -1,8 +1,8 @@
 // BF16 tensor-core product on the fifth-generation tensor cores (tcgen05):
 // C = alpha A B + beta C (+ bias) (-> GELU), FP32 in and out, BF16 operands,
-// FP32 accumulation in tensor memory.  Every contraction of the surrogate's
-// BF16 path and of its training (channel mixes, the truncated DFT along each
-// axis and their adjoints) is one call of this kernel on strided views.
+// FP32 accumulation in tensor memory.  The y and z transforms of the surrogate's
+// BF16 path and of its training run on it, and every other contraction where a
+// kernel of its own does not take the shape, as calls on strided views.
 //
 // A block of 128 threads computes a 128 x BN tile of C:
 //   * K runs in chunks of 64; the chunk's A (128 x 64) and B (BN x 64) tiles

@@ -17,8 +17,7 @@
 // between them in HBM.  At 240 x 240 x 200, width 32, a layer took 904 us for
 // the inverse (1.5 GB written) and 2040 us for the mix (1.5 GB read twice
 // over, 1.5 GB written), the projection 6806 + 2151 us around 5.9 GB of
-// hidden activations; now 690 us a layer and 1793 us (the whole
-// forward 28.0 -> 8.5 ms).  Every product keeps its
+// hidden activations; now 690 us a layer and 1793 us.  Every product keeps its
 // operands' rounding and its order of K steps, and the two sums of a layer
 // meet in FP32 in the epilogue as they did through memory, so the results are
 // the separate products' bit for bit.
