@@ -522,12 +522,15 @@ int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *c
  * branches (as bvf_batch_run_streams deals them over streams), recorded once
  * and replayed with a single graph launch on `stream`, so the host issues one
  * launch per sweep and the branches' kernels share the GPU.  The recording is
- * kept and replayed while the call's arguments, the contexts' tiles and
- * the step counts the contexts start from are those it was recorded for
- * (e.g. the same sweep after bvf_reset); anything else records anew, which
- * waits for `stream`.  Results are those of bvf_run_acoustic, bit for bit.
- * Contexts with a time budget, kernel timing or the test hook armed are
- * refused (BVF_E_ARG). */
+ * kept and replayed while the call's arguments, the contexts' tiles, the step
+ * counts they start from, their sources' plane number, speed, envelope and
+ * cycle count and the lengths of their material tables are those it was
+ * recorded for (e.g. the same sweep after bvf_reset, with other values on the
+ * source planes or other materials in tables of the same length); anything
+ * else records anew, which waits for `stream`.  Results are those of
+ * bvf_run_acoustic, bit for bit.  Contexts with a time budget, kernel timing
+ * or the test hook armed, or whose last bvf_set_materials was refused for its
+ * index, are refused (BVF_E_ARG). */
 int bvf_batch_run_graph(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int n_branches,
                         void *stream);
 

@@ -133,8 +133,8 @@ struct bvf_batch {
     std::vector<cudaEvent_t> side_ev;
     cudaEvent_t fork = nullptr;
     // bvf_batch_run_graph: the recorded graph, what it was recorded for (start
-    // steps, step counts, capture windows, z-chunks, branches) and the counter
-    // advances of one replay
+    // steps, step counts, capture windows, tiles, sources, table lengths,
+    // branches) and the counter advances of one replay
     cudaGraphExec_t gexec = nullptr;
     std::vector<long long> gsig;
     std::vector<long long> gdsteps, gddft;
@@ -1796,9 +1796,18 @@ int bvf_batch_run_graph(bvf_batch *b, const int *n_steps, const bvf_capture *cap
         if (c->budget_s > 0.0 || c->timing || c->hold)
             return fail(nullptr, BVF_E_ARG, "bvf_batch_run_graph: a context has a time budget, "
                                             "kernel timing or the test hook armed");
+        if (!c->have_materials)
+            return fail(nullptr, BVF_E_ARG, "bvf_batch_run_graph: a context has no valid materials");
         const bvf_capture cp = caps ? caps[d] : bvf_capture{-1, 0, 0};
+        // everything a recorded launch holds by value (make_params, step_param
+        // and the shared memory of n_mat materials); what it reads through the
+        // context's buffers may change under it
+        long long c0_bits = 0;
+        std::memcpy(&c0_bits, &c->c0, sizeof c0_bits);
         sig.insert(sig.end(), {c->steps, n_steps[d], cp.peak_from, cp.dft_start, cp.dft_steps,
-                               c->kchunk, c->tile.stress_rows, c->tile.velocity_rows});
+                               c->kchunk, c->tile.stress_rows, c->tile.velocity_rows,
+                               (long long)c->table.size(), c->have_source});
+        if (c->have_source) sig.insert(sig.end(), {c->k_src, c0_bits, c->envelope, c->n_cycles});
     }
     if (!b->gexec || sig != b->gsig) {
         // record the per-domain launches once, domains dealt round-robin over
