@@ -494,7 +494,7 @@ int bvf_plan_host(bvf_ctx *skull, bvf_ctx *water, const uint8_t *h_index,
  * bvf_batch_create: the contexts stay owned by the caller and must outlive
  * the batch; each needs its materials set, nx % 8 == 0 and at most 2 SLS
  * mechanisms, and all share the SLS count and storage type (BVF_E_ARG
- * otherwise).  Sources are taken from the contexts at each run. */
+ * otherwise).  Sources and materials are taken from the contexts at each run. */
 typedef struct bvf_batch bvf_batch;
 int bvf_batch_create(bvf_ctx *const *ctxs, int n, bvf_batch **out);
 void bvf_batch_destroy(bvf_batch *b);
@@ -505,7 +505,8 @@ void bvf_batch_destroy(bvf_batch *b);
  * (0: each context's default).  graph_steps > 0 captures that many steps in
  * a CUDA graph and replays it (launch overhead of one graph per graph_steps
  * steps); 0 launches the kernels directly.  Asynchronous on `stream`;
- * bvf_synchronize on each context reports its errors. */
+ * bvf_synchronize on each context reports its errors.  A context whose last
+ * bvf_set_materials was refused for its index is refused (BVF_E_ARG). */
 int bvf_batch_run(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int kchunk,
                   int graph_steps, void *stream);
 

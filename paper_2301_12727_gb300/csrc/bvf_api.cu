@@ -116,7 +116,8 @@ struct bvf_ctx {
 
 struct bvf_batch {
     std::vector<bvf_ctx *> ctx;       // not owned
-    int L = 0, h16 = 0, n_mat_max = 1;
+    int L = 0, h16 = 0;
+    int n_mat_max = 1;                // longest material table the grids below are for
     int grid_vel = 0, grid_str = 0;   // persistent grid sizes
     StressTmaMaps *d_sm = nullptr;    // [ctx.size()]
     VelocityTmaMaps *d_vm = nullptr;
@@ -1616,8 +1617,11 @@ int bvf_batch_run(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int
     const int n = (int)b->ctx.size();
     cudaStream_t s = (cudaStream_t)stream;
     long long total_steps = 0;
-    int n_max = 0;
+    int n_max = 0, n_mat_max = 1;
     for (int d = 0; d < n; ++d) {
+        if (!b->ctx[d]->have_materials)
+            return fail(nullptr, BVF_E_ARG, "bvf_batch_run: a context has no valid materials");
+        n_mat_max = std::max(n_mat_max, (int)b->ctx[d]->table.size());
         if (n_steps[d] < 0) return fail(nullptr, BVF_E_ARG, "bvf_batch_run: negative step count");
         if (caps && caps[d].dft_steps < 0)
             return fail(nullptr, BVF_E_ARG, "bvf_batch_run: negative dft_steps");
@@ -1625,6 +1629,12 @@ int bvf_batch_run(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int
         n_max = std::max(n_max, n_steps[d]);
     }
     if (kchunk < 0) return fail(nullptr, BVF_E_ARG, "bvf_batch_run: negative kchunk");
+    // the launches' shared memory holds the longest table the contexts have now
+    if (n_mat_max != b->n_mat_max) {
+        CK_FREE(batch_prepare(b->L, b->h16, n_mat_max, &b->grid_vel, &b->grid_str),
+                "bvf_batch_run: table length");
+        b->n_mat_max = n_mat_max;
+    }
     // device buffers: tensor maps and per-step tables
     if (b->steps_cap < (size_t)std::max<long long>(total_steps, 1)) {
         if (b->d_steps) cudaFree(b->d_steps);
