@@ -1407,11 +1407,14 @@ template <int L, typename T>
 static cudaError_t batch_prepare_t(int n_mat_max, int *gv, int *gs)
 {
     const size_t smv = VelLayout<T>::bytes(n_mat_max), sms = StressLayout<L, T>::bytes(n_mat_max);
-    cudaError_t e = cudaFuncSetAttribute(k_velocity_batch<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smv);
+    // the limits belong to the kernels, not to a batch: one value for every
+    // table length
+    const auto limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_velocity_batch<T>, limit,
+                                         (int)VelLayout<T>::bytes(BVF_MAX_MATERIALS));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_stress_batch<L, 4, T>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms);
+        e = cudaFuncSetAttribute(k_stress_batch<L, 4, T>, limit,
+                                 (int)StressLayout<L, T>::bytes(BVF_MAX_MATERIALS));
     int dev = 0, sm_count = 0, bv = 0, bs = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);

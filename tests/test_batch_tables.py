@@ -45,6 +45,31 @@ def test_shared_memory_follows_the_tables(tmp_path):
     host_cuda.run(HOST, tmp_path)
 
 
+LIMITS = r"""
+# 240 rows need more than the 48 KB every kernel may use: a batch of short
+# tables made afterwards leaves the long one's launches as they were
+NX, NY, NZ = 32, 16, 16
+steps = (ctypes.c_int * 1)(2)
+
+def batch(rows):
+    c = context(NX, NY, NZ, [WATER] * rows)
+    b = ctypes.c_void_p()
+    assert L.bvf_batch_create((ctypes.c_void_p * 1)(c), 1, ctypes.byref(b)) == OK
+    return b
+
+long = batch(240)
+assert L.bvf_batch_run(long, steps, None, 0, 0, None) == OK
+assert max(s for n, s in launched()) > 48 * 1024
+short = batch(2)
+for b in (short, long, short):
+    assert L.bvf_batch_run(b, steps, None, 0, 0, None) == OK, L.bvf_last_error(None)
+"""
+
+
+def test_a_batch_of_short_tables_leaves_the_limit_of_a_long_one(tmp_path):
+    host_cuda.run(LIMITS, tmp_path)
+
+
 @pytest.mark.gpu
 def test_gpu_longer_table_after_the_batch_was_made():
     """96 rows set after the batch was made from 2: the sweep equals
