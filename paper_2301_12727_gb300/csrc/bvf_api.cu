@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <vector>
@@ -152,6 +153,8 @@ int fail(bvf_ctx *c, int code, const std::string &msg)
 
 int cuda_fail(bvf_ctx *c, cudaError_t e, const char *where)
 {
+    // reported here: the next call's launches must not find it pending
+    (void)cudaGetLastError();
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
     return fail(c, e == cudaErrorMemoryAllocation ? BVF_E_NOMEM : BVF_E_CUDA, m);
 }
@@ -168,6 +171,34 @@ int cuda_fail(bvf_ctx *c, cudaError_t e, const char *where)
         cudaError_t e_ = (call);                             \
         if (e_ != cudaSuccess) return cuda_fail(c, e_, where); \
     } while (0)
+
+// Buffers made on first use: a call makes those of a group that are missing,
+// or, when one fails, gives back what it made, so that a later call finds the
+// whole group or none of it.  *made: whether this call made any.
+struct Buffer {
+    void **p;
+    size_t bytes;
+};
+cudaError_t make_group(std::initializer_list<Buffer> group, bool *made)
+{
+    std::vector<void **> mine;
+    cudaError_t e = cudaSuccess;
+    for (const Buffer &b : group) {
+        if (*b.p) continue;
+        if ((e = cudaMalloc(b.p, b.bytes)) != cudaSuccess) {
+            *b.p = nullptr;
+            break;
+        }
+        mine.push_back(b.p);
+    }
+    if (e != cudaSuccess)
+        for (void **p : mine) {
+            cudaFree(*p);
+            *p = nullptr;
+        }
+    *made = e == cudaSuccess && !mine.empty();
+    return e;
+}
 
 // Relaxation times 1 / (2 pi f_l), f_l log-spaced on [f0/3, 3 f0] (f0 if L = 1).
 std::vector<double> relaxation_times(double f0, int L)
@@ -479,11 +510,12 @@ StepParam step_param(const bvf_ctx *c, const bvf_capture &cp, long long n)
 // FP64 DFT sums of a context, allocated and zeroed on first use
 int ensure_dft(bvf_ctx *c, cudaStream_t s)
 {
-    if (c->dftC) return BVF_OK;
-    CK(cudaMalloc(&c->dftC, c->NP * sizeof(double)), "dft buffers");
-    CK(cudaMalloc(&c->dftS, c->NP * sizeof(double)), "dft buffers");
-    CK(cudaMemsetAsync(c->dftC, 0, c->NP * sizeof(double), s), "dft buffers");
-    CK(cudaMemsetAsync(c->dftS, 0, c->NP * sizeof(double), s), "dft buffers");
+    const size_t bytes = c->NP * sizeof(double);
+    bool made = false;
+    CK(make_group({{(void **)&c->dftC, bytes}, {(void **)&c->dftS, bytes}}, &made), "dft buffers");
+    if (!made) return BVF_OK;
+    CK(cudaMemsetAsync(c->dftC, 0, bytes, s), "dft buffers");
+    CK(cudaMemsetAsync(c->dftS, 0, bytes, s), "dft buffers");
     return BVF_OK;
 }
 
@@ -1092,23 +1124,25 @@ int bvf_run_thermal(bvf_ctx *c, const bvf_thermal *th, const double *d_amp, floa
     if (th->dt > dt_lim)
         return fail(c, BVF_E_ARG, "bvf_run_thermal: dt above the explicit stability limit");
     cudaStream_t s = (cudaStream_t)stream;
-    if (!c->T2) {
-        CK(cudaMalloc(&c->T2, c->N * sizeof(float)), "thermal buffers");
-        CK(cudaMalloc(&c->Q, c->N * sizeof(float)), "thermal buffers");
-        CK(cudaMalloc(&c->cemf, c->N * sizeof(float)), "thermal buffers");
-        CK(cudaMalloc(&c->q_bad, sizeof(int)), "thermal buffers");
-        CK(cudaMalloc(&c->tlut, BVF_MAX_MATERIALS * sizeof(ThermCoef)), "thermal buffers");
-        CK(cudaMalloc(&c->kface, (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float)),
-           "thermal buffers");
-    }
+    const size_t vol = c->N * sizeof(float);
+    bool made = false;
+    CK(make_group({{(void **)&c->T2, vol},
+                   {(void **)&c->Q, vol},
+                   {(void **)&c->cemf, vol},
+                   {(void **)&c->q_bad, sizeof(int)},
+                   {(void **)&c->tlut, BVF_MAX_MATERIALS * sizeof(ThermCoef)},
+                   {(void **)&c->kface,
+                    (size_t)BVF_MAX_MATERIALS * BVF_MAX_MATERIALS * sizeof(float)}},
+                  &made),
+       "thermal buffers");
     // TMA-fed steps where the rows are whole multiples of 16 bytes and both
     // temperature buffers can be mapped (BVF_NO_TMA forces the direct kernel)
     const bool want_tma = c->g.nx % 8 == 0 && !std::getenv("BVF_NO_TMA");
-    if (want_tma && !c->cls) {
+    if (want_tma) {
         const size_t bytes = c->index_pitch * c->g.ny * c->g.nz;
-        CK(cudaMalloc(&c->cls_of, BVF_MAX_MATERIALS), "thermal buffers");
-        CK(cudaMalloc(&c->cls, bytes), "thermal buffers");
-        CK(cudaMemsetAsync(c->cls, 0, bytes, s), "thermal buffers");
+        CK(make_group({{(void **)&c->cls_of, BVF_MAX_MATERIALS}, {(void **)&c->cls, bytes}}, &made),
+           "thermal buffers");
+        if (made) CK(cudaMemsetAsync(c->cls, 0, bytes, s), "thermal buffers");
     }
     ThermTmaMaps tmaps[2];
     bool th_tma = false;
@@ -1247,14 +1281,15 @@ int bvf_plan_host(bvf_ctx *skull, bvf_ctx *water, const uint8_t *h_index,
         return fail(skull, BVF_E_ARG, "bvf_plan_host: NULL argument");
     bvf_ctx *c = skull;
     const size_t N = c->N;
-    if (!c->h_index_d) {
-        CK(cudaMalloc(&c->h_index_d, N), "bvf_plan_host: staging");
-        CK(cudaMalloc(&c->h_peak_d, N * sizeof(float)), "bvf_plan_host: staging");
-        CK(cudaMalloc(&c->h_T_d, N * sizeof(float)), "bvf_plan_host: staging");
-        CK(cudaMalloc(&c->h_Tmax_d, N * sizeof(float)), "bvf_plan_host: staging");
-        CK(cudaMalloc(&c->h_amp_d, N * sizeof(double)), "bvf_plan_host: staging");
-        CK(cudaMalloc(&c->h_cem_d, N * sizeof(double)), "bvf_plan_host: staging");
-    }
+    bool made = false;
+    CK(make_group({{(void **)&c->h_index_d, N},
+                   {(void **)&c->h_peak_d, N * sizeof(float)},
+                   {(void **)&c->h_T_d, N * sizeof(float)},
+                   {(void **)&c->h_Tmax_d, N * sizeof(float)},
+                   {(void **)&c->h_amp_d, N * sizeof(double)},
+                   {(void **)&c->h_cem_d, N * sizeof(double)}},
+                  &made),
+       "bvf_plan_host: staging");
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaMemcpyAsync(c->h_index_d, h_index, N, cudaMemcpyHostToDevice, s), "bvf_plan_host: index in");
     const int rc = bvf_plan(skull, water, c->h_index_d, h_table, n_mat, h_water, bowl, k_src, pp,

@@ -1,0 +1,74 @@
+"""A device allocation that fails leaves a context that can go on: the call
+that needed it returns BVF_E_NOMEM, and the same call made again allocates
+what is missing and does all of its work, for every allocation of every call
+that makes buffers on first use."""
+from tests import host_cuda
+
+ACOUSTIC = r"""
+NX, NY, NZ = 32, 16, 16
+N = NX * NY * NZ
+cap = bvf.Capture(0, 1, 4)
+th = bvf.Thermal(1e-3, 3, 2, 0.3, 37.0, 2.2e6, 1.0)
+calls = {}
+
+def dft(c):
+    return lambda: L.bvf_run_acoustic(c, 2, ctypes.byref(cap), None)
+
+def thermal(c):
+    d = [buf(4 * N), buf(4 * N), buf(8 * N)]
+    return lambda: L.bvf_run_thermal(c, ctypes.byref(th), buf(8 * N), *d, None)
+
+def load(c):
+    # a snapshot with DFT sums, loaded into a context that has none yet
+    n = ctypes.c_size_t()
+    assert L.bvf_state_bytes(c, ctypes.byref(n)) == OK
+    full = context(NX, NY, NZ, [WATER])
+    assert dft(full)() == OK
+    snap = buf(n.value)
+    assert L.bvf_state_save(full, snap, n, None) == OK
+    return lambda: L.bvf_state_load(c, snap, n, None)
+
+def plan_host(c):
+    water = context(NX, NY, NZ, [WATER])
+    bowl = bvf.Bowl(8e-3, 9e-3, (ctypes.c_double * 3)(8e-3, 4e-3, -2e-2),
+                    (ctypes.c_double * 3)(0, 0, 1), 1e5, 1500.0, 0.25)
+    pp = bvf.PlanParams(4, 1, 3, 0.0, th, 0)
+    out = bvf.PlanOut()
+    h = [buf(N), buf(4 * N), buf(4 * N), buf(4 * N), buf(8 * N)]
+    mat = bvf.material_array([WATER])
+    # without kernels the water field is zero, which the plan refuses at its
+    # end: the work up to there is what counts
+    def call():
+        rc = L.bvf_plan_host(c, water, h[0], mat, 1, mat, ctypes.byref(bowl), 2, ctypes.byref(pp),
+                             h[1], h[2], h[3], h[4], ctypes.byref(out), None)
+        return OK if rc == ARG and b"zero water intensity" in L.bvf_last_error(None) else rc
+    return call
+
+for make in (dft, thermal, load, plan_host):
+    # what the call launches and allocates with nothing failing
+    c = context(NX, NY, NZ, [WATER])
+    call = make(c)
+    launched()
+    before = fake.fake_mallocs()
+    assert call() == OK, (make.__name__, L.bvf_last_error(None))
+    want, n = launched(), fake.fake_mallocs() - before
+    assert n > 1
+    L.bvf_destroy(c)
+    for k in range(1, n + 1):
+        c = context(NX, NY, NZ, [WATER])
+        call = make(c)
+        fake.fake_fail_malloc(k)
+        assert call() == NOMEM, (make.__name__, k)
+        launched()
+        before = fake.fake_mallocs()
+        assert call() == OK, (make.__name__, k, L.bvf_last_error(None))
+        assert launched() == want, (make.__name__, k)
+        assert fake.fake_mallocs() > before, (make.__name__, k)
+        # reset walks over the lazily made buffers
+        assert L.bvf_reset(c, None) == OK
+        L.bvf_destroy(c)
+"""
+
+
+def test_calls_after_a_failed_allocation(tmp_path):
+    host_cuda.run(ACOUSTIC, tmp_path)
