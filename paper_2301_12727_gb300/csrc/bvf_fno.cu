@@ -47,6 +47,8 @@ int fno_fail(int code, const std::string &msg)
 
 int fno_cuda(cudaError_t e, const char *where)
 {
+    // reported here: the next call's launches must not find it pending
+    (void)cudaGetLastError();
     std::string m = std::string(where) + ": " + cudaGetErrorString(e);
     return fno_fail(e == cudaErrorMemoryAllocation ? BVF_E_NOMEM : BVF_E_CUDA, m);
 }
@@ -1394,6 +1396,9 @@ int prepare_grid(bvf_fno *f, int nx, int ny, int nz)
     int rc;
     // buffers of an earlier grid may still be in use on some stream
     FCK(cudaDeviceSynchronize(), "bvf_fno_forward: sync before a grid change");
+    // no grid until all of it is there: a failed allocation below leaves some
+    // buffers released
+    f->nx = f->ny = f->nz = 0;
     if ((size_t)W * N > f->v_cap) {
         cudaFree(f->v0);
         cudaFree(f->v1);

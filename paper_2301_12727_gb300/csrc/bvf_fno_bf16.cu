@@ -60,12 +60,18 @@ int b16_fail(int code, const std::string &msg)
     return code;
 }
 
-#define BCK(call, where)                                                           \
-    do {                                                                           \
-        cudaError_t e_ = (call);                                                   \
-        if (e_ != cudaSuccess)                                                     \
-            return b16_fail(e_ == cudaErrorMemoryAllocation ? BVF_E_NOMEM : BVF_E_CUDA, \
-                            std::string(where) + ": " + cudaGetErrorString(e_));   \
+int b16_cuda(cudaError_t e, const std::string &where)
+{
+    // reported here: the next call's launches must not find it pending
+    (void)cudaGetLastError();
+    return b16_fail(e == cudaErrorMemoryAllocation ? BVF_E_NOMEM : BVF_E_CUDA,
+                    where + ": " + cudaGetErrorString(e));
+}
+
+#define BCK(call, where)                                   \
+    do {                                                   \
+        cudaError_t e_ = (call);                           \
+        if (e_ != cudaSuccess) return b16_cuda(e_, where); \
     } while (0)
 
 __host__ __device__ __forceinline__ int slot_freq(int j, int m) { return j < m ? j : j - 2 * m; }
@@ -507,7 +513,10 @@ template <typename P>
 int dalloc(bvf_fno_bf16 *t, P **p, size_t n, const char *what)
 {
     cudaError_t e = cudaMalloc((void **)p, n * sizeof(P));
-    if (e != cudaSuccess) return b16_fail(BVF_E_NOMEM, std::string("bvf_fno_bf16_create: ") + what);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return b16_fail(BVF_E_NOMEM, std::string("bvf_fno_bf16_create: ") + what);
+    }
     t->all.push_back(*p);
     return BVF_OK;
 }

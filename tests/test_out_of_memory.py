@@ -72,3 +72,55 @@ for make in (dft, thermal, load, plan_host):
 
 def test_calls_after_a_failed_allocation(tmp_path):
     host_cuda.run(ACOUSTIC, tmp_path)
+
+
+SURROGATE = r"""
+F = fno.lib()
+dims = fno.FnoDims(3, 16, 4, 2, 16, 1)
+n_w = F.bvf_fno_weight_count(ctypes.byref(dims))
+w = (ctypes.c_float * n_w)()
+
+def net():
+    f = ctypes.c_void_p()
+    assert F.bvf_fno_create(ctypes.byref(f), ctypes.byref(dims), w, n_w) == OK
+    return f
+
+def forward(f, nx, ny, nz):
+    n = 4 * nx * ny * nz
+    return F.bvf_fno_forward(f, nx, ny, nz, buf(3 * n), buf(n), None)
+
+small, large = (16, 12, 10), (32, 24, 20)
+f = net()
+launched()
+assert forward(f, *small) == OK
+want, before = launched(), fake.fake_mallocs()
+assert forward(f, *large) == OK
+n = fake.fake_mallocs() - before
+assert n > 4
+for k in range(1, n + 1):
+    f = net()
+    assert forward(f, *small) == OK
+    fake.fake_fail_malloc(k)
+    assert forward(f, *large) == NOMEM, k
+    # back on the grid it had: whatever the failed call gave up is made again
+    launched()
+    before = fake.fake_mallocs()
+    assert forward(f, *small) == OK, (k, L.bvf_last_error(None))
+    assert launched() == want and fake.fake_mallocs() > before, k
+    assert forward(f, *large) == OK
+    F.bvf_fno_destroy(f)
+
+# the BF16 network: a failed creation leaves no error behind for the next one
+for k in (1, 5, 20):
+    t = ctypes.c_void_p()
+    fake.fake_fail_malloc(k)
+    assert F.bvf_fno_bf16_create(ctypes.byref(t), ctypes.byref(dims), w, n_w, 16, 12, 10, 1) == NOMEM
+    assert not t.value
+    assert F.bvf_fno_bf16_create(ctypes.byref(t), ctypes.byref(dims), w, n_w, 16, 12, 10, 1) == OK
+    assert F.bvf_fno_bf16_forward(t, 1, buf(12 * 1920), buf(4 * 1920), None) == OK, L.bvf_last_error(None)
+    F.bvf_fno_bf16_destroy(t)
+"""
+
+
+def test_surrogate_after_a_failed_grid_change(tmp_path):
+    host_cuda.run(SURROGATE, tmp_path)
