@@ -1530,12 +1530,11 @@ int bvf_plan(bvf_ctx *skull, bvf_ctx *water, const uint8_t *d_index, const bvf_m
     // source plane exists and joined before the reductions (serial: `stream`)
     void *ws = stream;
     if (!pp->serial) {
-        if (!skull->side) {
-            e = cudaStreamCreateWithFlags(&skull->side, cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&skull->fork_ev, cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&skull->join_ev, cudaEventDisableTiming);
-            if (e != cudaSuccess) return done(cuda_fail(nullptr, e, "bvf_plan: second stream"));
-        }
+        // each by itself: a call after a failed one makes what is missing
+        if (!skull->side) e = cudaStreamCreateWithFlags(&skull->side, cudaStreamNonBlocking);
+        for (cudaEvent_t *ev : {&skull->fork_ev, &skull->join_ev})
+            if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return done(cuda_fail(nullptr, e, "bvf_plan: second stream"));
         e = cudaEventRecord(skull->fork_ev, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(skull->side, skull->fork_ev, 0);
         if (e != cudaSuccess) return done(cuda_fail(nullptr, e, "bvf_plan: fork"));
@@ -1774,6 +1773,26 @@ static int run_beside(bvf_batch *b, int d, int n_steps, const bvf_capture *caps,
     return rc;
 }
 
+// side streams and events of the batch, at least n of each and as many events
+// as streams
+static int batch_side_streams(bvf_batch *b, int n)
+{
+    while ((int)b->side.size() < n) {
+        cudaStream_t t = nullptr;
+        cudaEvent_t ev = nullptr;
+        CK_FREE(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking), "batch streams");
+        const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
+            cudaStreamDestroy(t);
+            return cuda_fail(nullptr, e, "batch streams");
+        }
+        b->side.push_back(t);
+        b->side_ev.push_back(ev);
+    }
+    if (!b->fork) CK_FREE(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "batch streams");
+    return BVF_OK;
+}
+
 int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *caps,
                           int n_streams, void *stream)
 {
@@ -1783,15 +1802,8 @@ int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *c
     for (int d = 0; d < n; ++d)
         if (n_steps[d] < 0) return fail(nullptr, BVF_E_ARG, "bvf_batch_run_streams: negative step count");
     cudaStream_t s = (cudaStream_t)stream;
-    while ((int)b->side.size() < n_streams) {
-        cudaStream_t t = nullptr;
-        CK_FREE(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking), "bvf_batch_run_streams");
-        b->side.push_back(t);
-        cudaEvent_t ev = nullptr;
-        CK_FREE(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "bvf_batch_run_streams");
-        b->side_ev.push_back(ev);
-    }
-    if (!b->fork) CK_FREE(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "bvf_batch_run_streams");
+    const int made = batch_side_streams(b, n_streams);
+    if (made != BVF_OK) return made;
     // fork: every side stream waits for the caller's stream
     CK_FREE(cudaEventRecord(b->fork, s), "bvf_batch_run_streams");
     for (int k = 0; k < n_streams; ++k)
@@ -1807,21 +1819,6 @@ int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *c
         CK_FREE(cudaEventRecord(b->side_ev[k], b->side[k]), "bvf_batch_run_streams");
         CK_FREE(cudaStreamWaitEvent(s, b->side_ev[k], 0), "bvf_batch_run_streams");
     }
-    return BVF_OK;
-}
-
-// side streams and events of the batch, at least n of each
-static int batch_side_streams(bvf_batch *b, int n)
-{
-    while ((int)b->side.size() < n) {
-        cudaStream_t t = nullptr;
-        CK_FREE(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking), "batch streams");
-        b->side.push_back(t);
-        cudaEvent_t ev = nullptr;
-        CK_FREE(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "batch streams");
-        b->side_ev.push_back(ev);
-    }
-    if (!b->fork) CK_FREE(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "batch streams");
     return BVF_OK;
 }
 

@@ -1,15 +1,33 @@
-"""A device allocation that fails leaves a context that can go on: the call
-that needed it returns BVF_E_NOMEM, and the same call made again allocates
-what is missing and does all of its work, for every allocation of every call
-that makes buffers on first use."""
+"""A device allocation, stream or event that cannot be made leaves a context
+that can go on: the call that needed it returns an error, and the same call
+made again makes what is missing and does all of its work, for every one of
+those that a call makes on first use."""
 from tests import host_cuda
 
-ACOUSTIC = r"""
+COMMON = r"""
 NX, NY, NZ = 32, 16, 16
 N = NX * NY * NZ
 cap = bvf.Capture(0, 1, 4)
 th = bvf.Thermal(1e-3, 3, 2, 0.3, 37.0, 2.2e6, 1.0)
-calls = {}
+
+def plan_host(c):
+    water = context(NX, NY, NZ, [WATER])
+    bowl = bvf.Bowl(8e-3, 9e-3, (ctypes.c_double * 3)(8e-3, 4e-3, -2e-2),
+                    (ctypes.c_double * 3)(0, 0, 1), 1e5, 1500.0, 0.25)
+    pp = bvf.PlanParams(4, 1, 3, 0.0, th, 0)
+    out = bvf.PlanOut()
+    h = [buf(N), buf(4 * N), buf(4 * N), buf(4 * N), buf(8 * N)]
+    mat = bvf.material_array([WATER])
+    # without kernels the water field is zero, which the plan refuses at its
+    # end: the work up to there is what counts
+    def call():
+        rc = L.bvf_plan_host(c, water, h[0], mat, 1, mat, ctypes.byref(bowl), 2, ctypes.byref(pp),
+                             h[1], h[2], h[3], h[4], ctypes.byref(out), None)
+        return OK if rc == ARG and b"zero water intensity" in L.bvf_last_error(None) else rc
+    return call
+"""
+
+ACOUSTIC = COMMON + r"""
 
 def dft(c):
     return lambda: L.bvf_run_acoustic(c, 2, ctypes.byref(cap), None)
@@ -27,22 +45,6 @@ def load(c):
     snap = buf(n.value)
     assert L.bvf_state_save(full, snap, n, None) == OK
     return lambda: L.bvf_state_load(c, snap, n, None)
-
-def plan_host(c):
-    water = context(NX, NY, NZ, [WATER])
-    bowl = bvf.Bowl(8e-3, 9e-3, (ctypes.c_double * 3)(8e-3, 4e-3, -2e-2),
-                    (ctypes.c_double * 3)(0, 0, 1), 1e5, 1500.0, 0.25)
-    pp = bvf.PlanParams(4, 1, 3, 0.0, th, 0)
-    out = bvf.PlanOut()
-    h = [buf(N), buf(4 * N), buf(4 * N), buf(4 * N), buf(8 * N)]
-    mat = bvf.material_array([WATER])
-    # without kernels the water field is zero, which the plan refuses at its
-    # end: the work up to there is what counts
-    def call():
-        rc = L.bvf_plan_host(c, water, h[0], mat, 1, mat, ctypes.byref(bowl), 2, ctypes.byref(pp),
-                             h[1], h[2], h[3], h[4], ctypes.byref(out), None)
-        return OK if rc == ARG and b"zero water intensity" in L.bvf_last_error(None) else rc
-    return call
 
 for make in (dft, thermal, load, plan_host):
     # what the call launches and allocates with nothing failing
@@ -124,3 +126,37 @@ for k in (1, 5, 20):
 
 def test_surrogate_after_a_failed_grid_change(tmp_path):
     host_cuda.run(SURROGATE, tmp_path)
+
+
+STREAMS = COMMON + r"""
+def batch(run):
+    def make(c):
+        b = ctypes.c_void_p()
+        ctxs = (ctypes.c_void_p * 2)(c, context(NX, NY, NZ, [WATER]))
+        steps = (ctypes.c_int * 2)(2, 2)
+        assert L.bvf_batch_create(ctxs, 2, ctypes.byref(b)) == OK
+        return lambda: run(b, steps, None, 3, None)
+    return make
+
+for make, objects in ((plan_host, 3), (batch(L.bvf_batch_run_streams), 7), (batch(L.bvf_batch_run_graph), 7)):
+    c = context(NX, NY, NZ, [WATER])
+    call = make(c)
+    launched()
+    assert call() == OK
+    want = launched()
+    for k in range(1, objects + 1):
+        c = context(NX, NY, NZ, [WATER])
+        call = make(c)
+        fake.fake_fail_object(k)
+        assert call() == bvf.BVF_E_CUDA, (objects, k)
+        launched()
+        assert call() == OK, (objects, k, L.bvf_last_error(None))
+        assert launched() == want, (objects, k)
+        fake.fake_fail_object(1)
+        assert call() == OK          # nothing left to make
+        fake.fake_fail_object(0)
+"""
+
+
+def test_calls_after_a_stream_or_event_that_could_not_be_made(tmp_path):
+    host_cuda.run(STREAMS, tmp_path)
