@@ -803,12 +803,15 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     const bool pad = padded != g.nx && 4LL * padded <= 5LL * g.nx && c->L <= 2 &&
                      (double)padded * g.ny * g.nz < 2147483648.0 && tensor_map_encoder() &&
                      !std::getenv("BVF_NO_TMA") && !(st_env && st_env[0] == '0');
-    cudaError_t e = pad ? alloc_state(c, padded) : cudaErrorMemoryAllocation;
-    if (e != cudaSuccess || !c->tma) {
-        free_state(c);
-        (void)cudaGetLastError();
-        e = alloc_state(c, g.nx);
+    cudaError_t e = cudaSuccess;
+    bool ready = false;
+    if (pad) {
+        e = alloc_state(c, padded);
+        ready = e == cudaSuccess && c->tma;
+        if (!ready) free_state(c);
+        if (e != cudaSuccess) (void)cudaGetLastError();     // answered by dense rows
     }
+    if (!ready) e = alloc_state(c, g.nx);
     if (e != cudaSuccess) {
         const int rc = cuda_fail(nullptr, e, "bvf_create: buffers");
         bvf_destroy(c);
