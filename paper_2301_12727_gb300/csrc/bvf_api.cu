@@ -768,6 +768,15 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
         return fail(nullptr, BVF_E_ARG, "bvf_create: bad physics (f0, qc or n_sls)");
     if ((double)g.nx * g.ny * g.nz >= 2147483648.0)
         return fail(nullptr, BVF_E_ARG, "bvf_create: grid of 2^31 voxels or more");
+    // the kernels index the voxels and each axis' CPML memories with 32 bits
+    const int W = g.n_pml > 0 ? 2 * g.n_pml + 1 : 0;
+    auto fits32 = [&](int row) {
+        const double widest = std::max({(double)g.nz * g.ny, (double)g.nz * row, (double)g.ny * row});
+        return (double)row * g.ny * g.nz < 2147483648.0 &&
+               (double)kNumCpmlSlots * W * widest < 2147483648.0;
+    };
+    if (!fits32(g.nx))
+        return fail(nullptr, BVF_E_ARG, "bvf_create: CPML memories of 2^31 elements or more");
     if ((phys->storage != BVF_STORAGE_F32 && phys->storage != BVF_STORAGE_F16) ||
         !(phys->p_ref >= 0.0) || std::isinf(phys->p_ref))
         return fail(nullptr, BVF_E_ARG, "bvf_create: bad storage or p_ref");
@@ -789,7 +798,7 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
         c->s_r = c->s_v * zw / (8.0 * g.dt);
     }
     c->P = g.n_pml;
-    c->W = g.n_pml > 0 ? 2 * g.n_pml + 1 : 0;
+    c->W = W;
     c->nmax = std::max(g.nx, std::max(g.ny, g.nz));
     c->tau_sigma = relaxation_times(phys->f0, c->L);
     if (const char *kc = std::getenv("BVF_KCHUNK")) c->kchunk = std::max(0, std::atoi(kc));
@@ -801,7 +810,7 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     const int padded = (g.nx + 7) / 8 * 8;
     const char *st_env = std::getenv("BVF_STRESS_TMA");
     const bool pad = padded != g.nx && 4LL * padded <= 5LL * g.nx && c->L <= 2 &&
-                     (double)padded * g.ny * g.nz < 2147483648.0 && tensor_map_encoder() &&
+                     fits32(padded) && tensor_map_encoder() &&
                      !std::getenv("BVF_NO_TMA") && !(st_env && st_env[0] == '0');
     cudaError_t e = cudaSuccess;
     bool ready = false;

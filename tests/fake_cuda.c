@@ -7,9 +7,13 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/mman.h>
+
+/* allocations above this are address space only: never touched, never freed */
+#define FAKE_LARGE ((size_t)256 << 20)
 
 static int g_fail_malloc, g_fail_object;        /* the n-th from now fails (0: none) */
-static long long g_mallocs, g_instantiated, g_launches, g_last_error_calls;
+static long long g_mallocs, g_malloc_bytes, g_instantiated, g_launches, g_last_error_calls;
 static size_t g_free_mem = (size_t)200 << 30;
 static int g_pending;                           /* error cudaGetLastError would return */
 static int g_read_u32 = -1;                     /* value of 4-byte copies to the host */
@@ -25,6 +29,7 @@ void fake_set_pending(int e) { g_pending = e; }
 int fake_pending(void) { return g_pending; }
 void fake_read_u32(int v) { g_read_u32 = v; }
 long long fake_mallocs(void) { return g_mallocs; }
+long long fake_malloc_bytes(void) { return g_malloc_bytes; }
 long long fake_instantiated(void) { return g_instantiated; }
 long long fake_launches(void) { return g_launches; }
 /* "name smem" of every launch since the last clear, one a line */
@@ -62,18 +67,44 @@ static cudaError_t failed(int *countdown, cudaError_t e)
 }
 
 /* memory */
+static void *g_large[256];
+static int g_n_large;
+static int is_large(const void *p)
+{
+    int i;
+    for (i = 0; i < g_n_large; ++i)
+        if (g_large[i] == p) return 1;
+    return 0;
+}
 cudaError_t cudaMalloc(void **p, size_t n)
 {
     ++g_mallocs;
-    if (failed(&g_fail_malloc, cudaErrorMemoryAllocation) || !(*p = calloc(1, n ? n : 1)))
-        return cudaErrorMemoryAllocation;
+    if (failed(&g_fail_malloc, cudaErrorMemoryAllocation)) return cudaErrorMemoryAllocation;
+    if (n > FAKE_LARGE)
+        *p = mmap(0, n, PROT_NONE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+    else
+        *p = calloc(1, n ? n : 1);
+    if (!*p || *p == MAP_FAILED) return cudaErrorMemoryAllocation;
+    if (n > FAKE_LARGE) {
+        if (g_n_large == 256) abort();
+        g_large[g_n_large++] = *p;
+    }
+    g_malloc_bytes += n;
     return cudaSuccess;
 }
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t s) { (void)s; return cudaMalloc(p, n); }
-cudaError_t cudaFree(void *p) { free(p); return cudaSuccess; }
+cudaError_t cudaFree(void *p)
+{
+    if (!is_large(p)) free(p);
+    return cudaSuccess;
+}
 cudaError_t cudaFreeAsync(void *p, cudaStream_t s) { (void)s; return cudaFree(p); }
 cudaError_t cudaMemGetInfo(size_t *f, size_t *t) { *f = g_free_mem; *t = (size_t)280 << 30; return cudaSuccess; }
-cudaError_t cudaMemset(void *p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemset(void *p, int v, size_t n)
+{
+    if (!is_large(p)) memset(p, v, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t s) { (void)s; return cudaMemset(p, v, n); }
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, enum cudaMemcpyKind k)
 {

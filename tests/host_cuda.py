@@ -18,7 +18,7 @@ L = bvf.lib()
 fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
 fake.fake_log.restype = ctypes.c_char_p
 fake.fake_free_mem.argtypes = [ctypes.c_size_t]
-for f in ("fake_mallocs", "fake_instantiated", "fake_launches"):
+for f in ("fake_mallocs", "fake_malloc_bytes", "fake_instantiated", "fake_launches"):
     getattr(fake, f).restype = ctypes.c_longlong
 OK, ARG, NOMEM = bvf.BVF_OK, bvf.BVF_E_ARG, bvf.BVF_E_NOMEM
 WATER = [1000.0, 1500.0, 0.0, 0.0, 0.0, 0.6, 4178.0, 0.0, 1.0]

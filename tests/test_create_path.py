@@ -36,3 +36,33 @@ for k in range(1, n + 1):
 
 def test_dense_rows_where_padded_ones_cannot_be_had(tmp_path):
     host_cuda.run(FALLBACK, tmp_path)
+
+
+INDEX_RANGE = r"""
+# the memories of an axis (six slabs of 2 n_pml + 1 layers) are indexed with 32
+# bits: 6 * 39 * 48 * 200000 elements of padded rows are too many where the
+# 6 * 39 * 41 * 200000 of dense rows are not
+def made(*shape, **kw):
+    before = fake.fake_malloc_bytes()
+    rc, c = create(*shape, **kw)
+    if rc == OK:
+        L.bvf_destroy(c)
+    return rc, fake.fake_malloc_bytes() - before
+
+def state_bytes(pitch, ny, nz, W):      # fields and CPML memories, FP32, no SLS
+    return 4 * (9 * pitch * ny * nz + 6 * W * (nz * ny + nz * pitch + ny * pitch))
+
+for ny, pitch in ((190000, 48), (200000, 41)):
+    rc, n = made(41, ny, 40, n_sls=0, n_pml=19)
+    low = state_bytes(pitch, ny, 40, 39)
+    # the peak map, the index and its padded copy, tables, the CPML profile
+    assert rc == OK and low < n < low + (4 * pitch + 41 + 48) * ny * 40 + (2 << 20) + (8 * pitch + 48) * ny, ny
+# dense rows beyond the range are refused
+assert made(41, 230000, 40, n_sls=0, n_pml=19)[0] == ARG
+assert made(800, 800, 800, n_sls=0, n_pml=340)[0] == ARG
+assert made(700, 700, 700, n_sls=0, n_pml=300)[0] == OK
+"""
+
+
+def test_cpml_memories_stay_within_32_bits(tmp_path):
+    host_cuda.run(INDEX_RANGE, tmp_path)
