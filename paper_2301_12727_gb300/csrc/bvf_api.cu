@@ -650,6 +650,27 @@ cudaError_t copy_sections(const bvf_ctx *c, const StateSections &t, char *b, boo
 
 Rows rows_of(const bvf_ctx *c) { return Rows{(unsigned)c->g.nx, (unsigned)c->pitch}; }
 
+// free memory of the current device, 0 where it cannot be told
+double free_memory()
+{
+    size_t avail = 0, all = 0;
+    if (cudaMemGetInfo(&avail, &all) == cudaSuccess) return (double)avail;
+    (void)cudaGetLastError();
+    return 0.0;
+}
+
+// Device memory of a context whose rows have `pitch` elements, with all it may
+// come to hold (within a few MB): state, CPML memories, peak map, index copies,
+// DFT sums, thermal buffers, conduction classes and the staging of
+// bvf_plan_host.
+double full_bytes(const bvf_ctx *c, int pitch)
+{
+    const double yz = (double)c->g.ny * c->g.nz, np = pitch * yz, n = c->g.nx * yz;
+    const double psi = kNumCpmlSlots * (yz + (double)pitch * (c->g.ny + c->g.nz)) * c->W * sizeof(float);
+    const double own = ((9.0 + 6.0 * c->L) * c->es + sizeof(float) + 2 * sizeof(double)) * np + psi;
+    return own + 3 * n + (3 * sizeof(float) + 29) * n;
+}
+
 void free_state(bvf_ctx *c)
 {
     void **bufs[] = {&c->fields, (void **)&c->psi, (void **)&c->peak, (void **)&c->index,
@@ -804,14 +825,17 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     if (const char *kc = std::getenv("BVF_KCHUNK")) c->kchunk = std::max(0, std::atoi(kc));
     // Rows padded to a multiple of 8 let the TMA-fed kernels take any nx: the
     // direct kernels, which load every halo by hand, need 653 us a step at 197
-    // x 211 x 163 against 320.  Up to a quarter more memory (nx of about 29
-    // and up); without it (or where a switch keeps a kernel direct) rows stay
-    // dense.
+    // x 211 x 163 against 320.  They take up to a quarter more memory, so only
+    // where the GPU has room left for two such contexts (a plan's skull and
+    // water) with all that they may come to hold; elsewhere (or where a switch
+    // keeps a kernel direct) rows stay dense, and what fitted with dense rows
+    // fits.
     const int padded = (g.nx + 7) / 8 * 8;
     const char *st_env = std::getenv("BVF_STRESS_TMA");
     const bool pad = padded != g.nx && 4LL * padded <= 5LL * g.nx && c->L <= 2 &&
                      fits32(padded) && tensor_map_encoder() &&
-                     !std::getenv("BVF_NO_TMA") && !(st_env && st_env[0] == '0');
+                     !std::getenv("BVF_NO_TMA") && !(st_env && st_env[0] == '0') &&
+                     2.0 * full_bytes(c, padded) <= free_memory();
     cudaError_t e = cudaSuccess;
     bool ready = false;
     if (pad) {

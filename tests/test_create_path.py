@@ -66,3 +66,46 @@ assert made(700, 700, 700, n_sls=0, n_pml=300)[0] == OK
 
 def test_cpml_memories_stay_within_32_bits(tmp_path):
     host_cuda.run(INDEX_RANGE, tmp_path)
+
+
+ROOM = r"""
+# A context of dense rows, with its DFT sums, thermal buffers and the staging of
+# bvf_plan_host, against the memory there is.  Where padded rows would take a
+# quarter more than dense ones (nx = 13), a program whose two contexts just fit
+# with dense rows finds room for both, in the order create, create, use, use.
+nx, ny, nz = 13, 64, 60
+N = nx * ny * nz
+cap, th = bvf.Capture(0, 1, 4), bvf.Thermal(1e-3, 2, 1, 0.3, 37.0, 2.2e6, 1.0)
+
+def use(c):
+    materials(c, N, [WATER])
+    assert L.bvf_run_acoustic(c, 1, ctypes.byref(cap), None) == OK
+    assert L.bvf_run_thermal(c, ctypes.byref(th), buf(8 * N), buf(4 * N), buf(4 * N), buf(8 * N), None) == OK
+
+def two_contexts(free):
+    start, cs = fake.fake_malloc_bytes(), []
+    for _ in range(2):
+        fake.fake_free_mem(max(0, int(free - (fake.fake_malloc_bytes() - start))))
+        rc, c = create(nx, ny, nz)
+        assert rc == OK
+        cs.append(c)
+    launched()
+    for c in cs:
+        use(c)
+    taken = fake.fake_malloc_bytes() - start
+    padded = [n for n, _ in launched()].count("k_velocity_tma")
+    return taken, padded
+
+staging = 29 * N
+dense, none = two_contexts(1)
+assert none == 0
+exact = dense + 2 * staging                 # what two dense contexts come to hold
+for free in (exact, 1.02 * exact, 1.1 * exact, 1.2 * exact, 1.3 * exact, 2 * exact):
+    taken, padded = two_contexts(free)
+    assert taken + 2 * staging <= free, (free / exact, padded)
+assert padded == 2                          # room enough: both padded
+"""
+
+
+def test_padded_rows_leave_room_for_what_dense_rows_held(tmp_path):
+    host_cuda.run(ROOM, tmp_path)
