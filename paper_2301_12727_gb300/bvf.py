@@ -32,7 +32,8 @@ EXPORTS = ("bvf_version", "bvf_courant_limit", "bvf_strerror", "bvf_create", "bv
            "bvf_rs_elements", "bvf_set_time_budget", "bvf_state_bytes", "bvf_state_save",
            "bvf_state_load", "bvf_test_withhold_copy", "bvf_bowl_array", "bvf_steer_weights",
            "bvf_time_reversal_plane", "bvf_batch_run_graph", "bvf_batch_tune_domains",
-           "bvf_set_tile", "bvf_get_tile", "bvf_batch_tune_graph", "bvf_plan_host")
+           "bvf_set_tile", "bvf_get_tile", "bvf_batch_tune_graph", "bvf_plan_host",
+           "bvf_test_withhold_tma")
 
 
 class BvfError(RuntimeError):
@@ -178,6 +179,7 @@ def lib():
         L.bvf_state_save.argtypes = [vp, vp, ctypes.c_size_t, vp]
         L.bvf_state_load.argtypes = [vp, vp, ctypes.c_size_t, vp]
         L.bvf_test_withhold_copy.argtypes = [vp, i, i, ctypes.c_uint]
+        L.bvf_test_withhold_tma.argtypes = [vp, i, i, ctypes.c_uint]
         L.bvf_bowl_array.argtypes = [ctypes.POINTER(Bowl), i, i, vp, ctypes.POINTER(i)]
         L.bvf_steer_weights.argtypes = [vp, i, vp, d, d]
         L.bvf_time_reversal_plane.argtypes = [vp, i, i, i, i, i, d, vp, vp]
@@ -368,6 +370,10 @@ def bvf_state_load(ctx, buf, stream=None):
 
 def bvf_test_withhold_copy(ctx, kernel, plane, wait_limit=0):
     _check(lib().bvf_test_withhold_copy(ctx, kernel, plane, wait_limit), ctx)
+
+
+def bvf_test_withhold_tma(ctx, kernel, plane, wait_limit=0):
+    _check(lib().bvf_test_withhold_tma(ctx, kernel, plane, wait_limit), ctx)
 
 
 def bvf_bowl_array(bowl: Bowl, n_rings, n_inner) -> np.ndarray:

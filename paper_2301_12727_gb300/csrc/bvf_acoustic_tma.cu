@@ -215,6 +215,8 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
         tma::load3d(smb + Lay::off_i + slot * IT_SLOT, &tm.idx, x0, y0, pl, bar);
     };
 
+    // test hook: plane kk's copies are armed but not issued
+    auto held = [&](int kk) { return p.hold == 1 && kk == p.hold_plane + 1; };
     // the index does not change during a run, so its copies go out before the
     // wait for the previous kernel of the stream
     if (tid == 0) {
@@ -224,14 +226,16 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
         *s_abort = -1;
         if (REUSE) tma::fence_async_smem();
         tma::mbar_expect_tx(&bars[0], A_BYTES + 4 * B_BYTES + 4 * C_BYTES + 2 * IT);
-        ldI(k0, 0, &bars[0]);
-        ldI(k0 + 1, 1, &bars[0]);
+        if (!held(k0)) {
+            ldI(k0, 0, &bars[0]);
+            ldI(k0 + 1, 1, &bars[0]);
+        }
     }
     if (!REUSE) {
         tma::pdl_wait();
         tma::pdl_launch_next();
     }
-    if (tid == 0) {
+    if (tid == 0 && !held(k0)) {
         ldA(k0, 0, &bars[0]);
         for (int d = 0; d < 4; ++d) ldB(k0 - 2 + d, d, &bars[0]);
         for (int d = 0; d < 4; ++d) ldC(k0 - 1 + d, d, &bars[0]);
@@ -286,7 +290,7 @@ __device__ __forceinline__ bool velocity_tile(const AcParams &p, const VelocityT
                 tma::fence_async_smem();
                 uint64_t *bar = &bars[(u + 1) & 1];
                 tma::mbar_expect_tx(bar, A_BYTES + B_BYTES + C_BYTES + IT);
-                if (!(p.hold == 1 && k == p.hold_plane)) {
+                if (!held(k + 1)) {
                     ldA(k + 1, (u + 1) % Lay::RA, bar);
                     ldB(k + 2, (u + 4) % Lay::RB, bar);
                     ldC(k + 3, (u + 4) % Lay::RC, bar);
@@ -1305,9 +1309,8 @@ static cudaError_t raise_smem_once(K kernel, size_t bytes, std::atomic<int> &don
     return e;
 }
 
-// z-planes per block of a launch: the context's choice, else the rule's (with
-// the test hook armed at least 8, so that the plane it names has look-ahead
-// copies).  Beside other domains' kernels the SMs are full whatever one launch
+// z-planes per block of a launch: the context's choice, else the rule's.
+// Beside other domains' kernels the SMs are full whatever one launch
 // does, and long chunks cost the least in all: 16 domains of 96 to 200 cells
 // in one graph take 101.2 ms with the batch rule's 8 to 10 planes, 104.5 with
 // the chunks that are the fastest for a domain alone.
@@ -1315,7 +1318,7 @@ static int chunk_or(const AcParams &p, int th, int rule)
 {
     if (p.kchunk > 0) return p.kchunk;
     if (p.crowd) return default_kchunk_tma(p.nx, p.ny, p.nz, th);
-    return p.hold ? std::min(p.nz, std::max(8, rule)) : rule;
+    return rule;
 }
 
 template <typename T, int TH, bool PAD>

@@ -2158,17 +2158,24 @@ int bvf_set_time_budget(bvf_ctx *c, double seconds)
 
 int bvf_test_withhold_copy(bvf_ctx *c, int kernel, int plane, unsigned wait_limit)
 {
-    if (!c) return fail(nullptr, BVF_E_ARG, "bvf_test_withhold_copy: NULL context");
+    if (c && kernel != 0 && c->g.nx % 8 != 0)
+        return fail(c, BVF_E_ARG, "bvf_test_withhold_copy: nx is not a multiple of 8");
+    return bvf_test_withhold_tma(c, kernel, plane, wait_limit);
+}
+
+int bvf_test_withhold_tma(bvf_ctx *c, int kernel, int plane, unsigned wait_limit)
+{
+    if (!c) return fail(nullptr, BVF_E_ARG, "bvf_test_withhold: NULL context");
     if (kernel == 0) {
         c->hold = 0;
         return BVF_OK;
     }
     if ((kernel < 1 || kernel > 3) || plane < 0 || plane >= c->g.nz)
         return fail(c, BVF_E_ARG,
-                    "bvf_test_withhold_copy: kernel must be 1, 2 or 3, plane inside the grid");
-    if (c->g.nx % 8 != 0 || (kernel < 3 ? !(kernel == 1 ? c->tma : c->tma_stress)
-                                        : std::getenv("BVF_NO_TMA") != nullptr))
-        return fail(c, BVF_E_ARG, "bvf_test_withhold_copy: this context does not use the TMA-fed kernel");
+                    "bvf_test_withhold: kernel must be 1, 2 or 3, plane inside the grid");
+    if (kernel < 3 ? !(kernel == 1 ? c->tma : c->tma_stress)
+                   : c->g.nx % 8 != 0 || std::getenv("BVF_NO_TMA") != nullptr)
+        return fail(c, BVF_E_ARG, "bvf_test_withhold: this context does not use the TMA-fed kernel");
     c->hold = kernel;
     c->hold_plane = plane;
     c->hold_limit = wait_limit;

@@ -32,7 +32,7 @@ long long fake_mallocs(void) { return g_mallocs; }
 long long fake_malloc_bytes(void) { return g_malloc_bytes; }
 long long fake_instantiated(void) { return g_instantiated; }
 long long fake_launches(void) { return g_launches; }
-/* "name smem" of every launch since the last clear, one a line */
+/* "name grid-x grid-y grid-z smem" of every launch since the last clear, one a line */
 const char *fake_log(void) { return g_log ? g_log : ""; }
 void fake_log_clear(void)
 {
@@ -40,14 +40,14 @@ void fake_log_clear(void)
     if (g_log) g_log[0] = 0;
 }
 
-static void launched(const void *fun, size_t smem)
+static void launched(const void *fun, struct dim3 g, size_t smem)
 {
     const char *name = "?";
-    char line[320];
+    char line[400];
     int i, n;
     for (i = 0; i < g_n_fun; ++i)
         if (g_fun[i].fun == fun) name = g_fun[i].name;
-    n = snprintf(line, sizeof line, "%s %zu\n", name, smem);
+    n = snprintf(line, sizeof line, "%s %u %u %u %zu\n", name, g.x, g.y, g.z, smem);
     if (g_log_len + n + 1 > g_log_cap) {
         g_log_cap = 2 * (g_log_len + n + 1);
         g_log = realloc(g_log, g_log_cap);
@@ -229,7 +229,7 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
     return cudaSuccess;
 }
 /* as the runtime: more than 48 KB only up to the kernel's own limit */
-static cudaError_t launch(const void *fun, size_t smem)
+static cudaError_t launch(const void *fun, struct dim3 g, size_t smem)
 {
     int i, lim = 48 * 1024;
     for (i = 0; i < g_n_smem; ++i)
@@ -238,19 +238,19 @@ static cudaError_t launch(const void *fun, size_t smem)
         g_pending = cudaErrorInvalidValue;
         return cudaErrorInvalidValue;
     }
-    launched(fun, smem);
+    launched(fun, g, smem);
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **a)
 {
     (void)a;
-    return launch(f, c->dynamicSmemBytes);
+    return launch(f, c->gridDim, c->dynamicSmemBytes);
 }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, struct dim3 g, struct dim3 b, void **a, size_t sm, cudaStream_t s)
 {
-    (void)g; (void)b; (void)a; (void)s;
-    return launch((const void *)k, sm);
+    (void)b; (void)a; (void)s;
+    return launch((const void *)k, g, sm);
 }
 static struct dim3 c_grid, c_block;
 static size_t c_smem;

@@ -47,11 +47,15 @@ def materials(c, n, table):
     rc = L.bvf_set_materials(c, buf(n), bvf.material_array(list(table)), len(table))
     assert rc == OK, L.bvf_last_error(c)
 
-def launched():
-    # (kernel name, dynamic shared memory) of every launch since the last call
-    rows = [r.rsplit(" ", 1) for r in fake.fake_log().decode().splitlines()]
+def launches():
+    # (kernel name, grid, dynamic shared memory) of every launch since the last call
+    rows = [r.rsplit(" ", 4) for r in fake.fake_log().decode().splitlines()]
     fake.fake_log_clear()
-    return [(re.search("k_[a-z0-9_]+", n).group(), int(s)) for n, s in rows]
+    return [(re.search("k_[a-z0-9_]+", n).group(), (int(x), int(y), int(z)), int(s))
+            for n, x, y, z, s in rows]
+
+def launched():
+    return [(n, s) for n, _, s in launches()]
 """
 
 
