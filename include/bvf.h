@@ -550,8 +550,11 @@ int bvf_batch_run_graph(bvf_batch *b, const int *n_steps, const bvf_capture *cap
  * height other than 0 or 8 are skipped for contexts without two SLS
  * mechanisms), keeps the fastest in the context (as bvf_set_tile; used by
  * bvf_run_acoustic and the run modes above) and writes it to h_best[d] (may
- * be NULL).  Leaves every context reset (bvf_reset).  Errors: BVF_E_ARG (a
- * height other than 0, 4, 8, 16 or a negative z-chunk). */
+ * be NULL).  Each domain is timed alone, so a z-chunk of 0 is the rule for a
+ * domain alone here, while the streams and graph modes then run it with the
+ * rule for domains side by side; bvf_batch_tune_graph times those.  Leaves
+ * every context reset (bvf_reset).  Errors: BVF_E_ARG (a height other than 0,
+ * 4, 8, 16 or a negative z-chunk). */
 int bvf_batch_tune_domains(bvf_batch *b, int trial_steps, const bvf_tile *candidates,
                            int n_candidates, bvf_tile *h_best, void *stream);
 

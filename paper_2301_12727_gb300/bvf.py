@@ -95,9 +95,12 @@ class Tile(ctypes.Structure):
                 ("kchunk", ctypes.c_int)]
 
 
-# candidates of the per-domain tile autotuner: (stress rows, velocity rows, z-planes per block)
+# candidates of the tile autotuners: (stress rows, velocity rows, z-planes per
+# block); 0 planes is each kernel's own rule, the fastest on most grids and, with
+# the default rows, what a context without tuning runs: the first candidate, so
+# that another has to be faster to replace it
 TILE_CANDIDATES = tuple((s, v, k) for s, v in ((8, 16), (8, 8), (16, 16))
-                        for k in (6, 8, 10, 13, 16))
+                        for k in (0, 6, 8, 10, 13, 16))
 
 
 class Stats(ctypes.Structure):
