@@ -825,11 +825,11 @@ int bvf_create(const bvf_grid *grid, const bvf_physics *phys, bvf_ctx **out)
     if (const char *kc = std::getenv("BVF_KCHUNK")) c->kchunk = std::max(0, std::atoi(kc));
     // Rows padded to a multiple of 8 let the TMA-fed kernels take any nx: the
     // direct kernels, which load every halo by hand, need 653 us a step at 197
-    // x 211 x 163 against 320.  They take up to a quarter more memory, so only
-    // where the GPU has room left for two such contexts (a plan's skull and
-    // water) with all that they may come to hold; elsewhere (or where a switch
-    // keeps a kernel direct) rows stay dense, and what fitted with dense rows
-    // fits.
+    // x 211 x 163 against 320.  Up to a quarter more elements (nx of 7, 13 to
+    // 15, 20 to 23, and every width from 26 on), and only where the GPU has room
+    // left for two such contexts (a plan's skull and water) with all that they
+    // may come to hold; elsewhere (or where a switch keeps a kernel direct)
+    // rows stay dense, and what fitted with dense rows fits.
     const int padded = (g.nx + 7) / 8 * 8;
     const char *st_env = std::getenv("BVF_STRESS_TMA");
     const bool pad = padded != g.nx && 4LL * padded <= 5LL * g.nx && c->L <= 2 &&
