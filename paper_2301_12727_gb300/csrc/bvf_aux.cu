@@ -3,7 +3,9 @@
 // and the E_L reductions (Sec. 2.4, Eq. 2).
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "bvf_stencil.cuh"
 #include "bvf_tma.cuh"
@@ -104,16 +106,70 @@ __global__ void k_amp_phase(const double *__restrict__ C, const double *__restri
 // multiplied by w_e = wr + i wi.
 //
 // The sum runs in tiles of 256 elements, FP32 within a tile and FP64 over the
-// tiles in their order.  A block of 32 points x 8 threads takes 8 tiles at a
-// time, one per thread of a point, and the first thread of the point adds the
-// 8 partial sums in order, so the result does not depend on the split.  The
-// sum is bound by its instructions (square root, sincospi and division of
-// every pair): one thread per point gave 225 blocks on 152 SMs at 240 x 240
-// points, half the SMs with one block of 8 warps, and 976 us; this takes
-// 650 us.  The elements (98 KB there) come from the L1, the same address for a
-// point's whole warp.
+// tiles in their order, in one of two ways with the same bits (see rs_split):
+//   k_rs_point  a thread per point, 256 points a block, the tile in shared
+//               memory;
+//   k_rs        a block of 32 points x 8 threads takes 8 tiles at a time, one
+//               per thread of a point, the elements (98 KB of 6150) from the L1
+//               at an address a point's whole warp shares, and the first thread
+//               of the point adds the 8 partial sums in order.
+// The sum is bound by its instructions (square root, sincospi and division of
+// every pair).  A thread per point gives 225 blocks on 152 SMs at 240 x 240
+// points, half the SMs with one block of 8 warps, and 976 us with 6150 elements;
+// eight take 650 us.
 constexpr int kRsTile = 256;             // elements per FP32 partial sum
 constexpr int kRsPts = 32, kRsGroups = 8;
+
+// one element's term added to a partial sum; weight() is its complex weight
+template <bool WT, class Weight>
+__device__ __forceinline__ void rs_add(float4 E, Weight weight, float x, float y, float zp,
+                                       float k_over_pi, float &pre, float &pim)
+{
+    const float ddx = x - E.x, ddy = y - E.y, ddz = zp - E.z;
+    const float r = sqrtf(fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz)));
+    float sn, cs;
+    sincospif(k_over_pi * r, &sn, &cs);
+    const float w = E.w / r;
+    if (WT) {                            // (wr + i wi)(sin kr + i cos kr)
+        const float2 W = weight();
+        pre = fmaf(w, fmaf(W.x, sn, -W.y * cs), pre);
+        pim = fmaf(w, fmaf(W.x, cs, W.y * sn), pim);
+    } else {
+        pre = fmaf(w, sn, pre);
+        pim = fmaf(w, cs, pim);
+    }
+}
+
+template <bool WT>
+__global__ void __launch_bounds__(kRsTile)
+    k_rs_point(const float4 *__restrict__ el, const float2 *__restrict__ wt, int ne, int nx, int ny,
+               float dx, float zp, float k_over_pi, double pref, float2 *__restrict__ out)
+{
+    __shared__ float4 s_el[kRsTile];
+    __shared__ float2 s_wt[WT ? kRsTile : 1];
+    const int q = blockIdx.x * kRsTile + threadIdx.x;
+    const bool live = q < nx * ny;
+    const float x = live ? (q % nx) * dx : 0.0f;
+    const float y = live ? (q / nx) * dx : 0.0f;
+    double re = 0.0, im = 0.0;
+    for (int base = 0; base < ne; base += kRsTile) {
+        if (base + (int)threadIdx.x < ne) {
+            s_el[threadIdx.x] = el[base + threadIdx.x];
+            if (WT) s_wt[threadIdx.x] = wt[base + threadIdx.x];
+        }
+        __syncthreads();
+        const int n = min(kRsTile, ne - base);
+        float pre = 0.0f, pim = 0.0f;
+        for (int e = 0; e < n; ++e) {
+            const float2 W = s_wt[WT ? e : 0];
+            rs_add<WT>(s_el[e], [&] { return W; }, x, y, zp, k_over_pi, pre, pim);
+        }
+        re += pre;
+        im += pim;
+        __syncthreads();
+    }
+    if (live) out[q] = make_float2((float)(pref * re), (float)(pref * im));
+}
 
 template <bool WT>
 __global__ void __launch_bounds__(kRsPts *kRsGroups)
@@ -131,22 +187,8 @@ __global__ void __launch_bounds__(kRsPts *kRsGroups)
         const int e0 = base + g * kRsTile, e1 = min(ne, e0 + kRsTile);
         float pre = 0.0f, pim = 0.0f;
 #pragma unroll 4
-        for (int e = e0; e < e1; ++e) {
-            const float4 E = __ldg(el + e);
-            const float ddx = x - E.x, ddy = y - E.y, ddz = zp - E.z;
-            const float r = sqrtf(fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz)));
-            float sn, cs;
-            sincospif(k_over_pi * r, &sn, &cs);
-            const float w = E.w / r;
-            if (WT) {                    // (wr + i wi)(sin kr + i cos kr)
-                const float2 W = __ldg(wt + e);
-                pre = fmaf(w, fmaf(W.x, sn, -W.y * cs), pre);
-                pim = fmaf(w, fmaf(W.x, cs, W.y * sn), pim);
-            } else {
-                pre = fmaf(w, sn, pre);
-                pim = fmaf(w, cs, pim);
-            }
-        }
+        for (int e = e0; e < e1; ++e)
+            rs_add<WT>(__ldg(el + e), [&] { return __ldg(wt + e); }, x, y, zp, k_over_pi, pre, pim);
         s_part[g][pt] = make_float2(pre, pim);
         __syncthreads();
         if (g == 0)
@@ -724,21 +766,56 @@ cudaError_t launch_amp_phase(const double *C, const double *S, size_t n, Rows r,
     return cudaGetLastError();
 }
 
+// Whether eight threads share a point: where that is estimated to be the faster
+// way.  The estimates (us, with b blocks per SM) are fits to both kernels' times
+// at 459 sizes, 32^2 to 2048^2 points and 256 to 4200 elements; the kernel they
+// pick is at most 3 % slower than the other.  Few elements leave most of the
+// eight threads idle (256 elements at 512 x 512 points: 324 us, 135 with a
+// thread per point), and many on a small plane leave a thread per point to a
+// serial chain (1024 at 64 x 64: 139 us, 62 with eight).  From about 900 x 900
+// points on the two are within 3 % of each other for any number of elements
+// above 1500.
+static bool rs_split(int points, int ne, bool weighted)
+{
+    constexpr int n_sm = 152;
+    // a thread per point: an element's latency, or the SM's share of its issue
+    const int blocks = (points + kRsTile - 1) / kRsTile, b1 = (blocks + n_sm - 1) / n_sm;
+    const double t_point = ne * std::max(0.137, 0.070 * b1 + 0.035);
+    // eight threads: the chain of a tile, and the issue of all of them
+    const double b8 = points / (double)(kRsPts * n_sm);
+    const double tile = b8 <= 6.6 ? (weighted ? 59.0 : 51.5)
+                                  : std::max(90.0, (weighted ? 46.0 : 40.0) + 4.5 * b8);
+    const int round = kRsTile * kRsGroups, rest = ne % round;
+    const double chain = tile * (ne / round + std::min(kRsTile, rest) / (double)kRsTile);
+    const double issue = (weighted ? 0.0088 : 0.0085) * b8 * ne;
+    return std::pow(std::pow(chain, 2.5) + std::pow(issue, 2.5), 0.4) < t_point;
+}
+
+template <bool WT>
+static cudaError_t launch_rs_t(const float4 *el, const float2 *wt, int ne, int nx, int ny, float dx,
+                               float zp, float k_over_pi, double pref, float2 *out, cudaStream_t s)
+{
+    const int n = nx * ny;
+    if (rs_split(n, ne, WT))
+        k_rs<WT><<<(n + kRsPts - 1) / kRsPts, dim3(kRsPts, kRsGroups), 0, s>>>(
+            el, wt, ne, nx, ny, dx, zp, k_over_pi, pref, out);
+    else
+        k_rs_point<WT><<<(n + kRsTile - 1) / kRsTile, kRsTile, 0, s>>>(el, wt, ne, nx, ny, dx, zp,
+                                                                       k_over_pi, pref, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_rs(const float4 *el, int ne, int nx, int ny, float dx, float zp, float k_over_pi,
                       double pref, float2 *out, cudaStream_t s)
 {
-    k_rs<false><<<(nx * ny + kRsPts - 1) / kRsPts, dim3(kRsPts, kRsGroups), 0, s>>>(
-        el, nullptr, ne, nx, ny, dx, zp, k_over_pi, pref, out);
-    return cudaGetLastError();
+    return launch_rs_t<false>(el, nullptr, ne, nx, ny, dx, zp, k_over_pi, pref, out, s);
 }
 
 cudaError_t launch_rs_weighted(const float4 *el, const float2 *wt, int ne, int nx, int ny,
                                float dx, float zp, float k_over_pi, double pref, float2 *out,
                                cudaStream_t s)
 {
-    k_rs<true><<<(nx * ny + kRsPts - 1) / kRsPts, dim3(kRsPts, kRsGroups), 0, s>>>(
-        el, wt, ne, nx, ny, dx, zp, k_over_pi, pref, out);
-    return cudaGetLastError();
+    return launch_rs_t<true>(el, wt, ne, nx, ny, dx, zp, k_over_pi, pref, out, s);
 }
 
 cudaError_t launch_classes(const uint8_t *idx, const uint8_t *cls, uint8_t *out, size_t n, Rows r,
