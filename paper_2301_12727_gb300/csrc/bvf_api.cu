@@ -594,58 +594,68 @@ StateSections state_sections(const bvf_ctx *c)
 }
 
 // rows of nx elements of `es` bytes between an array of the context (rows
-// pitch apart) and a dense one
-cudaError_t copy_rows(const bvf_ctx *c, void *dense, void *own, size_t rows, size_t es, bool out,
+// pitch apart) and a dense one with `tail` elements more, which become zero
+void add_rows(const bvf_ctx *c, RowSegs &q, void *dense, void *own, size_t rows, size_t es, bool out,
+              size_t tail = 0)
+{
+    const size_t nx = c->g.nx, pitch = c->pitch;
+    if (out)
+        q.add(dense, nx, own, pitch, nx, rows, es, tail);
+    else
+        q.add(own, pitch, dense, nx, nx, rows, es);
+}
+cudaError_t copy_rows(bvf_ctx *c, void *dense, void *own, size_t rows, size_t es, bool out,
                       cudaStream_t s)
 {
-    const size_t w = (size_t)c->g.nx * es, p = (size_t)c->pitch * es;
-    if (w == p)
-        return cudaMemcpyAsync(out ? dense : own, out ? own : dense, rows * w,
+    if (c->pitch == c->g.nx)
+        return cudaMemcpyAsync(out ? dense : own, out ? own : dense, rows * c->g.nx * es,
                                cudaMemcpyDeviceToDevice, s);
-    return out ? cudaMemcpy2DAsync(dense, w, own, p, w, rows, cudaMemcpyDeviceToDevice, s)
-               : cudaMemcpy2DAsync(own, p, dense, w, w, rows, cudaMemcpyDeviceToDevice, s);
+    RowSegs q;
+    add_rows(c, q, dense, own, rows, es, out);
+    c->launches++;
+    return launch_copy_rows(q, s);
 }
 
 // the snapshot's arrays between the context and the buffer at b
-cudaError_t copy_sections(const bvf_ctx *c, const StateSections &t, char *b, bool out,
-                          cudaStream_t s)
+cudaError_t copy_sections(bvf_ctx *c, const StateSections &t, char *b, bool out, cudaStream_t s)
 {
-    const size_t rows = (size_t)c->g.ny * c->g.nz, lf = (c->N + 63) & ~(size_t)63;
-    char *f = static_cast<char *>(c->fields);
+    const size_t rows = (size_t)c->g.ny * c->g.nz, L = c->L;
+    char *f = static_cast<char *>(c->fields), *psi = reinterpret_cast<char *>(c->psi);
+    auto whole = [&](char *snap, void *own, size_t bytes) {
+        return cudaMemcpyAsync(out ? (void *)snap : own, out ? own : (void *)snap, bytes,
+                               cudaMemcpyDeviceToDevice, s);
+    };
     cudaError_t e = cudaSuccess;
     if (c->pitch == c->g.nx) {
-        e = cudaMemcpyAsync(out ? b + t.off_fields : f, out ? f : b + t.off_fields, t.fields,
-                            cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess && t.psi)
-            e = cudaMemcpyAsync(out ? b + t.off_psi : (char *)c->psi,
-                                out ? (char *)c->psi : b + t.off_psi, t.psi,
-                                cudaMemcpyDeviceToDevice, s);
-    } else {
-        if (out) e = cudaMemsetAsync(b + t.off_fields, 0, t.fields, s);
-        // 9 arrays of rows of nx elements, then 6 of rows of nx L (the
-        // mechanisms of a voxel are adjacent)
-        for (int a = 0; a < 15 && e == cudaSuccess; ++a) {
-            const size_t L = c->L, n = a < 9 ? (size_t)a : 9 + (size_t)(a - 9) * L;
-            const size_t es = c->es * (a < 9 ? 1 : L);
-            if (es)
-                e = copy_rows(c, b + t.off_fields + n * lf * c->es, f + n * c->fstride * c->es, rows,
-                              es, out, s);
-        }
-        if (e == cudaSuccess && t.psi) {
-            char *d = b + t.off_psi, *own = reinterpret_cast<char *>(c->psi);
-            const size_t bx = kNumCpmlSlots * c->slab_x * sizeof(float);
-            e = cudaMemcpyAsync(out ? d : own, out ? own : d, bx, cudaMemcpyDeviceToDevice, s);
-            if (e == cudaSuccess)
-                e = copy_rows(c, d + bx, own + bx, (size_t)kNumCpmlSlots * c->W * (c->g.nz + c->g.ny),
-                              sizeof(float), out, s);
-        }
+        e = whole(b + t.off_fields, f, t.fields);
+        if (e == cudaSuccess && t.psi) e = whole(b + t.off_psi, psi, t.psi);
+        if (e == cudaSuccess) e = whole(b + t.off_peak, c->peak, t.peak);
+        if (e == cudaSuccess && c->dftC) e = whole(b + t.off_C, c->dftC, t.dft);
+        if (e == cudaSuccess && c->dftC) e = whole(b + t.off_S, c->dftS, t.dft);
+        return e;
     }
-    if (e == cudaSuccess) e = copy_rows(c, b + t.off_peak, c->peak, rows, sizeof(float), out, s);
+    // padded rows: 9 arrays of nx elements a row, 6 of nx L (the mechanisms of a
+    // voxel are adjacent), each up to a multiple of 64 elements in the snapshot
+    RowSegs q;
+    const size_t lf = (c->N + 63) & ~(size_t)63;
+    for (size_t a = 0; a < (L ? 15 : 9); ++a) {
+        const size_t k = a < 9 ? 1 : L, n = a < 9 ? a : 9 + (a - 9) * L;
+        add_rows(c, q, b + t.off_fields + n * lf * c->es, f + n * c->fstride * c->es, rows, c->es * k, out,
+                 lf - c->N);
+    }
+    if (t.psi) {
+        const size_t bx = kNumCpmlSlots * c->slab_x * sizeof(float);      // no padded rows
+        e = whole(b + t.off_psi, psi, bx);
+        add_rows(c, q, b + t.off_psi + bx, psi + bx, (size_t)kNumCpmlSlots * c->W * (c->g.nz + c->g.ny),
+                 sizeof(float), out);
+    }
+    add_rows(c, q, b + t.off_peak, c->peak, rows, sizeof(float), out);
     if (c->dftC) {
-        if (e == cudaSuccess) e = copy_rows(c, b + t.off_C, c->dftC, rows, sizeof(double), out, s);
-        if (e == cudaSuccess) e = copy_rows(c, b + t.off_S, c->dftS, rows, sizeof(double), out, s);
+        add_rows(c, q, b + t.off_C, c->dftC, rows, sizeof(double), out);
+        add_rows(c, q, b + t.off_S, c->dftS, rows, sizeof(double), out);
     }
-    return e;
+    c->launches++;
+    return e == cudaSuccess ? launch_copy_rows(q, s) : e;
 }
 
 Rows rows_of(const bvf_ctx *c) { return Rows{(unsigned)c->g.nx, (unsigned)c->pitch}; }
@@ -922,10 +932,12 @@ int bvf_set_materials(bvf_ctx *c, const uint8_t *d_index, const bvf_material *h_
                 pml[((size_t)ax * 2 + h) * c->nmax + s] = make_float2((float)a, (float)b);
             }
     CK(cudaMemcpy(c->index, d_index, c->N, cudaMemcpyDeviceToDevice), "copy index");
-    if (c->index_p)
-        CK(cudaMemcpy2D(c->index_p, c->index_pitch, c->index, c->g.nx, c->g.nx,
-                        (size_t)c->g.ny * c->g.nz, cudaMemcpyDeviceToDevice),
-           "copy padded index");
+    if (c->index_p) {
+        RowSegs q;
+        q.add(c->index_p, c->index_pitch, c->index, c->g.nx, c->g.nx, (size_t)c->g.ny * c->g.nz, 1);
+        CK(launch_copy_rows(q, 0), "copy padded index");
+        c->launches++;
+    }
     CK(cudaMemcpy(c->lut, lut.data(), n_mat * sizeof(MatCoef), cudaMemcpyHostToDevice), "copy lut");
     // buoyancy at a velocity point between cells of materials a and b: 2 / (rho_a + rho_b)
     std::vector<float> buoy((size_t)n_mat * n_mat);

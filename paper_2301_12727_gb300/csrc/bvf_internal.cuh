@@ -225,6 +225,23 @@ cudaError_t launch_velocity_tma(const AcParams &p, const VelocityTmaMaps &tm, cu
 cudaError_t launch_stress_tma(const AcParams &p, const StressTmaMaps &tm, cudaStream_t s);
 // st::StressCoef of each of n materials (slut: n * 32 bytes, 16-byte aligned)
 cudaError_t launch_stress_table(const MatCoef *lut, int n, float Lf, void *slut, cudaStream_t s);
+// copies of rows, pitches in units: w units of each row, then `tail` zeros
+// behind the last one
+struct RowSeg {
+    void *dst;
+    const void *src;
+    size_t dst_pitch, src_pitch, rows;
+    unsigned w, tail;
+    int unit;                // bytes: 1, 2, 4 or 8
+};
+struct RowSegs {
+    RowSeg s[20];
+    int n = 0;
+    // elements of es bytes (1, 2, 4 or 8), sizes and pitches in elements
+    void add(void *dst, size_t dst_pitch, const void *src, size_t src_pitch, size_t w, size_t rows,
+             size_t es, size_t tail = 0);
+};
+cudaError_t launch_copy_rows(const RowSegs &q, cudaStream_t s);
 cudaError_t launch_index_max(const uint8_t *idx, size_t n, unsigned *d_out, cudaStream_t s);
 // Read-outs of the context's arrays, whose rows of nx elements lie pitch apart,
 // into the caller's dense ones (launch_field_in: the other way).
