@@ -1310,7 +1310,7 @@ static cudaError_t raise_smem_once(K kernel, size_t bytes, std::atomic<int> &don
 }
 
 // z-planes per block of a launch: the context's choice, else the rule's.
-// Beside other domains' kernels the SMs are full whatever one launch
+// Where other domains fill the GPU the SMs are full whatever one launch
 // does, and long chunks cost the least in all: 16 domains of 96 to 200 cells
 // in one graph take 101.2 ms with the batch rule's 8 to 10 planes, 104.5 with
 // the chunks that are the fastest for a domain alone.

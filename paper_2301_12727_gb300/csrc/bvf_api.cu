@@ -88,7 +88,7 @@ struct bvf_ctx {
     long long steps = 0, launches = 0, thermal_steps = 0;
     double courant = 0.0;
     int kchunk = 0;                   // z-planes per block (0 = default)
-    bool crowd = false;               // enqueued beside other domains (batch calls)
+    bool crowd = false;               // enqueued beside domains that fill the GPU (batch calls)
     bvf_tile tile{0, 0, 0};           // tile of the TMA kernels (bvf_set_tile; 0 = default)
     bool tma = false;                 // velocity kernel fed by TMA
     bool tma_stress = false;          // stress kernel fed by TMA
@@ -1811,11 +1811,35 @@ int bvf_batch_run(bvf_batch *b, const int *n_steps, const bvf_capture *caps, int
     return BVF_OK;
 }
 
-// one domain's steps on `s`, beside the other domains' (crowd: see chunk_or)
-static int run_beside(bvf_batch *b, int d, int n_steps, const bvf_capture *caps, cudaStream_t s)
+// Whether domains dealt over `lanes` streams or graph branches fill the GPU with
+// the long z-chunks of the batch rule (see chunk_or), by the blocks of the
+// domains that run at a time.  Where the line lies differs: streams leave gaps
+// between launches that more blocks fill, and the paired FP16 tiles take half
+// the threads.  30 FP32 steps with long chunks and with those of a domain alone,
+// ms: graph 1.48 and 0.81 (2 of 64^3, 256 blocks), 2.09 and 2.02 (5 of 64^3,
+// 640), 2.35 and 2.44 (6 of 64^3, 768), 2.89 and 3.31 (8 of 64^3, 1024); streams
+// 3.15 and 2.98 (7 of 64^3, 896), 3.39 and 3.58 (4 of 80^3, 1200).  FP16: graph
+// 2.43 and 2.35 (896), 2.67 and 2.74 (1024); streams 3.79 and 3.60 (2 of 112^3,
+// 1568), 4.63 and 4.71 (2 of 128^3, 2048).
+static bool crowded(const bvf_batch *b, int lanes, bool graph)
+{
+    const int n = (int)b->ctx.size(), rounds = (n + lanes - 1) / lanes;
+    double blocks = 0.0;
+    for (const bvf_ctx *c : b->ctx) {
+        const bvf_grid &g = c->g;
+        const int kc = default_kchunk_tma(g.nx, g.ny, g.nz);
+        blocks += (double)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + kc - 1) / kc);
+    }
+    const double line = graph ? (b->h16 ? 1000.0 : 750.0) : (b->h16 ? 1800.0 : 912.0);
+    return n > 1 && blocks / rounds >= line;
+}
+
+// one domain's steps on `s`, beside the other domains'
+static int run_beside(bvf_batch *b, int d, int n_steps, const bvf_capture *caps, cudaStream_t s,
+                      bool crowd)
 {
     bvf_ctx *c = b->ctx[d];
-    c->crowd = b->ctx.size() > 1;
+    c->crowd = crowd;
     const int rc = bvf_run_acoustic(c, n_steps, caps ? &caps[d] : nullptr, s);
     c->crowd = false;
     return rc;
@@ -1858,7 +1882,7 @@ int bvf_batch_run_streams(bvf_batch *b, const int *n_steps, const bvf_capture *c
         CK_FREE(cudaStreamWaitEvent(b->side[k], b->fork, 0), "bvf_batch_run_streams");
     // domains dealt round-robin; each side stream runs its domains one after another
     for (int d = 0; d < n; ++d) {
-        const int rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_streams]);
+        const int rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_streams], crowded(b, n_streams, false));
         if (rc != BVF_OK) return rc;
         b->launches += 2LL * n_steps[d];
     }
@@ -1924,7 +1948,7 @@ int bvf_batch_run_graph(bvf_batch *b, const int *n_steps, const bvf_capture *cap
         for (int k = 0; k < n_branches && e == cudaSuccess; ++k)
             e = cudaStreamWaitEvent(b->side[k], b->fork, 0);
         for (int d = 0; d < n && e == cudaSuccess && rc == BVF_OK; ++d)
-            rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_branches]);
+            rc = run_beside(b, d, n_steps[d], caps, b->side[d % n_branches], crowded(b, n_branches, true));
         for (int k = 0; k < n_branches && e == cudaSuccess; ++k) {
             e = cudaEventRecord(b->side_ev[k], b->side[k]);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->side_ev[k], 0);

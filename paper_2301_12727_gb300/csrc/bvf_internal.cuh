@@ -108,7 +108,7 @@ struct AcParams {
     // rows of an x-y tile of the TMA-fed stress and velocity kernels: 4, 8 or
     // 16 (heights other than 8 with L = 2 only)
     int tile_y, tile_yv;
-    int crowd;           // other domains' kernels run beside this one (batched sweeps)
+    int crowd;           // domains that fill the GPU run beside this one (batched sweeps)
 };
 
 // Tensor maps of the TMA-fed acoustic kernels (x-y boxes of one z-plane).
