@@ -1109,7 +1109,8 @@ k_dftx_tc(const float *v, long R, int nx, int m, const float2 *__restrict__ tx, 
 // out[k][p] = q2[k] + sum_j Q2[k][j] GELU(q1[j] + sum_c Q1[j][c] v[c][p]) on
 // 128-point tiles: D[128 points][HP hidden] = A[128][W] B[W][HP] in TMEM, as
 // three TF32 products (A_lo B_hi + A_hi B_lo + A_hi B_hi) per K step of 8.
-// 128 threads: thread i owns point i of the tile (A staging and epilogue).
+// 256 threads: threads i and i + 128 share point i of the tile, half of its
+// channels to stage and half of its hidden columns in the epilogue each.
 struct ProjTcLayout {
     int HP, ncols, sAh, sAl, sBh, sBl, sq1, sq2, sred, bar, tmem, bytes;
     __host__ __device__ ProjTcLayout(int width, int hidden, int c_out)
@@ -1641,9 +1642,9 @@ int bvf_fno_forward(bvf_fno *f, int nx, int ny, int nz, const float *d_in, float
     const int rows_p = nz * ny;
     const float invN = (float)(1.0 / (double)N64);
     // the row pass: k_row_tc (layer output: inverse x transform, W v + b,
-    // GELU) and, when a further layer follows, k_dftx_tc (its forward x
-    // transform); grids whose rows do not fit shared memory take the unfused
-    // kernels
+    // GELU) and, when a further layer follows, its forward x transform (k_xfwd,
+    // or k_dftx_tc for rows TMA cannot fetch); grids whose rows do not fit shared
+    // memory take the unfused kernels
     const int kc_lift = ((d.c_in + 7) / 8) * 8;
     const int nb = 2 * m <= 16 ? 16 : 32;
     const DftxTcLayout dl(nb, nx);
